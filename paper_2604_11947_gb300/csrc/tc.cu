@@ -1065,6 +1065,36 @@ MatrixWs matrix_ws(int op, int64_t rows, int64_t cols, int sms, void *ws)
 }
 }  // namespace
 
+namespace {
+template <int SDP, typename TG>
+cudaError_t launch_ns_t(int64_t rows, int64_t cols, const void *G, int steps, const float coef[3], float eps, void *out,
+                        const Ctx &c)
+{
+    static std::atomic<uint8_t> smem_set[kMaxDev];
+    cudaError_t e = ensure_smem(tc::k_newton_schulz<SDP, TG>, tc::kNsMaxSmem, c.device, smem_set);
+    if (e != cudaSuccess) return e;
+    const bool tall = rows > cols;
+    const int64_t sd = tall ? cols : rows, ld = tall ? rows : cols;
+    const tc::NsLayout l = tc::ns_layout(SDP, ld);
+    e = launch_clustered(tc::k_newton_schulz<SDP, TG>, l.cl, tc::kNsThreads, l.bytes, l.cl, c.stream,
+                         static_cast<const TG *>(G), (int)sd, ld, tall ? 1 : 0, steps, coef[0], coef[1], coef[2], eps,
+                         static_cast<__nv_bfloat16 *>(out));
+    count_launches(1);
+    return e;
+}
+template <typename TG>
+cudaError_t launch_ns(int64_t rows, int64_t cols, const void *G, int steps, const float coef[3], float eps, void *out,
+                      const Ctx &c)
+{
+    switch (tc::ns_sdp(rows < cols ? rows : cols)) {
+    case 16: return launch_ns_t<16, TG>(rows, cols, G, steps, coef, eps, out, c);
+    case 32: return launch_ns_t<32, TG>(rows, cols, G, steps, coef, eps, out, c);
+    case 48: return launch_ns_t<48, TG>(rows, cols, G, steps, coef, eps, out, c);
+    default: return launch_ns_t<64, TG>(rows, cols, G, steps, coef, eps, out, c);
+    }
+}
+}  // namespace
+
 size_t matrix_ws_bytes(int op, int64_t rows, int64_t cols, int sms) { return matrix_ws(op, rows, cols, sms, nullptr).bytes; }
 
 bool matrix_supported(int64_t rows, int64_t cols)
@@ -1076,6 +1106,10 @@ cudaError_t tc_newton_schulz(int64_t rows, int64_t cols, const void *G, bool g_f
                              float eps, void *X_out, void *ws, const Ctx &c)
 {
     if (!al16(G) || !al16(X_out) || !al16(ws) || encode_fn() == nullptr) return cudaErrorNotSupported;
+    // a small side of up to 64 whose columns fit in a cluster's shared memory: one launch
+    if (tc::ns_fused_ok(rows, cols))
+        return g_f32 ? launch_ns<float>(rows, cols, G, steps, coef, eps, X_out, c)
+                     : launch_ns<__nv_bfloat16>(rows, cols, G, steps, coef, eps, X_out, c);
     const MatrixWs w = matrix_ws(RESBM_OP_NEWTON_SCHULZ, rows, cols, c.sm_count, ws);
     const int64_t n = rows * cols;
     __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(X_out);

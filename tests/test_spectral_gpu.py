@@ -92,3 +92,29 @@ def test_effective_rank_of_structured_matrices():
     Wq = torch.from_numpy(Q).to("cuda").to(torch.bfloat16)
     r = _reff(Wq)[2]
     assert abs(r - oracle.effective_rank(Wq.double().cpu().numpy())) <= 1e-4 * r and abs(r - 64) < 2.0
+
+
+# The one-launch form (a small side of up to 64, its columns over a cluster of 1 to 8 CTAs): the
+# smallest matrices, sides that are not multiples of 16, a last CTA with few or no columns, the
+# largest small side with the most columns that fit and the first side that takes the chain.
+# bounds: NS_FRO_TOL and NS_ELEM_TOL above (the same products and roundings)
+@pytest.mark.parametrize("shape", [(8, 8), (8, 72), (40, 520), (56, 1032), (24, 264), (64, 64), (64, 8192), (8192, 64),
+                                   (4104, 16), (72, 512)])
+def test_newton_schulz_one_launch_edges(shape):
+    G = torch.from_numpy(synth.matrix(*shape, seed=sum(shape))).to("cuda").float()
+    want = oracle.newton_schulz(G.double().cpu().numpy(), 5)
+    got = _ns(G)
+    fro = np.linalg.norm(got - want) / np.linalg.norm(want)
+    elem = np.max(np.abs(got - want)) / np.sqrt(np.mean(want ** 2))
+    assert fro <= NS_FRO_TOL and elem <= NS_ELEM_TOL, (fro, elem)
+    assert resbm.resbm_device_error() == 0
+
+
+@pytest.mark.parametrize("scale", [1e25, 1e-25, 0.0])
+def test_newton_schulz_extreme_scales(scale):
+    """Squares outside fp32's range (the norm's sum then runs in fp64), below it (the eps in the
+    denominator decides) and a zero matrix."""
+    G = (torch.from_numpy(synth.matrix(32, 512, seed=9)).to("cuda") * scale).float()
+    want = oracle.newton_schulz(G.double().cpu().numpy(), 5)
+    got = _ns(G)
+    assert np.isfinite(got).all() and np.linalg.norm(got - want) <= NS_FRO_TOL * np.linalg.norm(want) + 1e-30
