@@ -398,10 +398,10 @@ RESBM_API resbm_status resbm_newton_schulz(int64_t rows, int64_t cols, const voi
 /* The effective rank of a bf16 matrix W (rows x cols, row-major) as the appendix's spectral
  * analysis defines it, r_eff = sum_i sigma_i^2 / max_i sigma_i^2, computed as trace(S) /
  * lambda_max(S) for the Gram matrix S of W's smaller side (W^T W or W W^T; fp32 sums of the exact
- * bf16 products), lambda_max by power iteration on one CTA until the residual ||S v - lambda v||
- * is at most 1e-5 lambda ||v|| (at most 20000 iterations): some eigenvalue of S then lies within
- * 1e-5 (relative) of lambda (Bauer-Fike; the fp32 products put the residual's floor near 1e-6). `out` (device, 4 doubles): sigma_max^2, ||W||_F^2, r_eff, the iterations
- * taken. min(rows, cols) <= 4096. */
+ * bf16 products), lambda_max by restarted Lanczos until the residual ||S v - lambda v|| is at most
+ * 1e-5 lambda ||v|| (at most 20000 iterations, i.e. products with S): some eigenvalue of S then lies
+ * within 1e-5 (relative) of lambda (Bauer-Fike; the fp32 products put the residual's floor near
+ * 1e-6). `out` (device, 4 doubles): sigma_max^2, ||W||_F^2, r_eff, the iterations taken. min(rows, cols) <= 4096. */
 RESBM_API resbm_status resbm_effective_rank(int64_t rows, int64_t cols, const void *W, double *out,
                                   void *ws, size_t ws_bytes, void *stream);
 

@@ -1174,7 +1174,12 @@ cudaError_t tc_effective_rank(int64_t rows, int64_t cols, const void *W, double 
                          : wgrad(c, sd, sd, ld, W, W, w.gram, w.slots, &job, nullptr, false, false);
     if (e == cudaSuccess) e = reduce_jobs(job, tc::ReduceJob{nullptr, 0, 0, 0, nullptr, 0, 0, 0}, c);
     if (e == cudaSuccess) {
-        e = launch(tc::k_power_iter, 1, 1024, 0, c.stream, (const float *)w.gram, (int)sd, 20000, 1e-5f, out);
+        const uint32_t smem = (uint32_t)tc::lanczos_layout((int)sd).floats * 4;
+        static std::atomic<uint8_t> smem_set[kMaxDev];
+        e = ensure_smem(tc::k_lanczos_top, tc::kLzMaxSmem, c.device, smem_set);
+        if (e != cudaSuccess) return e;
+        e = launch_clustered(tc::k_lanczos_top, tc::kLzCl, tc::kLzThreads, smem, tc::kLzCl, c.stream,
+                             (const float *)w.gram, (int)sd, 20000, 1e-5f, out);
         count_launches(1);
     }
     return e;

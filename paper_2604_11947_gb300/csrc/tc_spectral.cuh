@@ -1,7 +1,7 @@
 // tc_spectral.cuh -- small kernels of the two matrix utilities around the bottleneck weights
 // (Sec. 3.4.2 and the appendix's spectral analysis): the Frobenius normalisation that starts
-// Muon's Newton-Schulz orthogonalisation, and the top eigenvalue of a Gram matrix W^T W by power
-// iteration for the effective rank r_eff = sum sigma_i^2 / max sigma_i^2 = trace(W^T W) /
+// Muon's Newton-Schulz orthogonalisation, and the top eigenvalue of a Gram matrix W^T W by
+// restarted Lanczos for the effective rank r_eff = sum sigma_i^2 / max sigma_i^2 = trace(W^T W) /
 // lambda_max(W^T W). The products themselves run on the tensor-core GEMM (tc_gemm.cuh).
 // Every sum here has a fixed order (per-block ranges, then the blocks in order): results are
 // bitwise reproducible.
@@ -353,93 +353,319 @@ __global__ void __launch_bounds__(kNsThreads, 1)
     sync_all();   // no CTA leaves while another may still write into it
 }
 
-// Power iteration on a symmetric positive semi-definite n x n fp32 matrix G (row-major) by one
-// CTA: v <- G v / ||G v|| from a fixed start vector, until the residual ||G v - lambda v|| of the
-// Rayleigh quotient lambda = v^T G v (||v|| = 1) is at most tol * lambda, or max_iter iterations.
-// For a symmetric matrix some eigenvalue lies within the residual of lambda (Bauer-Fike), so the
-// stop bounds the eigenvalue's relative error by tol even when the top eigenvalues are close
-// (where the Rayleigh quotient itself creeps slowly). out[0] = lambda_max,
-// out[1] = trace(G) (fp64 sum in index order), out[2] = trace / lambda_max (the effective rank
-// when G = W^T W), out[3] = iterations taken. The vectors live in shared memory (n <= kPowMaxN).
+// The largest eigenvalue of a symmetric positive semi-definite n x n fp32 matrix G (row-major) by
+// restarted Lanczos on one cluster of kLzCl CTAs. A cycle builds up to kLzK orthonormal vectors
+// q_0 .. q_{k-1} (every new vector orthogonalised twice against all earlier ones of the cycle) and
+// the tridiagonal projection of G on them; the cycle's top Ritz vector starts the next. Each cycle
+// begins with the check that ends the iteration: with v the start vector, lambda = v^T G v / v^T v
+// and the residual ||G v - lambda v|| / ||v|| (sums in fp64) at most tol * lambda. For a symmetric
+// matrix some eigenvalue then lies within the residual of lambda (Bauer-Fike), also when the top
+// eigenvalues are close. out[0] = lambda_max, out[1] = trace(G) (fp64), out[2] = trace / lambda_max
+// (the effective rank when G = W^T W), out[3] = products with G taken.
+//
+// What bounds it: latency. A step is one product with G (each CTA's rows, held in shared memory
+// where they fit: n = 512 is 128 KB a CTA) and three exchanges over the cluster (twice the
+// projections on the earlier vectors; the norm together with the new vector). Power iteration on one CTA
+// (the Gram matrix read from L2 by one SM, ~9 us a product) needed thousands of products where the
+// top eigenvalues are close, Lanczos ~100. Measured at n = 512 (W 8192 x 512, random): 25-40 ms by
+// power iteration, 0.65-0.71 ms by this kernel.
+// Every CTA takes each decision from the same sums, added in rank order: the cluster stays in
+// step, and results are bitwise reproducible.
 constexpr int kPowMaxN = 4096;
-__global__ void __launch_bounds__(1024) k_power_iter(const float *__restrict__ G, int n, int max_iter, float tol,
-                                                     double *__restrict__ out)
+constexpr int kLzCl = 8, kLzThreads = 512, kLzK = 32;
+constexpr uint32_t kLzMaxSmem = 216 * 1024;   // beside ~6 KB of static shared memory
+
+struct LanczosLayout {   // dynamic shared memory, in floats; rows: G's rows per CTA
+    int rows, v, y, q, g, floats;
+    bool g_in_smem;
+};
+__host__ __device__ inline LanczosLayout lanczos_layout(int n)
 {
-    __shared__ float v[kPowMaxN], y[kPowMaxN];
-    __shared__ double red[32];
-    __shared__ double bc;
+    LanczosLayout l;
+    l.rows = ((n + kLzCl - 1) / kLzCl + 3) / 4 * 4;
+    l.v = 0;                         // two full vectors
+    l.y = 2 * n;                     // this CTA's part of the current product
+    l.q = l.y + l.rows;              // this CTA's part of the cycle's vectors
+    l.g = l.q + kLzK * l.rows;
+    l.g_in_smem = (int64_t)l.g + (int64_t)l.rows * n <= (int64_t)kLzMaxSmem / 4;
+    l.floats = l.g_in_smem ? l.g + l.rows * n : l.g;
+    return l;
+}
+
+// The top eigenvector s (unnormalised) of the k x k tridiagonal matrix (diagonal a, off-diagonals
+// b[1 .. k-1]), one warp: the top eigenvalue by 33-section with Sturm counts (the pivots of
+// T - x I, one positive pivot per eigenvalue above x), then one step of inverse iteration from
+// the upper end of the last interval by the twisted factorisation (forward and backward pivots
+// meeting where they nearly cancel).
+__device__ __forceinline__ void tridiag_top(const float *a, const float *b, int k, float *d, float *u, float *s)
+{
+    const int lane = threadIdx.x & 31;
+    float lo = a[0], hi = a[0];
+    for (int i = 0; i < k; ++i) {
+        lo = fmaxf(lo, a[i]);
+        hi = fmaxf(hi, a[i] + (i > 0 ? fabsf(b[i]) : 0.0f) + (i + 1 < k ? fabsf(b[i + 1]) : 0.0f));
+    }
+    const float tiny = 1e-30f + 1e-14f * fabsf(hi);
+    hi += 1e-6f * fabsf(hi) + tiny;
+    for (int round = 0; round < 5; ++round) {
+        const float x = lo + (hi - lo) * ((float)(lane + 1) / 33.0f);
+        float p = a[0] - x;
+        bool above = p > 0.0f;
+        for (int i = 1; i < k; ++i) {
+            if (fabsf(p) < tiny) p = -tiny;
+            p = a[i] - x - __fdividef(b[i] * b[i], p);
+            above = above || p > 0.0f;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, above);
+        const int top = m ? 31 - __clz((int)m) : -1;   // the highest shift below the eigenvalue
+        const float nlo = lo + (hi - lo) * ((float)(top + 1) / 33.0f);
+        hi = lo + (hi - lo) * ((float)(top + 2) / 33.0f);
+        lo = nlo;
+    }
+    if (lane < 2) {   // lane 0: forward pivots d; lane 1: backward pivots u
+        float p = 0.0f;
+        for (int t = 0; t < k; ++t) {
+            const int i = lane == 0 ? t : k - 1 - t;
+            const float off = t == 0 ? 0.0f : lane == 0 ? b[i] : b[i + 1];
+            p = a[i] - hi - (t == 0 ? 0.0f : off * off / p);
+            if (fabsf(p) < tiny) p = -tiny;
+            (lane == 0 ? d : u)[i] = p;
+        }
+    }
+    __syncwarp();
+    if (lane == 0) {
+        int r = 0;
+        float best = 3.4e38f;
+        for (int i = 0; i < k; ++i) {
+            const float g = fabsf(d[i] + u[i] - (a[i] - hi));
+            if (g < best) { best = g; r = i; }
+        }
+        s[r] = 1.0f;
+        for (int i = r; i > 0; --i) s[i - 1] = -b[i] / d[i - 1] * s[i];
+        for (int i = r; i + 1 < k; ++i) s[i + 1] = -b[i + 1] / u[i + 1] * s[i];
+    }
+    __syncwarp();
+}
+
+__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster_f64(uint32_t addr, double v)
+{
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+}
+
+__global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__restrict__ G, int n, int max_iter, float tol,
+                                                               double *__restrict__ out)
+{
+    extern __shared__ float4 lz_smem4[];
+    float *sm = reinterpret_cast<float *>(lz_smem4);
+    __shared__ double slots[2][3][kLzCl];      // exchanged partial sums: [buffer][value][rank]
+    __shared__ float hslots[2][kLzK][kLzCl];   // the same for the projections
+    __shared__ double red[3][kLzThreads / 32];
+    __shared__ float hs[kLzK], al[kLzK], be[kLzK + 1], sv[kLzK], pd[kLzK], pu[kLzK];
+    const LanczosLayout L = lanczos_layout(n);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int NW = kLzThreads / 32;
+    const int rank = (int)cluster_rank();
+    const int row0 = rank * L.rows;
+    const int nr = n - row0 < 0 ? 0 : n - row0 < L.rows ? n - row0 : L.rows;
+    float *y = sm + L.y, *Q = sm + L.q;
     griddep_wait();
     griddep_launch_dependents();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+
+    const float *Gr = G + (int64_t)row0 * n;
+    if (L.g_in_smem) {
+        const float4 *src = reinterpret_cast<const float4 *>(Gr);
+        float4 *dst = reinterpret_cast<float4 *>(sm + L.g);
+        for (int e = tid; e < nr * n / 4; e += kLzThreads) dst[e] = src[e];
+        Gr = sm + L.g;
+    }
     // a fixed start with no special direction: 1 + 0.5 sin(0.7 j)
-    for (int j = tid; j < n; j += blockDim.x) v[j] = 1.0f + 0.5f * sinf(0.7f * (float)j);
-    __syncthreads();
-    // block-wide sum of per-thread doubles in a fixed order
-    auto block_sum = [&](double t) -> double {
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) red[warp] = t;
-        __syncthreads();
-        if (tid == 0) {
-            double s = 0.0;
-            for (int w = 0; w < nw; ++w) s += red[w];
-            bc = s;
+    for (int j = tid; j < n; j += kLzThreads) sm[j] = 1.0f + 0.5f * sinf(0.7f * (float)j);
+
+    // sums of NV doubles over the block (warp tree, then the warps in order); valid in lane v < NV of warp 0
+    auto block_sums = [&](auto &t) {
+        constexpr int NV = sizeof(t) / sizeof(double);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            for (int o = 16; o > 0; o >>= 1) t[v] += __shfl_xor_sync(0xffffffffu, t[v], o);
+            if (lane == 0) red[v][warp] = t[v];
         }
         __syncthreads();
-        const double r = bc;
-        __syncthreads();
+        double r = 0.0;
+        if (tid < NV)
+            for (int w = 0; w < NW; ++w) r += red[tid][w];
         return r;
     };
-    double nv = 0.0;
-    for (int j = tid; j < n; j += blockDim.x) nv += (double)v[j] * v[j];
-    nv = block_sum(nv);
-    const float s0 = (float)(1.0 / sqrt(nv));
-    for (int j = tid; j < n; j += blockDim.x) v[j] *= s0;
+    uint32_t buf = 0;   // exchange buffer of the next exchange
+    auto send = [&](int v, double x, int to) {
+        st_cluster_f64(map_shared(smem_u32(&slots[buf][v][rank]), (uint32_t)to), x);
+    };
+    auto total = [&](uint32_t b, int v) {
+        double s = 0.0;
+#pragma unroll
+        for (int p = 0; p < kLzCl; ++p) s += slots[b][v][p];
+        return s;
+    };
+
+    // the trace and the start vector's norm (this CTA's rows; exchanged over the cluster)
     __syncthreads();
-    double lam = 0.0;
-    int it = 0;
-    for (; it < max_iter; ++it) {
-        // y = G v: one warp per row, lanes along the row, a fixed reduction tree
-        for (int i = warp; i < n; i += nw) {
-            float acc = 0.0f;
-            for (int j = lane; j < n; j += 32) acc = fmaf(G[(int64_t)i * n + j], v[j], acc);
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) y[i] = acc;
-        }
-        __syncthreads();
-        double rq = 0.0, ny = 0.0, vv = 0.0;
-        for (int j = tid; j < n; j += blockDim.x) {
-            rq += (double)v[j] * y[j];
-            ny += (double)y[j] * y[j];
-            vv += (double)v[j] * v[j];
-        }
-        rq = block_sum(rq);
-        ny = block_sum(ny);
-        vv = block_sum(vv);
-        lam = rq / vv;   // the Rayleigh quotient of v (unit length up to fp32 rounding)
-        if (ny <= 0.0) break;   // G v = 0: G is zero on the start vector's span
-        // the residual ||G v - lam v|| / ||v||, summed element by element in fp64
-        double r2 = 0.0;
-        for (int j = tid; j < n; j += blockDim.x) {
-            const double t = (double)y[j] - lam * (double)v[j];
-            r2 += t * t;
-        }
-        const double res = sqrt(block_sum(r2) / vv);
-        const float s = (float)(1.0 / sqrt(ny));
-        for (int j = tid; j < n; j += blockDim.x) v[j] = y[j] * s;
-        __syncthreads();
-        if (res <= (double)tol * fabs(lam)) {
-            ++it;
-            break;
-        }
+    double t2[2] = {0.0, 0.0};
+    for (int i = tid; i < nr; i += kLzThreads) {
+        t2[0] += (double)Gr[(int64_t)i * n + row0 + i];
+        t2[1] += (double)sm[row0 + i] * sm[row0 + i];
     }
-    if (tid == 0) {
-        double tr = 0.0;
-        for (int i = 0; i < n; ++i) tr += (double)G[(int64_t)i * n + i];
+    double bs = block_sums(t2);
+    cluster_sync();   // every CTA runs before anything is written into it
+    if (tid < 2)
+        for (int p = 0; p < kLzCl; ++p) send(tid, bs, p);
+    cluster_sync();
+    const double trace = total(buf, 0);
+    float scale = (float)(1.0 / sqrt(total(buf, 1)));   // 1 / ||v||: v is kept unnormalised
+    buf ^= 1;
+    for (int i = tid; i < nr; i += kLzThreads) Q[i] = sm[row0 + i] * scale;
+
+    const int kmax = n < kLzK ? n : kLzK;
+    int cur = 0, j = 0, it = 0;
+    double lam = 0.0;
+    for (;;) {
+        __syncthreads();   // y of the previous step has been read
+        // y = scale * G v, one warp per four rows
+        {
+            const float4 *v4 = reinterpret_cast<const float4 *>(sm + cur * n);
+            for (int i0 = 4 * warp; i0 < nr; i0 += 4 * NW) {
+                const float4 *g4 = reinterpret_cast<const float4 *>(Gr + (int64_t)i0 * n);
+                float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                const int last = nr - i0 - 1;
+                for (int c = lane; c < n / 4; c += 32) {
+                    const float4 x = v4[c];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const float4 g = g4[(int64_t)(r < last ? r : last) * (n / 4) + c];
+                        acc[r] = fmaf(g.x, x.x, fmaf(g.y, x.y, fmaf(g.z, x.z, fmaf(g.w, x.w, acc[r]))));
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    for (int o = 16; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+                if (lane < 4 && lane <= last)
+                    y[i0 + lane] = scale * (lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3]);
+            }
+        }
+        __syncthreads();
+        if (j == 0) {   // lambda and the residual of the cycle's start vector
+            double t3[3] = {0.0, 0.0, 0.0};
+            for (int i = tid; i < nr; i += kLzThreads) {
+                const double v = Q[i], w = y[i];
+                t3[0] = fma(v, w, t3[0]);
+                t3[1] = fma(w, w, t3[1]);
+                t3[2] = fma(v, v, t3[2]);
+            }
+            bs = block_sums(t3);
+            if (tid < 3)
+                for (int p = 0; p < kLzCl; ++p) send(tid, bs, p);
+            cluster_sync();
+            const double vy = total(buf, 0), yy = total(buf, 1), vv = total(buf, 2);
+            buf ^= 1;
+            lam = vy / vv;
+            if (yy <= 0.0) break;   // G v = 0: G is zero on the start vector's span
+            if (!isfinite(lam)) {   // G holds infinities or NaN: no iteration changes that
+                it = max_iter;
+                break;
+            }
+            if (it < max_iter) ++it;
+            // ||y - lam v||^2 from the three fp64 sums (their rounding, ~1e-16 lam^2, is far below tol^2 lam^2)
+            const double r2 = yy - 2.0 * lam * vy + lam * lam * vv;
+            if (sqrt((r2 > 0.0 ? r2 : 0.0) / vv) <= (double)tol * fabs(lam) || it >= max_iter) break;
+            if (tid == 0) al[0] = (float)lam;
+            for (int i = tid; i < nr; i += kLzThreads) y[i] = fmaf(-(float)lam, Q[i], y[i]);
+        } else {
+            // the projections on the cycle's vectors removed (one warp per vector), twice: the vectors
+            // are orthogonal to E ~ eps, one pass leaves E G q behind, which the division by the new
+            // direction's norm (a tenth of ||G q|| for a flat spectrum) would let grow tenfold a step
+            ++it;
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {
+                for (int v = warp; v <= j; v += NW) {
+                    float h = 0.0f;
+                    for (int i = lane; i < nr; i += 32) h = fmaf(Q[v * L.rows + i], y[i], h);
+                    for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+                    if (lane < kLzCl)
+                        st_cluster_f32(map_shared(smem_u32(&hslots[pass][v][rank]), (uint32_t)lane), h);
+                }
+                cluster_sync();
+                if (tid <= j) {
+                    float h = 0.0f;
+#pragma unroll
+                    for (int p = 0; p < kLzCl; ++p) h += hslots[pass][tid][p];
+                    hs[tid] = h;
+                }
+                __syncthreads();
+                if (tid == 0) al[j] = pass ? al[j] + hs[j] : hs[j];
+                // eight threads per row (n = 512: one row each), every eighth vector a thread
+                for (int i = tid >> 3; i < L.rows; i += kLzThreads / 8) {
+                    float w = 0.0f;
+                    for (int v = tid & 7; v <= j; v += 8) w = fmaf(hs[v], Q[v * L.rows + i], w);
+                    w += __shfl_xor_sync(0xffffffffu, w, 1);
+                    w += __shfl_xor_sync(0xffffffffu, w, 2);
+                    w += __shfl_xor_sync(0xffffffffu, w, 4);
+                    if ((tid & 7) == 0 && i < nr) y[i] -= w;
+                }
+                __syncthreads();
+            }
+        }
+        __syncthreads();
+        // the new direction's norm, and the direction itself into every CTA's other vector
+        double t1[1] = {0.0};
+        for (int i = tid; i < nr; i += kLzThreads) t1[0] = fma((double)y[i], (double)y[i], t1[0]);
+        bs = block_sums(t1);
+        if (tid == 0)
+            for (int p = 0; p < kLzCl; ++p) send(0, bs, p);
+        const uint32_t vdst = smem_u32(sm + (cur ^ 1) * n + row0);
+        for (int e = tid; e < nr * kLzCl; e += kLzThreads)
+            st_cluster_f32(map_shared(vdst + 4u * (uint32_t)(e / kLzCl), (uint32_t)(e % kLzCl)), y[e / kLzCl]);
+        cluster_sync();
+        const float beta = (float)sqrt(total(buf, 0));
+        buf ^= 1;
+        if (j + 1 < kmax && it < max_iter && beta > 1e-6f * fabsf((float)lam)) {
+            if (tid == 0) be[j + 1] = beta;
+            scale = 1.0f / beta;
+            cur ^= 1;
+            ++j;
+            for (int i = tid; i < nr; i += kLzThreads) Q[j * L.rows + i] = y[i] * scale;
+            continue;   // (Q and be are read after later barriers)
+        }
+        // the cycle's top Ritz vector starts the next cycle
+        if (warp == 0) tridiag_top(al, be, j + 1, pd, pu, sv);
+        __syncthreads();
+        t1[0] = 0.0;
+        for (int i = tid; i < nr; i += kLzThreads) {
+            float w = 0.0f;
+            for (int v = 0; v <= j; ++v) w = fmaf(sv[v], Q[v * L.rows + i], w);
+            y[i] = w;
+            t1[0] = fma((double)w, (double)w, t1[0]);
+        }
+        bs = block_sums(t1);
+        if (tid == 0)
+            for (int p = 0; p < kLzCl; ++p) send(0, bs, p);
+        for (int e = tid; e < nr * kLzCl; e += kLzThreads)
+            st_cluster_f32(map_shared(vdst + 4u * (uint32_t)(e / kLzCl), (uint32_t)(e % kLzCl)), y[e / kLzCl]);
+        cluster_sync();
+        scale = (float)(1.0 / sqrt(total(buf, 0)));
+        buf ^= 1;
+        cur ^= 1;
+        j = 0;
+        for (int i = tid; i < nr; i += kLzThreads) Q[i] = y[i] * scale;
+    }
+    if (rank == 0 && tid == 0) {
         out[0] = lam;
-        out[1] = tr;
-        out[2] = lam > 0.0 ? tr / lam : 0.0;
+        out[1] = trace;
+        out[2] = lam > 0.0 ? trace / lam : 0.0;
         out[3] = (double)it;
     }
+    cluster_sync();   // no CTA leaves while another may still write into it
 }
 
 }  // namespace tc

@@ -118,3 +118,21 @@ def test_newton_schulz_extreme_scales(scale):
     want = oracle.newton_schulz(G.double().cpu().numpy(), 5)
     got = _ns(G)
     assert np.isfinite(got).all() and np.linalg.norm(got - want) <= NS_FRO_TOL * np.linalg.norm(want) + 1e-30
+
+
+@pytest.mark.parametrize("shape", [(8, 8), (8, 4096), (40, 4096), (264, 1000), (1032, 1024), (2048, 1536)])
+def test_effective_rank_lanczos_edges(shape):
+    """Fewer columns than a cycle's vectors, CTAs without rows, the Gram matrix too large for shared
+    memory; bounds as in test_effective_rank_matches_oracle."""
+    W = torch.from_numpy(synth.matrix(*shape, seed=sum(shape)) / np.sqrt(shape[0])).to("cuda").to(torch.bfloat16)
+    Wh = W.double().cpu().numpy()
+    lam, fro2, reff, iters = _reff(W)
+    assert 0 < iters < 20000
+    want = np.linalg.svd(Wh, compute_uv=False)[0] ** 2
+    assert abs(lam - want) <= 1e-4 * lam and abs(fro2 - np.sum(Wh * Wh)) <= 1e-5 * np.sum(Wh * Wh)
+    assert abs(reff - oracle.effective_rank(Wh)) <= 1e-4 * reff
+
+
+def test_effective_rank_of_a_zero_matrix():
+    out = _reff(torch.zeros(512, 64, dtype=torch.bfloat16, device="cuda"))
+    assert out[0] == 0.0 and out[1] == 0.0 and out[2] == 0.0 and out[3] == 0.0
