@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "narrow.cuh"
 
 namespace resbm {
 namespace {
@@ -213,7 +214,7 @@ cudaError_t weight_grad(int64_t M, int64_t N, int64_t T, LA la, LB lb, float *ou
 }
 
 struct GenericWs {
-    float *P, *Q, *dG, *dA, *part1, *part2;
+    float *P, *Q, *dG, *dA, *A, *part1, *part2;
 };
 
 GenericWs carve(const resbm_desc &d, int op, void *base, size_t *bytes)
@@ -237,6 +238,7 @@ GenericWs carve(const resbm_desc &d, int op, void *base, size_t *bytes)
     case RESBM_OP_ENCODE_BWD:
         g.P = w.take<float>(T * d.m);
         g.dA = w.take<float>(T * d.m);
+        if (narrow_ok(d)) g.A = w.take<float>(T * d.m);
         g.part1 = w.take<float>(S * d.d * d.m);
         g.part2 = w.take<float>(S * d.m * d.r);
         break;
@@ -252,6 +254,7 @@ cudaError_t enc_fwd_t(const resbm_desc &d, const T *X, const T *F, const T *We1,
                       T *B, float *P_save, void *ws, const Ctx &c)
 {
     GenericWs g = carve(d, RESBM_OP_ENCODE_FWD, ws, nullptr);
+    if (narrow_ok(d)) return narrow_encode_fwd<T>(d, X, F, We1, We2, B, P_save, c);
     float *P = P_save ? P_save : g.P;
     cudaError_t e = gemm(d.T, d.m, d.d, 1, LdRM<T>{F, d.d}, LdRM<T>{We1, d.m},
                          EpF32{P, d.m, 0}, c.stream);                       // P = F . We1
@@ -265,6 +268,7 @@ cudaError_t dec_fwd_t(const resbm_desc &d, const T *B, const T *Wd1, const T *Wd
                       void *ws, const Ctx &c)
 {
     GenericWs g = carve(d, RESBM_OP_DECODE_FWD, ws, nullptr);
+    if (narrow_ok(d)) return narrow_decode_fwd<T>(d, B, Wd1, Wd2, Y, c);
     cudaError_t e = gemm(d.T, d.m, d.r, 1, LdRM<T>{B, d.r}, LdRM<T>{Wd1, d.m},
                          EpF32{g.Q, d.m, 0}, c.stream);                     // Q = B . Wd1
     if (e != cudaSuccess) return e;
@@ -277,6 +281,7 @@ cudaError_t dec_bwd_t(const resbm_desc &d, const T *dY, const T *B, const T *Wd1
                       T *dB, float *dWd1, float *dWd2, void *ws, const Ctx &c)
 {
     GenericWs g = carve(d, RESBM_OP_DECODE_BWD, ws, nullptr);
+    if (narrow_ok(d)) return narrow_decode_bwd<T>(d, dY, B, Wd1, Wd2, dB, dWd1, dWd2, g.Q, g.dG, c);
     cudaError_t e = gemm(d.T, d.m, d.r, 1, LdRM<T>{B, d.r}, LdRM<T>{Wd1, d.m},
                          EpF32{g.Q, d.m, 0}, c.stream);                     // Q = B . Wd1
     if (e != cudaSuccess) return e;
@@ -301,6 +306,14 @@ cudaError_t enc_bwd_t(const resbm_desc &d, const T *dB, const T *F, const float 
     GenericWs g = carve(d, RESBM_OP_ENCODE_BWD, ws, nullptr);
     cudaError_t e = cudaSuccess;
     const float *P = P_save;
+    if (narrow_ok(d)) {
+        if (!P) {   // P = F . We1, the forward's own kernel (the same bits)
+            e = narrow_encode_fwd<T>(d, nullptr, F, We1, We2, nullptr, g.P, c);
+            if (e != cudaSuccess) return e;
+            P = g.P;
+        }
+        return narrow_encode_bwd<T>(d, dB, F, P, We1, We2, dF, dX, dWe1, dWe2, g.dA, g.A, c);
+    }
     if (!P) {
         e = gemm(d.T, d.m, d.d, 1, LdRM<T>{F, d.d}, LdRM<T>{We1, d.m}, EpF32{g.P, d.m, 0},
                  c.stream);                                                 // P = F . We1

@@ -200,8 +200,7 @@ __global__ void __launch_bounds__(kNsThreads, 1)
         double t = 0.0;
         for (int w = 0; w < kNsThreads / 32; ++w) t += red[w];
         if (L.cl > 1)
-            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(map_shared(smem_u32(&nslot[rank]), (uint32_t)tid)), "d"(t)
-                         : "memory");
+            st_cluster_f64(map_shared(smem_u32(&nslot[rank]), (uint32_t)tid), t);
         else
             nslot[0] = t;
     }
@@ -445,15 +444,6 @@ __device__ __forceinline__ void tridiag_top(const float *a, const float *b, int 
         for (int i = r; i + 1 < k; ++i) s[i + 1] = -b[i + 1] / u[i + 1] * s[i];
     }
     __syncwarp();
-}
-
-__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v)
-{
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster_f64(uint32_t addr, double v)
-{
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
 }
 
 __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__restrict__ G, int n, int max_iter, float tol,
