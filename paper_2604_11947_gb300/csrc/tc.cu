@@ -462,36 +462,46 @@ cudaError_t launch_enc_bwd(const resbm_desc &d, const void *dB, const void *F, c
 // K x N row-major, else N x K), all bf16 with row pitches equal to the stored widths.
 int gemm_bn(int64_t N) { return N > 128 ? 256 : 128; }
 
-// 256-row units (two 128-row MMAs sharing each B tile, GemmCfg's BM2) for 256-column products
-// without a lo half, where A is K-major (measured on GB300 at d = 8192, T = 32768, m = 512:
-// P = F . We1 and dQ = dY . Wd2^T 6 % and 3 % faster; the MN-major weight gradient dWe1 = F^T dP
-// 6 % slower), K (per split, for a weight gradient that may split it: wg) is long enough that a
-// unit's epilogue, no longer overlapped with the next unit's products, is short next to them,
-// and the 256-row units still give every SM one. RESBM_GEMM_BM2 (read at every call; a tuning
-// and testing knob): 0 never, 1 wherever the shape allows (either major). Both forms sum each
-// output element over K in the same order; a weight gradient's split count can differ.
-bool gemm_bm2(int64_t M, int64_t N, int64_t K, bool lo, bool a_mn, int sms, bool wg)
+// The unit of a product: 128 rows on one CTA; 256 rows on one CTA (two 128-row MMAs sharing each B tile,
+// GemmCfg's BM2); 256 rows on a CTA pair (two-CTA MMAs, k_gemm's PAIR).
+enum GemmForm { kGemmSingle, kGemmBm2, kGemmPair };
+
+char env_01(const char *name)
 {
-    if (gemm_bn(N) != 256 || lo) return false;
-    const char *v = getenv("RESBM_GEMM_BM2");
-    if (v && (v[0] == '0' || v[0] == '1') && v[1] == 0) return v[0] == '1';
-    if (a_mn || M <= 256 || K < 2048) return false;
+    const char *v = getenv(name);
+    return v && (v[0] == '0' || v[0] == '1') && v[1] == 0 ? v[0] : 0;
+}
+
+// Pairs take every 256-column product with at least two row blocks. RESBM_GEMM_MC=0 turns them off, and
+// RESBM_GEMM_BM2 = 0 / 1 never / always takes the one-CTA 256-row units where the shape allows (both read
+// at every call: tuning and testing knobs). Without pairs the one-CTA 256-row units are for products
+// without a lo half, where A is K-major, K (per split, for a weight gradient that may split it: wg) is
+// long enough that a unit's epilogue, not overlapped with the next unit's products, is short next to
+// them, and the units still give every SM one. Every form sums each output element over K in the same
+// order; a weight gradient's split count can differ.
+GemmForm gemm_form(int64_t M, int64_t N, int64_t K, bool lo, bool a_mn, int sms, bool wg)
+{
+    if (gemm_bn(N) != 256) return kGemmSingle;
+    const char bm2 = env_01("RESBM_GEMM_BM2");
+    if (bm2 == '1' && !lo) return kGemmBm2;
+    if (M > 128 && env_01("RESBM_GEMM_MC") != '0') return kGemmPair;
+    if (bm2 == '0' || lo || a_mn || M <= 256 || K < 2048) return kGemmSingle;
     int64_t units = ((M + 255) / 256) * ((N + 255) / 256);
     if (wg) units *= K / 2048 < 32 ? K / 2048 : 32;
-    return units >= sms;
+    return units >= sms ? kGemmBm2 : kGemmSingle;
 }
 
 // Split-K of a product with few output tiles (the weight gradients, K = tokens): enough splits
-// to give every SM a unit, at most 32 and at least four 64-deep K slices per split. rows: the
-// unit's rows (256 where gemm_bm2 holds).
-int gemm_splits(int64_t M, int64_t N, int64_t K, int sms, int rows = 128)
+// to give every SM (every pair of SMs) a unit, at most 32 and at least four 64-deep K slices per split.
+int gemm_splits(int64_t M, int64_t N, int64_t K, int sms, GemmForm form = kGemmSingle)
 {
-    const int bn = gemm_bn(N);
+    const int bn = gemm_bn(N), rows = form == kGemmSingle ? 128 : 256;
     const int64_t units = ((M + rows - 1) / rows) * ((N + bn - 1) / bn);
-    if (4 * units >= 3 * (int64_t)sms) return 1;
-    int64_t s = sms / units;
-    // 256-row units keep 2048 K per split (their epilogue is not overlapped with the next unit)
-    const int64_t kmax = rows == 256 ? (K / 2048 > 1 ? K / 2048 : 1) : (K + 255) / 256;
+    const int64_t workers = form == kGemmPair ? sms / 2 : sms;
+    if (4 * units >= 3 * workers) return 1;
+    int64_t s = workers / units;
+    // one-CTA 256-row units keep 2048 K per split (their epilogue is not overlapped with the next unit)
+    const int64_t kmax = form == kGemmBm2 ? (K / 2048 > 1 ? K / 2048 : 1) : (K + 255) / 256;
     if (s > kmax) s = kmax;
     if (s > 32) s = 32;
     if (s < 1) s = 1;
@@ -499,21 +509,21 @@ int gemm_splits(int64_t M, int64_t N, int64_t K, int sms, int rows = 128)
     return (int)((K + kc - 1) / kc);
 }
 
-// MC: CTA pairs sharing B by multicast (k_gemm); the grid is then two CTAs per co-resident pair,
-// at most one pair per pair unit (returns cudaErrorNotSupported, before launching, when no pair
+// PAIR: CTA pairs (k_gemm); the grid is then two CTAs per co-resident pair, at most one pair per pair unit
+// (returns cudaErrorNotSupported, before launching, when no pair
 // fits: the caller runs single CTAs).
 // TS: the output leaves by TMA stores through `mo` (k_gemm's TS form); otherwise `mo` is not read.
-template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool MC = false, bool BM2 = false, bool TS = false>
+template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = false, bool BM2 = false, bool TS = false>
 cudaError_t launch_gemm_t(const CUtensorMap &ma, const CUtensorMap &malo, const CUtensorMap &mb,
                           const tc::GemmShape &g, const tc::GemmEp &ep, const Ctx &c, const CUtensorMap *mo = nullptr)
 {
-    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS>;
+    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR>;
     const CUtensorMap &mout = mo ? *mo : ma;
-#define RESBM_KGEMM tc::k_gemm<BN, AMN, BMN, ALO, ENCP, MC, BM2, TS>
+#define RESBM_KGEMM tc::k_gemm<BN, AMN, BMN, ALO, ENCP, PAIR, BM2, TS>
     static std::atomic<uint8_t> smem_set[kMaxDev];
     cudaError_t e = ensure_smem(RESBM_KGEMM, Cfg::SMEM_BYTES, c.device, smem_set);
     if (e != cudaSuccess) return e;
-    if (MC) {
+    if (PAIR) {
         static std::atomic<int> fit[kMaxDev][2];
         const int pairs_fit = coresident_clusters(RESBM_KGEMM, 2, Cfg::THREADS,
                                                   Cfg::SMEM_BYTES, c.device, fit);
@@ -540,21 +550,12 @@ bool ts_enabled()
     return !(v && v[0] == '0' && v[1] == 0);
 }
 
-// Pairs sharing B by multicast for the 256-column products with at least two row blocks, unless
-// RESBM_GEMM_MC=0 (read at every launch; a tuning and testing knob: both forms compute the same
-// bits, each output element summed in the same order by one CTA).
-bool gemm_pairs(int bn, int64_t M)
-{
-    const char *v = getenv("RESBM_GEMM_MC");
-    return bn == 256 && M > 128 && !(v && v[0] == '0' && v[1] == 0);
-}
-
 // splits: 1 for every product whose epilogue is not a plain fp32 store; with splits > 1 the
 // epilogue must be GEP_F32 into `splits` slots of M x N (ep.split_stride apart). A_lo: the lo
-// half of A as a bf16 hi + lo pair (same shape and layout as A), or null. rows: the unit's rows
-// as the caller chose them (128 or 256), or 0 to choose here.
+// half of A as a bf16 hi + lo pair (same shape and layout as A), or null. form: the unit as the
+// caller chose it, or null to choose here.
 cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, bool a_mn, const void *B, bool b_mn,
-                 const tc::GemmEp &ep, int splits, const void *A_lo = nullptr, int rows = 0)
+                 const tc::GemmEp &ep, int splits, const void *A_lo = nullptr, const GemmForm *form = nullptr)
 {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     const int bn = gemm_bn(N);
@@ -565,8 +566,8 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
                      : a_mn ? make_map(&malo, A_lo, M, K, M * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
                             : make_map(&malo, A_lo, K, M, K * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
     const bool lo = A_lo != nullptr;
-    const bool bm2 = !lo && bn == 256 && (rows ? rows == 256 : gemm_bm2(M, N, K, lo, a_mn, c.sm_count, false));
-    const bool pair = !bm2 && gemm_pairs(bn, M);
+    const GemmForm fm = form ? *form : gemm_form(M, N, K, lo, a_mn, c.sm_count, false);
+    const bool bm2 = fm == kGemmBm2, pair = fm == kGemmPair;
     // K-major B: a pair's CTAs each load half of the B tile's rows
     const bool okB = b_mn ? make_map(&mbm, B, N, K, N * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
                           : make_map(&mbm, B, K, N, K * 2, 64, (uint32_t)(pair ? bn / 2 : bn), CU_TENSOR_MAP_SWIZZLE_128B);
@@ -657,13 +658,13 @@ tc::GemmEp ep_of(int mode, int act, void *out, int64_t ldo)
 cudaError_t wgrad(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, const void *B, float *W, float *slots,
                   tc::ReduceJob *job, const void *A_lo = nullptr, bool a_mn = true, bool b_mn = true)
 {
-    const int rows = gemm_bm2(M, N, K, A_lo != nullptr, a_mn, c.sm_count, true) ? 256 : 128;
-    const int s = gemm_splits(M, N, K, c.sm_count, rows);
+    const GemmForm fm = gemm_form(M, N, K, A_lo != nullptr, a_mn, c.sm_count, true);
+    const int s = gemm_splits(M, N, K, c.sm_count, fm);
     *job = tc::ReduceJob{nullptr, 0, 0, 0, nullptr, 0, 0, 0};
-    if (s <= 1) return gemm(c, M, N, K, A, a_mn, B, b_mn, ep_of(tc::GEP_F32, 0, W, N), 1, A_lo, rows);
+    if (s <= 1) return gemm(c, M, N, K, A, a_mn, B, b_mn, ep_of(tc::GEP_F32, 0, W, N), 1, A_lo, &fm);
     tc::GemmEp e = ep_of(tc::GEP_F32, 0, slots, N);
     e.split_stride = M * N;
-    cudaError_t err = gemm(c, M, N, K, A, a_mn, B, b_mn, e, s, A_lo, rows);
+    cudaError_t err = gemm(c, M, N, K, A, a_mn, B, b_mn, e, s, A_lo, &fm);
     if (err != cudaSuccess) return err;
     // the number of splits the launch took (gemm rounds K per split to 64)
     const int64_t kc = ((K + s - 1) / s + 63) / 64 * 64;
@@ -700,9 +701,12 @@ constexpr int64_t kDfLoMaxM = 64;
 
 size_t slot_floats(int64_t M, int64_t N, int64_t K, int sms)
 {
-    // room for either unit size (which one a launch takes can depend on RESBM_GEMM_BM2)
-    const int s1 = gemm_splits(M, N, K, sms, 128), s2 = gemm_splits(M, N, K, sms, 256);
-    const int s = s1 > s2 ? s1 : s2;
+    // room for every form (which one a launch takes can depend on the knobs)
+    int s = 1;
+    for (GemmForm f : {kGemmSingle, kGemmBm2, kGemmPair}) {
+        const int n = gemm_splits(M, N, K, sms, f);
+        if (n > s) s = n;
+    }
     return s > 1 ? (size_t)(s * M * N) : 0;
 }
 
@@ -1020,9 +1024,9 @@ cudaError_t tc_ffn_down_encode(const resbm_desc &d, int64_t f, const void *H, co
     e.slot_stride = d.T * d.m;
     e.pm = (int)d.m;
     cudaError_t err = cudaErrorNotSupported;
-    // (not in 256-row units: measured 0.31 -> 0.47 ms at T = 16384, f = 5632, d = 2048, the P
-    // partials' epilogue no longer hidden behind the next unit's products)
-    if (gemm_pairs(bn, d.T)) err = launch_gemm_t<256, false, true, false, true, true>(ma, ma, mb, g, e, c);
+    // (lo: never in one-CTA 256-row units: measured 0.31 -> 0.47 ms at T = 16384, f = 5632, d = 2048, the
+    // P partials' epilogue no longer hidden behind the next unit's products)
+    if (gemm_form(d.T, d.d, f, true, false, c.sm_count, false) == kGemmPair) err = launch_gemm_t<256, false, true, false, true, true>(ma, ma, mb, g, e, c);
     if (err == cudaErrorNotSupported)
         err = bn == 256 ? launch_gemm_t<256, false, true, false, true>(ma, ma, mb, g, e, c)
                         : launch_gemm_t<128, false, true, false, true>(ma, ma, mb, g, e, c);

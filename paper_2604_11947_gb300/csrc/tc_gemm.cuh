@@ -36,26 +36,49 @@
 namespace resbm {
 namespace tc {
 
-// tma_load_2d multicast to the CTAs of the cluster in cta_mask: the box lands at the same
-// shared-memory offset in each of them and completes its bytes on the mbarrier at the same
-// offset in each (this GPU's own memory only).
-__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const CUtensorMap *m, int32_t x, int32_t y, uint32_t bar,
-                                               uint16_t cta_mask)
+// ---- CTA pairs (cta_group::2): the two CTAs of a cluster of 2 work on one 256-row tile -------------
+// tma_load_2d whose bytes complete on an mbarrier of either CTA of the pair (`bar` from map_shared)
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *m, int32_t x, int32_t y, uint32_t bar)
 {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
-        " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(bar), "h"(cta_mask)
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
 
-// mma_commit arriving on the mbarrier at the same offset in every CTA of the cluster in cta_mask.
-__device__ __forceinline__ void mma_commit_mc(uint32_t bar, uint16_t cta_mask)
+// D (+)= A * B over both CTAs, issued by one thread of the even CTA: A's rows 0..127 and the first half
+// of B's columns from its own shared memory, the rest from the odd CTA's (the same offsets); each CTA's
+// TMEM receives its own 128 rows of D.
+__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                              bool accumulate)
 {
     asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-        "h"(cta_mask)
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate)
         : "memory");
+}
+
+// Arrive on the mbarrier at the same offset in the CTAs of `mask` (3: both, 1: the even one) when every
+// pair MMA issued so far has completed.
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t mask = 3)
+{
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+        "h"(mask)
+        : "memory");
+}
+
+// tmem_alloc / tmem_dealloc of a pair: executed by one warp of each of the two CTAs
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t dst, uint32_t ncols)
+{
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(ncols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols)
+{
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
 // The element-wise step after the product (acc = the fp32 accumulator of one output element at
@@ -131,21 +154,23 @@ struct GemmShape {
 
 // BM2: 256-row units, two 128-row A sub-tiles per stage against one B tile, the two halves'
 // accumulators side by side in TMEM (one unit at a time: no accumulator double buffering).
+// PAIR: CTA pairs (cta_group::2) on 256-row units: a stage of each CTA holds its own 128 rows of A and
+// half of the B tile.
 // TS: the output tile leaves by TMA stores from shared-memory staging boxes, two per half of the
 // epilogue warps (128 rows x 64 columns of bf16, 128-byte swizzle; one fills while the other's
 // store reads it), for the products that write T x d bf16 tensors: per-thread 16-byte stores of
 // 32 different rows per warp instruction made the epilogue, not the products, set such a
 // product's pace.
-template <int BN_, bool ALO_ = false, bool BM2_ = false, bool TS_ = false> struct GemmCfg {
+template <int BN_, bool ALO_ = false, bool BM2_ = false, bool TS_ = false, bool PAIR_ = false> struct GemmCfg {
     static constexpr int BN = BN_;
     static constexpr uint32_t A_TILE = 128 * 64 * 2;        // 128 rows x 64 K, bf16
     static constexpr uint32_t A_STAGE = A_TILE * (ALO_ ? 2 : 1) * (BM2_ ? 2 : 1);   // hi (+ lo), per half
-    static constexpr uint32_t B_STAGE = BN_ * 64 * 2;       // BN rows x 64 K, bf16
+    static constexpr uint32_t B_STAGE = (PAIR_ ? BN_ / 2 : BN_) * 64 * 2;   // BN (PAIR: BN / 2) rows x 64 K, bf16
     static constexpr uint32_t STAGE = A_STAGE + B_STAGE;
     static constexpr uint32_t STG_HALF = 128 * 64 * 2;      // TS: one staging box
     static constexpr uint32_t STG_BYTES = TS_ ? 4 * STG_HALF : 0;   // two per half
-    // 4 stages at BN = 256, 6 at 128 (3, 4 with lo; 3 for BM2); TS: 3 at BN = 256 (2 with lo)
-    // beside its four boxes, from a larger share of the 227 KB
+    // 4 stages at BN = 256, 6 at 128 (3, 4 with lo; 3 for BM2; PAIR: 6 and 8, 4 and 5 with lo); TS: 3 at
+    // BN = 256 (2 with lo; PAIR: 5 and 3) beside its four boxes, from a larger share of the 227 KB
     static constexpr int NST = ((TS_ ? 224 : 200) * 1024 - (int)STG_BYTES) / (int)STAGE;
     static constexpr uint32_t OFF_STG = NST * STAGE;        // 1024-aligned (STAGE is)
     static constexpr uint32_t SMEM_BYTES = NST * STAGE + STG_BYTES + 1024;
@@ -338,21 +363,22 @@ __device__ __forceinline__ void gemm_epilogue_ts(const GemmEp &ep, int64_t row, 
 // instead of gemm_epilogue.
 // BM2 (GemmCfg): units of 256 rows (two 128-row MMAs per K step sharing the B tile, ~128 flop per
 // shared-memory byte against ~85), for long K where a unit's epilogue is short next to its
-// products; not with ALO or MC.
-// MC: CTA pairs (clusters of 2) take the row blocks 2p and 2p + 1 of the same column block and K
-// split; each CTA loads its own A tile and half of the B tile, multicast into both CTAs, so each
-// reads 2/3 of a stage's bytes from L2. A stage's `empty` barrier then takes an arrival from both
-// CTAs' MMA commits (multicast), so neither refills it before both have read it. (For K-major B
-// the tensor map's box is BN / 2 rows.)
-template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool MC = false, bool BM2 = false,
+// products; not with ALO or PAIR.
+// PAIR: CTA pairs (clusters of 2) run 256-row units with two-CTA MMAs (cta_group::2, 256 x BN x 16): CTA
+// `rank` loads the rows 128 * rank .. + 127 of A and half of the B tile, all bytes counted on the even
+// CTA's `full` barrier; the even CTA's MMA thread issues for both, and its commits free the stage and
+// publish the accumulators in both (multicast). Each SM reads 96 operand rows a K step for 128 x 256
+// products instead of 384 / 2, and 32 KB instead of 48 KB a stage keep six in flight.
+// (For K-major B the tensor map's box is BN / 2 rows.)
+template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = false, bool BM2 = false,
           bool TS = false>
 __global__ void __launch_bounds__(320, 1)
     k_gemm(const __grid_constant__ CUtensorMap tma, const __grid_constant__ CUtensorMap tma_lo,
            const __grid_constant__ CUtensorMap tmb, const __grid_constant__ CUtensorMap tmo, const GemmShape g,
            const GemmEp ep)
 {
-    using C = GemmCfg<BN, ALO, BM2, TS>;
-    static_assert(!(BM2 && (ALO || MC)), "256-row units without hi + lo A or pairs");
+    using C = GemmCfg<BN, ALO, BM2, TS, PAIR>;
+    static_assert(!(BM2 && (ALO || PAIR)), "256-row units without hi + lo A or pairs");
     static_assert(!(TS && (ENCP || BM2)), "TMA-store epilogue: plain 128-row units");
     constexpr int MH = BM2 ? 2 : 1;   // 128-row halves per unit (g.nm counts units of 128 * MH rows)
     griddep_wait();               // the previous kernel of the stream has completed
@@ -371,35 +397,38 @@ __global__ void __launch_bounds__(320, 1)
     };
     // this CTA's units: every gridDim.x-th from blockIdx.x, or for a pair every (gridDim.x / 2)-th
     // pair unit from the cluster index, the row block 2 * (pair row block) + rank
-    const uint32_t crank = MC ? cluster_rank() : 0u;
-    const int64_t u_first = MC ? (int64_t)cluster_index() : (int64_t)blockIdx.x;
-    const int64_t u_step = MC ? (int64_t)(gridDim.x / 2) : (int64_t)gridDim.x;
+    const uint32_t crank = PAIR ? cluster_rank() : 0u;
+    const int64_t u_first = PAIR ? (int64_t)cluster_index() : (int64_t)blockIdx.x;
+    const int64_t u_step = PAIR ? (int64_t)(gridDim.x / 2) : (int64_t)gridDim.x;
     GemmShape gp = g;
-    if (MC) {
+    if (PAIR) {
         gp.nm = (g.nm + 1) / 2;
         gp.units = (int64_t)gp.nm * gp.nn * gp.splits;
     }
     auto unit_of = [&](int64_t u, int &mb, int &nb, int &ks) {
         gemm_unit(gp, u, mb, nb, ks);
-        if (MC) mb = 2 * mb + (int)crank;   // past the last row block: loads read zeros, nothing is stored
+        if (PAIR) mb = 2 * mb + (int)crank;   // past the last row block: loads read zeros, nothing is stored
     };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::NST; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
-            mbar_init(smem_u32(&empty[s]), MC ? 2 : 1);
+            mbar_init(smem_u32(&empty[s]), 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&acc_full[i]), 1);
-            mbar_init(smem_u32(&acc_empty[i]), C::EPI);
+            mbar_init(smem_u32(&acc_empty[i]), PAIR ? 2 * C::EPI / 32 : C::EPI);   // PAIR: both CTAs' warps, on the even CTA
         }
         mbar_init(smem_u32(&done_bar), 1);
         fence_mbar_init();
     }
-    if (warp == 1) tmem_alloc(smem_u32(&tmem_base_sh), C::TMEM_COLS);
+    if (warp == 1) {
+        if (PAIR) tmem_alloc_pair(smem_u32(&tmem_base_sh), C::TMEM_COLS);
+        else tmem_alloc(smem_u32(&tmem_base_sh), C::TMEM_COLS);
+    }
     tc_fence_before();
     __syncthreads();
-    if (MC) cluster_sync();   // the peer's barriers exist before anything is multicast to them
+    if (PAIR) cluster_sync();   // the peer's barriers exist before anything arrives on them
     tc_fence_after();
     const uint32_t tmem = tmem_base_sh;
 
@@ -422,8 +451,17 @@ __global__ void __launch_bounds__(320, 1)
                         ok = false;
                         break;
                     }
-                    const uint32_t bar = smem_u32(&full[s]);
-                    mbar_expect_tx(bar, C::STAGE);
+                    uint32_t bar = smem_u32(&full[s]);
+                    if (!PAIR) {
+                        mbar_expect_tx(bar, C::STAGE);
+                    } else {   // both CTAs' bytes on the even CTA's barrier
+                        if (crank == 0) mbar_expect_tx(bar, 2 * C::STAGE);
+                        bar = map_shared(bar, 0);
+                    }
+                    auto load = [&](uint32_t dst, const CUtensorMap *m, int32_t x, int32_t y) {
+                        if (PAIR) tma_load_2d_pair(dst, m, x, y, bar);
+                        else tma_load_2d(dst, m, x, y, bar);
+                    };
                     const uint32_t adst = smem_u32(smem + s * C::STAGE), bdst = adst + C::A_STAGE;
                     const int32_t kx = (int32_t)(k0 + 64 * kb);
                     if (BM2) {   // the unit's two 128-row A sub-tiles
@@ -438,25 +476,23 @@ __global__ void __launch_bounds__(320, 1)
                             }
                         }
                     } else if (!AMN) {
-                        tma_load_2d(adst, &tma, kx, mb * 128, bar);
-                        if (ALO) tma_load_2d(adst + C::A_TILE, &tma_lo, kx, mb * 128, bar);
+                        load(adst, &tma, kx, mb * 128);
+                        if (ALO) load(adst + C::A_TILE, &tma_lo, kx, mb * 128);
                     } else {
-                        tma_load_2d(adst, &tma, mb * 128, kx, bar);
-                        tma_load_2d(adst + 8192, &tma, mb * 128 + 64, kx, bar);
+                        load(adst, &tma, mb * 128, kx);
+                        load(adst + 8192, &tma, mb * 128 + 64, kx);
                         if (ALO) {
-                            tma_load_2d(adst + C::A_TILE, &tma_lo, mb * 128, kx, bar);
-                            tma_load_2d(adst + C::A_TILE + 8192, &tma_lo, mb * 128 + 64, kx, bar);
+                            load(adst + C::A_TILE, &tma_lo, mb * 128, kx);
+                            load(adst + C::A_TILE + 8192, &tma_lo, mb * 128 + 64, kx);
                         }
                     }
-                    if (MC) {   // this CTA's half of B, into both CTAs of the pair
+                    if (PAIR) {   // this CTA's half of B
                         if (!BMN) {
-                            tma_load_2d_mc(bdst + crank * (BN / 2) * 128, &tmb, kx, nb * BN + (int)crank * (BN / 2), bar, 3);
+                            load(bdst, &tmb, kx, nb * BN + (int)crank * (BN / 2));
                         } else {
 #pragma unroll
-                            for (int j = 0; j < BN / 128; ++j) {
-                                const int jj = (int)crank * (BN / 128) + j;
-                                tma_load_2d_mc(bdst + jj * 8192, &tmb, nb * BN + 64 * jj, kx, bar, 3);
-                            }
+                            for (int j = 0; j < BN / 128; ++j)
+                                load(bdst + j * 8192, &tmb, nb * BN + (int)crank * (BN / 2) + 64 * j, kx);
                         }
                     } else if (!BMN) {
                         tma_load_2d(bdst, &tmb, kx, nb * BN, bar);
@@ -466,20 +502,19 @@ __global__ void __launch_bounds__(320, 1)
                     }
                 }
             }
-            // drain the loads still in flight before the CTA may exit (for a pair this includes the
-            // peer's multicast halves), and for a pair the last MMA commits of both CTAs on this
-            // CTA's stage barriers
+            // drain the loads still in flight before the CTA may exit; a pair's CTAs wait for the MMAs
+            // that read them (whose commits arrive on both CTAs' stage barriers)
             const uint32_t n = it < (uint32_t)C::NST ? it : (uint32_t)C::NST;
             for (uint32_t k = 0; k < n; ++k) {
                 const uint32_t j = it - 1 - k;
-                mbar_wait(smem_u32(&full[j % C::NST]), (j / C::NST) & 1);
-                if (MC && ok) mbar_wait(smem_u32(&empty[j % C::NST]), (j / C::NST) & 1);
+                if (!PAIR) mbar_wait(smem_u32(&full[j % C::NST]), (j / C::NST) & 1);
+                else if (ok) mbar_wait(smem_u32(&empty[j % C::NST]), (j / C::NST) & 1);
             }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (elect_one()) {
-            constexpr uint32_t idesc = idesc_bf16(128, BN, AMN, BMN);
+        if ((!PAIR || crank == 0) && elect_one()) {   // a pair's even CTA issues for both
+            constexpr uint32_t idesc = idesc_bf16(PAIR ? 256 : 128, BN, AMN, BMN);
             // stage-0 descriptors, advanced by (byte offset >> 4) in the start-address field.
             // K-major: rows of 128 bytes (64 K), 8-row groups 1024 bytes apart, a K step of 16 =
             // 32 bytes. MN-major: 64-wide blocks of 64 K rows (8 KB) 8192 bytes apart along M/N,
@@ -511,22 +546,28 @@ __global__ void __launch_bounds__(320, 1)
                     const uint64_t so = (uint64_t)((s * C::STAGE) >> 4);
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
+                        if (PAIR) {
+                            mma_bf16_pair(d_tmem, ad0 + so + kk * AK, bd0 + so + kk * BK, idesc, kb > 0 || kk > 0);
+                            if (ALO)
+                                mma_bf16_pair(d_tmem, ad0 + so + (C::A_TILE >> 4) + kk * AK, bd0 + so + kk * BK, idesc, true);
+                            continue;
+                        }
                         mma_bf16(d_tmem, ad0 + so + kk * AK, bd0 + so + kk * BK, idesc, kb > 0 || kk > 0);
                         if (ALO) mma_bf16(d_tmem, ad0 + so + (C::A_TILE >> 4) + kk * AK, bd0 + so + kk * BK, idesc, true);
                         if (BM2)   // the second 128-row half into the next BN columns
                             mma_bf16(d_tmem + BN, ad0 + so + (C::A_TILE >> 4) + kk * AK, bd0 + so + kk * BK, idesc,
                                      kb > 0 || kk > 0);
                     }
-                    // the stage is free once these MMAs are done (for a pair: once both CTAs' are)
-                    if (MC)
-                        mma_commit_mc(smem_u32(&empty[s]), 3);
-                    else
-                        mma_commit(smem_u32(&empty[s]));
+                    // the stage is free once these MMAs are done (a pair's: in both CTAs)
+                    if (PAIR) mma_commit_pair(smem_u32(&empty[s]));
+                    else mma_commit(smem_u32(&empty[s]));
                 }
                 if (!ok) break;
-                mma_commit(smem_u32(&acc_full[ab]));
+                if (PAIR) mma_commit_pair(smem_u32(&acc_full[ab]));
+                else mma_commit(smem_u32(&acc_full[ab]));
             }
-            mma_commit(smem_u32(&done_bar));
+            if (PAIR) mma_commit_pair(smem_u32(&done_bar), 1);
+            else mma_commit(smem_u32(&done_bar));
             mbar_wait(smem_u32(&done_bar), 0);
         }
     } else {
@@ -615,7 +656,14 @@ __global__ void __launch_bounds__(320, 1)
                 }
                 if (h == MH - 1) {
                     tc_fence_before();
-                    mbar_arrive(smem_u32(&acc_empty[ab]));   // this accumulator may be overwritten
+                    // this accumulator may be overwritten (the arrival orders the TMEM reads above only; a
+                    // cluster-scope release would wait for the warp's stores, ~3000 cycles a unit)
+                    if (PAIR) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_remote(map_shared(smem_u32(&acc_empty[ab]), 0));
+                    } else {
+                        mbar_arrive(smem_u32(&acc_empty[ab]));
+                    }
                 }
                 if (ENCP && row < g.M) {
                     float *dst = ep.pslots + (int64_t)(nb * 2 + half) * ep.slot_stride + row * ep.pm;
@@ -631,11 +679,12 @@ __global__ void __launch_bounds__(320, 1)
     if (TS && warp >= 2 && (warp & 3) == 0 && lane == 0) bulk_wait<0>();   // the output tiles' stores are done
     tc_fence_before();
     __syncthreads();
+    if (PAIR) cluster_sync();   // neither CTA of a pair leaves, or frees TMEM, while the other may still address it
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, C::TMEM_COLS);
+        if (PAIR) tmem_dealloc_pair(tmem, C::TMEM_COLS);
+        else tmem_dealloc(tmem, C::TMEM_COLS);
     }
-    if (MC) cluster_sync();   // neither CTA of a pair leaves while the other may still address it
 }
 
 // The encoder's end after the fused down-projection, one token row per warp: lane j < m sums

@@ -1,0 +1,31 @@
+"""The GEMM chain's units on CTA pairs (two-CTA MMAs) against its single-CTA units (RESBM_GEMM_MC=0): the
+per-token outputs bit for bit (every element summed over K in the same order), the weight gradients, whose
+split count may differ, to fp32 accumulation in another order."""
+import pytest
+import torch
+
+from gpu_helpers import gpu_step, host_inputs, to_dev
+from paper_2604_11947_gb300 import resbm, synth
+
+pytestmark = pytest.mark.gpu
+
+# one row past a block, an odd number of row blocks (a pair's second CTA idle), ragged columns and K
+SHAPES = [(129, 264, 136, 144), (257, 520, 264, 136), (385, 512, 256, 512), (700, 328, 320, 264)]
+
+
+@pytest.mark.parametrize("T,d,r,m", SHAPES)
+def test_pairs_match_single_ctas(T, d, r, m, monkeypatch):
+    cfg = synth.BoundaryConfig("pairs_%d" % T, T=T, d=d, r=r, m=m)
+    dev = {k: to_dev(v, cfg) for k, v in host_inputs(cfg).items()}
+    flags = resbm.RESBM_FLAG_GEMM
+    pairs = gpu_step(cfg, dev, flags=flags)
+    monkeypatch.setenv("RESBM_GEMM_MC", "0")
+    single = gpu_step(cfg, dev, flags=flags)
+    for k in ("B", "P", "Y", "dB", "dF", "dX"):
+        assert torch.equal(pairs[k], single[k]), k
+    for k in ("dWe1", "dWe2", "dWd1", "dWd2"):
+        err = (pairs[k] - single[k]).abs().max() / single[k].square().mean().sqrt()
+        # sums of up to 700 terms, each partial rounded to 2^-24: sqrt(700) 2^-24 = 1.6e-6 of the RMS
+        # for one element, six times that for the largest of 2.7e5: 1e-5, bound ten times it
+        assert err <= 1e-4, (k, float(err))
+    assert resbm.resbm_device_error() == 0
