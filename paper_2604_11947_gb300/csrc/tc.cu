@@ -42,9 +42,10 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
     return fn;
 }
 
-// 2D bf16 tensor map over a row-major matrix (outer rows x inner columns, row pitch in bytes).
+// 2D bf16 (or fp32) tensor map over a row-major matrix (outer rows x inner columns, row pitch in bytes).
 bool make_map(CUtensorMap *m, const void *ptr, uint64_t inner, uint64_t outer, uint64_t pitch_bytes,
-              uint32_t box_inner, uint32_t box_outer, CUtensorMapSwizzle swz)
+              uint32_t box_inner, uint32_t box_outer, CUtensorMapSwizzle swz,
+              CUtensorMapDataType type = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16)
 {
     auto fn = encode_fn();
     if (!fn) return false;
@@ -52,8 +53,7 @@ bool make_map(CUtensorMap *m, const void *ptr, uint64_t inner, uint64_t outer, u
     cuuint64_t strides[1] = {pitch_bytes};
     cuuint32_t box[2] = {box_inner, box_outer};
     cuuint32_t es[2] = {1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+    return fn(m, type, 2, const_cast<void *>(ptr), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -512,32 +512,34 @@ int gemm_splits(int64_t M, int64_t N, int64_t K, int sms, GemmForm form = kGemmS
 // PAIR: CTA pairs (k_gemm); the grid is then two CTAs per co-resident pair, at most one pair per pair unit
 // (returns cudaErrorNotSupported, before launching, when no pair
 // fits: the caller runs single CTAs).
-// TS: the output leaves by TMA stores through `mo` (k_gemm's TS form); otherwise `mo` is not read.
-template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = false, bool BM2 = false, bool TS = false>
+// TS: the outputs leave by TMA stores through `out` (k_gemm's TS forms; ENCP: F through out->o if it is
+// stored); otherwise `out` is not read.
+struct GemmOutMaps {
+    CUtensorMap o, o2, lo;
+};
+template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = false, bool BM2 = false, int TS = 0>
 cudaError_t launch_gemm_t(const CUtensorMap &ma, const CUtensorMap &malo, const CUtensorMap &mb,
-                          const tc::GemmShape &g, const tc::GemmEp &ep, const Ctx &c, const CUtensorMap *mo = nullptr)
+                          const tc::GemmShape &g, const tc::GemmEp &ep, const Ctx &c, const GemmOutMaps *out = nullptr)
 {
-    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR>;
-    const CUtensorMap &mout = mo ? *mo : ma;
-#define RESBM_KGEMM tc::k_gemm<BN, AMN, BMN, ALO, ENCP, PAIR, BM2, TS>
+    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP>;
+    const GemmOutMaps none{ma, ma, ma};   // not read
+    const GemmOutMaps &mo = out ? *out : none;
+    auto kernel = tc::k_gemm<BN, AMN, BMN, ALO, ENCP, PAIR, BM2, TS>;
     static std::atomic<uint8_t> smem_set[kMaxDev];
-    cudaError_t e = ensure_smem(RESBM_KGEMM, Cfg::SMEM_BYTES, c.device, smem_set);
+    cudaError_t e = ensure_smem(kernel, Cfg::SMEM_BYTES, c.device, smem_set);
     if (e != cudaSuccess) return e;
     if (PAIR) {
         static std::atomic<int> fit[kMaxDev][2];
-        const int pairs_fit = coresident_clusters(RESBM_KGEMM, 2, Cfg::THREADS,
-                                                  Cfg::SMEM_BYTES, c.device, fit);
+        const int pairs_fit = coresident_clusters(kernel, 2, Cfg::THREADS, Cfg::SMEM_BYTES, c.device, fit);
         const int64_t pair_units = (int64_t)((g.nm + 1) / 2) * g.nn * g.splits;
         const int64_t pairs = pair_units < pairs_fit ? pair_units : pairs_fit;
         if (pairs < 1) return cudaErrorNotSupported;
-        e = launch_clustered(RESBM_KGEMM, (unsigned)(2 * pairs), Cfg::THREADS,
-                             Cfg::SMEM_BYTES, 2, c.stream, ma, malo, mb, mout, g, ep);
+        e = launch_clustered(kernel, (unsigned)(2 * pairs), Cfg::THREADS, Cfg::SMEM_BYTES, 2, c.stream, ma, malo, mb, mo.o,
+                             mo.o2, mo.lo, g, ep);
     } else {
         const int64_t grid = g.units < c.sm_count ? g.units : c.sm_count;
-        e = launch(RESBM_KGEMM, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, c.stream, ma,
-                   malo, mb, mout, g, ep);
+        e = launch(kernel, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, c.stream, ma, malo, mb, mo.o, mo.o2, mo.lo, g, ep);
     }
-#undef RESBM_KGEMM
     count_launches(1);
     return e;
 }
@@ -548,6 +550,46 @@ bool ts_enabled()
 {
     const char *v = getenv("RESBM_GEMM_TS");
     return !(v && v[0] == '0' && v[1] == 0);
+}
+
+// The TMA-store form of an epilogue and its output maps: 1 for one bf16 output (Y, dF, B, dB), 2 for the
+// pre-activation and the activation's bf16 pair (P, A; Q, G; dQ; dP, A), 0 for the rest (fp32 outputs of
+// long sums, the Newton-Schulz steps), and for pointers or pitches TMA does not take.
+int gemm_ts(const tc::GemmEp &ep, int64_t M, int64_t N, bool lo, GemmOutMaps *m)
+{
+    if (!ts_enabled()) return 0;
+    bool ok = true;
+    auto map = [&](CUtensorMap *t, const void *p, int64_t ld, bool f32, uint32_t cols) {
+        const int64_t pitch = ld * (f32 ? 4 : 2);
+        ok = ok && al16(p) && pitch % 16 == 0 &&
+             make_map(t, p, N, M, pitch, cols, 32, cols * (f32 ? 4 : 2) == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                      f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
+    };
+    switch (ep.mode) {
+    case tc::GEP_BF16:
+    case tc::GEP_ADD_AUX:
+    case tc::GEP_DF:
+        map(&m->o, ep.out, ep.ldo, false, 64);
+        m->o2 = m->lo = m->o;
+        return ok ? 1 : 0;
+    case tc::GEP_P_A:
+    case tc::GEP_ACT:
+    case tc::GEP_DACT: {
+        if (lo) return 0;
+        const bool p_a = ep.mode == tc::GEP_P_A;
+        const void *act = p_a ? ep.out2 : ep.out;   // the bf16 activation (or dQ, dP): always there
+        map(p_a ? &m->o2 : &m->o, act, p_a ? ep.ldo2 : ep.ldo, false, 32);
+        const CUtensorMap &a = p_a ? m->o2 : m->o;
+        m->lo = a;
+        if (ep.lo) map(&m->lo, ep.lo, p_a ? ep.ldo2 : ep.ldo, false, 32);
+        CUtensorMap *other = p_a ? &m->o : &m->o2;   // P, Q (fp32) or A (bf16)
+        const void *po = p_a ? ep.out : ep.out2;
+        *other = a;
+        if (po) map(other, po, p_a ? ep.ldo : ep.ldo2, ep.mode != tc::GEP_DACT, 32);
+        return ok ? 2 : 0;
+    }
+    }
+    return 0;
 }
 
 // splits: 1 for every product whose epilogue is not a plain fp32 store; with splits > 1 the
@@ -589,30 +631,27 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
         if (a_mn && b_mn) return launch_gemm_t<256, true, true, false, false, false, true>(ma, malo, mbm, g, ep, c);
         return cudaErrorNotSupported;
     }
-    // TMA-store epilogue for the pairs' plain bf16 outputs (Y = G . Wd2 + pad(B), dF = dP . We1^T)
-    CUtensorMap mo;
-    const bool ts = bn == 256 && !bm2 && !a_mn && !(b_mn && lo) && g.splits == 1 &&
-                    (ep.mode == tc::GEP_BF16 || ep.mode == tc::GEP_ADD_AUX || ep.mode == tc::GEP_DF) &&
-                    al16(ep.out) && (ep.ldo * 2) % 16 == 0 && ts_enabled() &&
-                    make_map(&mo, ep.out, N, M, ep.ldo * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B);
-    if (ts && pair) {
-        cudaError_t e = b_mn ? launch_gemm_t<256, false, true, false, false, true, false, true>(ma, malo, mbm, g, ep, c, &mo)
-                        : lo ? launch_gemm_t<256, false, false, true, false, true, false, true>(ma, malo, mbm, g, ep, c, &mo)
-                             : launch_gemm_t<256, false, false, false, false, true, false, true>(ma, malo, mbm, g, ep, c, &mo);
-        if (e != cudaErrorNotSupported) return e;
-        // no pair fits: single CTAs need the whole-tile box for K-major B
-        if (!b_mn && !make_map(&mbm, B, K, N, K * 2, 64, (uint32_t)bn, CU_TENSOR_MAP_SWIZZLE_128B))
-            return cudaErrorInvalidValue;
-    }
-    if (ts) {   // single CTAs
-        return b_mn ? launch_gemm_t<256, false, true, false, false, false, false, true>(ma, malo, mbm, g, ep, c, &mo)
-               : lo ? launch_gemm_t<256, false, false, true, false, false, false, true>(ma, malo, mbm, g, ep, c, &mo)
-                    : launch_gemm_t<256, false, false, false, false, false, false, true>(ma, malo, mbm, g, ep, c, &mo);
+    // TMA-store epilogues: on pairs, and for the products of up to 128 columns
+    GemmOutMaps mo;
+    const int ts = (pair || bn == 128) && !a_mn && g.splits == 1 ? gemm_ts(ep, M, N, lo, &mo) : 0;
+    if (ts && bn == 128) {
+        if (ts == 2) return b_mn ? launch_gemm_t<128, false, true, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo)
+                                 : launch_gemm_t<128, false, false, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo);
+        if (b_mn) return lo ? launch_gemm_t<128, false, true, true, false, false, false, 1>(ma, malo, mbm, g, ep, c, &mo)
+                            : launch_gemm_t<128, false, true, false, false, false, false, 1>(ma, malo, mbm, g, ep, c, &mo);
+        return lo ? launch_gemm_t<128, false, false, true, false, false, false, 1>(ma, malo, mbm, g, ep, c, &mo)
+                  : launch_gemm_t<128, false, false, false, false, false, false, 1>(ma, malo, mbm, g, ep, c, &mo);
     }
     if (pair) {
         cudaError_t e = cudaErrorNotSupported;
-        if (!a_mn && b_mn) e = lo ? launch_gemm_t<256, false, true, true, false, true>(ma, malo, mbm, g, ep, c)
-                                  : launch_gemm_t<256, false, true, false, false, true>(ma, malo, mbm, g, ep, c);
+        if (ts == 2) e = b_mn ? launch_gemm_t<256, false, true, false, false, true, false, 2>(ma, malo, mbm, g, ep, c, &mo)
+                              : launch_gemm_t<256, false, false, false, false, true, false, 2>(ma, malo, mbm, g, ep, c, &mo);
+        else if (ts && b_mn) e = lo ? launch_gemm_t<256, false, true, true, false, true, false, 1>(ma, malo, mbm, g, ep, c, &mo)
+                                    : launch_gemm_t<256, false, true, false, false, true, false, 1>(ma, malo, mbm, g, ep, c, &mo);
+        else if (ts) e = lo ? launch_gemm_t<256, false, false, true, false, true, false, 1>(ma, malo, mbm, g, ep, c, &mo)
+                            : launch_gemm_t<256, false, false, false, false, true, false, 1>(ma, malo, mbm, g, ep, c, &mo);
+        else if (!a_mn && b_mn) e = lo ? launch_gemm_t<256, false, true, true, false, true>(ma, malo, mbm, g, ep, c)
+                                       : launch_gemm_t<256, false, true, false, false, true>(ma, malo, mbm, g, ep, c);
         else if (!a_mn && !b_mn) e = lo ? launch_gemm_t<256, false, false, true, false, true>(ma, malo, mbm, g, ep, c)
                                         : launch_gemm_t<256, false, false, false, false, true>(ma, malo, mbm, g, ep, c);
         else if (a_mn && b_mn) e = lo ? launch_gemm_t<256, true, true, true, false, true>(ma, malo, mbm, g, ep, c)
@@ -1023,13 +1062,15 @@ cudaError_t tc_ffn_down_encode(const resbm_desc &d, int64_t f, const void *H, co
     e.pslots = static_cast<float *>(ws);
     e.slot_stride = d.T * d.m;
     e.pm = (int)d.m;
+    GemmOutMaps mo{ma, ma, ma};
+    if (F_out && !make_map(&mo.o, F_out, d.d, d.T, d.d * 2, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
     cudaError_t err = cudaErrorNotSupported;
     // (lo: never in one-CTA 256-row units: measured 0.31 -> 0.47 ms at T = 16384, f = 5632, d = 2048, the
     // P partials' epilogue no longer hidden behind the next unit's products)
-    if (gemm_form(d.T, d.d, f, true, false, c.sm_count, false) == kGemmPair) err = launch_gemm_t<256, false, true, false, true, true>(ma, ma, mb, g, e, c);
+    if (gemm_form(d.T, d.d, f, true, false, c.sm_count, false) == kGemmPair) err = launch_gemm_t<256, false, true, false, true, true>(ma, ma, mb, g, e, c, &mo);
     if (err == cudaErrorNotSupported)
-        err = bn == 256 ? launch_gemm_t<256, false, true, false, true>(ma, ma, mb, g, e, c)
-                        : launch_gemm_t<128, false, true, false, true>(ma, ma, mb, g, e, c);
+        err = bn == 256 ? launch_gemm_t<256, false, true, false, true>(ma, ma, mb, g, e, c, &mo)
+                        : launch_gemm_t<128, false, true, false, true>(ma, ma, mb, g, e, c, &mo);
     if (err != cudaSuccess) return err;
     err = launch(tc::k_enc_finish, (unsigned)((d.T + 7) / 8), 256, 0, c.stream, (const float *)ws,
                  (int)ffn_slots(d), d.T * d.m, d.T, (int)d.m, (int)d.r, d.act, P,

@@ -121,30 +121,6 @@ struct GemmEp {
     int pm;
 };
 
-// P partial of one row over 32 columns: pacc[j] += sum over c of f[c] * We1[col + c][j], j < m
-// (m a multiple of 8, at most 32); We1's rows are read through L1 (every lane of a warp reads the
-// same rows: broadcasts)
-__device__ __forceinline__ void enc_partial32(const __nv_bfloat16 *__restrict__ we1, int m, int64_t col,
-                                              const float (&f)[32], int nv, float (&pacc)[32])
-{
-#pragma unroll
-    for (int c = 0; c < 32; ++c) {   // fully unrolled: f is indexed by constants only
-        if (c >= nv) break;
-        const uint4 *w = reinterpret_cast<const uint4 *>(we1 + (col + c) * m);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (8 * q >= m) break;
-            const uint4 u = __ldg(w + q);
-            const uint32_t ww[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                pacc[8 * q + 2 * e] = fmaf(f[c], __uint_as_float(ww[e] << 16), pacc[8 * q + 2 * e]);
-                pacc[8 * q + 2 * e + 1] = fmaf(f[c], __uint_as_float(ww[e] & 0xFFFF0000u), pacc[8 * q + 2 * e + 1]);
-            }
-        }
-    }
-}
-
 struct GemmShape {
     int64_t M, N, K;
     int64_t kc;          // K per split, a multiple of 64
@@ -156,23 +132,28 @@ struct GemmShape {
 // accumulators side by side in TMEM (one unit at a time: no accumulator double buffering).
 // PAIR: CTA pairs (cta_group::2) on 256-row units: a stage of each CTA holds its own 128 rows of A and
 // half of the B tile.
-// TS: the output tile leaves by TMA stores from shared-memory staging boxes, two per half of the
-// epilogue warps (128 rows x 64 columns of bf16, 128-byte swizzle; one fills while the other's
-// store reads it), for the products that write T x d bf16 tensors: per-thread 16-byte stores of
-// 32 different rows per warp instruction made the epilogue, not the products, set such a
-// product's pace.
-template <int BN_, bool ALO_ = false, bool BM2_ = false, bool TS_ = false, bool PAIR_ = false> struct GemmCfg {
+// TS: the outputs leave by TMA stores from shared-memory boxes, two 4 KB boxes per epilogue warp (one
+// fills while the other's store reads it), each warp on its own: no barrier between warps. 1: one bf16
+// output in boxes of 32 rows x 64 columns (128-byte swizzle); 2: up to two bf16 and one fp32 output in
+// boxes of 32 rows x 32 columns (64- and 128-byte rows). Per-thread 16-byte stores put 32 different rows
+// in a warp instruction: they, not the products, set the pace where K is short.
+// ENCP: one box of 32 rows x 64 columns per warp (F as the partial P's operand, and for F's store) and
+// We1's rows of the unit's columns.
+template <int BN_, bool ALO_ = false, bool BM2_ = false, int TS_ = 0, bool PAIR_ = false, bool ENCP_ = false> struct GemmCfg {
     static constexpr int BN = BN_;
     static constexpr uint32_t A_TILE = 128 * 64 * 2;        // 128 rows x 64 K, bf16
     static constexpr uint32_t A_STAGE = A_TILE * (ALO_ ? 2 : 1) * (BM2_ ? 2 : 1);   // hi (+ lo), per half
     static constexpr uint32_t B_STAGE = (PAIR_ ? BN_ / 2 : BN_) * 64 * 2;   // BN (PAIR: BN / 2) rows x 64 K, bf16
     static constexpr uint32_t STAGE = A_STAGE + B_STAGE;
-    static constexpr uint32_t STG_HALF = 128 * 64 * 2;      // TS: one staging box
-    static constexpr uint32_t STG_BYTES = TS_ ? 4 * STG_HALF : 0;   // two per half
-    // 4 stages at BN = 256, 6 at 128 (3, 4 with lo; 3 for BM2; PAIR: 6 and 8, 4 and 5 with lo); TS: 3 at
-    // BN = 256 (2 with lo; PAIR: 5 and 3) beside its four boxes, from a larger share of the 227 KB
-    static constexpr int NST = ((TS_ ? 224 : 200) * 1024 - (int)STG_BYTES) / (int)STAGE;
+    static constexpr uint32_t BOX = 32 * 128;               // a staging box: 32 rows of 128 bytes
+    static constexpr uint32_t STG_WARP = TS_ ? 2 * BOX : ENCP_ ? BOX : 0;   // per epilogue warp
+    static constexpr uint32_t WE1_HALF = 128 * 64;          // ENCP: 128 columns' rows of We1 (up to 32 wide)
+    static constexpr uint32_t STG_BYTES = 8 * STG_WARP + (ENCP_ ? 2 * WE1_HALF : 0);
+    // stages: 4 at BN = 256, 6 at 128 (3, 4 with lo; 3 for BM2; PAIR: 6 and 8, 4 and 5 with lo); beside the
+    // boxes of TS 3 at BN = 256 (2 with lo; PAIR: 5 and 3), from a larger share of the 227 KB
+    static constexpr int NST = ((STG_BYTES ? 224 : 200) * 1024 - (int)STG_BYTES) / (int)STAGE;
     static constexpr uint32_t OFF_STG = NST * STAGE;        // 1024-aligned (STAGE is)
+    static constexpr uint32_t OFF_WE1 = OFF_STG + 8 * STG_WARP;
     static constexpr uint32_t SMEM_BYTES = NST * STAGE + STG_BYTES + 1024;
     static_assert(SMEM_BYTES <= 232448 - 512, "shared memory budget");
     static constexpr uint32_t TMEM_COLS = 2 * BN_;          // two accumulators
@@ -357,8 +338,8 @@ __device__ __forceinline__ void gemm_epilogue_ts(const GemmEp &ep, int64_t row, 
     }
 }
 
-// tma_lo: the lo matrix of A (same shape and layout as A; read only with ALO); tmo: the output
-// (bf16, N x M, boxes of 64 columns x 128 rows, 128-byte swizzle; read only with TS)
+// tma_lo: the lo matrix of A (same shape and layout as A; read only with ALO); tmo, tmo2, tmol: the
+// outputs ep.out, ep.out2 and ep.lo in the boxes of the TS form (read only with TS; ENCP: tmo, if ep.out)
 // ENCP: the epilogue of the encoder fused into the FFN down-projection (the GemmEp ENCP fields)
 // instead of gemm_epilogue.
 // BM2 (GemmCfg): units of 256 rows (two 128-row MMAs per K step sharing the B tile, ~128 flop per
@@ -371,15 +352,16 @@ __device__ __forceinline__ void gemm_epilogue_ts(const GemmEp &ep, int64_t row, 
 // products instead of 384 / 2, and 32 KB instead of 48 KB a stage keep six in flight.
 // (For K-major B the tensor map's box is BN / 2 rows.)
 template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = false, bool BM2 = false,
-          bool TS = false>
+          int TS = 0>
 __global__ void __launch_bounds__(320, 1)
     k_gemm(const __grid_constant__ CUtensorMap tma, const __grid_constant__ CUtensorMap tma_lo,
-           const __grid_constant__ CUtensorMap tmb, const __grid_constant__ CUtensorMap tmo, const GemmShape g,
+           const __grid_constant__ CUtensorMap tmb, const __grid_constant__ CUtensorMap tmo,
+           const __grid_constant__ CUtensorMap tmo2, const __grid_constant__ CUtensorMap tmol, const GemmShape g,
            const GemmEp ep)
 {
-    using C = GemmCfg<BN, ALO, BM2, TS, PAIR>;
+    using C = GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP>;
     static_assert(!(BM2 && (ALO || PAIR)), "256-row units without hi + lo A or pairs");
-    static_assert(!(TS && (ENCP || BM2)), "TMA-store epilogue: plain 128-row units");
+    static_assert(!(TS && (ENCP || BM2)), "TMA-store epilogue: plain 128-row units or pairs");
     constexpr int MH = BM2 ? 2 : 1;   // 128-row halves per unit (g.nm counts units of 128 * MH rows)
     griddep_wait();               // the previous kernel of the stream has completed
     griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
@@ -576,107 +558,223 @@ __global__ void __launch_bounds__(320, 1)
         const int half = (warp - 2) >> 2;       // which half of the BN columns
         const int rin = q * 32 + lane;          // row within the 128-row block
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        uint32_t ti = 0, stg_it = 0;   // units; TS staging boxes filled
+        uint32_t ti = 0, stg_it = 0;   // units; staging boxes filled
+        uint8_t *const boxes = smem + C::OFF_STG + (warp - 2) * C::STG_WARP;   // this warp's
+        // the next box, once its previous store has read it
+        auto next_box = [&]() -> uint8_t * {
+            if (lane == 0) bulk_wait_read<1>();
+            __syncwarp();
+            return boxes + (stg_it++ & 1) * C::BOX;
+        };
+        // the warp's writes to the box are complete: store it at (col, row0)
+        auto store_box = [&](const CUtensorMap &m, const uint8_t *box, int64_t col, int64_t row0) {
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                tma_store_2d(&m, (int32_t)col, (int32_t)row0, smem_u32(box));
+                bulk_commit();
+            }
+        };
+        // 32 values of this thread's row as bf16, to bytes [at, at + 64) of the box row (pitch bytes)
+        auto put_bf16 = [&](uint8_t *box, const float (&v)[32], uint32_t at, uint32_t pitch) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint32_t pk[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) pk[i] = pack_bf16(v[8 * e + 2 * i], v[8 * e + 2 * i + 1]);
+                *reinterpret_cast<uint4 *>(box + swz_offset((uint32_t)lane, at + 16 * e, pitch)) =
+                    make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            }
+        };
+        auto release_acc = [&](uint32_t ab) {   // every read of the accumulator is complete: it may be overwritten
+            tc_fence_before();
+            if (PAIR) {
+                // (the arrival orders the TMEM reads only; a cluster-scope release would wait for the warp's
+                // stores, ~3000 cycles a unit)
+                __syncwarp();
+                if (lane == 0) mbar_arrive_remote(map_shared(smem_u32(&acc_empty[ab]), 0));
+            } else {
+                mbar_arrive(smem_u32(&acc_empty[ab]));
+            }
+        };
         bool ok = true;
         for (int64_t u = u_first; u < gp.units && ok; u += u_step, ++ti) {
             int mb, nb, ks;
             unit_of(u, mb, nb, ks);
             const uint32_t ab = BM2 ? 0u : (ti & 1);
+            if (ENCP) {   // this half's rows of We1 (zeros past the last column), while the products run
+                constexpr int HC = BN / 2;
+                uint8_t *w = smem + C::OFF_WE1 + half * C::WE1_HALF;
+                named_barrier(1 + half, 128);   // the previous unit's have been read
+                const int per = ep.pm / 8;      // 16-byte pieces per row, rows 64 bytes apart
+                for (int e = (int)threadIdx.x - 64 - 128 * half; e < HC * per; e += 128) {
+                    const int c = e / per, x = e - c * per;
+                    const int64_t col = (int64_t)nb * BN + half * HC + c;
+                    const uint4 v = col < g.N ? __ldg(reinterpret_cast<const uint4 *>(ep.we1 + col * ep.pm) + x)
+                                              : make_uint4(0u, 0u, 0u, 0u);
+                    *reinterpret_cast<uint4 *>(w + swz_offset((uint32_t)c, 16 * x, 64)) = v;
+                }
+                named_barrier(1 + half, 128);
+            }
             ok = mbar_wait(smem_u32(&acc_full[ab]), BM2 ? (ti & 1) : ((ti >> 1) & 1));
             tc_fence_after();
             if (!ok) break;
+            if (ENCP) {
+                // F as the FFN's bf16 output, 64 columns at a time in the warp's box (stored from there if
+                // asked), then its share of P = F . We1 by warp MMAs on the box (m16n8k16: the tile's 128
+                // tokens x 16 or 32 columns of P are too narrow for the idle TMEM columns, of which there
+                // are none). On CUDA cores, one row per thread with We1 by broadcast loads, this took
+                // 37 us a unit against 23 us of products.
+                float pacc[2][4][4];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) pacc[i >> 4][(i >> 2) & 3][i & 3] = 0.0f;
+                const int64_t row0 = (int64_t)mb * 128 + q * 32;
+                const uint32_t box = smem_u32(boxes), wb = smem_u32(smem + C::OFF_WE1 + half * C::WE1_HALF);
+                const int nt8 = ep.pm / 8;
+#pragma unroll 1
+                for (int c0 = 0; c0 < BN / 2; c0 += 64) {
+                    const uint32_t acc_col = ab * BN + half * (BN / 2) + c0;
+                    float v[2][32];
+                    tmem_ld32(tmem + lane_base + acc_col, v[0]);   // warp-collective: every lane
+                    tmem_ld32(tmem + lane_base + acc_col + 32, v[1]);
+                    if (lane == 0) bulk_wait_read<0>();            // the box's previous store has read it
+                    tmem_ld_wait();
+                    tmem_regs_ready(v[0]);
+                    tmem_regs_ready(v[1]);
+                    if (c0 + 64 >= BN / 2) release_acc(ab);
+                    __syncwarp();                                  // (and every lane its previous fragments)
+                    put_bf16(boxes, v[0], 0, 128);
+                    put_bf16(boxes, v[1], 64, 128);
+                    const int64_t col = (int64_t)nb * BN + half * (BN / 2) + c0;
+                    if (ep.out && row0 < g.M && col < g.N) store_box(tmo, boxes, col, row0);
+                    else __syncwarp();
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        uint32_t af[2][4];
+#pragma unroll
+                        for (int mt = 0; mt < 2; ++mt)
+                            ldsm4(af[mt], box + swz_offset(16 * mt + (lane & 15), 32 * k + 16 * (lane >> 4), 128));
+#pragma unroll
+                        for (int n = 0; n < 4; n += 2) {
+                            if (n >= nt8) break;
+                            uint32_t bf[4];   // (for an odd count of 8-column tiles the last is read and not used)
+                            ldsm4t(bf, wb + swz_offset(c0 + 16 * k + (lane & 15), 16 * n + 16 * (lane >> 4), 64));
+#pragma unroll
+                            for (int mt = 0; mt < 2; ++mt) {
+                                mma16816(pacc[mt][n], af[mt], bf[0], bf[1]);
+                                if (n + 1 < nt8) mma16816(pacc[mt][n + 1], af[mt], bf[2], bf[3]);
+                            }
+                        }
+                    }
+                }
+                float *slot = ep.pslots + (int64_t)(nb * 2 + half) * ep.slot_stride;
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int64_t row = row0 + 16 * mt + 8 * h + (lane >> 2);
+                        if (row >= g.M) continue;
+#pragma unroll
+                        for (int n = 0; n < 4; ++n)
+                            if (n < nt8)
+                                *reinterpret_cast<float2 *>(slot + row * ep.pm + 8 * n + 2 * (lane & 3)) =
+                                    make_float2(pacc[mt][n][2 * h], pacc[mt][n][2 * h + 1]);
+                    }
+                continue;
+            }
+            if (TS) {
+                const int64_t row0 = (int64_t)mb * 128 + q * 32, row = row0 + lane;
+                constexpr int CW = TS == 1 ? 64 : 32;   // columns at a time
+#pragma unroll 1
+                for (int c0 = half * (BN / 2); c0 < (half + 1) * (BN / 2); c0 += CW) {
+                    const int64_t col0 = (int64_t)nb * BN + c0;
+                    const bool last = c0 + CW >= (half + 1) * (BN / 2);
+                    float v[CW / 32][32];
+#pragma unroll
+                    for (int h = 0; h < CW / 32; ++h) tmem_ld32(tmem + lane_base + ab * BN + c0 + 32 * h, v[h]);   // warp-collective
+                    if (row0 >= g.M || col0 >= g.N) {   // nothing of it exists (the same for the whole warp)
+                        tmem_ld_wait();
+                        if (last) release_acc(ab);
+                        continue;
+                    }
+                    if (TS == 1) {
+                        uint8_t *box = next_box();
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int h = 0; h < CW / 32; ++h) tmem_regs_ready(v[h]);
+                        if (last) release_acc(ab);
+#pragma unroll
+                        for (int h = 0; h < CW / 32; ++h) {
+                            const int64_t col = col0 + 32 * h;
+                            gemm_epilogue_ts(ep, row, col, v[h], g.N - col < 32 ? (int)(g.N - col) : 32, row < g.M && col < g.N);
+                            put_bf16(box, v[h], 64 * h, 128);
+                        }
+                        store_box(tmo, box, col0, row0);
+                    } else {
+                        // x: the pre-activation (P, Q) the element-wise step works on
+                        const int nv = g.N - col0 < 32 ? (int)(g.N - col0) : 32;
+                        float x[32];
+                        if (ep.mode == GEP_DACT && row < g.M)
+                            ld_f32x32(static_cast<const float *>(ep.aux) + row * ep.lda + col0, x, nv);
+                        tmem_ld_wait();
+                        tmem_regs_ready(v[0]);
+                        if (last) release_acc(ab);
+                        float *f32 = static_cast<float *>(ep.mode == GEP_P_A ? ep.out : ep.mode == GEP_ACT ? ep.out2 : nullptr);
+                        if (f32) {   // P or Q
+                            uint8_t *box = next_box();
+#pragma unroll
+                            for (int e = 0; e < 8; ++e)
+                                *reinterpret_cast<float4 *>(box + swz_offset((uint32_t)lane, 16 * e, 128)) =
+                                    make_float4(v[0][4 * e], v[0][4 * e + 1], v[0][4 * e + 2], v[0][4 * e + 3]);
+                            store_box(ep.mode == GEP_P_A ? tmo : tmo2, box, col0, row0);
+                        }
+                        if (ep.mode == GEP_DACT) {
+                            float dx[32];
+                            dact_fast_row<32>(ep.act, x, dx);
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) v[0][j] *= dx[j];
+                        } else {
+                            act_fast_row<32>(ep.act, v[0]);
+                        }
+                        uint8_t *box = next_box();
+                        put_bf16(box, v[0], 0, 64);
+                        store_box(ep.mode == GEP_P_A ? tmo2 : tmo, box, col0, row0);
+                        if (ep.lo) {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) v[0][j] -= __bfloat162float(__float2bfloat16_rn(v[0][j]));
+                            box = next_box();
+                            put_bf16(box, v[0], 0, 64);
+                            store_box(tmol, box, col0, row0);
+                        }
+                        if (ep.mode == GEP_DACT && ep.out2) {   // A = phi(P)
+                            act_fast_row<32>(ep.act, x);
+                            box = next_box();
+                            put_bf16(box, x, 0, 64);
+                            store_box(tmo2, box, col0, row0);
+                        }
+                    }
+                }
+                continue;
+            }
 #pragma unroll 1
             for (int h = 0; h < MH; ++h) {   // the unit's 128-row halves (one unless BM2)
                 const int64_t row = (int64_t)mb * (128 * MH) + 128 * h + rin;
                 const uint32_t acc_col = (ab + (uint32_t)h) * BN;
-                float pacc[32];
-                if (ENCP) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) pacc[j] = 0.0f;
-                }
-                if (TS) {
-                    // 64 columns at a time through this half's two staging boxes in turn, each
-                    // stored by one thread
-                    const bool issuer = q == 0 && lane == 0;
 #pragma unroll 1
-                    for (int c0 = half * (BN / 2); c0 < (half + 1) * (BN / 2); c0 += 64, ++stg_it) {
-                        uint8_t *stg = smem + C::OFF_STG + (2 * half + (stg_it & 1)) * C::STG_HALF;
-                        if (issuer) bulk_wait_read<1>();   // the box's previous store has read it
-                        named_barrier(1 + half, 128);
-                        float v2[2][32];
-                        tmem_ld32(tmem + lane_base + acc_col + c0, v2[0]);   // warp-collective: every lane
-                        tmem_ld32(tmem + lane_base + acc_col + c0 + 32, v2[1]);
-                        tmem_ld_wait();
-                        tmem_regs_ready(v2[0]);
-                        tmem_regs_ready(v2[1]);
-#pragma unroll
-                        for (int hh = 0; hh < 2; ++hh) {
-                            const int64_t col = (int64_t)nb * BN + c0 + 32 * hh;
-                            const int nv = g.N - col < 32 ? (int)(g.N - col) : 32;
-                            gemm_epilogue_ts(ep, row, col, v2[hh], nv, row < g.M && col < g.N);
-                            uint32_t pk[16];
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) {
-                                __nv_bfloat162 b2 = __floats2bfloat162_rn(v2[hh][2 * e], v2[hh][2 * e + 1]);
-                                pk[e] = *reinterpret_cast<uint32_t *>(&b2);
-                            }
-#pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                *reinterpret_cast<uint4 *>(stg + swz_offset((uint32_t)rin, 64 * hh + 16 * e, 128)) =
-                                    make_uint4(pk[4 * e], pk[4 * e + 1], pk[4 * e + 2], pk[4 * e + 3]);
-                        }
-                        fence_async_smem();
-                        named_barrier(1 + half, 128);
-                        const int64_t row0 = (int64_t)mb * (128 * MH) + 128 * h, col0 = (int64_t)nb * BN + c0;
-                        if (issuer && row0 < g.M && col0 < g.N) {   // boxes past the tensor: nothing to store
-                            tma_store_2d(&tmo, (int32_t)col0, (int32_t)row0, smem_u32(stg));
-                            bulk_commit();
-                        }
-                    }
-                }
-#pragma unroll 1
-                for (int c = half * (BN / 2); c < (TS ? half * (BN / 2) : (half + 1) * (BN / 2)); c += 32) {
+                for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
                     float v[32];
                     tmem_ld32(tmem + lane_base + acc_col + c, v);   // warp-collective: every lane
                     tmem_ld_wait();
                     tmem_regs_ready<32>(v);
                     const int64_t col = (int64_t)nb * BN + c;
-                    if (col < g.N && row < g.M) {
-                        const int nv = g.N - col < 32 ? (int)(g.N - col) : 32;
-                        if (ENCP) {
-                            // F as the FFN's bf16 output, then its share of P = F . We1
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) v[j] = __bfloat162float(__float2bfloat16_rn(v[j]));
-                            if (ep.out) st_bf16x32(static_cast<__nv_bfloat16 *>(ep.out) + row * ep.ldo + col, v, nv);
-                            enc_partial32(ep.we1, ep.pm, col, v, nv, pacc);
-                        } else {
-                            gemm_epilogue(ep, row, col, v, nv, ks);
-                        }
-                    }
+                    if (col < g.N && row < g.M)
+                        gemm_epilogue(ep, row, col, v, g.N - col < 32 ? (int)(g.N - col) : 32, ks);
                 }
-                if (h == MH - 1) {
-                    tc_fence_before();
-                    // this accumulator may be overwritten (the arrival orders the TMEM reads above only; a
-                    // cluster-scope release would wait for the warp's stores, ~3000 cycles a unit)
-                    if (PAIR) {
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive_remote(map_shared(smem_u32(&acc_empty[ab]), 0));
-                    } else {
-                        mbar_arrive(smem_u32(&acc_empty[ab]));
-                    }
-                }
-                if (ENCP && row < g.M) {
-                    float *dst = ep.pslots + (int64_t)(nb * 2 + half) * ep.slot_stride + row * ep.pm;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (4 * q < ep.pm)
-                            reinterpret_cast<float4 *>(dst)[q] =
-                                make_float4(pacc[4 * q], pacc[4 * q + 1], pacc[4 * q + 2], pacc[4 * q + 3]);
-                }
+                if (h == MH - 1) release_acc(ab);
             }
         }
     }
-    if (TS && warp >= 2 && (warp & 3) == 0 && lane == 0) bulk_wait<0>();   // the output tiles' stores are done
+    if ((TS || ENCP) && warp >= 2 && lane == 0) bulk_wait<0>();   // this warp's stores are done
     tc_fence_before();
     __syncthreads();
     if (PAIR) cluster_sync();   // neither CTA of a pair leaves, or frees TMEM, while the other may still address it
