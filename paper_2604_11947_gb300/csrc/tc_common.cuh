@@ -507,6 +507,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return *reinterpret_cast<uint32_t *>(&h);
 }
 
+// Two bf16 sums (each added in fp32, rounded once)
+__device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b)
+{
+    return pack_bf16(__uint_as_float(a << 16) + __uint_as_float(b << 16),
+                     __uint_as_float(a & 0xFFFF0000u) + __uint_as_float(b & 0xFFFF0000u));
+}
+
 // Swizzle mode of a K-major or MN-major operand whose rows are `row_bytes` (32, 64 or 128).
 __host__ __device__ constexpr Swz swz_for(uint32_t row_bytes)
 {

@@ -164,8 +164,10 @@ template <int BN_, bool ALO_ = false, bool BM2_ = false, int TS_ = 0, bool PAIR_
 
 __device__ __forceinline__ void gemm_unit(const GemmShape &g, int64_t u, int &mb, int &nb, int &ks)
 {
-    nb = (int)(u % g.nn);
     const int64_t rest = u / g.nn;
+    // the column blocks rotate with the row block: with a fixed start the grid's stride gave some CTAs
+    // every column block that carries the identity path's extra work and others none
+    nb = (int)((u + rest) % g.nn);
     mb = (int)(rest % g.nm);
     ks = (int)(rest / g.nm);
 }
@@ -313,28 +315,33 @@ __device__ __forceinline__ void gemm_epilogue(const GemmEp &ep, int64_t row, int
     }
 }
 
-// TS: the values of an output tile's 32 columns as gemm_epilogue computes them, without its bf16
-// store (the caller stages them for a TMA store). Only GEP_BF16, GEP_ADD_AUX and GEP_DF; GEP_DF's
-// dX[:, :r] read-modify-write still goes to global memory. in_rows: row < M and col < N.
-__device__ __forceinline__ void gemm_epilogue_ts(const GemmEp &ep, int64_t row, int64_t col, float (&v)[32], int nv,
-                                                 bool in_rows)
+// rmw[row][col] += aux[row][col] (bf16, added in fp32) for the 32 rows from row0 (rows < M) and the columns
+// [col0, col1), one warp, in whole 128-byte row pieces (eight lanes a row). One row per thread between the
+// accumulator and the store this cost 9000 cycles a box of 64 columns. (16 rows at a time: 32 made the
+// epilogue loop spill.)
+__device__ __forceinline__ void rmw_rows(const GemmEp &ep, int64_t row0, int64_t M, int64_t col0, int64_t col1)
 {
-    if (!in_rows) return;
-    if (ep.mode == GEP_ADD_AUX && col < ep.aux_cols) {
-        const int na = ep.aux_cols - col < nv ? (int)(ep.aux_cols - col) : nv;
-        float x[32];
-        ld_bf16x32(static_cast<const __nv_bfloat16 *>(ep.aux) + row * ep.lda + col, x, na);
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (; col0 < col1; col0 += 64) {
+        const int64_t col = col0 + 8 * (lane & 7);
+        if (col >= col1) continue;
+#pragma unroll 1
+        for (int64_t row = row0 + (lane >> 3); row < row0 + 32; row += 16) {
+            uint4 x[4], y[4];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = j < na ? v[j] + x[j] : v[j];
-    } else if (ep.mode == GEP_DF && ep.rmw && col < ep.aux_cols) {
-        const int na = ep.aux_cols - col < nv ? (int)(ep.aux_cols - col) : nv;
-        float x[32], y[32];
-        __nv_bfloat16 *r = ep.rmw + row * ep.ldr + col;
-        ld_bf16x32(r, y, na);
-        ld_bf16x32(static_cast<const __nv_bfloat16 *>(ep.aux) + row * ep.lda + col, x, na);
+            for (int i = 0; i < 4; ++i)
+                if (row + 4 * i < M) {
+                    x[i] = __ldg(reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(ep.aux) + (row + 4 * i) * ep.lda + col));
+                    y[i] = *reinterpret_cast<const uint4 *>(ep.rmw + (row + 4 * i) * ep.ldr + col);
+                }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) y[j] += x[j];
-        st_bf16x32(r, y, na);
+            for (int i = 0; i < 4; ++i)
+                if (row + 4 * i < M)
+                    *reinterpret_cast<uint4 *>(ep.rmw + (row + 4 * i) * ep.ldr + col) =
+                        make_uint4(add_bf16x2(y[i].x, x[i].x), add_bf16x2(y[i].y, x[i].y), add_bf16x2(y[i].z, x[i].z),
+                                   add_bf16x2(y[i].w, x[i].w));
+        }
     }
 }
 
@@ -616,6 +623,11 @@ __global__ void __launch_bounds__(320, 1)
                 }
                 named_barrier(1 + half, 128);
             }
+            const int64_t ts_row0 = (int64_t)mb * 128 + q * 32, ts_col0 = (int64_t)nb * BN + half * (BN / 2);
+            if (TS == 1 && ep.mode == GEP_DF && ep.rmw) {
+                const int64_t end = ts_col0 + BN / 2 < ep.aux_cols ? ts_col0 + BN / 2 : ep.aux_cols;
+                if (ts_col0 < end) rmw_rows(ep, ts_row0, g.M, ts_col0, end);   // dX[:, :r] += dB, while the products run
+            }
             ok = mbar_wait(smem_u32(&acc_full[ab]), BM2 ? (ti & 1) : ((ti >> 1) & 1));
             tc_fence_after();
             if (!ok) break;
@@ -683,7 +695,7 @@ __global__ void __launch_bounds__(320, 1)
                 continue;
             }
             if (TS) {
-                const int64_t row0 = (int64_t)mb * 128 + q * 32, row = row0 + lane;
+                const int64_t row0 = ts_row0, row = row0 + lane;
                 constexpr int CW = TS == 1 ? 64 : 32;   // columns at a time
 #pragma unroll 1
                 for (int c0 = half * (BN / 2); c0 < (half + 1) * (BN / 2); c0 += CW) {
@@ -706,27 +718,33 @@ __global__ void __launch_bounds__(320, 1)
 #pragma unroll
                         for (int h = 0; h < CW / 32; ++h) {
                             const int64_t col = col0 + 32 * h;
-                            gemm_epilogue_ts(ep, row, col, v[h], g.N - col < 32 ? (int)(g.N - col) : 32, row < g.M && col < g.N);
+                            if (ep.mode == GEP_ADD_AUX && row < g.M && col < ep.aux_cols) {   // the identity path's columns
+                                const int na = ep.aux_cols - col < 32 ? (int)(ep.aux_cols - col) : 32;
+                                float x[32];
+                                ld_bf16x32(static_cast<const __nv_bfloat16 *>(ep.aux) + row * ep.lda + col, x, na);
+#pragma unroll
+                                for (int j = 0; j < 32; ++j) v[h][j] = j < na ? v[h][j] + x[j] : v[h][j];
+                            }
                             put_bf16(box, v[h], 64 * h, 128);
                         }
                         store_box(tmo, box, col0, row0);
                     } else {
                         // x: the pre-activation (P, Q) the element-wise step works on
-                        const int nv = g.N - col0 < 32 ? (int)(g.N - col0) : 32;
                         float x[32];
+                        uint8_t *box = next_box();
                         if (ep.mode == GEP_DACT && row < g.M)
-                            ld_f32x32(static_cast<const float *>(ep.aux) + row * ep.lda + col0, x, nv);
+                            ld_f32x32(static_cast<const float *>(ep.aux) + row * ep.lda + col0, x, g.N - col0 < 32 ? (int)(g.N - col0) : 32);
                         tmem_ld_wait();
                         tmem_regs_ready(v[0]);
                         if (last) release_acc(ab);
                         float *f32 = static_cast<float *>(ep.mode == GEP_P_A ? ep.out : ep.mode == GEP_ACT ? ep.out2 : nullptr);
                         if (f32) {   // P or Q
-                            uint8_t *box = next_box();
 #pragma unroll
                             for (int e = 0; e < 8; ++e)
                                 *reinterpret_cast<float4 *>(box + swz_offset((uint32_t)lane, 16 * e, 128)) =
                                     make_float4(v[0][4 * e], v[0][4 * e + 1], v[0][4 * e + 2], v[0][4 * e + 3]);
                             store_box(ep.mode == GEP_P_A ? tmo : tmo2, box, col0, row0);
+                            box = next_box();
                         }
                         if (ep.mode == GEP_DACT) {
                             float dx[32];
@@ -736,7 +754,6 @@ __global__ void __launch_bounds__(320, 1)
                         } else {
                             act_fast_row<32>(ep.act, v[0]);
                         }
-                        uint8_t *box = next_box();
                         put_bf16(box, v[0], 0, 64);
                         store_box(ep.mode == GEP_P_A ? tmo2 : tmo, box, col0, row0);
                         if (ep.lo) {
