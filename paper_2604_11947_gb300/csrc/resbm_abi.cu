@@ -191,9 +191,14 @@ template <size_t N> bool any_overlap(const Range (&outs)[N], const Range *ins, s
     return false;
 }
 
-// Which kernels run an op: the fused tensor-core kernels where they take the shape (unless a
-// flag says otherwise), else the tensor-core GEMM chain, else the portable CUDA-core kernels.
+// Which kernels run an op: the fused tensor-core kernels where they take the shape and are the faster
+// ones (unless a flag says otherwise), else the tensor-core GEMM chain, else the portable CUDA-core kernels.
 bool use_tc(const resbm_desc &d, int op)
+{
+    return !(d.flags & (RESBM_FLAG_GENERIC | RESBM_FLAG_GEMM)) && tc_supported(d, op) && tc_preferred(d, op);
+}
+// ... and where the chain does not take the call's pointers after all
+bool can_tc(const resbm_desc &d, int op)
 {
     return !(d.flags & (RESBM_FLAG_GENERIC | RESBM_FLAG_GEMM)) && tc_supported(d, op);
 }
@@ -423,6 +428,10 @@ resbm_status run_decode_bwd(const resbm_desc &d, const void *dY, const void *B, 
         cudaError_t e = gemm_decode_bwd(d, dY, B, Wd1, Wd2, dB, dWd1, dWd2, ws, c);
         if (e != cudaErrorNotSupported) return finish(e);
     }
+    if (can_tc(d, RESBM_OP_DECODE_BWD)) {   // gradients that are not 16-byte aligned
+        cudaError_t e = tc_decode_bwd(d, dY, B, Wd1, Wd2, dB, dWd1, dWd2, ws, c, after_independent);
+        if (e != cudaErrorNotSupported) return finish(e);
+    }
     return finish(generic_decode_bwd(d, dY, B, Wd1, Wd2, dB, dWd1, dWd2, ws, c));
 }
 
@@ -470,7 +479,7 @@ resbm_status run_decode_fwd_rmsnorm(const resbm_desc &d, const void *B, const vo
                                     const void *gamma, float eps, void *Y, void *N, void *ws, const Ctx &c)
 {
     if (d.T == 0) return RESBM_OK;
-    if (use_tc(d, RESBM_OP_DECODE_FWD)) {
+    if (can_tc(d, RESBM_OP_DECODE_FWD)) {
         cudaError_t e = tc_decode_fwd_rmsnorm(d, B, Wd1, Wd2, gamma, eps, Y, N, ws, c);
         if (e != cudaErrorNotSupported) return finish(e);
     }

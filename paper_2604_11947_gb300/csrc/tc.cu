@@ -218,14 +218,6 @@ BwdShape bwd_shape(void (*kernel)(KArgs...), int64_t T, int sms, int threads, ui
 
 bool tc_width_ok(int64_t m) { return m == 16 || m == 32 || m == 64 || m == 128; }
 
-// Persistent grid: one CTA per SM, at most one per 128-token tile (token_range).
-int grid_tokens(const Ctx &c, int64_t T)
-{
-    int64_t g = (T + 127) / 128;
-    if (g > c.sm_count) g = c.sm_count;
-    return (int)(g < 1 ? 1 : g);
-}
-
 // NORM (k_dec_fwd): 0 Y; 1 Y and the row sums of squares into ss; 2 N = RMSNorm(Y) * gamma into Y
 template <int M, int NORM = 0>
 cudaError_t launch_dec_fwd(const resbm_desc &d, const void *B, const void *Wd1, const void *Wd2, void *Y,
@@ -280,7 +272,7 @@ cudaError_t launch_enc_fwd(const resbm_desc &d, const void *X, const void *F, co
     int cl = 1;
     int64_t grid = tiles < c.sm_count ? (tiles < 1 ? 1 : tiles) : c.sm_count;
     const int forced = forced_cluster();
-    if (Cfg::SPLIT && forced != 1 && (forced != 0 || tiles > c.sm_count)) {
+    if (forced != 1 && (forced != 0 || tiles > c.sm_count)) {
         static std::atomic<int> fit[kMaxDev][2];
         int64_t pairs = tiles < c.sm_count / 2 ? (tiles < 1 ? 1 : tiles) : c.sm_count / 2;
         if (pairs >= 1 && coresident_clusters(tc::k_enc_fwd<M>, 2, Cfg::THREADS, Cfg::SMEM_BYTES, c.device, fit) >= pairs) {
@@ -414,11 +406,15 @@ EncBwdWs enc_bwd_ws(const resbm_desc &d, int sms, int grid, void *ws)
     WsCarver c(ws);
     w.P = c.take<float>(d.T * d.m);
     char *rest = c.take<char>(0);
-    const int nt = d.m <= 16 ? tc::EncBwdCfg<16>::NT : d.m <= 32 ? tc::EncBwdCfg<32>::NT : tc::EncBwdCfg<64>::NT;
+    const int nt = d.m <= 16 ? tc::EncBwdCfg<16>::NT : tc::EncBwdCfg<32>::NT;
     w.plan = bwd_plan(d, sms, grid, nt, d.m * d.r, ws ? rest : nullptr);
     w.bytes = c.used + w.plan.bytes;
     return w;
 }
+
+// P = F . We1 alone, by the kernel that the encoder forward takes for the shape, so that it matches a
+// saved P bit for bit
+cudaError_t recompute_P(const resbm_desc &d, const void *F, const void *We1, const void *We2, float *P, const Ctx &c);
 
 template <int M>
 cudaError_t launch_enc_bwd(const resbm_desc &d, const void *dB, const void *F, const float *P, const void *We1,
@@ -441,8 +437,8 @@ cudaError_t launch_enc_bwd(const resbm_desc &d, const void *dB, const void *F, c
         !make_map(&m_df16, dF, d.d, d.T, d.d * 2, 64, 16, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_db, dB, d.r, d.T, d.r * 2, M, 128, swizzle_for(Cfg::RB)))
         return cudaErrorInvalidValue;
-    if (!P) {  // P = F . We1 with the forward kernel (no B), so it matches a saved P bit for bit
-        e = launch_enc_fwd<M>(d, nullptr, F, We1, We2, nullptr, w.P, c);
+    if (!P) {
+        e = recompute_P(d, F, We1, We2, w.P, c);
         if (e != cudaSuccess) return e;
         P = w.P;
     }
@@ -694,13 +690,15 @@ tc::GemmEp ep_of(int mode, int act, void *out, int64_t ldo)
 // sum them (in slot order) is returned in `job` (job->blocks = 0: nothing to reduce).
 // A_lo: A as a bf16 hi + lo pair (or null). a_mn / b_mn: the operand majors (both MN-major for the
 // weight gradients, whose K is the tokens).
+// tr: W receives the transpose (N x M), by way of the slots (at least one) and the reduction; so does a W
+// that is not 16-byte aligned.
 cudaError_t wgrad(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, const void *B, float *W, float *slots,
-                  tc::ReduceJob *job, const void *A_lo = nullptr, bool a_mn = true, bool b_mn = true)
+                  tc::ReduceJob *job, const void *A_lo = nullptr, bool a_mn = true, bool b_mn = true, bool tr = false)
 {
     const GemmForm fm = gemm_form(M, N, K, A_lo != nullptr, a_mn, c.sm_count, true);
     const int s = gemm_splits(M, N, K, c.sm_count, fm);
     *job = tc::ReduceJob{nullptr, 0, 0, 0, nullptr, 0, 0, 0};
-    if (s <= 1) return gemm(c, M, N, K, A, a_mn, B, b_mn, ep_of(tc::GEP_F32, 0, W, N), 1, A_lo, &fm);
+    if (s <= 1 && !tr && al16(W)) return gemm(c, M, N, K, A, a_mn, B, b_mn, ep_of(tc::GEP_F32, 0, W, N), 1, A_lo, &fm);
     tc::GemmEp e = ep_of(tc::GEP_F32, 0, slots, N);
     e.split_stride = M * N;
     cudaError_t err = gemm(c, M, N, K, A, a_mn, B, b_mn, e, s, A_lo, &fm);
@@ -708,7 +706,7 @@ cudaError_t wgrad(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, 
     // the number of splits the launch took (gemm rounds K per split to 64)
     const int64_t kc = ((K + s - 1) / s + 63) / 64 * 64;
     const int64_t ns = (K + kc - 1) / kc;
-    *job = reduce_job(slots, ns, M, N, W, 0, al16(W), (int64_t)c.sm_count * 8);
+    *job = reduce_job(slots, ns, M, N, W, tr, al16(W), (int64_t)c.sm_count * 8);
     return cudaSuccess;
 }
 
@@ -749,6 +747,10 @@ size_t slot_floats(int64_t M, int64_t N, int64_t K, int sms)
     return s > 1 ? (size_t)(s * M * N) : 0;
 }
 
+// dWd1 = B^T . dQ takes dQ as a hi + lo pair (as dQ^T . B, transposed by its reduction) up to m = r = 64,
+// where the chain runs in place of a fused kernel that does.
+bool dwd1_pair(const resbm_desc &d) { return d.m == d.r && d.m <= 64; }
+
 GemmWs gemm_ws(const resbm_desc &d, int op, int sms, void *ws, bool have_P)
 {
     GemmWs w;
@@ -766,14 +768,17 @@ GemmWs gemm_ws(const resbm_desc &d, int op, int sms, void *ws, bool have_P)
         w.dQ = cv.take<__nv_bfloat16>(T * m);
         w.dQ_lo = cv.take<__nv_bfloat16>(T * m);
         w.slots1 = cv.take<float>(slot_floats(m, D, T, sms));   // dWd2
-        w.slots2 = cv.take<float>(slot_floats(r, m, T, sms));   // dWd1
+        const size_t s2 = slot_floats(r, m, T, sms);            // dWd1
+        w.slots2 = cv.take<float>(dwd1_pair(d) && s2 < (size_t)(r * m) ? (size_t)(r * m) : s2);
     } else if (op == RESBM_OP_ENCODE_BWD) {
         if (!have_P) w.P = cv.take<float>(T * m);
         w.A = cv.take<__nv_bfloat16>(T * m);
         w.dP = cv.take<__nv_bfloat16>(T * m);
         if (m <= kDfLoMaxM) w.dP_lo = cv.take<__nv_bfloat16>(T * m);
-        w.slots1 = cv.take<float>(slot_floats(D, m, T, sms));   // dWe1
-        w.slots2 = cv.take<float>(slot_floats(m, r, T, sms));   // dWe2
+        // dWe1, dWe2: at least one slot each, for gradients that are not 16-byte aligned
+        const size_t s1 = slot_floats(D, m, T, sms), s2 = slot_floats(m, r, T, sms);
+        w.slots1 = cv.take<float>(s1 ? s1 : (size_t)(D * m));
+        w.slots2 = cv.take<float>(s2 ? s2 : (size_t)(m * r));
     }
     w.bytes = cv.used;
     return w;
@@ -789,9 +794,40 @@ bool tc_supported(const resbm_desc &d, int op)
         const int64_t nch = d.m <= 32 ? 256 : 128;
         return d.d % nch == 0;
     }
-    if (op == RESBM_OP_ENCODE_FWD) return d.d % 64 == 0;
-    if (op == RESBM_OP_DECODE_BWD || op == RESBM_OP_ENCODE_BWD) return d.m <= 64 && d.d % 128 == 0;
+    if (op == RESBM_OP_ENCODE_FWD) return d.m <= 64 && d.d % 64 == 0;
+    if (op == RESBM_OP_DECODE_BWD) return d.m <= 64 && d.d % 128 == 0;
+    if (op == RESBM_OP_ENCODE_BWD) return d.m <= 32 && d.d % 128 == 0;
     return false;
+}
+
+// Fused kernel or chain of products, where both take the shape. A CTA of a fused kernel streams whole
+// 128-token tiles through all of d, so few tokens leave most SMs without work, and the backward kernels
+// write one d x m partial gradient per CTA or cluster, which weighs against their one pass over the data
+// when a CTA gets few tokens; the chain spreads both over the chip but reads the T x d input of a backward
+// op twice and takes three to six launches (20 to 30 us at least). Measured, us, fused / chain (T x d):
+//   encode fwd  m = 16: 1000 x 4096 24 / 19, 4096 x 4096 17 / 20;  m = 32: 1000 x 512 13 / 9, 4096 x 1024
+//               10.7 / 11.2, 16384 x 2048 19 / 22;  m = 64: 256 x 512 16 / 11, 32768 x 8192 106 / 105,
+//               65536 x 4096 98 / 112;  m = 128: 256 x 512 39 / 12 ... 65536 x 4096 155 / 124 (no fused kernel)
+//   decode fwd  m = 64: 1000 x 4096 10 / 10, 65536 x 4096 82 / 103;  m = 128: 1000 x 512 17 / 12, 32768 x 8192
+//               104 / 103, 65536 x 4096 121 / 115
+//   decode bwd  m = 32: 1000 x 4096 38 / 34, 16384 x 2048 30 / 44;  m = 64: 1000 x 512 21 / 31, 1000 x 4096
+//               71 / 39, 65536 x 1024 97 / 110, 16384 x 2048 54 / 51, 32768 x 8192 234 / 223
+//   encode bwd  m = 16: 1000 x 4096 59 / 22, 4096 x 4096 50 / 32, 16384 x 8192 119 / 127;  m = 32: 1000 x 512
+//               16 / 21, 4096 x 4096 70 / 31, 16384 x 2048 42 / 55, 32768 x 8192 259 / 219, 65536 x 4096
+//               200 / 235;  m = 64: 256 x 512 26 / 21 ... 65536 x 4096 485 / 235 (no fused kernel)
+// RESBM_CLUSTER set (the fused kernels' cluster size is being forced) keeps the fused kernels.
+bool tc_preferred(const resbm_desc &d, int op)
+{
+    if (forced_cluster() || !gemm_supported(d, op)) return true;
+    switch (op) {
+    case RESBM_OP_ENCODE_FWD:
+        return d.m == 16 ? !(d.T <= 2048 && d.d >= 2048) : d.m == 32 ? !(d.T <= 2048 && d.d >= 512) : d.T > 32768;
+    case RESBM_OP_DECODE_FWD: return d.m <= 64;
+    case RESBM_OP_DECODE_BWD: return d.m <= 32 || d.d < 2048;
+    case RESBM_OP_ENCODE_BWD:
+        return d.m == 16 ? d.d < 1024 + d.T / 2 : d.T > 38912 || d.d < 512 + d.T / 5;
+    }
+    return true;
 }
 
 size_t tc_ws_bytes(const resbm_desc &d, int op, int sms)
@@ -810,7 +846,6 @@ cudaError_t tc_encode_fwd(const resbm_desc &d, const void *X, const void *F, con
     case 16: return launch_enc_fwd<16>(d, X, F, We1, We2, B, P, c);
     case 32: return launch_enc_fwd<32>(d, X, F, We1, We2, B, P, c);
     case 64: return launch_enc_fwd<64>(d, X, F, We1, We2, B, P, c);
-    case 128: return launch_enc_fwd<128>(d, X, F, We1, We2, B, P, c);
     }
     return cudaErrorNotSupported;
 }
@@ -823,7 +858,6 @@ cudaError_t tc_decode_fwd(const resbm_desc &d, const void *B, const void *Wd1, c
     case 16: return launch_dec_fwd<16>(d, B, Wd1, Wd2, Y, c);
     case 32: return launch_dec_fwd<32>(d, B, Wd1, Wd2, Y, c);
     case 64: return launch_dec_fwd<64>(d, B, Wd1, Wd2, Y, c);
-    case 128: return launch_dec_fwd<128>(d, B, Wd1, Wd2, Y, c);
     }
     return cudaErrorNotSupported;
 }
@@ -890,7 +924,6 @@ cudaError_t tc_encode_bwd(const resbm_desc &d, const void *dB, const void *F, co
     switch (d.m) {
     case 16: return launch_enc_bwd<16>(d, dB, F, P, We1, We2, dF, dX, dWe1, dWe2, ws, c);
     case 32: return launch_enc_bwd<32>(d, dB, F, P, We1, We2, dF, dX, dWe1, dWe2, ws, c);
-    case 64: return launch_enc_bwd<64>(d, dB, F, P, We1, We2, dF, dX, dWe1, dWe2, ws, c);
     }
     return cudaErrorNotSupported;
 }
@@ -966,27 +999,37 @@ cudaError_t gemm_decode_bwd(const resbm_desc &d, const void *dY, const void *B, 
     e3.lda = d.d;
     e3.aux_cols = d.merge_identity ? d.r : 0;
     if (e == cudaSuccess) e = gemm(c, d.T, d.r, d.m, w.dQ, false, Wd1, false, e3, 1, w.dQ_lo);
-    // dWd2 = (G_hi + G_lo)^T . dY, dWd1 = B^T . dQ (sums over the tokens)
+    // dWd2 = (G_hi + G_lo)^T . dY, dWd1 = B^T . dQ (sums over the tokens; dQ as hi + lo up to m = r = 64)
     tc::ReduceJob j2, j1;
     if (e == cudaSuccess) e = wgrad(c, d.m, d.d, d.T, w.G, dY, dWd2, w.slots1, &j2, w.G_lo);
-    if (e == cudaSuccess) e = wgrad(c, d.r, d.m, d.T, B, w.dQ, dWd1, w.slots2, &j1);
+    if (e == cudaSuccess)
+        e = dwd1_pair(d) ? wgrad(c, d.m, d.r, d.T, w.dQ, B, dWd1, w.slots2, &j1, w.dQ_lo, true, true, true)
+                         : wgrad(c, d.r, d.m, d.T, B, w.dQ, dWd1, w.slots2, &j1);
     if (e == cudaSuccess) e = reduce_jobs(j1, j2, c);
     return e;
 }
 
+namespace {
+cudaError_t recompute_P(const resbm_desc &d, const void *F, const void *We1, const void *We2, float *P, const Ctx &c)
+{
+    if (!(d.flags & RESBM_FLAG_GEMM) && tc_supported(d, RESBM_OP_ENCODE_FWD) && tc_preferred(d, RESBM_OP_ENCODE_FWD) &&
+        al16(We2))
+        return d.m == 16   ? launch_enc_fwd<16>(d, nullptr, F, We1, We2, nullptr, P, c)
+               : d.m == 32 ? launch_enc_fwd<32>(d, nullptr, F, We1, We2, nullptr, P, c)
+                           : launch_enc_fwd<64>(d, nullptr, F, We1, We2, nullptr, P, c);
+    return gemm(c, d.T, d.m, d.d, F, false, We1, true, ep_of(tc::GEP_F32, 0, P, d.m), 1);
+}
+}  // namespace
+
 cudaError_t gemm_encode_bwd(const resbm_desc &d, const void *dB, const void *F, const float *P, const void *We1,
                             const void *We2, void *dF, void *dX, float *dWe1, float *dWe2, void *ws, const Ctx &c)
 {
-    if (!al16(dB) || !al16(F) || (P && !al16(P)) || !al16(We1) || !al16(We2) || !al16(dF) || (dX && !al16(dX)) ||
-        !al16(dWe1) || !al16(dWe2) || !al16(ws))
+    if (!al16(dB) || !al16(F) || (P && !al16(P)) || !al16(We1) || !al16(We2) || !al16(dF) || (dX && !al16(dX)) || !al16(ws))
         return cudaErrorNotSupported;
     const GemmWs w = gemm_ws(d, RESBM_OP_ENCODE_BWD, c.sm_count, ws, P != nullptr);
     cudaError_t e = cudaSuccess;
-    if (!P) {   // P = F . We1, the forward's own product (the same launch shape, so the same bits)
-        tc::GemmEp e0 = ep_of(tc::GEP_P_A, d.act, w.P, d.m);
-        e0.out2 = w.A;   // overwritten below; the forward writes A too
-        e0.ldo2 = d.m;
-        e = gemm(c, d.T, d.m, d.d, F, false, We1, true, e0, 1);
+    if (!P) {
+        e = recompute_P(d, F, We1, We2, w.P, c);
         P = w.P;
     }
     // dP = (dB . We2^T) * phi'(P), and A = phi(P) for dWe2

@@ -8,6 +8,8 @@ namespace resbm {
 // Whether the tensor-core kernels handle this descriptor for `op` (bf16 I/O, shapes that fit
 // their tiles); otherwise the portable kernels run.
 bool tc_supported(const resbm_desc &d, int op);
+// Whether they are the better choice there against the GEMM chain below.
+bool tc_preferred(const resbm_desc &d, int op);
 
 // Reads (and optionally clears) the error word of the tensor-core kernels; synchronizing.
 cudaError_t tc_device_error(unsigned int *code, bool clear);

@@ -38,14 +38,15 @@ template <int M_> struct EncBwdCfg {
     static constexpr int M = M_;
     static constexpr int R = M_;
     static constexpr int MS = M_ < 32 ? 32 : M_;                 // TMEM columns per m-wide accumulator
-    static constexpr int NT = M_ <= 32 ? 4 : 2;                  // tiles per group
+    static_assert(M_ <= 32, "wider bottlenecks run as a chain of products");
+    static constexpr int NT = 4;                                 // tiles per group
     static constexpr int NSF = 3;                                // F ring depth
-    static constexpr int NW = M_ <= 16 ? 4 : M_ <= 32 ? 2 : 3;   // We1 slice ring depth
-    static constexpr int CLMAX = M_ <= 32 ? 4 : 1;               // CTAs per cluster (weight-gradient exchange)
+    static constexpr int NW = M_ <= 16 ? 4 : 2;                  // We1 slice ring depth
+    static constexpr int CLMAX = 4;                              // CTAs per cluster (weight-gradient exchange)
     static constexpr int CL_MIN_TOKENS = 256;                 // clusters only from this many tokens per CTA
     static constexpr int NWB = CLMAX > 1 ? 3 : 2;                // dWe1 accumulators in TMEM
-    static constexpr int NDA = M_ <= 32 ? NT : 1;                // dA TMEM regions (a ring)
-    static constexpr bool DPLO = M_ <= 32;                       // dP kept as bf16 hi + lo for dF
+    static constexpr int NDA = NT;                               // dA TMEM regions (a ring)
+    static constexpr bool DPLO = true;                           // dP kept as bf16 hi + lo for dF
     static constexpr uint32_t RB = M_ * 2;                       // row bytes (= swizzle) of r / m wide tiles
     static constexpr uint32_t F_STAGE = 128 * 128 * 2;
     static constexpr uint32_t STG_HALF = 128 * 64 * 2;           // dF staging: 128 rows x 64 columns

@@ -33,7 +33,8 @@ template <int M_> struct EncFwdCfg {
     static constexpr uint32_t F_BYTES = 128 * 128;                      // 128 rows x 64 bf16
     static constexpr uint32_t W_BYTES = 64 * M_ * 2;                    // 64 rows x m bf16
     static constexpr uint32_t STAGE_BYTES = F_BYTES + W_BYTES;
-    static constexpr int NSTAGE = M_ <= 32 ? 8 : (M_ == 64 ? 6 : 3);   // chunk slots
+    static_assert(M_ <= 64, "wider bottlenecks run as a chain of products");
+    static constexpr int NSTAGE = M_ <= 32 ? 8 : 6;                      // chunk slots
     // chunks per ring stage (one barrier, one wait per stage): two consecutive 64-column chunks
     // of a tile share a stage for m <= 32 (a tile's odd last chunk fills half a stage); per CTA
     // the stream is paced by stages in flight, and 32 KB of F per stage streams faster than 16
@@ -47,9 +48,8 @@ template <int M_> struct EncFwdCfg {
     static constexpr uint32_t OFF_STAGE = 0;
     static constexpr uint32_t OFF_A = NSTAGE * STAGE_BYTES;             // A = phi(P): hi tile, then lo tile
     static constexpr uint32_t OFF_WE2T = OFF_A + 2 * A_TILE;            // We2^T [r][m], K-major
-    static constexpr bool SPLIT = M_ <= 64;                              // tiles shared within a pair
     static constexpr uint32_t OFF_RX = OFF_WE2T + WE2T_BYTES;           // the peer's partial P [128][m] fp32
-    static constexpr uint32_t SMEM_BYTES = OFF_RX + (SPLIT ? 128 * M_ * 4 : 0) + 1024;
+    static constexpr uint32_t SMEM_BYTES = OFF_RX + 128 * M_ * 4 + 1024;
     static_assert(SMEM_BYTES <= 232448 - 512, "shared memory budget");
     static constexpr uint32_t ACC_STRIDE = M_ < 32 ? 32 : M_;          // TMEM columns per accumulator
     static constexpr uint32_t TM_E = 2 * ACC_STRIDE;                    // E = A . We2 (r columns)
@@ -117,8 +117,8 @@ __global__ void __launch_bounds__(192, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nk = (int)(a.d / 64);
     const bool want_b = a.B != nullptr;
-    const uint32_t cl = C::SPLIT ? cluster_size() : 1u;
-    const EncFwdWork wk = enc_fwd_work(a.T, nk, cl, C::SPLIT ? cluster_rank() : 0u, cluster_index(), gridDim.x / cl);
+    const uint32_t cl = cluster_size();
+    const EncFwdWork wk = enc_fwd_work(a.T, nk, cl, cluster_rank(), cluster_index(), gridDim.x / cl);
     const int ntiles = (int)(wk.t_end - wk.t_begin);
     // the tiles that need E = A . We2 (all but a tile whose partial P goes to the peer)
     const int e_tiles = ntiles - (wk.send_first ? 1 : 0);
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(192, 1)
     }
     tc_fence_before();
     __syncthreads();
-    if (C::SPLIT && cl > 1) cluster_sync();   // the peer's barrier is armed before anything is pushed
+    if (cl > 1) cluster_sync();   // the peer's barrier is armed before anything is pushed
     tc_fence_after();
     const uint32_t tmem = tmem_base_sh;
 
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(192, 1)
             tmem_ld_row<C::M>(tmem + lane_base + ab * C::ACC_STRIDE, p);
             tc_fence_before();
             mbar_arrive(smem_u32(&acc_empty[ab]));
-            if (C::SPLIT) {
+            {
                 constexpr int V4 = C::M / 4, SW = V4 < 8 ? V4 - 1 : 7;   // float4 per row, swizzle mask
                 const uint32_t rx = smem_u32(smem + C::OFF_RX) + (uint32_t)row * (C::M * 4);
                 if (ti == 0 && wk.send_first) {
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(192, 1)
         tc_fence_after();
         tmem_dealloc(tmem, C::TMEM_COLS);
     }
-    if (C::SPLIT && cl > 1) cluster_sync();   // no peer addresses this CTA's shared memory any more
+    if (cl > 1) cluster_sync();   // no peer addresses this CTA's shared memory any more
 }
 
 }  // namespace tc
