@@ -805,8 +805,8 @@ bool tc_supported(const resbm_desc &d, int op)
 // write one d x m partial gradient per CTA or cluster, which weighs against their one pass over the data
 // when a CTA gets few tokens; the chain spreads both over the chip but reads the T x d input of a backward
 // op twice and takes three to six launches (20 to 30 us at least). Measured, us, fused / chain (T x d):
-//   encode fwd  m = 16: 1000 x 4096 24 / 19, 4096 x 4096 17 / 20;  m = 32: 1000 x 512 13 / 9, 4096 x 1024
-//               10.7 / 11.2, 16384 x 2048 19 / 22;  m = 64: 256 x 512 16 / 11, 32768 x 8192 106 / 105,
+//   encode fwd  m = 16: 1000 x 4096 24 / 19, 4096 x 4096 17 / 20;  m = 32: 1000 x 512 13 / 9 (but in a
+//               step 39 / 40 in all), 1000 x 4096 29 / 18, 4096 x 1024 10.7 / 11.2, 16384 x 2048 19 / 22;  m = 64: 256 x 512 16 / 11, 32768 x 8192 106 / 105,
 //               65536 x 4096 98 / 112;  m = 128: 256 x 512 39 / 12 ... 65536 x 4096 155 / 124 (no fused kernel)
 //   decode fwd  m = 64: 1000 x 4096 10 / 10, 65536 x 4096 82 / 103;  m = 128: 1000 x 512 17 / 12, 32768 x 8192
 //               104 / 103, 65536 x 4096 121 / 115
@@ -821,7 +821,7 @@ bool tc_preferred(const resbm_desc &d, int op)
     if (forced_cluster() || !gemm_supported(d, op)) return true;
     switch (op) {
     case RESBM_OP_ENCODE_FWD:
-        return d.m == 16 ? !(d.T <= 2048 && d.d >= 2048) : d.m == 32 ? !(d.T <= 2048 && d.d >= 512) : d.T > 32768;
+        return d.m == 16 ? !(d.T <= 2048 && d.d >= 2048) : d.m == 32 ? !(d.T <= 2048 && d.d >= 1024) : d.T > 32768;
     case RESBM_OP_DECODE_FWD: return d.m <= 64;
     case RESBM_OP_DECODE_BWD: return d.m <= 32 || d.d < 2048;
     case RESBM_OP_ENCODE_BWD:
@@ -1262,12 +1262,14 @@ cudaError_t tc_effective_rank(int64_t rows, int64_t cols, const void *W, double 
                          : wgrad(c, sd, sd, ld, W, W, w.gram, w.slots, &job, nullptr, false, false);
     if (e == cudaSuccess) e = reduce_jobs(job, tc::ReduceJob{nullptr, 0, 0, 0, nullptr, 0, 0, 0}, c);
     if (e == cudaSuccess) {
-        const uint32_t smem = (uint32_t)tc::lanczos_layout((int)sd).floats * 4;
-        static std::atomic<uint8_t> smem_set[kMaxDev];
-        e = ensure_smem(tc::k_lanczos_top, tc::kLzMaxSmem, c.device, smem_set);
+        const bool small = sd <= tc::kLzSmallN;
+        auto kernel = small ? tc::k_lanczos_small : tc::k_lanczos_top;
+        const uint32_t smem = 4u * (uint32_t)(small ? tc::lanczos_small((int)sd).floats : tc::lanczos_layout((int)sd).floats);
+        static std::atomic<uint8_t> set_small[kMaxDev], set_top[kMaxDev];
+        e = ensure_smem(kernel, tc::kLzMaxSmem, c.device, small ? set_small : set_top);
         if (e != cudaSuccess) return e;
-        e = launch_clustered(tc::k_lanczos_top, tc::kLzCl, tc::kLzThreads, smem, tc::kLzCl, c.stream,
-                             (const float *)w.gram, (int)sd, 20000, 1e-5f, out);
+        e = launch_clustered(kernel, tc::kLzCl, tc::kLzThreads, smem, tc::kLzCl, c.stream, (const float *)w.gram, (int)sd,
+                             20000, 1e-5f, out);
         count_launches(1);
     }
     return e;

@@ -419,6 +419,212 @@ __device__ __forceinline__ void tridiag_top(const float *a, const float *b, int 
     __syncwarp();
 }
 
+// The form for n <= kLzSmallN: every CTA keeps the whole of the cycle's vectors and repeats their
+// orthogonalisation, so that a step's only exchange is the product itself (each CTA's rows of G v into
+// every CTA's copy). With the vectors spread over the cluster (k_lanczos_top) a step takes three
+// exchanges with a remote store's round trip each: W 8192 x 512, 614 us a call against 370 us.
+// A cycle also ends early when the residual estimate |beta s_k| of its top Ritz pair, taken after 8 and
+// 16 vectors, is below half the stop.
+constexpr int kLzSmallN = 512;
+struct LanczosSmall {   // dynamic shared memory, in floats
+    int rows, y, g, floats;
+};
+__host__ __device__ inline LanczosSmall lanczos_small(int n)
+{
+    LanczosSmall l;
+    l.rows = ((n + kLzCl - 1) / kLzCl + 3) / 4 * 4;
+    l.y = kLzK * n;          // after the cycle's vectors: the products, two buffers
+    l.g = l.y + 2 * n;       // this CTA's rows of G
+    l.floats = l.g + l.rows * n;
+    return l;
+}
+
+__global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_small(const float *__restrict__ G, int n, int max_iter, float tol,
+                                                                 double *__restrict__ out)
+{
+    extern __shared__ float4 lz_smem4[];
+    float *sm = reinterpret_cast<float *>(lz_smem4);
+    constexpr int NW = kLzThreads / 32;
+    __shared__ double red[3][NW];
+    __shared__ float fred[NW], hs[kLzK], al[kLzK], be[kLzK + 1], sv[kLzK], pd[kLzK], pu[kLzK];
+    __shared__ int stop_early;
+    const LanczosSmall L = lanczos_small(n);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = (int)cluster_rank(), row0 = rank * L.rows;
+    const int nr = n - row0 < 0 ? 0 : n - row0 < L.rows ? n - row0 : L.rows;
+    float *Q = sm;
+    const float *Gr = sm + L.g;
+    griddep_wait();
+    griddep_launch_dependents();
+    {
+        const float4 *src = reinterpret_cast<const float4 *>(G + (int64_t)row0 * n);
+        float4 *dst = reinterpret_cast<float4 *>(sm + L.g);
+        for (int e = tid; e < nr * n / 4; e += kLzThreads) dst[e] = src[e];
+    }
+    // block-wide sums in a fixed order (a warp's tree, then the warps in order), on every thread
+    auto sums = [&](auto &t) {
+        constexpr int NV = sizeof(t) / sizeof(double);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            for (int o = 16; o > 0; o >>= 1) t[v] += __shfl_xor_sync(0xffffffffu, t[v], o);
+            if (lane == 0) red[v][warp] = t[v];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            t[v] = 0.0;
+            for (int w = 0; w < NW; ++w) t[v] += red[v][w];
+        }
+        __syncthreads();
+    };
+    // (n <= kLzThreads: one element per thread)
+    const bool on = tid < n;
+    // a fixed start with no special direction: 1 + 0.5 sin(0.7 j); the trace from G itself
+    double t2[2];
+    float q = on ? 1.0f + 0.5f * sinf(0.7f * (float)tid) : 0.0f;
+    t2[0] = on ? (double)G[(int64_t)tid * n + tid] : 0.0;
+    t2[1] = (double)q * q;
+    sums(t2);
+    const double trace = t2[0];
+    if (on) Q[tid] = q * (float)(1.0 / sqrt(t2[1]));
+    cluster_sync();   // every CTA runs before anything is written into it (and Q, G are complete)
+
+    const int kmax = n < kLzK ? n : kLzK;
+    int j = 0, it = 0;
+    uint32_t buf = 0;
+    double lam = 0.0;
+    for (;;) {
+        // y = G q_j, one warp per four rows, every row's sum into all CTAs' copies
+        {
+            const float4 *v4 = reinterpret_cast<const float4 *>(Q + j * n);
+            const uint32_t ydst = smem_u32(sm + L.y + buf * n);
+            for (int i0 = 4 * warp; i0 < nr; i0 += 4 * NW) {
+                const float4 *g4 = reinterpret_cast<const float4 *>(Gr + i0 * n);
+                float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                const int last = nr - i0 - 1;
+                for (int c = lane; c < n / 4; c += 32) {
+                    const float4 x = v4[c];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const float4 g = g4[(r < last ? r : last) * (n / 4) + c];
+                        acc[r] = fmaf(g.x, x.x, fmaf(g.y, x.y, fmaf(g.z, x.z, fmaf(g.w, x.w, acc[r]))));
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    for (int o = 16; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+                const int r = lane & 3;   // eight CTAs x four rows
+                if (r <= last)
+                    st_cluster_f32(map_shared(ydst + 4u * (uint32_t)(row0 + i0 + r), (uint32_t)(lane >> 2)),
+                                   r == 0 ? acc[0] : r == 1 ? acc[1] : r == 2 ? acc[2] : acc[3]);
+            }
+        }
+        cluster_sync();
+        float *y = sm + L.y + buf * n;
+        buf ^= 1;
+        float w = on ? y[tid] : 0.0f;   // this thread's element of the new direction
+        if (j == 0) {   // lambda and the residual of the cycle's start vector
+            const double v = on ? (double)Q[tid] : 0.0;
+            double t3[3] = {v * w, (double)w * w, v * v};
+            sums(t3);
+            lam = t3[0] / t3[2];
+            if (t3[1] <= 0.0) break;   // G v = 0: G is zero on the start vector's span
+            if (!isfinite(lam)) {      // G holds infinities or NaN: no iteration changes that
+                it = max_iter;
+                break;
+            }
+            if (it < max_iter) ++it;
+            // ||y - lam v||^2 from the three fp64 sums (their rounding, ~1e-16 lam^2, is far below tol^2 lam^2)
+            const double r2 = t3[1] - 2.0 * lam * t3[0] + lam * lam * t3[2];
+            if (sqrt((r2 > 0.0 ? r2 : 0.0) / t3[2]) <= (double)tol * fabs(lam) || it >= max_iter) break;
+            if (tid == 0) al[0] = (float)lam;
+            if (on) w = fmaf(-(float)lam, Q[tid], w);
+        } else {
+            // the projections on the cycle's vectors removed, twice (see k_lanczos_top)
+            ++it;
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {
+                if (pass) {
+                    if (on) y[tid] = w;
+                    __syncthreads();
+                }
+                for (int v = warp; v <= j; v += NW) {
+                    float h = 0.0f;
+                    for (int i = lane; i < n; i += 32) h = fmaf(Q[v * n + i], y[i], h);
+                    for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+                    if (lane == 0) hs[v] = h;
+                }
+                __syncthreads();
+                if (tid == 0) al[j] = pass ? al[j] + hs[j] : hs[j];
+                if (on) {
+                    float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
+                    int v = 0;
+                    for (; v + 4 <= j + 1; v += 4) {
+                        s0 = fmaf(hs[v], Q[v * n + tid], s0);
+                        s1 = fmaf(hs[v + 1], Q[(v + 1) * n + tid], s1);
+                        s2 = fmaf(hs[v + 2], Q[(v + 2) * n + tid], s2);
+                        s3 = fmaf(hs[v + 3], Q[(v + 3) * n + tid], s3);
+                    }
+                    for (; v <= j; ++v) s0 = fmaf(hs[v], Q[v * n + tid], s0);
+                    w -= (s0 + s1) + (s2 + s3);
+                }
+            }
+        }
+        float b2 = w * w;
+        for (int o = 16; o > 0; o >>= 1) b2 += __shfl_xor_sync(0xffffffffu, b2, o);
+        if (lane == 0) fred[warp] = b2;
+        __syncthreads();
+        b2 = 0.0f;
+#pragma unroll
+        for (int x = 0; x < NW; ++x) b2 += fred[x];
+        const float beta = sqrtf(b2);
+        bool more = j + 1 < kmax && it < max_iter && beta > 1e-6f * fabsf((float)lam);
+        bool have_s = false;
+        if (more && (j + 1 == 8 || j + 1 == 16)) {
+            if (warp == 0) {
+                tridiag_top(al, be, j + 1, pd, pu, sv);
+                if (lane == 0) {
+                    float s2 = 0.0f;
+                    for (int v = 0; v <= j; ++v) s2 = fmaf(sv[v], sv[v], s2);
+                    stop_early = beta * fabsf(sv[j]) <= 0.5f * tol * fabsf((float)lam) * sqrtf(s2);
+                }
+            }
+            __syncthreads();
+            if (stop_early) {
+                more = false;
+                have_s = true;
+            }
+        }
+        if (more) {
+            if (tid == 0) be[j + 1] = beta;
+            ++j;
+            if (on) Q[j * n + tid] = w * (1.0f / beta);
+            __syncthreads();
+            continue;
+        }
+        // the cycle's top Ritz vector starts the next cycle
+        if (!have_s) {
+            if (warp == 0) tridiag_top(al, be, j + 1, pd, pu, sv);
+            __syncthreads();
+        }
+        float z = 0.0f;
+        if (on)
+            for (int v = 0; v <= j; ++v) z = fmaf(sv[v], Q[v * n + tid], z);
+        double t1[1] = {(double)z * z};
+        sums(t1);
+        if (on) Q[tid] = z * (float)(1.0 / sqrt(t1[0]));
+        j = 0;
+        __syncthreads();
+    }
+    if (rank == 0 && tid == 0) {
+        out[0] = lam;
+        out[1] = trace;
+        out[2] = lam > 0.0 ? trace / lam : 0.0;
+        out[3] = (double)it;
+    }
+    cluster_sync();   // no CTA leaves while another may still write into it
+}
+
 __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__restrict__ G, int n, int max_iter, float tol,
                                                                double *__restrict__ out)
 {

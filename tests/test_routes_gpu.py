@@ -11,7 +11,7 @@ from test_parity_gpu import _compare_all
 pytestmark = pytest.mark.gpu
 
 # T, d, r = m
-SHAPES = [(2048, 2048, 16), (2049, 2048, 16), (700, 1408, 16), (2048, 512, 32), (2049, 512, 32), (1000, 768, 32),
+SHAPES = [(2048, 2048, 16), (2049, 2048, 16), (700, 1408, 16), (2048, 1024, 32), (2049, 1024, 32), (1000, 768, 32),
           (520, 2048, 64), (520, 1920, 64), (300, 256, 64), (260, 512, 128)]
 
 
