@@ -106,6 +106,15 @@ inline bool ns_fused_ok(int64_t rows, int64_t cols)
     return sd <= kNsMaxSd && ld <= (1 << 20) && ns_layout(ns_sdp(sd), ld).bytes <= kNsMaxSmem;
 }
 
+// four consecutive elements as fp32
+__device__ __forceinline__ float4 ns_load4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+__device__ __forceinline__ float4 ns_load4(const __nv_bfloat16 *p)
+{
+    const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p));
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xFFFF0000u));
+}
+
 // SDP: sd rounded up to 16 (the padding rows and columns of X are zeros and stay zeros)
 template <int SDP, typename TG>
 __global__ void __launch_bounds__(kNsThreads, 1)
@@ -126,38 +135,45 @@ __global__ void __launch_bounds__(kNsThreads, 1)
         if (L.cl > 1) cluster_sync();
         else __syncthreads();
     };
-    // element e of this CTA's part in memory order: (row i, column l) of the wide orientation
-    const int ne = sd * nl;
+    // four consecutive elements of this CTA's part in memory order (sd, ld and nl are multiples of 8):
+    // tall, row i .. i + 3 of column l of the wide orientation; wide, row i, columns l .. l + 3
+    const int nq = sd * nl / 4;
     auto place = [&](int e, int &i, int &l) -> int64_t {
-        if (tall) {
-            l = e / sd;
-            i = e - l * sd;
-            return (l0 + l) * (int64_t)sd + i;
-        }
-        i = e / nl;
-        l = e - i * nl;
-        return (int64_t)i * ld + l0 + l;
+        const int per = (tall ? sd : nl) / 4;
+        const int a = e / per, b = 4 * (e - a * per);
+        i = tall ? b : a;
+        l = tall ? a : b;
+        return tall ? (l0 + l) * (int64_t)sd + i : (int64_t)i * ld + l0 + l;
     };
+    auto load4 = [&](int e, int &i, int &l) { return ns_load4(G + place(e, i, l)); };
     // ||G||_F^2: squares in fp32 with their rounding errors carried along (two-term sums, ~2^-46
     // relative), or in fp64 where they leave fp32's range
     double s;
     {
         float hi = 0.0f, lo = 0.0f;
-        for (int e = tid; e < ne; e += kNsThreads) {
+#pragma unroll 4
+        for (int e = tid; e < nq; e += kNsThreads) {
             int i, l;
-            const float v = to_f32(G[place(e, i, l)]);
-            const float p = v * v, pe = fmaf(v, v, -p);
-            const float t = hi + p, bb = t - hi;
-            lo += (hi - (t - bb)) + (p - bb) + pe;
-            hi = t;
+            const float4 v4 = load4(e, i, l);
+            const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float p = v[k] * v[k], pe = fmaf(v[k], v[k], -p);
+                const float t = hi + p, bb = t - hi;
+                lo += (hi - (t - bb)) + (p - bb) + pe;
+                hi = t;
+            }
         }
         s = (double)hi + (double)lo;
         if (!(hi < 1e37f)) {   // overflow (or NaN): again in fp64
             s = 0.0;
-            for (int e = tid; e < ne; e += kNsThreads) {
+            for (int e = tid; e < nq; e += kNsThreads) {
                 int i, l;
-                const double v = to_f32(G[place(e, i, l)]);
-                s = fma(v, v, s);
+                const float4 v = load4(e, i, l);
+                s = fma((double)v.x, (double)v.x, s);
+                s = fma((double)v.y, (double)v.y, s);
+                s = fma((double)v.z, (double)v.z, s);
+                s = fma((double)v.w, (double)v.w, s);
             }
         }
     }
@@ -181,10 +197,20 @@ __global__ void __launch_bounds__(kNsThreads, 1)
     s = 0.0;
     for (int p = 0; p < L.cl; ++p) s += nslot[p];
     const float inv = (float)(1.0 / (sqrt(s) + (double)eps));
-    for (int e = tid; e < ne; e += kNsThreads) {
+#pragma unroll 4
+    for (int e = tid; e < nq; e += kNsThreads) {
         int i, l;
-        const float v = to_f32(G[place(e, i, l)]);
-        *reinterpret_cast<__nv_bfloat16 *>(sm + L.x + i * L.xs + 2 * l) = __float2bfloat16_rn(v * inv);
+        const float4 v = load4(e, i, l);
+        uint8_t *x = sm + L.x + i * L.xs + 2 * l;
+        const uint32_t p01 = pack_bf16(v.x * inv, v.y * inv), p23 = pack_bf16(v.z * inv, v.w * inv);
+        if (tall) {
+            *reinterpret_cast<uint16_t *>(x) = (uint16_t)p01;
+            *reinterpret_cast<uint16_t *>(x + L.xs) = (uint16_t)(p01 >> 16);
+            *reinterpret_cast<uint16_t *>(x + 2 * L.xs) = (uint16_t)p23;
+            *reinterpret_cast<uint16_t *>(x + 3 * L.xs) = (uint16_t)(p23 >> 16);
+        } else {
+            *reinterpret_cast<uint2 *>(x) = make_uint2(p01, p23);
+        }
     }
     __syncthreads();
 
@@ -317,10 +343,18 @@ __global__ void __launch_bounds__(kNsThreads, 1)
         }
         __syncthreads();
     }
-    for (int e = tid; e < ne; e += kNsThreads) {
+    for (int e = tid; e < nq; e += kNsThreads) {
         int i, l;
         const int64_t at = place(e, i, l);
-        out[at] = *reinterpret_cast<const __nv_bfloat16 *>(sm + L.x + i * L.xs + 2 * l);
+        const uint8_t *x = sm + L.x + i * L.xs + 2 * l;
+        uint2 v;
+        if (tall) {
+            auto get = [&](int k) { return (uint32_t) * reinterpret_cast<const uint16_t *>(x + k * L.xs); };
+            v = make_uint2(get(0) | get(1) << 16, get(2) | get(3) << 16);
+        } else {
+            v = *reinterpret_cast<const uint2 *>(x);
+        }
+        *reinterpret_cast<uint2 *>(out + at) = v;
     }
     sync_all();   // no CTA leaves while another may still write into it
 }
