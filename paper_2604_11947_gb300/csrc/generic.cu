@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(256) k_rmsnorm(const E *__restrict__ Y, const 
 // the dgamma sums of the columns it owns in shared memory (no two threads touch a column), so the
 // result does not depend on timing or on the device. The second pass over the row re-reads it
 // (from L1 / L2). dY may equal dY_out (read before written by the same thread) or be null.
-constexpr int kNormBwdBlocks = 1024;   // ~7 resident per SM on 152 SMs: rows in flight hide the load latency
+constexpr int kNormBwdBlocks = 608;   // four per SM on 152 SMs (a fixed number: the sums' order does not depend on the device)
 constexpr int kNormBwdMaxD = 16384;
 
 template <typename E, int V> struct VecOf;
@@ -432,6 +432,8 @@ __global__ void __launch_bounds__(256) k_rmsnorm_bwd(const E *__restrict__ Y, co
     extern __shared__ float dgs[];   // d: this block's dgamma sums, column j owned by thread (j / V) % 256
     __shared__ float2 part[2][8];
     using L = VecOf<E, V>;
+    griddep_wait();
+    griddep_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t nv = d / V;
     for (int64_t q = tid; q < nv; q += 256)
@@ -507,55 +509,63 @@ __global__ void __launch_bounds__(256) k_rmsnorm_bwd(const E *__restrict__ Y, co
     for (int64_t j = tid; j < d; j += 256) dg_part[(int64_t)blockIdx.x * d + j] = dgs[j];
 }
 
-// The vector path for rows of at most 256 * KV vectors: each thread keeps its vectors of Y, dN and
-// dY (as loaded, 16 bytes each) in registers from the first pass to the second, so a row costs one
-// trip to memory, and loads dY with Y and dN. The same sums in the same order as k_rmsnorm_bwd, so
-// the same bits.
+// The vector path for rows of at most 256 * KV vectors: each thread keeps its vectors of Y, dN and dY (as
+// loaded, 16 bytes each) in registers from the first pass to the second, so a row costs one trip to memory,
+// with the next row's loads in flight meanwhile; gamma and the dgamma sums of the thread's columns stay in
+// registers too. The same sums in the same order as k_rmsnorm_bwd, so the same bits. Bound by memory (4 d
+// elements a row): T = 16384, d = 2048 59 us (4.5 TB/s) without the prefetch and with the dgamma sums in
+// shared memory.
 template <typename E, int V, int KV>
-__global__ void __launch_bounds__(256) k_rmsnorm_bwd_reg(const E *__restrict__ Y, const E *__restrict__ gamma, float eps,
-                                                         const E *__restrict__ dN, const E *dY, E *dYo,
-                                                         float *__restrict__ dg_part, int64_t rows, int64_t d)
+__global__ void __launch_bounds__(256, KV == 1 ? 4 : KV == 2 ? 2 : 1)
+    k_rmsnorm_bwd_reg(const E *__restrict__ Y, const E *__restrict__ gamma, float eps, const E *__restrict__ dN,
+                      const E *dY, E *dYo, float *__restrict__ dg_part, int64_t rows, int64_t d)
 {
-    extern __shared__ float dgs[];
     __shared__ float2 part[2][8];
     using L = VecOf<E, V>;
+    griddep_wait();
+    griddep_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t nv = d / V;
+    const int nv = (int)(d / V);
+    float acc[KV][V];
+    uint4 rg[KV];
 #pragma unroll
     for (int k = 0; k < KV; ++k) {
-        const int64_t q = tid + 256 * k;
-        if (q < nv)
+        const int q = tid + 256 * k;
+        rg[k] = q < nv ? *reinterpret_cast<const uint4 *>(gamma + q * V) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-            for (int i = 0; i < V; ++i) dgs[q * V + i] = 0.0f;
+        for (int i = 0; i < V; ++i) acc[k][i] = 0.0f;
     }
     const int64_t r0 = rows * blockIdx.x / gridDim.x, r1 = rows * (blockIdx.x + 1) / gridDim.x;
-    for (int64_t t = r0; t < r1; ++t) {
-        uint4 ry[KV], rn[KV], ro[KV];
-#pragma unroll
-        for (int k = 0; k < KV; ++k) {   // every load of the row in flight before the first use
-            const int64_t q = tid + 256 * k;
-            if (q < nv) {
-                ry[k] = *reinterpret_cast<const uint4 *>(Y + t * d + q * V);
-                rn[k] = *reinterpret_cast<const uint4 *>(dN + t * d + q * V);
-                ro[k] = dY ? *reinterpret_cast<const uint4 *>(dY + t * d + q * V) : make_uint4(0u, 0u, 0u, 0u);
-            }
-        }
-        float sy = 0.0f, sg = 0.0f;
+    uint4 ry[KV], rn[KV], ro[KV];
+    auto load = [&](int64_t t, uint4 (&y)[KV], uint4 (&n)[KV], uint4 (&o)[KV]) {
 #pragma unroll
         for (int k = 0; k < KV; ++k) {
-            const int64_t q = tid + 256 * k;
+            const int q = tid + 256 * k;
             if (q < nv) {
+                y[k] = *reinterpret_cast<const uint4 *>(Y + t * d + q * V);
+                n[k] = *reinterpret_cast<const uint4 *>(dN + t * d + q * V);
+                o[k] = dY ? *reinterpret_cast<const uint4 *>(dY + t * d + q * V) : make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+    };
+    if (r0 < r1) load(r0, ry, rn, ro);
+    for (int64_t t = r0; t < r1; ++t) {
+        uint4 ny[KV], nn[KV], no[KV];
+        if (t + 1 < r1) load(t + 1, ny, nn, no);   // (dY_out may be dY: each row is read before it is written)
+        float sy = 0.0f, sg = 0.0f;
+#pragma unroll
+        for (int k = 0; k < KV; ++k)
+            if (tid + 256 * k < nv) {
                 float a[V], b[V], gm[V];
                 L::unpack(ry[k], a);
                 L::unpack(rn[k], b);
-                L::load(gamma + q * V, gm);
+                L::unpack(rg[k], gm);
 #pragma unroll
                 for (int i = 0; i < V; ++i) {
                     sy = fmaf(a[i], a[i], sy);
                     sg = fmaf(b[i] * gm[i], a[i], sg);
                 }
             }
-        }
         for (int o = 16; o > 0; o >>= 1) {
             sy += __shfl_xor_sync(0xffffffffu, sy, o);
             sg += __shfl_xor_sync(0xffffffffu, sg, o);
@@ -573,44 +583,48 @@ __global__ void __launch_bounds__(256) k_rmsnorm_bwd_reg(const E *__restrict__ Y
         const float kk = s * s * s * Sg / (float)d;
 #pragma unroll
         for (int k = 0; k < KV; ++k) {
-            const int64_t q = tid + 256 * k;
+            const int q = tid + 256 * k;
             if (q < nv) {
-                float a[V], b[V], gm[V], o[V], acc[V];
+                float a[V], b[V], gm[V], o[V];
                 L::unpack(ry[k], a);
                 L::unpack(rn[k], b);
                 L::unpack(ro[k], o);
-                L::load(gamma + q * V, gm);
-#pragma unroll
-                for (int i = 0; i < V; i += 4) {
-                    const float4 u = *reinterpret_cast<const float4 *>(dgs + q * V + i);
-                    acc[i] = u.x; acc[i + 1] = u.y; acc[i + 2] = u.z; acc[i + 3] = u.w;
-                }
+                L::unpack(rg[k], gm);
 #pragma unroll
                 for (int i = 0; i < V; ++i) {
                     o[i] += s * (b[i] * gm[i]) - a[i] * kk;
-                    acc[i] = fmaf(b[i], a[i] * s, acc[i]);
+                    acc[k][i] = fmaf(b[i], a[i] * s, acc[k][i]);
                 }
-#pragma unroll
-                for (int i = 0; i < V; i += 4)
-                    *reinterpret_cast<float4 *>(dgs + q * V + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
                 L::store(dYo + t * d + q * V, o);
             }
+            ry[k] = ny[k];
+            rn[k] = nn[k];
+            ro[k] = no[k];
         }
     }
-    __syncthreads();
-    for (int64_t j = tid; j < d; j += 256) dg_part[(int64_t)blockIdx.x * d + j] = dgs[j];
+#pragma unroll
+    for (int k = 0; k < KV; ++k) {
+        const int q = tid + 256 * k;
+        if (q < nv)
+#pragma unroll
+            for (int i = 0; i < V; i += 4)
+                *reinterpret_cast<float4 *>(dg_part + (int64_t)blockIdx.x * d + q * V + i) =
+                    make_float4(acc[k][i], acc[k][i + 1], acc[k][i + 2], acc[k][i + 3]);
+    }
 }
 
 // dgamma[j] = the blocks' partials summed by a fixed two-level tree: warp w of a CTA sums the
 // partials of blocks [w G, (w + 1) G) in block order (eight loads in flight) for the CTA's 32
-// columns, then the eight group sums are added in group order. CTA x covers columns 32 x .. + 31.
-__global__ void __launch_bounds__(256) k_rmsnorm_dgamma(const float *__restrict__ dg_part, int nblocks, int64_t d,
+// columns, then the 32 group sums are added in group order. CTA x covers columns 32 x .. + 31.
+__global__ void __launch_bounds__(1024) k_rmsnorm_dgamma(const float *__restrict__ dg_part, int nblocks, int64_t d,
                                                         float *__restrict__ dgamma)
 {
-    __shared__ float gs[8][32];
+    __shared__ float gs[32][32];
+    griddep_wait();
+    griddep_launch_dependents();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t j = (int64_t)blockIdx.x * 32 + lane;
-    const int G = (nblocks + 7) / 8;
+    const int G = (nblocks + 31) / 32;
     const int b0 = w * G, b1 = b0 + G < nblocks ? b0 + G : nblocks;
     float a = 0.0f;
     if (j < d) {
@@ -629,7 +643,7 @@ __global__ void __launch_bounds__(256) k_rmsnorm_dgamma(const float *__restrict_
     if (w == 0 && j < d) {
         float t = 0.0f;
 #pragma unroll
-        for (int g = 0; g < 8; ++g) t += gs[g][lane];
+        for (int g = 0; g < 32; ++g) t += gs[g][lane];
         dgamma[j] = t;
     }
 }
@@ -654,29 +668,32 @@ cudaError_t generic_rmsnorm_bwd(const resbm_desc &d, const void *Y, const void *
         // the register-cached vector path up to 4 vectors a thread (bf16 d <= 8192, fp32 d <= 4096)
         const int64_t nv = d.d / (d.dtype == RESBM_F32 ? 4 : 8);
         const int kv = !vec ? 0 : nv <= 256 ? 1 : nv <= 512 ? 2 : nv <= 1024 ? 4 : 0;
-        if (d.dtype == RESBM_F32) {
-            auto k = kv == 1 ? k_rmsnorm_bwd_reg<float, 4, 1> : kv == 2 ? k_rmsnorm_bwd_reg<float, 4, 2>
-                   : kv == 4 ? k_rmsnorm_bwd_reg<float, 4, 4> : vec ? k_rmsnorm_bwd<float, 4> : k_rmsnorm_bwd<float, 1>;
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e == cudaSuccess)
-                k<<<nb, 256, smem, c.stream>>>((const float *)Y, (const float *)gamma, eps, (const float *)dN,
-                                              (const float *)dY, (float *)dY_out, part, d.T, d.d);
-        } else {
-            using bf = __nv_bfloat16;
-            auto k = kv == 1 ? k_rmsnorm_bwd_reg<bf, 8, 1> : kv == 2 ? k_rmsnorm_bwd_reg<bf, 8, 2>
-                   : kv == 4 ? k_rmsnorm_bwd_reg<bf, 8, 4> : vec ? k_rmsnorm_bwd<bf, 8> : k_rmsnorm_bwd<bf, 1>;
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e == cudaSuccess)
-                k<<<nb, 256, smem, c.stream>>>((const bf *)Y, (const bf *)gamma, eps, (const bf *)dN, (const bf *)dY,
-                                              (bf *)dY_out, part, d.T, d.d);
-        }
+        // (the register-cached forms keep the dgamma sums in registers)
+        auto run = [&](auto k, auto tag) -> cudaError_t {
+            using E = decltype(tag);
+            const size_t sm = kv ? 0 : smem;
+            if (sm) {
+                const cudaError_t a = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                if (a != cudaSuccess) return a;
+            }
+            return launch_pdl(k, dim3(nb), dim3(256), sm, c, (const E *)Y, (const E *)gamma, eps, (const E *)dN,
+                              (const E *)dY, (E *)dY_out, part, d.T, d.d);
+        };
+        using bf = __nv_bfloat16;
+        if (d.dtype == RESBM_F32)
+            e = run(kv == 1 ? k_rmsnorm_bwd_reg<float, 4, 1> : kv == 2 ? k_rmsnorm_bwd_reg<float, 4, 2>
+                    : kv == 4 ? k_rmsnorm_bwd_reg<float, 4, 4> : vec ? k_rmsnorm_bwd<float, 4> : k_rmsnorm_bwd<float, 1>, 0.0f);
+        else
+            e = run(kv == 1 ? k_rmsnorm_bwd_reg<bf, 8, 1> : kv == 2 ? k_rmsnorm_bwd_reg<bf, 8, 2>
+                    : kv == 4 ? k_rmsnorm_bwd_reg<bf, 8, 4> : vec ? k_rmsnorm_bwd<bf, 8> : k_rmsnorm_bwd<bf, 1>, bf());
         count_launches(1);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     const int64_t gb = (d.d + 31) / 32;
     if (d.T > 0) {
-        k_rmsnorm_dgamma<<<(unsigned)gb, 256, 0, c.stream>>>(part, nb, d.d, dgamma);
+        e = launch_pdl(k_rmsnorm_dgamma, dim3((unsigned)gb), dim3(1024), 0, c, (const float *)part, nb, d.d, dgamma);
+        if (e != cudaSuccess) return e;
     } else {
         e = cudaMemsetAsync(dgamma, 0, (size_t)d.d * sizeof(float), c.stream);
         if (e != cudaSuccess) return e;

@@ -18,6 +18,24 @@ struct Ctx {
     int sm_count;
 };
 
+// A launch with programmatic stream serialization (see launch_clustered in tc.cu): the kernel waits for its
+// predecessor itself (griddep_wait).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, const Ctx &c, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c.stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // Bump-allocates 256-byte aligned regions out of the caller's workspace (or, with a null
 // base, only measures them).
 struct WsCarver {
