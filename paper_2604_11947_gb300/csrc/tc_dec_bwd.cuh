@@ -107,8 +107,6 @@ __global__ void __launch_bounds__(192, 1)
               const __grid_constant__ CUtensorMap tm_yr, const DecBwdArgs a)
 {
     using C = DecBwdCfg<M_>;
-    if (!a.after_independent) griddep_wait();   // the previous kernel of the stream has completed
-    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ uint64_t y_full[C::NSY], y_empty[C::NSY], w_full[C::NW], w_empty[C::NW];
@@ -166,7 +164,13 @@ __global__ void __launch_bounds__(192, 1)
         fence_mbar_init();
         xg.arm_first();
     }
+    // Barriers, TMEM and (in clusters) the peers are set up before the wait for the previous kernel, whose last
+    // CTAs may still run: only what follows touches global memory.
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_sh), C::TMEM_COLS);
+    __syncthreads();
+    if (C::CLMAX > 1 && xg.cl > 1) cluster_sync();   // every CTA's barriers are initialized before any exchange
+    if (!a.after_independent) griddep_wait();   // the previous kernel of the stream has completed
+    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     if (warp >= 2) {  // Wd1 (r x m) and Wd1^T (m x r) as swizzled K-major operands
         const int et = threadIdx.x - 64;
         for (int e = et; e < C::R * C::M; e += 128) {
@@ -179,7 +183,6 @@ __global__ void __launch_bounds__(192, 1)
     }
     tc_fence_before();
     __syncthreads();
-    if (C::CLMAX > 1 && xg.cl > 1) cluster_sync();   // every CTA's barriers are initialized before any exchange
     tc_fence_after();
     const uint32_t tmem = tmem_base_sh;
 

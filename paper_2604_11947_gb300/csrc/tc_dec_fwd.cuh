@@ -123,8 +123,6 @@ __global__ void __launch_bounds__(320, 1)
 {
     using C = DecFwdCfg<M_>;
     static_assert(NORM >= 0 && NORM <= 2, "0: Y; 1: Y and row sums of squares; 2: the normalised rows");
-    griddep_wait();               // the previous kernel of the stream has completed
-    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ uint64_t w_full[C::NSTAGE], w_empty[C::NSTAGE];
@@ -161,7 +159,11 @@ __global__ void __launch_bounds__(320, 1)
         mbar_init(smem_u32(&done_bar), 1);
         fence_mbar_init();
     }
+    // Barriers and TMEM are set up before the wait for the previous kernel, whose last
+    // CTAs may still run: only what follows touches global memory.
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_sh), C::TMEM_COLS);
+    griddep_wait();               // the previous kernel of the stream has completed
+    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     if (warp >= 2) {  // Wd1^T (m x r) as a swizzled K-major operand: NB blocks of GB-byte rows
         for (int e = threadIdx.x - 64; e < C::R * C::M; e += C::EPI) {
             const int k = e / C::M, n = e % C::M;   // Wd1[k][n]

@@ -91,8 +91,6 @@ __global__ void __launch_bounds__(192, 1)
               const EncBwdArgs a)
 {
     using C = EncBwdCfg<M_>;
-    griddep_wait();               // the previous kernel of the stream has completed
-    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ uint64_t f_full[C::NSF], f_empty[C::NSF], w_full[C::NW], w_empty[C::NW];
@@ -150,7 +148,13 @@ __global__ void __launch_bounds__(192, 1)
         fence_mbar_init();
         xg.arm_first();
     }
+    // Barriers, TMEM and (in clusters) the peers are set up before the wait for the previous kernel, whose last
+    // CTAs may still run: only what follows touches global memory.
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_sh), C::TMEM_COLS);
+    __syncthreads();
+    if (C::CLMAX > 1 && xg.cl > 1) cluster_sync();   // every CTA's barriers are initialized before any exchange
+    griddep_wait();               // the previous kernel of the stream has completed
+    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     if (warp >= 2) {  // We2 (m x r) as a swizzled K-major operand
         for (int e = threadIdx.x - 64; e < C::M * C::R; e += 128)
             *reinterpret_cast<__nv_bfloat16 *>(smem + C::OFF_WE2 + swz_offset(e / C::R, 2 * (e % C::R), C::RB)) = a.We2[e];
@@ -158,7 +162,6 @@ __global__ void __launch_bounds__(192, 1)
     }
     tc_fence_before();
     __syncthreads();
-    if (C::CLMAX > 1 && xg.cl > 1) cluster_sync();   // every CTA's barriers are initialized before any exchange
     tc_fence_after();
     const uint32_t tmem = tmem_base_sh;
 

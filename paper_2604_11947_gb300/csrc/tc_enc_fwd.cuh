@@ -106,8 +106,6 @@ __global__ void __launch_bounds__(192, 1)
               const __grid_constant__ CUtensorMap tm_we1, const EncFwdArgs a)
 {
     using C = EncFwdCfg<M_>;
-    griddep_wait();               // the previous kernel of the stream has completed
-    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ uint64_t full[C::NST], empty[C::NST];
@@ -147,8 +145,17 @@ __global__ void __launch_bounds__(192, 1)
         fence_mbar_init();
         // the peer's partial P of the shared tile: 128 rows of m fp32
         if (wk.recv_last) mbar_expect_tx(smem_u32(&rx_full), 128 * C::M * 4);
+        tma_prefetch_desc(&tm_f128);
+        tma_prefetch_desc(&tm_f16);
+        tma_prefetch_desc(&tm_we1);
     }
+    // Barriers, TMEM and (in clusters) the peers are set up before the wait for the previous kernel, whose last
+    // CTAs may still run: only what follows touches global memory.
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_sh), C::TMEM_COLS);
+    __syncthreads();
+    if (cl > 1) cluster_sync();   // the peer's barrier is armed before anything is pushed
+    griddep_wait();               // the previous kernel of the stream has completed
+    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     if (warp >= 2 && want_b) {  // We2^T (r x m) as a swizzled K-major operand: NB blocks of GB-byte rows
         for (int e = threadIdx.x - 64; e < C::M * C::R; e += 128) {
             const int k = e / C::R, n = e % C::R;   // We2[k][n]
@@ -160,7 +167,6 @@ __global__ void __launch_bounds__(192, 1)
     }
     tc_fence_before();
     __syncthreads();
-    if (cl > 1) cluster_sync();   // the peer's barrier is armed before anything is pushed
     tc_fence_after();
     const uint32_t tmem = tmem_base_sh;
 
@@ -168,9 +174,6 @@ __global__ void __launch_bounds__(192, 1)
         // ---------------- producer ----------------
         if (elect_one()) {
             const uint64_t stream_pol = l2_evict_first();   // read once
-            tma_prefetch_desc(&tm_f128);
-            tma_prefetch_desc(&tm_f16);
-            tma_prefetch_desc(&tm_we1);
             uint32_t it = 0;
             bool ok = true;
             for (int ti = 0; ti < ntiles && ok; ++ti) {

@@ -370,8 +370,6 @@ __global__ void __launch_bounds__(320, 1)
     static_assert(!(BM2 && (ALO || PAIR)), "256-row units without hi + lo A or pairs");
     static_assert(!(TS && (ENCP || BM2)), "TMA-store epilogue: plain 128-row units or pairs");
     constexpr int MH = BM2 ? 2 : 1;   // 128-row halves per unit (g.nm counts units of 128 * MH rows)
-    griddep_wait();               // the previous kernel of the stream has completed
-    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ uint64_t full[C::NST], empty[C::NST], acc_full[2], acc_empty[2], done_bar;
@@ -419,6 +417,10 @@ __global__ void __launch_bounds__(320, 1)
     __syncthreads();
     if (PAIR) cluster_sync();   // the peer's barriers exist before anything arrives on them
     tc_fence_after();
+    // Barriers, TMEM and the pair were set up before the wait for the previous kernel, whose last
+    // CTAs may still run: only what follows touches global memory.
+    griddep_wait();               // the previous kernel of the stream has completed
+    griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     const uint32_t tmem = tmem_base_sh;
 
     if (warp == 0) {
