@@ -391,11 +391,13 @@ resbm_status run_encode_fwd(const resbm_desc &d, const void *X, const void *F, c
     return finish(generic_encode_fwd(d, X, F, We1, We2, B, P, ws, c));
 }
 
-// on_tc (nullable): set when the tensor-core kernel (one launch, no scratch) ran
+// on_tc (nullable): set when the tensor-core kernel (one launch, no scratch) ran; kept_q (nullable): set when
+// the chain of products ran and left Q and phi(Q) in ws for the decoder backward
 resbm_status run_decode_fwd(const resbm_desc &d, const void *B, const void *Wd1, const void *Wd2,
-                            void *Y, void *ws, const Ctx &c, bool *on_tc = nullptr)
+                            void *Y, void *ws, const Ctx &c, bool *on_tc = nullptr, bool *kept_q = nullptr)
 {
     if (on_tc) *on_tc = false;
+    if (kept_q) *kept_q = false;
     if (d.T == 0) return RESBM_OK;
     if (use_tc(d, RESBM_OP_DECODE_FWD)) {
         cudaError_t e = tc_decode_fwd(d, B, Wd1, Wd2, Y, ws, c);
@@ -405,8 +407,12 @@ resbm_status run_decode_fwd(const resbm_desc &d, const void *B, const void *Wd1,
         }
     }
     if (use_gemm(d, RESBM_OP_DECODE_FWD)) {
-        cudaError_t e = gemm_decode_fwd(d, B, Wd1, Wd2, Y, ws, c);
-        if (e != cudaErrorNotSupported) return finish(e);
+        const bool keep = kept_q && !use_tc(d, RESBM_OP_DECODE_BWD);
+        cudaError_t e = gemm_decode_fwd(d, B, Wd1, Wd2, Y, ws, c, keep);
+        if (e != cudaErrorNotSupported) {
+            if (keep) *kept_q = e == cudaSuccess;
+            return finish(e);
+        }
     }
     return finish(generic_decode_fwd(d, B, Wd1, Wd2, Y, ws, c));
 }
@@ -414,7 +420,7 @@ resbm_status run_decode_fwd(const resbm_desc &d, const void *B, const void *Wd1,
 // after_independent: see tc_decode_bwd (the boundary step, right after its decoder forward)
 resbm_status run_decode_bwd(const resbm_desc &d, const void *dY, const void *B, const void *Wd1,
                             const void *Wd2, void *dB, float *dWd1, float *dWd2, void *ws,
-                            const Ctx &c, bool after_independent = false)
+                            const Ctx &c, bool after_independent = false, bool have_q = false)
 {
     if (d.T == 0) {
         resbm_status s = zero_f32(dWd1, d.r * d.m, c.stream);
@@ -425,7 +431,7 @@ resbm_status run_decode_bwd(const resbm_desc &d, const void *dY, const void *B, 
         if (e != cudaErrorNotSupported) return finish(e);
     }
     if (use_gemm(d, RESBM_OP_DECODE_BWD)) {
-        cudaError_t e = gemm_decode_bwd(d, dY, B, Wd1, Wd2, dB, dWd1, dWd2, ws, c);
+        cudaError_t e = gemm_decode_bwd(d, dY, B, Wd1, Wd2, dB, dWd1, dWd2, ws, c, have_q);
         if (e != cudaErrorNotSupported) return finish(e);
     }
     if (can_tc(d, RESBM_OP_DECODE_BWD)) {   // gradients that are not 16-byte aligned
@@ -563,15 +569,15 @@ resbm_status enqueue_step(const resbm_desc &d, const resbm_step_args &a, void *w
         inner = l.inner;
     }
     if (s == RESBM_OK) s = run_encode_fwd(e, a.X, a.F, a.We1, We2, a.B, P, inner, c);
-    bool dec_fwd_tc = false;
-    if (s == RESBM_OK) s = run_decode_fwd(e, a.B, Wd1, a.Wd2, a.Y, inner, c, &dec_fwd_tc);
+    bool dec_fwd_tc = false, kept_q = false;
+    if (s == RESBM_OK) s = run_decode_fwd(e, a.B, Wd1, a.Wd2, a.Y, inner, c, &dec_fwd_tc, &kept_q);
     if (s == RESBM_OK && fwd_done) s = finish(cudaEventRecord(fwd_done, c.stream));
     if (s == RESBM_OK && bwd_ready) s = finish(cudaStreamWaitEvent(c.stream, bwd_ready, 0));
     // the decoder backward reads dY and B, not the decoder forward's Y, and the tensor-core
     // decoder forward uses no scratch: with nothing queued between the two kernels the backward
     // starts as the forward's CTAs leave (tc_decode_bwd)
     const bool overlap = dec_fwd_tc && fwd_done == nullptr && bwd_ready == nullptr;
-    if (s == RESBM_OK) s = run_decode_bwd(e, a.dY, a.B, Wd1, a.Wd2, a.dB, dWd1, a.dWd2, inner, c, overlap);
+    if (s == RESBM_OK) s = run_decode_bwd(e, a.dY, a.B, Wd1, a.Wd2, a.dB, dWd1, a.dWd2, inner, c, overlap, kept_q);
     if (s == RESBM_OK)
         s = run_encode_bwd(e, a.dB, a.F, P, a.We1, We2, a.dF, a.dX, a.dWe1, dWe2, inner, c);
     return s;

@@ -341,7 +341,7 @@ tc::ReduceJob reduce_job(const float *part, int64_t slots, int64_t rows, int64_t
 {
     int64_t g = (rows * cols / 4 + 31) / 32;
     if (g > cap) g = cap;
-    return tc::ReduceJob{part, slots, rows, cols, out, transpose, out4, (int)(g < 1 ? 1 : g)};
+    return tc::ReduceJob{part, slots, rows, cols, out, transpose, out4, (int)(g < 1 ? 1 : g), nullptr};
 }
 cudaError_t launch_reduce(const tc::ReduceJob &small, tc::ReduceJob big, const Ctx &c)
 {
@@ -548,9 +548,9 @@ bool ts_enabled()
     return !(v && v[0] == '0' && v[1] == 0);
 }
 
-// The TMA-store form of an epilogue and its output maps: 1 for one bf16 output (Y, dF, B, dB), 2 for the
-// pre-activation and the activation's bf16 pair (P, A; Q, G; dQ; dP, A), 0 for the rest (fp32 outputs of
-// long sums, the Newton-Schulz steps), and for pointers or pitches TMA does not take.
+// The TMA-store form of an epilogue and its output maps: 1 for one bf16 output (Y, dF, B, dB, the Newton-Schulz
+// steps), 2 for the pre-activation and the activation's bf16 pair (P, A; Q, G; dQ; dP, A), 0 for the rest (fp32
+// outputs of long sums), and for pointers or pitches TMA does not take.
 int gemm_ts(const tc::GemmEp &ep, int64_t M, int64_t N, bool lo, GemmOutMaps *m)
 {
     if (!ts_enabled()) return 0;
@@ -565,6 +565,7 @@ int gemm_ts(const tc::GemmEp &ep, int64_t M, int64_t N, bool lo, GemmOutMaps *m)
     case tc::GEP_BF16:
     case tc::GEP_ADD_AUX:
     case tc::GEP_DF:
+    case tc::GEP_AXPBY:
         map(&m->o, ep.out, ep.ldo, false, 64);
         m->o2 = m->lo = m->o;
         return ok ? 1 : 0;
@@ -697,7 +698,7 @@ cudaError_t wgrad(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, 
 {
     const GemmForm fm = gemm_form(M, N, K, A_lo != nullptr, a_mn, c.sm_count, true);
     const int s = gemm_splits(M, N, K, c.sm_count, fm);
-    *job = tc::ReduceJob{nullptr, 0, 0, 0, nullptr, 0, 0, 0};
+    *job = tc::ReduceJob{};
     if (s <= 1 && !tr && al16(W)) return gemm(c, M, N, K, A, a_mn, B, b_mn, ep_of(tc::GEP_F32, 0, W, N), 1, A_lo, &fm);
     tc::GemmEp e = ep_of(tc::GEP_F32, 0, slots, N);
     e.split_stride = M * N;
@@ -713,7 +714,7 @@ cudaError_t wgrad(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, 
 cudaError_t reduce_jobs(const tc::ReduceJob &a, const tc::ReduceJob &b, const Ctx &c)
 {
     if (a.blocks == 0 && b.blocks == 0) return cudaSuccess;
-    const tc::ReduceJob none{nullptr, 0, 0, 0, nullptr, 0, 0, 0};
+    const tc::ReduceJob none{};
     const tc::ReduceJob &first = a.blocks ? a : none;
     const tc::ReduceJob &second = a.blocks ? (b.blocks ? b : none) : b;
     const int blocks = first.blocks + second.blocks;
@@ -960,12 +961,18 @@ cudaError_t gemm_encode_fwd(const resbm_desc &d, const void *X, const void *F, c
 }
 
 cudaError_t gemm_decode_fwd(const resbm_desc &d, const void *B, const void *Wd1, const void *Wd2, void *Y, void *ws,
-                            const Ctx &c)
+                            const Ctx &c, bool keep_q)
 {
     if (!al16(B) || !al16(Wd1) || !al16(Wd2) || !al16(Y) || !al16(ws)) return cudaErrorNotSupported;
-    const GemmWs w = gemm_ws(d, RESBM_OP_DECODE_FWD, c.sm_count, ws, true);
-    // G = phi(B . Wd1)
-    cudaError_t e = gemm(c, d.T, d.m, d.r, B, false, Wd1, true, ep_of(tc::GEP_ACT, d.act, w.G, d.m), 1);
+    const GemmWs w = gemm_ws(d, keep_q ? RESBM_OP_DECODE_BWD : RESBM_OP_DECODE_FWD, c.sm_count, ws, true);
+    // G = phi(B . Wd1); keep_q: with Q and G's remainder, where the decoder backward looks for them
+    tc::GemmEp e1 = ep_of(tc::GEP_ACT, d.act, w.G, d.m);
+    if (keep_q) {
+        e1.out2 = w.Q;
+        e1.ldo2 = d.m;
+        e1.lo = w.G_lo;
+    }
+    cudaError_t e = gemm(c, d.T, d.m, d.r, B, false, Wd1, true, e1, 1);
     if (e != cudaSuccess) return e;
     // Y = G . Wd2 (+ B on the first r columns: the zero-padding identity path)
     tc::GemmEp e2 = ep_of(tc::GEP_ADD_AUX, d.act, Y, d.d);
@@ -976,7 +983,7 @@ cudaError_t gemm_decode_fwd(const resbm_desc &d, const void *B, const void *Wd1,
 }
 
 cudaError_t gemm_decode_bwd(const resbm_desc &d, const void *dY, const void *B, const void *Wd1, const void *Wd2,
-                            void *dB, float *dWd1, float *dWd2, void *ws, const Ctx &c)
+                            void *dB, float *dWd1, float *dWd2, void *ws, const Ctx &c, bool have_q)
 {
     if (!al16(dY) || !al16(B) || !al16(Wd1) || !al16(Wd2) || !al16(dB) || !al16(dWd1) || !al16(dWd2) || !al16(ws))
         return cudaErrorNotSupported;
@@ -986,7 +993,7 @@ cudaError_t gemm_decode_bwd(const resbm_desc &d, const void *dY, const void *B, 
     e1.out2 = w.Q;
     e1.ldo2 = d.m;
     e1.lo = w.G_lo;
-    cudaError_t e = gemm(c, d.T, d.m, d.r, B, false, Wd1, true, e1, 1);
+    cudaError_t e = have_q ? cudaSuccess : gemm(c, d.T, d.m, d.r, B, false, Wd1, true, e1, 1);
     // dQ = (dY . Wd2^T) * phi'(Q)
     tc::GemmEp e2 = ep_of(tc::GEP_DACT, d.act, w.dQ, d.m);
     e2.aux = w.Q;
@@ -1144,6 +1151,8 @@ MatrixWs matrix_ws(int op, int64_t rows, int64_t cols, int sms, void *ws)
         w.X = cv.take<__nv_bfloat16>(rows * cols);
         w.A = cv.take<__nv_bfloat16>(sd * sd);
         w.Bm = cv.take<__nv_bfloat16>(sd * sd);
+        if (ld >= 2048) w.slots = cv.take<float>(slot_floats(sd, sd, ld, sms));   // (shorter: one launch is quicker)
+        if (slot_floats(sd, sd, ld, sms) == 0) w.slots = nullptr;
     } else {
         w.gram = cv.take<float>(sd * sd);
         w.slots = cv.take<float>(slot_floats(sd, sd, ld, sms));
@@ -1224,19 +1233,28 @@ cudaError_t tc_newton_schulz(int64_t rows, int64_t cols, const void *G, bool g_f
     const int64_t sd = wide ? rows : cols;
     for (int k = 0; k < steps && e == cudaSuccess; ++k) {
         // A = X X^T (wide) or X^T X (tall): the s x s Gram matrix of the iterate
-        e = wide ? gemm(c, sd, sd, cols, cur, false, cur, false, ep_of(tc::GEP_BF16, 0, w.A, sd), 1)
-                 : gemm(c, sd, sd, rows, cur, true, cur, true, ep_of(tc::GEP_BF16, 0, w.A, sd), 1);
+        // (split over the long side where it has few tiles: 512 x 512 from 8192 columns took four pairs 42 us)
+        tc::ReduceJob job{};
+        if (w.slots) {
+            e = wgrad(c, sd, sd, wide ? cols : rows, cur, cur, nullptr, w.slots, &job, nullptr, !wide, !wide, true);
+            job.transpose = 0;   // (wgrad's way by the slots; the Gram matrix is stored as it is)
+            job.out_bf16 = w.A;
+            if (e == cudaSuccess) e = reduce_jobs(job, tc::ReduceJob{}, c);
+        } else {
+            e = wide ? gemm(c, sd, sd, cols, cur, false, cur, false, ep_of(tc::GEP_BF16, 0, w.A, sd), 1)
+                     : gemm(c, sd, sd, rows, cur, true, cur, true, ep_of(tc::GEP_BF16, 0, w.A, sd), 1);
+        }
         // Bm = b A + c A A
         tc::GemmEp eb = ep_of(tc::GEP_AXPBY, 0, w.Bm, sd);
         eb.aux = w.A;
-        eb.lda = sd;
+        eb.lda = eb.aux_cols = sd;
         eb.alpha = coef[2];
         eb.beta = coef[1];
         if (e == cudaSuccess) e = gemm(c, sd, sd, sd, w.A, false, w.A, true, eb, 1);
         // X <- a X + Bm X (wide) or a X + X Bm (tall; Bm is symmetric)
         tc::GemmEp ex = ep_of(tc::GEP_AXPBY, 0, nxt, cols);
         ex.aux = cur;
-        ex.lda = cols;
+        ex.lda = ex.aux_cols = cols;
         ex.alpha = 1.0f;
         ex.beta = coef[0];
         if (e == cudaSuccess)
@@ -1260,7 +1278,7 @@ cudaError_t tc_effective_rank(int64_t rows, int64_t cols, const void *W, double 
     tc::ReduceJob job;
     cudaError_t e = tall ? wgrad(c, sd, sd, ld, W, W, w.gram, w.slots, &job)
                          : wgrad(c, sd, sd, ld, W, W, w.gram, w.slots, &job, nullptr, false, false);
-    if (e == cudaSuccess) e = reduce_jobs(job, tc::ReduceJob{nullptr, 0, 0, 0, nullptr, 0, 0, 0}, c);
+    if (e == cudaSuccess) e = reduce_jobs(job, tc::ReduceJob{}, c);
     if (e == cudaSuccess) {
         const bool small = sd <= tc::kLzSmallN;
         auto kernel = small ? tc::k_lanczos_small : tc::k_lanczos_top;

@@ -52,11 +52,13 @@ bool gemm_supported(const resbm_desc &d, int op);
 size_t gemm_ws_bytes(const resbm_desc &d, int op, int sms);
 cudaError_t gemm_encode_fwd(const resbm_desc &d, const void *X, const void *F, const void *We1,
                             const void *We2, void *B, float *P_save, void *ws, const Ctx &c);
+// keep_q (the boundary step, whose decoder backward follows on the same workspace): Q = B . Wd1 and phi(Q)
+// as a hi + lo pair stay there, and gemm_decode_bwd with have_q does not compute them again.
 cudaError_t gemm_decode_fwd(const resbm_desc &d, const void *B, const void *Wd1, const void *Wd2,
-                            void *Y, void *ws, const Ctx &c);
+                            void *Y, void *ws, const Ctx &c, bool keep_q = false);
 cudaError_t gemm_decode_bwd(const resbm_desc &d, const void *dY, const void *B, const void *Wd1,
                             const void *Wd2, void *dB, float *dWd1, float *dWd2, void *ws,
-                            const Ctx &c);
+                            const Ctx &c, bool have_q = false);
 cudaError_t gemm_encode_bwd(const resbm_desc &d, const void *dB, const void *F, const float *P_save,
                             const void *We1, const void *We2, void *dF, void *dX, float *dWe1,
                             float *dWe2, void *ws, const Ctx &c);

@@ -605,13 +605,16 @@ struct ReduceJob {
     float *out;
     int transpose, out4;
     int blocks;
+    __nv_bfloat16 *out_bf16;   // if set: the sums rounded to bf16 here instead (untransposed, 8-byte aligned)
 };
 
 // element e4 (four consecutive values) of the job's result
 __device__ __forceinline__ void reduce_store(const ReduceJob &j, int64_t e4, const float4 &t)
 {
     const int64_t e = 4 * e4;
-    if (j.transpose) {
+    if (j.out_bf16) {
+        reinterpret_cast<uint2 *>(j.out_bf16)[e4] = make_uint2(pack_bf16(t.x, t.y), pack_bf16(t.z, t.w));
+    } else if (j.transpose) {
         const int64_t rr = e / j.cols, cc = e - rr * j.cols;
         j.out[(cc + 0) * j.rows + rr] = t.x;
         j.out[(cc + 1) * j.rows + rr] = t.y;

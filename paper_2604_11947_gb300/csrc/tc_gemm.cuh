@@ -720,12 +720,18 @@ __global__ void __launch_bounds__(320, 1)
 #pragma unroll
                         for (int h = 0; h < CW / 32; ++h) {
                             const int64_t col = col0 + 32 * h;
-                            if (ep.mode == GEP_ADD_AUX && row < g.M && col < ep.aux_cols) {   // the identity path's columns
+                            // the identity path's columns; AXPBY: every column
+                            if ((ep.mode == GEP_ADD_AUX || ep.mode == GEP_AXPBY) && row < g.M && col < ep.aux_cols) {
                                 const int na = ep.aux_cols - col < 32 ? (int)(ep.aux_cols - col) : 32;
                                 float x[32];
                                 ld_bf16x32(static_cast<const __nv_bfloat16 *>(ep.aux) + row * ep.lda + col, x, na);
+                                if (ep.mode == GEP_AXPBY) {
 #pragma unroll
-                                for (int j = 0; j < 32; ++j) v[h][j] = j < na ? v[h][j] + x[j] : v[h][j];
+                                    for (int j = 0; j < 32; ++j) v[h][j] = fmaf(ep.alpha, v[h][j], ep.beta * x[j]);
+                                } else {
+#pragma unroll
+                                    for (int j = 0; j < 32; ++j) v[h][j] = j < na ? v[h][j] + x[j] : v[h][j];
+                                }
                             }
                             put_bf16(box, v[h], 64 * h, 128);
                         }
@@ -750,7 +756,8 @@ __global__ void __launch_bounds__(320, 1)
                         }
                         if (ep.mode == GEP_DACT) {
                             float dx[32];
-                            dact_fast_row<32>(ep.act, x, dx);
+                            if (ep.out2) act_dact_fast_row<32>(ep.act, x, x, dx);   // (one exponential for both)
+                            else dact_fast_row<32>(ep.act, x, dx);
 #pragma unroll
                             for (int j = 0; j < 32; ++j) v[0][j] *= dx[j];
                         } else {
@@ -766,7 +773,6 @@ __global__ void __launch_bounds__(320, 1)
                             store_box(tmol, box, col0, row0);
                         }
                         if (ep.mode == GEP_DACT && ep.out2) {   // A = phi(P)
-                            act_fast_row<32>(ep.act, x);
                             box = next_box();
                             put_bf16(box, x, 0, 64);
                             store_box(tmo2, box, col0, row0);

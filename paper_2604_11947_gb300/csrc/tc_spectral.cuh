@@ -55,10 +55,15 @@ __global__ void __launch_bounds__(256) k_scale_bf16(const T *__restrict__ x, int
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    s = 0.0;
-#pragma unroll
-    for (int w = 0; w < kSqBlocks / 32; ++w) s += red[w];
-    const float inv = (float)(1.0 / (sqrt(s) + (double)eps));
+    // (one thread's square root and division: fp64 units are few, 256 threads' took 10 us)
+    __shared__ float inv_sh;
+    if (threadIdx.x == 0) {
+        s = 0.0;
+        for (int w = 0; w < kSqBlocks / 32; ++w) s += red[w];
+        inv_sh = (float)(1.0 / (sqrt(s) + (double)eps));
+    }
+    __syncthreads();
+    const float inv = inv_sh;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         y[i] = __float2bfloat16_rn(ld_f(x, i) * inv);
 }
