@@ -549,16 +549,16 @@ bool ts_enabled()
 }
 
 // The TMA-store form of an epilogue and its output maps: 1 for one bf16 output (Y, dF, B, dB, the Newton-Schulz
-// steps), 2 for the pre-activation and the activation's bf16 pair (P, A; Q, G; dQ; dP, A), 0 for the rest (fp32
-// outputs of long sums), and for pointers or pitches TMA does not take.
-int gemm_ts(const tc::GemmEp &ep, int64_t M, int64_t N, bool lo, GemmOutMaps *m)
+// steps), 2 for the pre-activation and the activation's bf16 pair (P, A; Q, G; dQ; dP, A), or one fp32
+// output (the weight gradients' slots), 0 for the rest, and for pointers or pitches TMA does not take.
+int gemm_ts(const tc::GemmEp &ep, int64_t M, int64_t N, int splits, bool lo, GemmOutMaps *m)
 {
     if (!ts_enabled()) return 0;
     bool ok = true;
-    auto map = [&](CUtensorMap *t, const void *p, int64_t ld, bool f32, uint32_t cols) {
+    auto map = [&](CUtensorMap *t, const void *p, int64_t ld, bool f32, uint32_t cols, int64_t rows = 0) {
         const int64_t pitch = ld * (f32 ? 4 : 2);
         ok = ok && al16(p) && pitch % 16 == 0 &&
-             make_map(t, p, N, M, pitch, cols, 32, cols * (f32 ? 4 : 2) == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+             make_map(t, p, N, rows ? rows : M, pitch, cols, 32, cols * (f32 ? 4 : 2) == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                       f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
     };
     switch (ep.mode) {
@@ -569,10 +569,15 @@ int gemm_ts(const tc::GemmEp &ep, int64_t M, int64_t N, bool lo, GemmOutMaps *m)
         map(&m->o, ep.out, ep.ldo, false, 64);
         m->o2 = m->lo = m->o;
         return ok ? 1 : 0;
+    case tc::GEP_F32:   // (split: one slot of M rows after the other, so the boxes of 32 rows may not cross M)
+        if (ep.ldo != N || (splits > 1 && (M % 32 || ep.split_stride != M * N))) return 0;
+        map(&m->o, ep.out, ep.ldo, true, 32, M * splits);
+        m->o2 = m->lo = m->o;
+        return ok ? 2 : 0;
     case tc::GEP_P_A:
     case tc::GEP_ACT:
     case tc::GEP_DACT: {
-        if (lo) return 0;
+        if (lo || (ep.mode == tc::GEP_DACT && ep.lo && ep.out2)) return 0;   // (a box holds two bf16 outputs)
         const bool p_a = ep.mode == tc::GEP_P_A;
         const void *act = p_a ? ep.out2 : ep.out;   // the bf16 activation (or dQ, dP): always there
         map(p_a ? &m->o2 : &m->o, act, p_a ? ep.ldo2 : ep.ldo, false, 32);
@@ -630,7 +635,10 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
     }
     // TMA-store epilogues: on pairs, and for the products of up to 128 columns
     GemmOutMaps mo;
-    const int ts = (pair || bn == 128) && !a_mn && g.splits == 1 ? gemm_ts(ep, M, N, lo, &mo) : 0;
+    // (an fp32 output on pairs only: beside the boxes the 128-column products keep 5 stages instead of 6, and
+    // dWe1 of d = 8192, m = 128 went 84 -> 91 us)
+    const bool ts_ok = ep.mode == tc::GEP_F32 ? pair && !lo : (pair || bn == 128) && !a_mn && g.splits == 1;
+    const int ts = ts_ok ? gemm_ts(ep, M, N, g.splits, lo, &mo) : 0;
     if (ts && bn == 128) {
         if (ts == 2) return b_mn ? launch_gemm_t<128, false, true, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo)
                                  : launch_gemm_t<128, false, false, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo);
@@ -641,8 +649,9 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
     }
     if (pair) {
         cudaError_t e = cudaErrorNotSupported;
-        if (ts == 2) e = b_mn ? launch_gemm_t<256, false, true, false, false, true, false, 2>(ma, malo, mbm, g, ep, c, &mo)
-                              : launch_gemm_t<256, false, false, false, false, true, false, 2>(ma, malo, mbm, g, ep, c, &mo);
+        if (ts == 2 && a_mn) e = launch_gemm_t<256, true, true, false, false, true, false, 2>(ma, malo, mbm, g, ep, c, &mo);
+        else if (ts == 2) e = b_mn ? launch_gemm_t<256, false, true, false, false, true, false, 2>(ma, malo, mbm, g, ep, c, &mo)
+                                   : launch_gemm_t<256, false, false, false, false, true, false, 2>(ma, malo, mbm, g, ep, c, &mo);
         else if (ts && b_mn) e = lo ? launch_gemm_t<256, false, true, true, false, true, false, 1>(ma, malo, mbm, g, ep, c, &mo)
                                     : launch_gemm_t<256, false, true, false, false, true, false, 1>(ma, malo, mbm, g, ep, c, &mo);
         else if (ts) e = lo ? launch_gemm_t<256, false, false, true, false, true, false, 1>(ma, malo, mbm, g, ep, c, &mo)

@@ -134,8 +134,8 @@ struct GemmShape {
 // half of the B tile.
 // TS: the outputs leave by TMA stores from shared-memory boxes, two 4 KB boxes per epilogue warp (one
 // fills while the other's store reads it), each warp on its own: no barrier between warps. 1: one bf16
-// output in boxes of 32 rows x 64 columns (128-byte swizzle); 2: up to two bf16 and one fp32 output in
-// boxes of 32 rows x 32 columns (64- and 128-byte rows). Per-thread 16-byte stores put 32 different rows
+// output in boxes of 32 rows x 64 columns (128-byte swizzle); 2: an fp32 output in boxes of 32 rows x 32
+// columns and / or up to two bf16 outputs of 32 x 32 in one box (64-byte rows). Per-thread 16-byte stores put 32 different rows
 // in a warp instruction: they, not the products, set the pace where K is short.
 // ENCP: one box of 32 rows x 64 columns per warp (F as the partial P's operand, and for F's store) and
 // We1's rows of the unit's columns.
@@ -745,13 +745,14 @@ __global__ void __launch_bounds__(320, 1)
                         tmem_ld_wait();
                         tmem_regs_ready(v[0]);
                         if (last) release_acc(ab);
-                        float *f32 = static_cast<float *>(ep.mode == GEP_P_A ? ep.out : ep.mode == GEP_ACT ? ep.out2 : nullptr);
-                        if (f32) {   // P or Q
+                        float *f32 = static_cast<float *>(ep.mode == GEP_ACT ? ep.out2 : ep.mode == GEP_DACT ? nullptr : ep.out);
+                        if (f32) {   // P, Q, or a plain fp32 output
 #pragma unroll
                             for (int e = 0; e < 8; ++e)
                                 *reinterpret_cast<float4 *>(box + swz_offset((uint32_t)lane, 16 * e, 128)) =
                                     make_float4(v[0][4 * e], v[0][4 * e + 1], v[0][4 * e + 2], v[0][4 * e + 3]);
-                            store_box(ep.mode == GEP_P_A ? tmo : tmo2, box, col0, row0);
+                            store_box(ep.mode == GEP_ACT ? tmo2 : tmo, box, col0, row0 + (int64_t)ks * g.M);
+                            if (ep.mode == GEP_F32) continue;
                             box = next_box();
                         }
                         if (ep.mode == GEP_DACT) {
@@ -763,19 +764,23 @@ __global__ void __launch_bounds__(320, 1)
                         } else {
                             act_fast_row<32>(ep.act, v[0]);
                         }
+                        // the bf16 result in the box's first half, its remainder or A = phi(P) in the second
                         put_bf16(box, v[0], 0, 64);
-                        store_box(ep.mode == GEP_P_A ? tmo2 : tmo, box, col0, row0);
+                        const CUtensorMap *second = nullptr;
                         if (ep.lo) {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) v[0][j] -= __bfloat162float(__float2bfloat16_rn(v[0][j]));
-                            box = next_box();
-                            put_bf16(box, v[0], 0, 64);
-                            store_box(tmol, box, col0, row0);
+                            for (int j = 0; j < 32; ++j) x[j] = v[0][j] - __bfloat162float(__float2bfloat16_rn(v[0][j]));
+                            second = &tmol;
+                        } else if (ep.mode == GEP_DACT && ep.out2) {
+                            second = &tmo2;
                         }
-                        if (ep.mode == GEP_DACT && ep.out2) {   // A = phi(P)
-                            box = next_box();
-                            put_bf16(box, x, 0, 64);
-                            store_box(tmo2, box, col0, row0);
+                        if (second) put_bf16(box + C::BOX / 2, x, 0, 64);
+                        fence_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            tma_store_2d(ep.mode == GEP_P_A ? &tmo2 : &tmo, (int32_t)col0, (int32_t)row0, smem_u32(box));
+                            if (second) tma_store_2d(second, (int32_t)col0, (int32_t)row0, smem_u32(box + C::BOX / 2));
+                            bulk_commit();
                         }
                     }
                 }
@@ -829,7 +834,15 @@ __global__ void __launch_bounds__(256) k_enc_finish(const float *__restrict__ ps
     float p = 0.0f;
     if (lane < m) {
         const float *src = pslots + t * m + lane;
-        for (int s = 0; s < nslots; ++s) p += src[s * slot_stride];
+        int s = 0;
+        for (; s + 8 <= nslots; s += 8) {   // eight loads in flight, added in slot order
+            float x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = __ldcs(src + (s + u) * slot_stride);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) p += x[u];
+        }
+        for (; s < nslots; ++s) p += src[s * slot_stride];
         if (P) P[t * m + lane] = p;
     }
     const float a = lane < m ? act_f(act, p) : 0.0f;
