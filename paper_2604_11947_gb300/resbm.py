@@ -193,19 +193,28 @@ def workspace(desc: resbm_desc, op: int, device="cuda") -> torch.Tensor:
 
 
 def _p(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return t
-    return t.data_ptr()
+    """The address of a tensor's data (an int is an address already, None stays None)."""
+    try:
+        return t.data_ptr()
+    except AttributeError:
+        if t is None or isinstance(t, int):
+            return t
+        raise
 
 
 def _nbytes(t):
     return 0 if t is None else t.numel() * t.element_size()
 
 
+# The current stream's handle without building a torch.cuda.Stream around it (3 us a call on the host;
+# a small step's launches take ~20), where this torch has the accessor.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     return stream if isinstance(stream, int) else stream.cuda_stream
 
