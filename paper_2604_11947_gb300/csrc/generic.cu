@@ -774,6 +774,43 @@ cudaError_t generic_encode_bwd(const resbm_desc &d, const void *dB, const void *
                       (const bf *)We2, (bf *)dF, (bf *)dX, dWe1, dWe2, ws, c));
 }
 
+namespace {
+size_t carve_narrow_step(const resbm_desc &d, void *ws, float *(&s)[4])
+{
+    WsCarver w(ws);
+    for (float *&p : s) p = w.take<float>(d.T * d.m);
+    return w.used;
+}
+template <typename E>
+cudaError_t narrow_step_t(const resbm_desc &d, const resbm_step_args &a, const void *We2, const void *Wd1, float *P, float *dWe2,
+                          float *dWd1, float *const (&s)[4], const Ctx &c)
+{
+    auto in = [](const void *p) { return static_cast<const E *>(p); };
+    auto out = [](void *p) { return static_cast<E *>(p); };
+    return narrow_step<E>(d, in(a.X), in(a.F), in(a.dY), in(a.We1), in(We2), in(Wd1), in(a.Wd2), out(a.B), P, out(a.Y),
+                          out(a.dB), out(a.dF), out(a.dX), a.dWe1, dWe2, dWd1, a.dWd2, s, c);
+}
+}  // namespace
+
+bool narrow_step_ok(const resbm_desc &d)
+{
+    // the grids of k_narrow_dec and k_narrow_wgrad in 32 bits
+    return narrow_ok(d) && d.T > 0 && ((d.T + kNT - 1) / kNT) * ((d.d + kNThr - 1) / kNThr + 1) < (int64_t)INT32_MAX / 2;
+}
+size_t narrow_step_ws_bytes(const resbm_desc &d)
+{
+    float *s[4];
+    return narrow_ok(d) ? carve_narrow_step(d, nullptr, s) : 0;
+}
+cudaError_t generic_narrow_step(const resbm_desc &d, const resbm_step_args &a, const void *We2, const void *Wd1, float *P,
+                                float *dWe2, float *dWd1, void *ws, const Ctx &c)
+{
+    float *s[4];
+    carve_narrow_step(d, ws, s);
+    return d.dtype == RESBM_F32 ? narrow_step_t<float>(d, a, We2, Wd1, P, dWe2, dWd1, s, c)
+                                : narrow_step_t<__nv_bfloat16>(d, a, We2, Wd1, P, dWe2, dWd1, s, c);
+}
+
 cudaError_t fill_identity(const resbm_desc &d, void *out, const Ctx &c)
 {
     const int64_t n = d.r;

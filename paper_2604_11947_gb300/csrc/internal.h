@@ -65,6 +65,12 @@ cudaError_t generic_decode_bwd(const resbm_desc &d, const void *dY, const void *
 cudaError_t generic_encode_bwd(const resbm_desc &d, const void *dB, const void *F,
                                const float *P_save, const void *We1, const void *We2, void *dF,
                                void *dX, float *dWe1, float *dWe2, void *ws, const Ctx &c);
+// The four ops of a boundary step in four launches on the portable narrow kernels (m, r <= 32). P: T x m, given.
+// ws: narrow_step_ws_bytes(d).
+bool narrow_step_ok(const resbm_desc &d);
+size_t narrow_step_ws_bytes(const resbm_desc &d);
+cudaError_t generic_narrow_step(const resbm_desc &d, const resbm_step_args &a, const void *We2, const void *Wd1, float *P,
+                                float *dWe2, float *dWd1, void *ws, const Ctx &c);
 // Backward of N = RMSNorm(Y) * gamma with an incoming dY added (dY may be null or equal dY_out):
 // dY_out (T x d, the descriptor's dtype) and dgamma (d, fp32). ws: rmsnorm_bwd_ws_bytes(d).
 bool rmsnorm_bwd_supported(const resbm_desc &d);

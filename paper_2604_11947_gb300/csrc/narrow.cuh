@@ -64,22 +64,24 @@ struct NarrowIn {
     float *G;             // decode: phi(Q) (T x m)
 };
 
-// MP: m rounded up to 4, 8, 16 or 32; lane j + MP * s of a warp takes column j of tokens s, s + 32 / MP, ...
-template <typename E, int MP, bool DEC>
-__global__ void __launch_bounds__(kNThr) k_narrow_in(const NarrowIn a)
+struct NarrowInSmem {
+    __align__(16) float zs[kNT][kNChunk + 4];
+    float rows1[kNT * 33], rows2[kNT * 33], vs[kNW * 33];
+};
+
+// One tile. MP: m rounded up to 4, 8, 16 or 32; lane j + MP * s of a warp takes column j of tokens s, s + 32 / MP, ...
+template <typename E, int MP, bool DEC> __device__ __forceinline__ void narrow_in_tile(const NarrowIn &a, int64_t tile, NarrowInSmem &sh)
 {
-    __shared__ __align__(16) float zs[kNT][kNChunk + 4];
+    auto &zs = sh.zs;
+    float *rows1 = sh.rows1, *rows2 = sh.rows2, *vs = sh.vs;
     float *part = &zs[0][0];   // [warp][token][column], once the products have read zs
     static_assert(kNThr / 32 * kNT * MP <= kNT * (kNChunk + 4), "the warps' parts fit in the staged rows");
-    __shared__ float rows1[kNT * 33], rows2[kNT * 33], vs[kNW * 33];
     constexpr int TPW = 32 / MP, NA = kNT / TPW > 0 ? kNT / TPW : 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int j = lane % MP, ts = lane / MP;
-    const int64_t t0 = (int64_t)blockIdx.x * kNT;
+    const int64_t t0 = tile * kNT;
     const int nt = a.T - t0 < kNT ? (int)(a.T - t0) : kNT;
     const E *Z = static_cast<const E *>(a.Z) + t0 * a.d, *W = static_cast<const E *>(a.W);
-    griddep_wait();
-    griddep_launch_dependents();
     stage_mat(static_cast<const E *>(a.V), DEC ? a.r : a.m, DEC ? a.m : a.r, vs);
     if (DEC) stage_rows(static_cast<const E *>(a.X) + t0 * a.r, a.r, nt, a.r, rows1);
     float acc[NA];
@@ -153,6 +155,14 @@ __global__ void __launch_bounds__(kNThr) k_narrow_in(const NarrowIn a)
     }
 }
 
+template <typename E, int MP, bool DEC> __global__ void __launch_bounds__(kNThr) k_narrow_in(const NarrowIn a)
+{
+    __shared__ NarrowInSmem sh;
+    griddep_wait();
+    griddep_launch_dependents();
+    narrow_in_tile<E, MP, DEC>(a, blockIdx.x, sh);
+}
+
 struct NarrowOut {
     const void *In;       // T x r: B (decode forward) or dB (encode backward)
     const void *V;        // Wd1 (r x m) or We2 (m x r)
@@ -165,19 +175,23 @@ struct NarrowOut {
     float *dP, *A;        // encode backward: T x m each
 };
 
+template <bool ENC> struct NarrowOutSmem {
+    __align__(16) float gs[kNW][kNT];                // the m-wide rows, [j][token]
+    float in[kNT * 33], vs[kNW * 33];
+    float ws[ENC ? kNThr * 33 : 1];                  // ENC: this block's columns of W
+};
+
+// One tile and block of 256 columns
 template <typename E, bool ENC>
-__global__ void __launch_bounds__(kNThr) k_narrow_out(const NarrowOut a)
+__device__ __forceinline__ void narrow_out_tile(const NarrowOut &a, int64_t tile, int64_t cblk, NarrowOutSmem<ENC> &sh)
 {
-    __shared__ float ws[kNThr * 33];                 // ENC: this block's columns of W
-    __shared__ float in[kNT * 33], vs[kNW * 33];
-    __shared__ __align__(16) float gs[kNW][kNT];     // the m-wide rows, [j][token]
+    float *ws = sh.ws, *in = sh.in, *vs = sh.vs;
+    auto &gs = sh.gs;
     const int tid = threadIdx.x;
-    const int64_t t0 = (int64_t)blockIdx.x * kNT, c0 = (int64_t)blockIdx.y * kNThr;
+    const int64_t t0 = tile * kNT, c0 = cblk * kNThr;
     const int nt = a.T - t0 < kNT ? (int)(a.T - t0) : kNT;
     const int nc = a.d - c0 < kNThr ? (int)(a.d - c0) : kNThr;
     const E *W = static_cast<const E *>(a.W);
-    griddep_wait();
-    griddep_launch_dependents();
     stage_mat(static_cast<const E *>(a.V), ENC ? a.m : a.r, ENC ? a.r : a.m, vs);
     stage_rows(static_cast<const E *>(a.In) + t0 * a.r, a.r, nt, a.r, in);
     if (ENC)   // We1 (d x m): contiguous rows of m
@@ -197,14 +211,14 @@ __global__ void __launch_bounds__(kNThr) k_narrow_out(const NarrowOut a)
             float f = 0.0f, df = 0.0f;
             if (t < nt) act_and_dact(a.act, a.P[(t0 + t) * a.m + k], f, df);
             s *= df;
-            if (blockIdx.y == 0 && t < nt) {
+            if (cblk == 0 && t < nt) {
                 a.dP[(t0 + t) * a.m + k] = s;
                 a.A[(t0 + t) * a.m + k] = f;
             }
         }
         gs[k][t] = s;
     }
-    if (ENC && a.dX && blockIdx.y == 0)   // dX[:, :r] += dB
+    if (ENC && a.dX && cblk == 0)   // dX[:, :r] += dB
         for (int e = tid; e < nt * a.r; e += kNThr) {
             const int t = e / a.r, n = e - t * a.r;
             E *x = static_cast<E *>(a.dX) + (t0 + t) * a.d + n;
@@ -237,6 +251,32 @@ __global__ void __launch_bounds__(kNThr) k_narrow_out(const NarrowOut a)
         }
 }
 
+template <typename E, bool ENC> __global__ void __launch_bounds__(kNThr) k_narrow_out(const NarrowOut a)
+{
+    __shared__ NarrowOutSmem<ENC> sh;
+    griddep_wait();
+    griddep_launch_dependents();
+    narrow_out_tile<E, ENC>(a, blockIdx.x, blockIdx.y, sh);
+}
+
+// The step's two decoder ops in one launch (both read B only): blocks [0, tiles) run the backward's tiles, the
+// rest the forward's
+template <typename E, int MP> __global__ void __launch_bounds__(kNThr) k_narrow_dec(const NarrowOut o, const NarrowIn i, int tiles)
+{
+    __shared__ union {
+        NarrowInSmem in;
+        NarrowOutSmem<false> out;
+    } sh;
+    griddep_wait();
+    griddep_launch_dependents();
+    if ((int)blockIdx.x < tiles) {
+        narrow_in_tile<E, MP, true>(i, blockIdx.x, sh.in);
+    } else {
+        const int64_t k = (int64_t)blockIdx.x - tiles;
+        narrow_out_tile<E, false>(o, k % tiles, k / tiles, sh.out);
+    }
+}
+
 struct NarrowWgrad {
     const void *Z;        // T x d: dY or F
     const float *V;       // T x m: phi(Q) or dP
@@ -249,10 +289,19 @@ struct NarrowWgrad {
     int small_mr;         // 1: m x r
 };
 
-// blockIdx.x / 8: the cluster's 64 columns of the d x m gradient, or (the last cluster) the small one
+// One backward op's two gradients, or (jobs == 2: the step) both ops', the clusters' first half the first op's.
+// Within a job, blockIdx.x / 8: the cluster's 64 columns of the d x m gradient, or (the last) the small one
+struct NarrowWgrads {
+    NarrowWgrad job[2];
+    int jobs;
+};
 template <typename E, int MP>
-__global__ void __launch_bounds__(kNThr) k_narrow_wgrad(const NarrowWgrad a)
+__global__ void __launch_bounds__(kNThr) k_narrow_wgrad(const NarrowWgrads w)
 {
+    const int per_job = (int)gridDim.x / w.jobs;   // CTAs
+    const bool second = (int)blockIdx.x >= per_job;
+    const NarrowWgrad &a = w.job[second ? 1 : 0];
+    const int cta = (int)blockIdx.x - (second ? per_job : 0);
     constexpr int TC = 64;                                   // tokens staged at a time
     __shared__ __align__(16) float buf[4 * 64 * (MP + 1) > TC * (MP + 33) ? 4 * 64 * (MP + 1) : TC * (MP + 33)];
     float(*vs)[MP] = reinterpret_cast<float(*)[MP]>(buf);
@@ -261,8 +310,8 @@ __global__ void __launch_bounds__(kNThr) k_narrow_wgrad(const NarrowWgrad a)
     __shared__ float slots[kNCl][kNW * kNW / kNCl];          // the owned sums from every rank
     const int tid = threadIdx.x;
     const int rank = (int)cluster_rank();
-    const int64_t chunk = blockIdx.x / kNCl;
-    const bool is_small = chunk == (int64_t)(gridDim.x / kNCl) - 1;
+    const int64_t chunk = cta / kNCl;
+    const bool is_small = chunk == per_job / kNCl - 1;
     const int64_t tb = a.T * rank / kNCl, te = a.T * (rank + 1) / kNCl;   // this CTA's tokens
     griddep_wait();
     griddep_launch_dependents();
@@ -394,65 +443,122 @@ template <typename E, bool ENC> cudaError_t narrow_out(const NarrowOut &a, const
     return launch_narrow(k_narrow_out<E, ENC>, dim3((unsigned)((a.T + kNT - 1) / kNT), (unsigned)((a.d + kNThr - 1) / kNThr)),
                          1, a, c);
 }
-template <typename E> cudaError_t narrow_wgrad(const NarrowWgrad &a, const Ctx &c)
+template <typename E> cudaError_t narrow_wgrad(const NarrowWgrads &w, const Ctx &c)
 {
-    const dim3 grid((unsigned)(kNCl * ((a.d + 63) / 64 + 1)));
-    return a.m <= 4    ? launch_narrow(k_narrow_wgrad<E, 4>, grid, kNCl, a, c)
-           : a.m <= 8  ? launch_narrow(k_narrow_wgrad<E, 8>, grid, kNCl, a, c)
-           : a.m <= 16 ? launch_narrow(k_narrow_wgrad<E, 16>, grid, kNCl, a, c)
-                       : launch_narrow(k_narrow_wgrad<E, 32>, grid, kNCl, a, c);
+    const NarrowWgrad &a = w.job[0];
+    const dim3 grid((unsigned)(w.jobs * kNCl * ((a.d + 63) / 64 + 1)));
+    return a.m <= 4    ? launch_narrow(k_narrow_wgrad<E, 4>, grid, kNCl, w, c)
+           : a.m <= 8  ? launch_narrow(k_narrow_wgrad<E, 8>, grid, kNCl, w, c)
+           : a.m <= 16 ? launch_narrow(k_narrow_wgrad<E, 16>, grid, kNCl, w, c)
+                       : launch_narrow(k_narrow_wgrad<E, 32>, grid, kNCl, w, c);
 }
 
+// ---- each op's arguments --------------------------------------------------------------------------
 template <typename E>
-cudaError_t narrow_encode_fwd(const resbm_desc &d, const E *X, const E *F, const E *We1, const E *We2, E *B, float *P,
-                              const Ctx &c)
+NarrowIn narrow_enc_in(const resbm_desc &d, const E *X, const E *F, const E *We1, const E *We2, E *B, float *P)
 {
     NarrowIn a{};
     a.Z = F; a.W = We1; a.sk = d.m; a.sj = 1; a.T = d.T; a.d = d.d;
     a.m = (int)d.m; a.r = (int)d.r; a.act = d.act;
     a.V = We2; a.X = X; a.out = B; a.P = P;
-    return narrow_in<E, false>(a, c);
+    return a;
 }
-template <typename E>
-cudaError_t narrow_decode_fwd(const resbm_desc &d, const E *B, const E *Wd1, const E *Wd2, E *Y, const Ctx &c)
+template <typename E> NarrowOut narrow_dec_out(const resbm_desc &d, const E *B, const E *Wd1, const E *Wd2, E *Y)
 {
     NarrowOut a{};
     a.In = B; a.V = Wd1; a.W = Wd2; a.sj = d.d; a.sc = 1; a.T = d.T; a.d = d.d;
     a.m = (int)d.m; a.r = (int)d.r; a.act = d.act; a.merge = d.merge_identity;
     a.out = Y;
-    return narrow_out<E, false>(a, c);
+    return a;
+}
+template <typename E>
+NarrowIn narrow_dec_in(const resbm_desc &d, const E *dY, const E *B, const E *Wd1, const E *Wd2, E *dB, float *G, float *dQ)
+{
+    NarrowIn a{};
+    a.Z = dY; a.W = Wd2; a.sk = 1; a.sj = d.d; a.T = d.T; a.d = d.d;
+    a.m = (int)d.m; a.r = (int)d.r; a.act = d.act; a.merge = d.merge_identity;
+    a.V = Wd1; a.X = B; a.out = dB; a.P = dQ; a.G = G;
+    return a;
+}
+template <typename E>
+NarrowWgrad narrow_dec_wgrad(const resbm_desc &d, const E *dY, const E *B, const float *G, const float *dQ, float *dWd1, float *dWd2)
+{
+    NarrowWgrad w{};
+    w.Z = dY; w.V = G; w.out = dWd2; w.sc = 1; w.sj = d.d; w.T = d.T; w.d = d.d; w.m = (int)d.m; w.r = (int)d.r;
+    w.io = B; w.U = dQ; w.small = dWd1; w.small_mr = 0;
+    return w;
+}
+template <typename E>
+NarrowOut narrow_enc_out(const resbm_desc &d, const E *dB, const float *P, const E *We1, const E *We2, E *dF, E *dX, float *dP,
+                         float *A)
+{
+    NarrowOut a{};
+    a.In = dB; a.V = We2; a.W = We1; a.sj = 1; a.sc = d.m; a.T = d.T; a.d = d.d;
+    a.m = (int)d.m; a.r = (int)d.r; a.act = d.act;
+    a.P = P; a.out = dF; a.dX = dX; a.dP = dP; a.A = A;
+    return a;
+}
+template <typename E>
+NarrowWgrad narrow_enc_wgrad(const resbm_desc &d, const E *F, const E *dB, const float *dP, const float *A, float *dWe1, float *dWe2)
+{
+    NarrowWgrad w{};
+    w.Z = F; w.V = dP; w.out = dWe1; w.sc = d.m; w.sj = 1; w.T = d.T; w.d = d.d; w.m = (int)d.m; w.r = (int)d.r;
+    w.io = dB; w.U = A; w.small = dWe2; w.small_mr = 1;
+    return w;
+}
+
+// ---- the ops, and the step ---------------------------------------------------------------------------
+template <typename E>
+cudaError_t narrow_encode_fwd(const resbm_desc &d, const E *X, const E *F, const E *We1, const E *We2, E *B, float *P,
+                              const Ctx &c)
+{
+    return narrow_in<E, false>(narrow_enc_in(d, X, F, We1, We2, B, P), c);
+}
+template <typename E>
+cudaError_t narrow_decode_fwd(const resbm_desc &d, const E *B, const E *Wd1, const E *Wd2, E *Y, const Ctx &c)
+{
+    return narrow_out<E, false>(narrow_dec_out(d, B, Wd1, Wd2, Y), c);
 }
 // G, dQ: T x m fp32 scratch
 template <typename E>
 cudaError_t narrow_decode_bwd(const resbm_desc &d, const E *dY, const E *B, const E *Wd1, const E *Wd2, E *dB, float *dWd1,
                               float *dWd2, float *G, float *dQ, const Ctx &c)
 {
-    NarrowIn a{};
-    a.Z = dY; a.W = Wd2; a.sk = 1; a.sj = d.d; a.T = d.T; a.d = d.d;
-    a.m = (int)d.m; a.r = (int)d.r; a.act = d.act; a.merge = d.merge_identity;
-    a.V = Wd1; a.X = B; a.out = dB; a.P = dQ; a.G = G;
-    const cudaError_t e = narrow_in<E, true>(a, c);
+    const cudaError_t e = narrow_in<E, true>(narrow_dec_in(d, dY, B, Wd1, Wd2, dB, G, dQ), c);
     if (e != cudaSuccess) return e;
-    NarrowWgrad w{};
-    w.Z = dY; w.V = G; w.out = dWd2; w.sc = 1; w.sj = d.d; w.T = d.T; w.d = d.d; w.m = a.m; w.r = a.r;
-    w.io = B; w.U = dQ; w.small = dWd1; w.small_mr = 0;
-    return narrow_wgrad<E>(w, c);
+    return narrow_wgrad<E>(NarrowWgrads{{narrow_dec_wgrad(d, dY, B, G, dQ, dWd1, dWd2), {}}, 1}, c);
 }
 // dP, A: T x m fp32 scratch
 template <typename E>
 cudaError_t narrow_encode_bwd(const resbm_desc &d, const E *dB, const E *F, const float *P, const E *We1, const E *We2,
                               E *dF, E *dX, float *dWe1, float *dWe2, float *dP, float *A, const Ctx &c)
 {
-    NarrowOut a{};
-    a.In = dB; a.V = We2; a.W = We1; a.sj = 1; a.sc = d.m; a.T = d.T; a.d = d.d;
-    a.m = (int)d.m; a.r = (int)d.r; a.act = d.act;
-    a.P = P; a.out = dF; a.dX = dX; a.dP = dP; a.A = A;
-    const cudaError_t e = narrow_out<E, true>(a, c);
+    const cudaError_t e = narrow_out<E, true>(narrow_enc_out(d, dB, P, We1, We2, dF, dX, dP, A), c);
     if (e != cudaSuccess) return e;
-    NarrowWgrad w{};
-    w.Z = F; w.V = dP; w.out = dWe1; w.sc = d.m; w.sj = 1; w.T = d.T; w.d = d.d; w.m = a.m; w.r = a.r;
-    w.io = dB; w.U = A; w.small = dWe2; w.small_mr = 1;
-    return narrow_wgrad<E>(w, c);
+    return narrow_wgrad<E>(NarrowWgrads{{narrow_enc_wgrad(d, F, dB, dP, A, dWe1, dWe2), {}}, 1}, c);
+}
+// The four ops in four launches instead of six (every output the same bits): the decoder's forward and
+// backward together, and all four weight gradients. Small steps are launches and their latency: T = 512,
+// d = 256, r = 2 fp32 20 us of GPU time and 11 us of enqueueing in six. scratch: four T x m fp32 matrices.
+template <typename E>
+cudaError_t narrow_step(const resbm_desc &d, const E *X, const E *F, const E *dY, const E *We1, const E *We2, const E *Wd1,
+                        const E *Wd2, E *B, float *P, E *Y, E *dB, E *dF, E *dX, float *dWe1, float *dWe2, float *dWd1,
+                        float *dWd2, float *const (&scratch)[4], const Ctx &c)
+{
+    float *G = scratch[0], *dQ = scratch[1], *dP = scratch[2], *A = scratch[3];
+    cudaError_t e = narrow_encode_fwd<E>(d, X, F, We1, We2, B, P, c);
+    if (e != cudaSuccess) return e;
+    const NarrowOut o = narrow_dec_out(d, B, Wd1, Wd2, Y);
+    const NarrowIn i = narrow_dec_in(d, dY, B, Wd1, Wd2, dB, G, dQ);
+    const int tiles = (int)((d.T + kNT - 1) / kNT);
+    const dim3 grid((unsigned)(tiles * (1 + (d.d + kNThr - 1) / kNThr)));
+    auto kernel = d.m <= 4 ? k_narrow_dec<E, 4> : d.m <= 8 ? k_narrow_dec<E, 8> : d.m <= 16 ? k_narrow_dec<E, 16> : k_narrow_dec<E, 32>;
+    e = launch_pdl(kernel, grid, dim3(kNThr), 0, c, o, i, tiles);
+    count_launches(1);
+    if (e == cudaSuccess) e = narrow_out<E, true>(narrow_enc_out(d, dB, P, We1, We2, dF, dX, dP, A), c);
+    if (e != cudaSuccess) return e;
+    return narrow_wgrad<E>(
+        NarrowWgrads{{narrow_dec_wgrad(d, dY, B, G, dQ, dWd1, dWd2), narrow_enc_wgrad(d, F, dB, dP, A, dWe1, dWe2)}, 2}, c);
 }
 
 }  // namespace

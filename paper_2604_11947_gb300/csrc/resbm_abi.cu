@@ -270,6 +270,9 @@ size_t step_ws_bytes(const resbm_desc &d)
         size_t b = ws_for(d, op);
         if (b > inner) inner = b;
     }
+    // the portable narrow kernels run the step in fewer launches with more scratch live at a time
+    const size_t n = narrow_step_ws_bytes(d) + (is_linear(d) ? carve_linear(d, nullptr).bytes : 0);
+    if (n > inner) inner = n;
     w.take<char>(inner);
     return w.used;
 }
@@ -568,6 +571,10 @@ resbm_status enqueue_step(const resbm_desc &d, const resbm_step_args &a, void *w
         dWd1 = l.dW1;
         inner = l.inner;
     }
+    // no tensor-core path for any op, and nothing to wait for in between: the portable kernels' own step
+    bool portable = narrow_step_ok(e) && !fwd_done && !bwd_ready;
+    for (int op = RESBM_OP_ENCODE_FWD; op <= RESBM_OP_ENCODE_BWD; ++op) portable = portable && !use_tc(e, op) && !use_gemm(e, op);
+    if (s == RESBM_OK && portable) return finish(generic_narrow_step(e, a, We2, Wd1, P, dWe2, dWd1, inner, c));
     if (s == RESBM_OK) s = run_encode_fwd(e, a.X, a.F, a.We1, We2, a.B, P, inner, c);
     bool dec_fwd_tc = false, kept_q = false;
     if (s == RESBM_OK) s = run_decode_fwd(e, a.B, Wd1, a.Wd2, a.Y, inner, c, &dec_fwd_tc, &kept_q);
