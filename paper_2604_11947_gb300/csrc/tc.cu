@@ -513,14 +513,14 @@ int gemm_splits(int64_t M, int64_t N, int64_t K, int sms, GemmForm form = kGemmS
 struct GemmOutMaps {
     CUtensorMap o, o2, lo;
 };
-template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = false, bool BM2 = false, int TS = 0>
+template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = false, bool BM2 = false, int TS = 0, bool RB = false>
 cudaError_t launch_gemm_t(const CUtensorMap &ma, const CUtensorMap &malo, const CUtensorMap &mb,
                           const tc::GemmShape &g, const tc::GemmEp &ep, const Ctx &c, const GemmOutMaps *out = nullptr)
 {
-    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP>;
+    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB>;
     const GemmOutMaps none{ma, ma, ma};   // not read
     const GemmOutMaps &mo = out ? *out : none;
-    auto kernel = tc::k_gemm<BN, AMN, BMN, ALO, ENCP, PAIR, BM2, TS>;
+    auto kernel = tc::k_gemm<BN, AMN, BMN, ALO, ENCP, PAIR, BM2, TS, RB>;
     static std::atomic<uint8_t> smem_set[kMaxDev];
     cudaError_t e = ensure_smem(kernel, Cfg::SMEM_BYTES, c.device, smem_set);
     if (e != cudaSuccess) return e;
@@ -533,7 +533,7 @@ cudaError_t launch_gemm_t(const CUtensorMap &ma, const CUtensorMap &malo, const 
         e = launch_clustered(kernel, (unsigned)(2 * pairs), Cfg::THREADS, Cfg::SMEM_BYTES, 2, c.stream, ma, malo, mb, mo.o,
                              mo.o2, mo.lo, g, ep);
     } else {
-        const int64_t grid = g.units < c.sm_count ? g.units : c.sm_count;
+        const int64_t grid = RB ? (g.M + g.rpc - 1) / g.rpc : g.units < c.sm_count ? g.units : c.sm_count;
         e = launch(kernel, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, c.stream, ma, malo, mb, mo.o, mo.o2, mo.lo, g, ep);
     }
     count_launches(1);
@@ -627,6 +627,7 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
     g.nm = (int)(bm2 ? (M + 255) / 256 : (M + 127) / 128);
     g.nn = (int)((N + bn - 1) / bn);
     g.units = (int64_t)g.nm * g.nn * g.splits;
+    g.rpc = 0;
     if (bm2) {
         if (!a_mn && b_mn) return launch_gemm_t<256, false, true, false, false, false, true>(ma, malo, mbm, g, ep, c);
         if (!a_mn && !b_mn) return launch_gemm_t<256, false, false, false, false, false, true>(ma, malo, mbm, g, ep, c);
@@ -639,6 +640,22 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
     // dWe1 of d = 8192, m = 128 went 84 -> 91 us)
     const bool ts_ok = ep.mode == tc::GEP_F32 ? pair && !lo : (pair || bn == 128) && !a_mn && g.splits == 1;
     const int ts = ts_ok ? gemm_ts(ep, M, N, g.splits, lo, &mo) : 0;
+    if (ts == 2 && bn == 128 && g.nm > c.sm_count && K >= 1024) {   // P, dQ of m <= 128: row-balanced units
+        const int64_t rpc = (M + 32 * (int64_t)c.sm_count - 1) / (32 * (int64_t)c.sm_count) * 32;
+        if (rpc < INT32_MAX) {
+            const bool narrow = N <= 64;
+            CUtensorMap mrest, mbr;
+            if (!make_map(&mrest, A, K, M, K * 2, 64, rpc % 128 ? (uint32_t)(rpc % 128) : 128u, CU_TENSOR_MAP_SWIZZLE_128B) ||
+                !(b_mn ? make_map(&mbr, B, N, K, N * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
+                       : make_map(&mbr, B, K, N, K * 2, 64, narrow ? 64 : 128, CU_TENSOR_MAP_SWIZZLE_128B)))
+                return cudaErrorInvalidValue;
+            g.rpc = (int)rpc;
+            if (narrow) return b_mn ? launch_gemm_t<64, false, true, false, false, false, false, 2, true>(ma, mrest, mbr, g, ep, c, &mo)
+                                    : launch_gemm_t<64, false, false, false, false, false, false, 2, true>(ma, mrest, mbr, g, ep, c, &mo);
+            return b_mn ? launch_gemm_t<128, false, true, false, false, false, false, 2, true>(ma, mrest, mbr, g, ep, c, &mo)
+                        : launch_gemm_t<128, false, false, false, false, false, false, 2, true>(ma, mrest, mbr, g, ep, c, &mo);
+        }
+    }
     if (ts && bn == 128) {
         if (ts == 2) return b_mn ? launch_gemm_t<128, false, true, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo)
                                  : launch_gemm_t<128, false, false, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo);
@@ -1105,7 +1122,7 @@ cudaError_t tc_ffn_down_encode(const resbm_desc &d, int64_t f, const void *H, co
     if (!make_map(&ma, H, f, d.T, f * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&mb, W2, d.d, f, d.d * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
-    tc::GemmShape g;
+    tc::GemmShape g{};
     g.M = d.T;
     g.N = d.d;
     g.K = f;

@@ -126,6 +126,12 @@ struct GemmShape {
     int64_t kc;          // K per split, a multiple of 64
     int nm, nn, splits;
     int64_t units;       // nm * nn * splits
+    // Row-balanced launch (one column block, one split, more row blocks than CTAs): CTA b takes the rows
+    // [b * rpc, (b + 1) * rpc), rpc a multiple of 32, in 128-row units and a last one of rpc % 128 rows; 0: off.
+    // Such a product is bound by reading A, and with whole 128-row blocks some CTAs read one block more than
+    // others (256 blocks on 152 SMs: 2 against 1; 224 rows each instead). What it reads at is the bytes in flight,
+    // so these launches keep one store box a warp and 64-column tiles where N allows: 6 stages of 16 KB of A, or 8.
+    int rpc;
 };
 
 // BM2: 256-row units, two 128-row A sub-tiles per stage against one B tile, the two halves'
@@ -133,20 +139,22 @@ struct GemmShape {
 // PAIR: CTA pairs (cta_group::2) on 256-row units: a stage of each CTA holds its own 128 rows of A and
 // half of the B tile.
 // TS: the outputs leave by TMA stores from shared-memory boxes, two 4 KB boxes per epilogue warp (one
-// fills while the other's store reads it), each warp on its own: no barrier between warps. 1: one bf16
+// fills while the other's store reads it; RB: one box), each warp on its own: no barrier between warps. 1: one bf16
 // output in boxes of 32 rows x 64 columns (128-byte swizzle); 2: an fp32 output in boxes of 32 rows x 32
 // columns and / or up to two bf16 outputs of 32 x 32 in one box (64-byte rows). Per-thread 16-byte stores put 32 different rows
 // in a warp instruction: they, not the products, set the pace where K is short.
 // ENCP: one box of 32 rows x 64 columns per warp (F as the partial P's operand, and for F's store) and
 // We1's rows of the unit's columns.
-template <int BN_, bool ALO_ = false, bool BM2_ = false, int TS_ = 0, bool PAIR_ = false, bool ENCP_ = false> struct GemmCfg {
+template <int BN_, bool ALO_ = false, bool BM2_ = false, int TS_ = 0, bool PAIR_ = false, bool ENCP_ = false, bool RB_ = false>
+struct GemmCfg {
     static constexpr int BN = BN_;
     static constexpr uint32_t A_TILE = 128 * 64 * 2;        // 128 rows x 64 K, bf16
     static constexpr uint32_t A_STAGE = A_TILE * (ALO_ ? 2 : 1) * (BM2_ ? 2 : 1);   // hi (+ lo), per half
     static constexpr uint32_t B_STAGE = (PAIR_ ? BN_ / 2 : BN_) * 64 * 2;   // BN (PAIR: BN / 2) rows x 64 K, bf16
     static constexpr uint32_t STAGE = A_STAGE + B_STAGE;
     static constexpr uint32_t BOX = 32 * 128;               // a staging box: 32 rows of 128 bytes
-    static constexpr uint32_t STG_WARP = TS_ ? 2 * BOX : ENCP_ ? BOX : 0;   // per epilogue warp
+    static constexpr int NBOX = TS_ && !RB_ ? 2 : TS_ || ENCP_ ? 1 : 0;      // boxes per epilogue warp
+    static constexpr uint32_t STG_WARP = NBOX * BOX;
     static constexpr uint32_t WE1_HALF = 128 * 64;          // ENCP: 128 columns' rows of We1 (up to 32 wide)
     static constexpr uint32_t STG_BYTES = 8 * STG_WARP + (ENCP_ ? 2 * WE1_HALF : 0);
     // stages: 4 at BN = 256, 6 at 128 (3, 4 with lo; 3 for BM2; PAIR: 6 and 8, 4 and 5 with lo); beside the
@@ -345,7 +353,8 @@ __device__ __forceinline__ void rmw_rows(const GemmEp &ep, int64_t row0, int64_t
     }
 }
 
-// tma_lo: the lo matrix of A (same shape and layout as A; read only with ALO); tmo, tmo2, tmol: the
+// tma_lo: the lo matrix of A (same shape and layout as A; read only with ALO; RB: A in boxes of the last
+// unit's rows); tmo, tmo2, tmol: the
 // outputs ep.out, ep.out2 and ep.lo in the boxes of the TS form (read only with TS; ENCP: tmo, if ep.out)
 // ENCP: the epilogue of the encoder fused into the FFN down-projection (the GemmEp ENCP fields)
 // instead of gemm_epilogue.
@@ -358,15 +367,19 @@ __device__ __forceinline__ void rmw_rows(const GemmEp &ep, int64_t row0, int64_t
 // publish the accumulators in both (multicast). Each SM reads 96 operand rows a K step for 128 x 256
 // products instead of 384 / 2, and 32 KB instead of 48 KB a stage keep six in flight.
 // (For K-major B the tensor map's box is BN / 2 rows.)
+// RB: row-balanced units (GemmShape::rpc).
 template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = false, bool BM2 = false,
-          int TS = 0>
+          int TS = 0, bool RB = false>
 __global__ void __launch_bounds__(320, 1)
     k_gemm(const __grid_constant__ CUtensorMap tma, const __grid_constant__ CUtensorMap tma_lo,
            const __grid_constant__ CUtensorMap tmb, const __grid_constant__ CUtensorMap tmo,
            const __grid_constant__ CUtensorMap tmo2, const __grid_constant__ CUtensorMap tmol, const GemmShape g,
            const GemmEp ep)
 {
-    using C = GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP>;
+    using C = GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB>;
+    // (a compile-time property so that the other launches keep their index arithmetic)
+    constexpr bool ROWS = RB;
+    static_assert(!RB || (BN <= 128 && !AMN && !ALO && !ENCP && !PAIR && !BM2 && TS), "row-balanced: K-major A, one column block");
     static_assert(!(BM2 && (ALO || PAIR)), "256-row units without hi + lo A or pairs");
     static_assert(!(TS && (ENCP || BM2)), "TMA-store epilogue: plain 128-row units or pairs");
     constexpr int MH = BM2 ? 2 : 1;   // 128-row halves per unit (g.nm counts units of 128 * MH rows)
@@ -385,17 +398,26 @@ __global__ void __launch_bounds__(320, 1)
     // this CTA's units: every gridDim.x-th from blockIdx.x, or for a pair every (gridDim.x / 2)-th
     // pair unit from the cluster index, the row block 2 * (pair row block) + rank
     const uint32_t crank = PAIR ? cluster_rank() : 0u;
-    const int64_t u_first = PAIR ? (int64_t)cluster_index() : (int64_t)blockIdx.x;
-    const int64_t u_step = PAIR ? (int64_t)(gridDim.x / 2) : (int64_t)gridDim.x;
+    const int64_t u_first = PAIR ? (int64_t)cluster_index() : ROWS ? 0 : (int64_t)blockIdx.x;
+    const int64_t u_step = PAIR ? (int64_t)(gridDim.x / 2) : ROWS ? 1 : (int64_t)gridDim.x;
     GemmShape gp = g;
+    if (ROWS) gp.units = (g.rpc + 127) / 128;
     if (PAIR) {
         gp.nm = (g.nm + 1) / 2;
         gp.units = (int64_t)gp.nm * gp.nn * gp.splits;
     }
     auto unit_of = [&](int64_t u, int &mb, int &nb, int &ks) {
+        if (ROWS) {
+            mb = (int)u;
+            nb = ks = 0;
+            return;
+        }
         gemm_unit(gp, u, mb, nb, ks);
         if (PAIR) mb = 2 * mb + (int)crank;   // past the last row block: loads read zeros, nothing is stored
     };
+    // first row of a unit, and the end of the rows this CTA may store
+    auto row_of = [&](int mb) { return (ROWS ? (int64_t)blockIdx.x * g.rpc : (int64_t)0) + (int64_t)mb * 128; };
+    const int64_t m_end = ROWS && (int64_t)(blockIdx.x + 1) * g.rpc < g.M ? (int64_t)(blockIdx.x + 1) * g.rpc : g.M;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::NST; ++s) {
@@ -427,7 +449,7 @@ __global__ void __launch_bounds__(320, 1)
         // ---------------- producer ----------------
         if (elect_one()) {
             tma_prefetch_desc(&tma);
-            if (ALO) tma_prefetch_desc(&tma_lo);
+            if (ALO || ROWS) tma_prefetch_desc(&tma_lo);
             tma_prefetch_desc(&tmb);
             uint32_t it = 0;
             bool ok = true;
@@ -443,8 +465,9 @@ __global__ void __launch_bounds__(320, 1)
                         break;
                     }
                     uint32_t bar = smem_u32(&full[s]);
+                    const bool rest = ROWS && (mb + 1) * 128 > g.rpc;   // the shorter last unit: its own box (tma_lo)
                     if (!PAIR) {
-                        mbar_expect_tx(bar, C::STAGE);
+                        mbar_expect_tx(bar, rest ? (uint32_t)(g.rpc % 128) * 128u + C::B_STAGE : C::STAGE);
                     } else {   // both CTAs' bytes on the even CTA's barrier
                         if (crank == 0) mbar_expect_tx(bar, 2 * C::STAGE);
                         bar = map_shared(bar, 0);
@@ -467,7 +490,7 @@ __global__ void __launch_bounds__(320, 1)
                             }
                         }
                     } else if (!AMN) {
-                        load(adst, &tma, kx, mb * 128);
+                        load(adst, rest ? &tma_lo : &tma, kx, (int32_t)row_of(mb));
                         if (ALO) load(adst + C::A_TILE, &tma_lo, kx, mb * 128);
                     } else {
                         load(adst, &tma, mb * 128, kx);
@@ -571,9 +594,9 @@ __global__ void __launch_bounds__(320, 1)
         uint8_t *const boxes = smem + C::OFF_STG + (warp - 2) * C::STG_WARP;   // this warp's
         // the next box, once its previous store has read it
         auto next_box = [&]() -> uint8_t * {
-            if (lane == 0) bulk_wait_read<1>();
+            if (lane == 0) bulk_wait_read<(C::NBOX > 1 ? 1 : 0)>();
             __syncwarp();
-            return boxes + (stg_it++ & 1) * C::BOX;
+            return C::NBOX > 1 ? boxes + (stg_it++ & 1) * C::BOX : boxes;
         };
         // the warp's writes to the box are complete: store it at (col, row0)
         auto store_box = [&](const CUtensorMap &m, const uint8_t *box, int64_t col, int64_t row0) {
@@ -625,10 +648,10 @@ __global__ void __launch_bounds__(320, 1)
                 }
                 named_barrier(1 + half, 128);
             }
-            const int64_t ts_row0 = (int64_t)mb * 128 + q * 32, ts_col0 = (int64_t)nb * BN + half * (BN / 2);
+            const int64_t ts_row0 = row_of(mb) + q * 32, ts_col0 = (int64_t)nb * BN + half * (BN / 2);
             if (TS == 1 && ep.mode == GEP_DF && ep.rmw) {
                 const int64_t end = ts_col0 + BN / 2 < ep.aux_cols ? ts_col0 + BN / 2 : ep.aux_cols;
-                if (ts_col0 < end) rmw_rows(ep, ts_row0, g.M, ts_col0, end);   // dX[:, :r] += dB, while the products run
+                if (ts_col0 < end) rmw_rows(ep, ts_row0, m_end, ts_col0, end);   // dX[:, :r] += dB, while the products run
             }
             ok = mbar_wait(smem_u32(&acc_full[ab]), BM2 ? (ti & 1) : ((ti >> 1) & 1));
             tc_fence_after();
@@ -706,7 +729,7 @@ __global__ void __launch_bounds__(320, 1)
                     float v[CW / 32][32];
 #pragma unroll
                     for (int h = 0; h < CW / 32; ++h) tmem_ld32(tmem + lane_base + ab * BN + c0 + 32 * h, v[h]);   // warp-collective
-                    if (row0 >= g.M || col0 >= g.N) {   // nothing of it exists (the same for the whole warp)
+                    if (row0 >= m_end || col0 >= g.N) {   // nothing of it exists (the same for the whole warp)
                         tmem_ld_wait();
                         if (last) release_acc(ab);
                         continue;
@@ -721,7 +744,7 @@ __global__ void __launch_bounds__(320, 1)
                         for (int h = 0; h < CW / 32; ++h) {
                             const int64_t col = col0 + 32 * h;
                             // the identity path's columns; AXPBY: every column
-                            if ((ep.mode == GEP_ADD_AUX || ep.mode == GEP_AXPBY) && row < g.M && col < ep.aux_cols) {
+                            if ((ep.mode == GEP_ADD_AUX || ep.mode == GEP_AXPBY) && row < m_end && col < ep.aux_cols) {
                                 const int na = ep.aux_cols - col < 32 ? (int)(ep.aux_cols - col) : 32;
                                 float x[32];
                                 ld_bf16x32(static_cast<const __nv_bfloat16 *>(ep.aux) + row * ep.lda + col, x, na);
@@ -740,7 +763,7 @@ __global__ void __launch_bounds__(320, 1)
                         // x: the pre-activation (P, Q) the element-wise step works on
                         float x[32];
                         uint8_t *box = next_box();
-                        if (ep.mode == GEP_DACT && row < g.M)
+                        if (ep.mode == GEP_DACT && row < m_end)
                             ld_f32x32(static_cast<const float *>(ep.aux) + row * ep.lda + col0, x, g.N - col0 < 32 ? (int)(g.N - col0) : 32);
                         tmem_ld_wait();
                         tmem_regs_ready(v[0]);

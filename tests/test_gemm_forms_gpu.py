@@ -29,3 +29,18 @@ def test_pairs_match_single_ctas(T, d, r, m, monkeypatch):
         # for one element, six times that for the largest of 2.7e5: 1e-5, bound ten times it
         assert err <= 1e-4, (k, float(err))
     assert resbm.resbm_device_error() == 0
+
+
+@pytest.mark.parametrize("T,d,r", [(19457, 1024, 128), (20011, 1032, 64), (38913, 1024, 40), (45000, 1024, 72)])
+def test_row_balanced_units_match_whole_blocks(T, d, r, monkeypatch):
+    """More row blocks than SMs and one column block: rows spread evenly over the CTAs (the last unit of each
+    shorter), against 128-row blocks (RESBM_GEMM_TS=0, which also stores without TMA): the same bits."""
+    cfg = synth.BoundaryConfig("rows_%d" % T, T=T, d=d, r=min(r, d), m=r)
+    dev = {k: to_dev(v, cfg) for k, v in host_inputs(cfg).items()}
+    flags = resbm.RESBM_FLAG_GEMM
+    got = gpu_step(cfg, dev, flags=flags)
+    monkeypatch.setenv("RESBM_GEMM_TS", "0")
+    want = gpu_step(cfg, dev, flags=flags)
+    for k in ("B", "P", "Y", "dB", "dF", "dX", "dWe1", "dWe2", "dWd1", "dWd2"):
+        assert torch.equal(got[k], want[k]), k
+    assert resbm.resbm_device_error() == 0
