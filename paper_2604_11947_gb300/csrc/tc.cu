@@ -429,12 +429,11 @@ cudaError_t launch_enc_bwd(const resbm_desc &d, const void *dB, const void *F, c
                                   Cfg::CL_MIN_TOKENS, c.device, fit, false);
     const EncBwdWs w = enc_bwd_ws(d, c.sm_count, sh.grid, ws);
     const BwdPlan &p = w.plan;
-    CUtensorMap m_f128, m_f16, m_we1, m_df128, m_df16, m_db;
+    CUtensorMap m_f128, m_f16, m_we1, m_df32, m_db;
     if (!make_map(&m_f128, F, d.d, d.T, d.d * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_f16, F, d.d, d.T, d.d * 2, 64, 16, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_we1, We1, d.m, d.d, d.m * 2, M, 128, swizzle_for(Cfg::RB)) ||
-        !make_map(&m_df128, dF, d.d, d.T, d.d * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m_df16, dF, d.d, d.T, d.d * 2, 64, 16, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map(&m_df32, dF, d.d, d.T, d.d * 2, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_db, dB, d.r, d.T, d.r * 2, M, 128, swizzle_for(Cfg::RB)))
         return cudaErrorInvalidValue;
     if (!P) {
@@ -445,7 +444,7 @@ cudaError_t launch_enc_bwd(const resbm_desc &d, const void *dB, const void *F, c
     tc::EncBwdArgs a{P, static_cast<const __nv_bfloat16 *>(We2), static_cast<__nv_bfloat16 *>(dX),
                      tc::WgradArgs{p.part_big, p.nch}, p.part_small, d.T, d.d, d.act, p.max_groups};
     e = launch_clustered(tc::k_enc_bwd<M>, p.grid, Cfg::THREADS, Cfg::SMEM_BYTES, sh.cl, c.stream, m_f128, m_f16,
-                         m_we1, m_df128, m_df16, m_db, a);
+                         m_we1, m_df32, m_db, a);
     count_launches(1);
     if (e != cudaSuccess) return e;
     const int64_t cap = (int64_t)c.sm_count * 8;

@@ -49,13 +49,13 @@ template <int M_> struct EncBwdCfg {
     static constexpr bool DPLO = true;                           // dP kept as bf16 hi + lo for dF
     static constexpr uint32_t RB = M_ * 2;                       // row bytes (= swizzle) of r / m wide tiles
     static constexpr uint32_t F_STAGE = 128 * 128 * 2;
-    static constexpr uint32_t STG_HALF = 128 * 64 * 2;           // dF staging: 128 rows x 64 columns
+    static constexpr uint32_t STG_BOX = 32 * 64 * 2;             // dF staging: 32 rows x 64 columns, two per warp
     static constexpr uint32_t W_STAGE = 128 * RB;                // We1 slice: 128 rows x m
     static constexpr uint32_t TILE = 128 * RB;                   // 128 tokens x r (or m) columns
     static constexpr uint32_t WE2_BYTES = M_ * R * 2;
     static constexpr uint32_t OFF_F = 0;
     static constexpr uint32_t OFF_STG = OFF_F + NSF * F_STAGE;
-    static constexpr uint32_t OFF_W = OFF_STG + 2 * STG_HALF;
+    static constexpr uint32_t OFF_W = OFF_STG + 8 * STG_BOX;
     static constexpr uint32_t OFF_DP = OFF_W + NW * W_STAGE;     // dP (hi) tiles [token][m]
     static constexpr uint32_t OFF_DPLO = OFF_DP + NT * TILE;     // dP lo tiles (if DPLO)
     static constexpr uint32_t OFF_WE2 = OFF_DPLO + (DPLO ? NT * TILE : 0);  // We2 [m][r], K-major
@@ -86,8 +86,8 @@ struct EncBwdArgs {
 template <int M_>
 __global__ void __launch_bounds__(192, 1)
     k_enc_bwd(const __grid_constant__ CUtensorMap tm_f128, const __grid_constant__ CUtensorMap tm_f16,
-              const __grid_constant__ CUtensorMap tm_we1, const __grid_constant__ CUtensorMap tm_df128,
-              const __grid_constant__ CUtensorMap tm_df16, const __grid_constant__ CUtensorMap tm_db,
+              const __grid_constant__ CUtensorMap tm_we1, const __grid_constant__ CUtensorMap tm_df32,
+              const __grid_constant__ CUtensorMap tm_db,
               const EncBwdArgs a)
 {
     using C = EncBwdCfg<M_>;
@@ -366,7 +366,8 @@ __global__ void __launch_bounds__(192, 1)
         const int row = q * 32 + lane;
         const int et = threadIdx.x - 64;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        uint32_t cit = 0, dfit = 0, sit = 0, u = 0;
+        uint32_t cit = 0, dfit = 0, u = 0;
+        uint8_t *const boxes = smem + C::OFF_STG + (warp - 2) * 2 * C::STG_BOX;   // this warp's
         bool ok = true;
         for (int g = 0; g < ngroups && ok; ++g) {
             int tb, te;
@@ -471,52 +472,44 @@ __global__ void __launch_bounds__(192, 1)
                     const uint32_t ad_buf = dfit & 1;
                     ok = mbar_wait(smem_u32(&df_full[ad_buf]), (dfit >> 1) & 1);
                     tc_fence_after();
+                    if (q * 32 >= valid) {   // all of the warp's rows lie past the tokens (the tensor's last tile)
+                        tc_fence_before();
+                        mbar_arrive(smem_u32(&df_empty[ad_buf]));
+                    } else {
 #pragma unroll
-                    for (int h = 0; h < 2; ++h, ++sit) {
-                        const uint32_t sb = sit & 1;
-                        if (et == 0) bulk_wait_read<1>();   // staging half sb is free again
-                        named_barrier(1, 128);
-                        uint8_t *stg = smem + C::OFF_STG + sb * C::STG_HALF;
-                        // a warp whose rows all lie past the valid tokens has nothing to store
-                        const int gqend = (q * 32 < valid) ? 2 : 0;
-                        float v2[2][32];
-                        if (gqend) {   // the half's 64 columns, both TMEM loads in flight
+                        for (int h = 0; h < 2; ++h) {
+                            // 32 rows x 64 columns through one of the warp's two boxes (the other's store may
+                            // still be reading it), each warp on its own: with 128-row boxes and two barriers of
+                            // the four warps a box, the epilogue was as slow as the stream
+                            uint8_t *stg = boxes + h * C::STG_BOX;
+                            float v2[2][32];
                             tmem_ld32(tmem + lane_base + C::TM_DF + ad_buf * 128 + h * 64, v2[0]);
                             tmem_ld32(tmem + lane_base + C::TM_DF + ad_buf * 128 + h * 64 + 32, v2[1]);
+                            if (lane == 0) bulk_wait_read<1>();   // the box's previous store has read it
+                            __syncwarp();
                             tmem_ld_wait();
                             tmem_regs_ready(v2[0]);
                             tmem_regs_ready(v2[1]);
-                        }
-#pragma unroll
-                        for (int gq = 0; gq < 2; ++gq) {
-                            if (gq >= gqend) break;
-                            float (&v)[32] = v2[gq];
-                            uint32_t p[16];
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) {
-                                __nv_bfloat162 hh = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
-                                p[e] = *reinterpret_cast<uint32_t *>(&hh);
+                            if (h == 1) {
+                                tc_fence_before();
+                                mbar_arrive(smem_u32(&df_empty[ad_buf]));
                             }
 #pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                *reinterpret_cast<uint4 *>(stg + swz_offset(row, gq * 64 + 16 * e, 128)) =
-                                    make_uint4(p[4 * e], p[4 * e + 1], p[4 * e + 2], p[4 * e + 3]);
-                        }
-                        if (h == 1) {
-                            tc_fence_before();
-                            mbar_arrive(smem_u32(&df_empty[ad_buf]));
-                        }
-                        fence_async_smem();
-                        named_barrier(1, 128);
-                        if (et == 0) {
-                            const int x = cc * 128 + 64 * h;
-                            if (valid == 128) {
-                                tma_store_2d_hint(&tm_df128, x, (int32_t)t0, smem_u32(stg), l2_evict_first());
-                            } else {
-                                for (int rgi = 0; rgi * 16 < valid; ++rgi)
-                                    tma_store_2d_hint(&tm_df16, x, (int32_t)(t0 + 16 * rgi), smem_u32(stg) + rgi * 2048, l2_evict_first());
+                            for (int gq = 0; gq < 2; ++gq)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    uint32_t pk[4];
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k) pk[k] = pack_bf16(v2[gq][8 * e + 2 * k], v2[gq][8 * e + 2 * k + 1]);
+                                    *reinterpret_cast<uint4 *>(stg + swz_offset((uint32_t)lane, gq * 64 + 16 * e, 128)) =
+                                        make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                                }
+                            fence_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {   // (rows past the tensor are not stored)
+                                tma_store_2d_hint(&tm_df32, cc * 128 + 64 * h, (int32_t)(t0 + q * 32), smem_u32(stg), l2_evict_first());
+                                bulk_commit();
                             }
-                            bulk_commit();
                         }
                     }
                     if (i == tb && pend >= 0) {
@@ -559,7 +552,7 @@ __global__ void __launch_bounds__(192, 1)
             }
             tc_fence_before();
         }
-        if (et == 0) bulk_wait<0>();
+        if (lane == 0) bulk_wait<0>();
     }
 
     tc_fence_before();
