@@ -224,10 +224,9 @@ cudaError_t launch_dec_fwd(const resbm_desc &d, const void *B, const void *Wd1, 
                            const Ctx &c, float *ss = nullptr, const float *rstd = nullptr, const float *gamma32 = nullptr)
 {
     using Cfg = tc::DecFwdCfg<M>;
-    CUtensorMap m_wd2, m_y128, m_y16, m_b;
+    CUtensorMap m_wd2, m_y32, m_b;
     if (!make_map(&m_wd2, Wd2, d.d, d.m, d.d * 2, 64, M, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m_y128, Y, d.d, d.T, d.d * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m_y16, Y, d.d, d.T, d.d * 2, 64, 16, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map(&m_y32, Y, d.d, d.T, d.d * 2, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_b, B, d.r, d.T, d.r * 2, Cfg::GB / 2, 128, swizzle_for(Cfg::GB)))
         return cudaErrorInvalidValue;
     static std::atomic<uint8_t> smem_set[kMaxDev];
@@ -238,8 +237,7 @@ cudaError_t launch_dec_fwd(const resbm_desc &d, const void *B, const void *Wd1, 
     // one CTA per SM, at most one per (tile, chunk) unit (the decoder forward splits tiles by columns)
     int64_t units = ((d.T + 127) / 128) * (d.d / Cfg::NCH);
     const int grid = (int)(units < c.sm_count ? (units < 1 ? 1 : units) : c.sm_count);
-    e = launch(tc::k_dec_fwd<M, NORM>, grid, Cfg::THREADS, Cfg::SMEM_BYTES, c.stream, m_wd2, m_y128, m_y16,
-               m_b, a);
+    e = launch(tc::k_dec_fwd<M, NORM>, grid, Cfg::THREADS, Cfg::SMEM_BYTES, c.stream, m_wd2, m_y32, m_b, a);
     count_launches(1);
     return e;
 }

@@ -55,7 +55,8 @@ template <int M_> struct DecFwdCfg {
     static constexpr int SPB = GB / 32;                // 16-element K steps per block
     static constexpr uint32_t W_STAGE_BYTES = M_ * NCH * 2;
     static constexpr uint32_t TILE_BYTES = 128 * M_ * 2;   // 128 tokens x r (or m) bf16, NB blocks
-    static constexpr uint32_t STG_BYTES = 128 * NCH * 2;
+    static constexpr uint32_t BOX = 32 * 64 * 2;           // staging box: 32 rows x 64 columns
+    static constexpr int WBOX = 2 * (NCH / 128);           // per epilogue warp: two chunks' worth
     static constexpr uint32_t WD1T_BYTES = R * M_ * 2;
     // shared-memory map (offsets from a 1024-aligned base)
     static constexpr uint32_t OFF_W = 0;
@@ -66,7 +67,7 @@ template <int M_> struct DecFwdCfg {
     static constexpr uint32_t OFF_G = OFF_W + NSTAGE * W_STAGE_BYTES;   // NGB G tiles [token][m]
     static constexpr uint32_t OFF_B = OFF_G + NGB * TILE_BYTES;          // NGB B tiles [token][r] (TMA)
     static constexpr uint32_t OFF_STG = OFF_B + NGB * TILE_BYTES;
-    static constexpr uint32_t OFF_WD1T = OFF_STG + 2 * STG_BYTES;       // Wd1^T [m][r], K-major
+    static constexpr uint32_t OFF_WD1T = OFF_STG + 8 * WBOX * BOX;       // Wd1^T [m][r], K-major
     static constexpr uint32_t SMEM_BYTES = OFF_WD1T + WD1T_BYTES + 1024;  // + alignment slack
     static_assert(SMEM_BYTES <= 232448 - 512, "shared memory budget");
     static constexpr uint32_t TMEM_COLS = 2 * NCH;
@@ -117,8 +118,8 @@ __global__ void __launch_bounds__(256) k_row_rstd(const float *__restrict__ ss, 
 // tile's Y chunks (G . Wd2_chunk, + B on the first r columns), storing them by TMA.
 template <int M_, int NORM = 0>
 __global__ void __launch_bounds__(320, 1)
-    k_dec_fwd(const __grid_constant__ CUtensorMap tm_wd2, const __grid_constant__ CUtensorMap tm_y128,
-              const __grid_constant__ CUtensorMap tm_y16, const __grid_constant__ CUtensorMap tm_b,
+    k_dec_fwd(const __grid_constant__ CUtensorMap tm_wd2, const __grid_constant__ CUtensorMap tm_y32,
+              const __grid_constant__ CUtensorMap tm_b,
               const DecFwdArgs a)
 {
     using C = DecFwdCfg<M_>;
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(320, 1)
         }
         for (int i = 0; i < C::NGB; ++i) {
             mbar_init(smem_u32(&b_full[i]), 1);
-            mbar_init(smem_u32(&b_empty[i]), 1);
+            mbar_init(smem_u32(&b_empty[i]), C::EPI / 32);
             mbar_init(smem_u32(&g_full[i]), 1);
         }
         mbar_init(smem_u32(&done_bar), 1);
@@ -319,6 +320,7 @@ __global__ void __launch_bounds__(320, 1)
         const int et = threadIdx.x - 64;    // 0..255
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
         uint32_t acc_it = 0, store_it = 0;
+        uint8_t *const boxes = smem + C::OFF_STG + (warp - 2) * C::WBOX * C::BOX;   // this warp's
         bool ok = true;
         // G = phi(Q) -> bf16 -> G buffer k % NGB (K-major, NB blocks of GB-byte rows), for segment
         // k's tile whose first `valid` rows are tokens
@@ -367,7 +369,7 @@ __global__ void __launch_bounds__(320, 1)
             const int valid = valid_of(tile);
             const uint8_t *bbuf = smem + C::OFF_B + (k % C::NGB) * C::TILE_BYTES;
             const float rstd = (NORM == 2 && row < valid) ? a.rstd[t0 + row] : 0.0f;   // this row's 1 / RMS
-            for (int c = c0; c < c1 && ok; ++c, ++acc_it, ++store_it) {
+            for (int c = c0; c < c1 && ok; ++c, ++acc_it) {
                 if (C::LOOKAHEAD && c == c1 - 1 && has_next) {   // the next tile's G (its Q was issued before this chunk)
                     int64_t nt;
                     int n0, n1;
@@ -376,26 +378,30 @@ __global__ void __launch_bounds__(320, 1)
                     if (!ok) break;
                 }
                 const uint32_t ab = acc_it & 1;
-                const uint32_t sb = store_it & 1;
                 ok = mbar_wait(smem_u32(&acc_full[ab]), (acc_it >> 1) & 1);
                 tc_fence_after();
-                if (et == 0) bulk_wait_read<1>();  // staging buffer sb is free again
-                named_barrier(1, C::EPI);
-                uint8_t *stg = smem + C::OFF_STG + sb * C::STG_BYTES;
-                // a warp whose 32 rows all lie past the tile's valid tokens has nothing to store
-                const int gend = (q * 32 < valid) ? C::NCH : 0;
+                const bool rows_in = q * 32 < valid;    // else all of the warp's rows lie past the tokens
                 float2 ssq = make_float2(0.0f, 0.0f);   // NORM = 1: this row's sums of squares (even, odd columns)
-                // 64 columns (two TMEM loads in flight) at a time: one staging box
+                // 64 columns (two TMEM loads in flight) at a time through one of the warp's boxes of 32 rows,
+                // each warp on its own (no barrier between the warps: a chunk's four boxes of 128 rows with two
+                // barriers around them took every warp as long as the slowest)
 #pragma unroll
                 for (int gh = 0; gh < C::NCH / 128; ++gh) {
                     const int g2 = half * (C::NCH / 128) + gh;   // this warp's boxes of the chunk
-                    if (g2 * 64 >= gend) break;
+                    if (!rows_in) break;
                     float v2[2][32];
                     tmem_ld32(tmem + lane_base + ab * C::NCH + g2 * 64, v2[0]);
                     tmem_ld32(tmem + lane_base + ab * C::NCH + g2 * 64 + 32, v2[1]);
+                    if (lane == 0) bulk_wait_read<C::WBOX - 1>();   // the box's previous store has read it
+                    __syncwarp();
+                    uint8_t *box = boxes + (store_it++ % C::WBOX) * C::BOX;
                     tmem_ld_wait();
                     tmem_regs_ready(v2[0]);
                     tmem_regs_ready(v2[1]);
+                    if (gh == C::NCH / 128 - 1) {
+                        tc_fence_before();
+                        mbar_arrive(smem_u32(&acc_empty[ab]));
+                    }
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int g = 2 * g2 + h;   // columns [g*32, g*32+32) of the chunk
@@ -444,36 +450,28 @@ __global__ void __launch_bounds__(320, 1)
                                 }
                             }
                         }
-                        // columns [g*32, g*32+32) of the chunk: box g/2, bytes (g%2)*64 .. +64
-                        uint8_t *box = stg + (g >> 1) * 16384;
-                        const uint32_t b0 = (g & 1) * 64;
+                        // columns [g*32, g*32+32) of the chunk: bytes h * 64 .. + 64 of the box's rows
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
-                            *reinterpret_cast<uint4 *>(box + swz_offset(row, b0 + 16 * i, 128)) =
+                            *reinterpret_cast<uint4 *>(box + swz_offset((uint32_t)lane, 64 * h + 16 * i, 128)) =
                                 make_uint4(p[4 * i], p[4 * i + 1], p[4 * i + 2], p[4 * i + 3]);
+                    }
+                    fence_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {   // (rows past the tensor are not stored)
+                        tma_store_2d_hint(&tm_y32, c * C::NCH + 64 * g2, (int32_t)(t0 + q * 32), smem_u32(box), l2_evict_first());
+                        bulk_commit();
                     }
                 }
                 if (NORM == 1 && row < valid) a.ss[(int64_t)(2 * c + half) * a.T + t0 + row] = ssq.x + ssq.y;
-                tc_fence_before();
-                mbar_arrive(smem_u32(&acc_empty[ab]));
-                fence_async_smem();
-                named_barrier(1, C::EPI);
-                if (et == 0) {
-                    // the segment's first chunk is drained: its B rows are no longer read (the Q
-                    // product and the identity path of chunk 0 are done)
-                    if (c == c0) mbar_arrive(smem_u32(&b_empty[k % C::NGB]));
-                    const uint32_t sbase = smem_u32(stg);
-                    for (int b = 0; b < C::NCH / 64; ++b) {
-                        const int x = c * C::NCH + 64 * b;
-                        if (valid == 128) {
-                            tma_store_2d_hint(&tm_y128, x, (int32_t)t0, sbase + b * 16384, l2_evict_first());
-                        } else {
-                            for (int rg = 0; rg * 16 < valid; ++rg)
-                                tma_store_2d_hint(&tm_y16, x, (int32_t)(t0 + 16 * rg), sbase + b * 16384 + rg * 2048, l2_evict_first());
-                        }
-                    }
-                    bulk_commit();
+                if (!rows_in) {
+                    tc_fence_before();
+                    mbar_arrive(smem_u32(&acc_empty[ab]));
                 }
+                // the segment's first chunk is drained: this warp reads its B rows no longer (the Q
+                // product and the identity path of chunk 0 are done)
+                __syncwarp();
+                if (c == c0 && lane == 0) mbar_arrive(smem_u32(&b_empty[k % C::NGB]));
             }
             if (!C::LOOKAHEAD && ok && has_next) {   // one G buffer: the next tile's G after this segment
                 int64_t nt;
@@ -482,7 +480,7 @@ __global__ void __launch_bounds__(320, 1)
                 make_g(k + 1, valid_of(nt));
             }
         }
-        if (et == 0) bulk_wait<0>();
+        if (lane == 0) bulk_wait<0>();
     }
 
     tc_fence_before();
