@@ -622,7 +622,21 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
     g.kc = ((K + g.splits - 1) / g.splits + 63) / 64 * 64;
     g.splits = (int)((K + g.kc - 1) / g.kc);
     g.nm = (int)(bm2 ? (M + 255) / 256 : (M + 127) / 128);
-    g.nn = (int)((N + bn - 1) / bn);
+    g.bnv = bn;
+    if (pair && a_mn && b_mn && g.splits == 1) {
+        // a weight gradient with about as many tiles as pairs: narrower tiles where that evens the last round out
+        // (dWd2 of m = 512, d = 8192: 64 tiles of 256 columns on 76 pairs, 74 of 224)
+        const int64_t m2 = (M + 255) / 256, pairs = c.sm_count / 2 > 0 ? c.sm_count / 2 : 1;
+        int64_t best = 0;
+        for (int w : {256, 224, 192, 160}) {
+            const int64_t cost = (m2 * ((N + w - 1) / w) + pairs - 1) / pairs * w;
+            if (best == 0 || cost < best) {
+                best = cost;
+                g.bnv = w;
+            }
+        }
+    }
+    g.nn = (int)((N + g.bnv - 1) / g.bnv);
     g.units = (int64_t)g.nm * g.nn * g.splits;
     g.rpc = 0;
     if (bm2) {
@@ -677,7 +691,10 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
         else if (a_mn && b_mn) e = lo ? launch_gemm_t<256, true, true, true, false, true>(ma, malo, mbm, g, ep, c)
                                       : launch_gemm_t<256, true, true, false, false, true>(ma, malo, mbm, g, ep, c);
         if (e != cudaErrorNotSupported) return e;
-        // no pair fits: single CTAs need the whole-tile box for K-major B
+        // no pair fits: whole tiles, and single CTAs need the whole-tile box for K-major B
+        g.bnv = bn;
+        g.nn = (int)((N + bn - 1) / bn);
+        g.units = (int64_t)g.nm * g.nn * g.splits;
         if (!b_mn && !make_map(&mbm, B, K, N, K * 2, 64, (uint32_t)bn, CU_TENSOR_MAP_SWIZZLE_128B))
             return cudaErrorInvalidValue;
     }
@@ -1127,6 +1144,7 @@ cudaError_t tc_ffn_down_encode(const resbm_desc &d, int64_t f, const void *H, co
     g.kc = (f + 63) / 64 * 64;
     g.nm = (int)((d.T + 127) / 128);
     g.nn = (int)((d.d + bn - 1) / bn);
+    g.bnv = bn;
     g.units = (int64_t)g.nm * g.nn;
     tc::GemmEp e{};
     e.out = F_out;

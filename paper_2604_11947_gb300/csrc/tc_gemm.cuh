@@ -132,6 +132,7 @@ struct GemmShape {
     // others (256 blocks on 152 SMs: 2 against 1; 224 rows each instead). What it reads at is the bytes in flight,
     // so these launches keep one store box a warp and 64-column tiles where N allows: 6 stages of 16 KB of A, or 8.
     int rpc;
+    int bnv;             // columns per unit (BN; on pairs with an MN-major A a multiple of 32 up to BN)
 };
 
 // BM2: 256-row units, two 128-row A sub-tiles per stage against one B tile, the two halves'
@@ -379,6 +380,7 @@ __global__ void __launch_bounds__(320, 1)
     using C = GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB>;
     // (a compile-time property so that the other launches keep their index arithmetic)
     constexpr bool ROWS = RB;
+    const int bnv = PAIR && AMN ? g.bnv : BN;
     static_assert(!RB || (BN <= 128 && !AMN && !ALO && !ENCP && !PAIR && !BM2 && TS), "row-balanced: K-major A, one column block");
     static_assert(!(BM2 && (ALO || PAIR)), "256-row units without hi + lo A or pairs");
     static_assert(!(TS && (ENCP || BM2)), "TMA-store epilogue: plain 128-row units or pairs");
@@ -501,12 +503,13 @@ __global__ void __launch_bounds__(320, 1)
                         }
                     }
                     if (PAIR) {   // this CTA's half of B
+                        // (a narrower unit's half ends inside the tile: what lies past it is loaded and not read)
                         if (!BMN) {
-                            load(bdst, &tmb, kx, nb * BN + (int)crank * (BN / 2));
+                            load(bdst, &tmb, kx, nb * bnv + (int)crank * (bnv / 2));
                         } else {
 #pragma unroll
                             for (int j = 0; j < BN / 128; ++j)
-                                load(bdst + j * 8192, &tmb, nb * BN + (int)crank * (BN / 2) + 64 * j, kx);
+                                load(bdst + j * 8192, &tmb, nb * bnv + (int)crank * (bnv / 2) + 64 * j, kx);
                         }
                     } else if (!BMN) {
                         tma_load_2d(bdst, &tmb, kx, nb * BN, bar);
@@ -528,7 +531,7 @@ __global__ void __launch_bounds__(320, 1)
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
         if ((!PAIR || crank == 0) && elect_one()) {   // a pair's even CTA issues for both
-            constexpr uint32_t idesc = idesc_bf16(PAIR ? 256 : 128, BN, AMN, BMN);
+            const uint32_t idesc = idesc_bf16(PAIR ? 256 : 128, (uint32_t)bnv, AMN, BMN);
             // stage-0 descriptors, advanced by (byte offset >> 4) in the start-address field.
             // K-major: rows of 128 bytes (64 K), 8-row groups 1024 bytes apart, a K step of 16 =
             // 32 bytes. MN-major: 64-wide blocks of 64 K rows (8 KB) 8192 bytes apart along M/N,
@@ -724,12 +727,12 @@ __global__ void __launch_bounds__(320, 1)
                 constexpr int CW = TS == 1 ? 64 : 32;   // columns at a time
 #pragma unroll 1
                 for (int c0 = half * (BN / 2); c0 < (half + 1) * (BN / 2); c0 += CW) {
-                    const int64_t col0 = (int64_t)nb * BN + c0;
+                    const int64_t col0 = (int64_t)nb * bnv + c0;
                     const bool last = c0 + CW >= (half + 1) * (BN / 2);
                     float v[CW / 32][32];
 #pragma unroll
                     for (int h = 0; h < CW / 32; ++h) tmem_ld32(tmem + lane_base + ab * BN + c0 + 32 * h, v[h]);   // warp-collective
-                    if (row0 >= m_end || col0 >= g.N) {   // nothing of it exists (the same for the whole warp)
+                    if (row0 >= m_end || col0 >= g.N || c0 >= bnv) {   // nothing of it exists (the same for the whole warp)
                         tmem_ld_wait();
                         if (last) release_acc(ab);
                         continue;
@@ -819,8 +822,8 @@ __global__ void __launch_bounds__(320, 1)
                     tmem_ld32(tmem + lane_base + acc_col + c, v);   // warp-collective: every lane
                     tmem_ld_wait();
                     tmem_regs_ready<32>(v);
-                    const int64_t col = (int64_t)nb * BN + c;
-                    if (col < g.N && row < g.M)
+                    const int64_t col = (int64_t)nb * bnv + c;
+                    if (col < g.N && row < g.M && c < bnv)
                         gemm_epilogue(ep, row, col, v, g.N - col < 32 ? (int)(g.N - col) : 32, ks);
                 }
                 if (h == MH - 1) release_acc(ab);

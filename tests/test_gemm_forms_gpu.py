@@ -44,3 +44,18 @@ def test_row_balanced_units_match_whole_blocks(T, d, r, monkeypatch):
     for k in ("B", "P", "Y", "dB", "dF", "dX", "dWe1", "dWe2", "dWd1", "dWd2"):
         assert torch.equal(got[k], want[k]), k
     assert resbm.resbm_device_error() == 0
+
+
+@pytest.mark.parametrize("T,d,m", [(300, 8192, 512), (260, 8168, 264), (192, 7424, 384)])
+def test_narrower_gradient_tiles_match_single_ctas(T, d, m, monkeypatch):
+    """Weight gradients whose tiles are narrowed to even out the last round of pairs (d x m and m x d, the last
+    tile ragged), against single CTAs (RESBM_GEMM_MC=0): one split in both, so the same bits."""
+    cfg = synth.BoundaryConfig("vn_%d" % d, T=T, d=d, r=m, m=m)
+    dev = {k: to_dev(v, cfg) for k, v in host_inputs(cfg).items()}
+    flags = resbm.RESBM_FLAG_GEMM
+    got = gpu_step(cfg, dev, flags=flags)
+    monkeypatch.setenv("RESBM_GEMM_MC", "0")
+    want = gpu_step(cfg, dev, flags=flags)
+    for k in ("dWe1", "dWd2", "dF", "Y"):
+        assert torch.equal(got[k], want[k]), k
+    assert resbm.resbm_device_error() == 0
