@@ -652,7 +652,12 @@ __global__ void __launch_bounds__(1024) k_rmsnorm_dgamma(const float *__restrict
 
 int rmsnorm_bwd_blocks(int64_t rows) { return (int)(rows < kNormBwdBlocks ? (rows < 1 ? 1 : rows) : kNormBwdBlocks); }
 bool rmsnorm_bwd_supported(const resbm_desc &d) { return d.d >= 1 && d.d <= kNormBwdMaxD; }
-size_t rmsnorm_bwd_ws_bytes(const resbm_desc &d) { return (size_t)rmsnorm_bwd_blocks(d.T) * (size_t)d.d * sizeof(float); }
+// (room for 1024 blocks' partials: the size callers have been told so far stays what the call asks for)
+size_t rmsnorm_bwd_ws_bytes(const resbm_desc &d)
+{
+    const int64_t n = d.T < 1 ? 1 : d.T < 1024 ? d.T : 1024;
+    return (size_t)n * (size_t)d.d * sizeof(float);
+}
 
 cudaError_t generic_rmsnorm_bwd(const resbm_desc &d, const void *Y, const void *gamma, float eps, const void *dN,
                                 const void *dY, void *dY_out, float *dgamma, void *ws, const Ctx &c)
