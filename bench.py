@@ -98,9 +98,9 @@ def measured_peaks():
             "source": "fallback"}
 
 
-# The files that define the fused boundary kernels the bench workload runs (their device code;
-# their launch rules in tc.cu have not changed since these files were split out): the committed
-# DRAM traffic is valid while these hash the same.
+# The files that define the fused boundary kernels the bench workload runs (their device code):
+# the committed DRAM traffic is valid while these hash the same. Their launch rules are in tc.cu: a
+# change of a grid or a cluster size there needs a fresh capture too.
 BENCH_KERNEL_FILES = ("common.cuh", "tc_common.cuh", "tc_wgrad.cuh", "tc_enc_fwd.cuh", "tc_dec_fwd.cuh",
                       "tc_dec_bwd.cuh", "tc_enc_bwd.cuh")
 

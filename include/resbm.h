@@ -43,8 +43,9 @@
  *   - Results are deterministic: the same inputs, descriptor and device give the same bits.
  *     (The tensor-core backward kernels run in thread-block clusters of 1, 2 or 4 CTAs and the
  *     encoder forward in pairs, chosen from the device's occupancy and T; the environment
- *     variable RESBM_CLUSTER=1, 2 or 4 forces the backward size where it fits, and 1 also runs
- *     the encoder forward as single CTAs. Each choice is deterministic; different choices add in
+ *     variable RESBM_CLUSTER=1, 2 or 4 forces the backward size where it fits, 1 also runs the
+ *     encoder forward as single CTAs, and any of the three keeps those kernels where the chain of
+ *     products would be chosen. Each choice is deterministic; different choices add in
  *     different fixed orders, so results may differ between them in the last bits.)
  *   - T = 0 is valid: nothing is read, weight gradients are set to zero.
  *   - The scratch memory `ws` (device, >= resbm_workspace_bytes(...) bytes, 256-byte aligned)
@@ -101,8 +102,9 @@ typedef enum {
  * NULL). Everything else, the identity path included, is as in the two-layer form. */
 #define RESBM_FLAG_LINEAR 2u
 /* Run every op as its chain of tensor-core products with fused element-wise steps (the path
- * the library takes by itself for bf16 shapes the fused boundary kernels do not cover, e.g.
- * m = r = 512, or the backward at m = 128, or m != r) even where the fused kernels would run.
+ * the library takes by itself for bf16 shapes the fused boundary kernels do not cover or are
+ * slower at, e.g. m = r >= 128, m != r, the encoder backward at m = 64, or few wide tokens) even
+ * where the fused kernels would run.
  * bf16 only, d, r and m multiples of 8, 16-byte aligned pointers; otherwise the portable
  * kernels run. For testing and comparing the two tensor-core paths. */
 #define RESBM_FLAG_GEMM 4u

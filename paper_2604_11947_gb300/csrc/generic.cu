@@ -1,6 +1,7 @@
 // generic.cu -- the portable CUDA-core path of the ResBM boundary bottleneck.
 //
-// Every product of Sec. 3.2 (and of its chain-rule backward) runs through one tiled FFMA
+// Bottlenecks of up to 32 columns run on the kernels of narrow.cuh. For wider ones every product of
+// Sec. 3.2 (and of its chain-rule backward) runs through one tiled FFMA
 // kernel whose operand loaders and epilogue are small functors: the nonlinearity, its
 // derivative, the identity-path add of Eq. generalized_transformer_equation and the rounding
 // to the I/O dtype are folded into loads and stores. It handles every shape and both dtypes

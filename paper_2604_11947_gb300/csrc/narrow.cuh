@@ -12,8 +12,8 @@
 //
 // What bounds it: at T = 512, d = 256, r = 2 the step moves 2 MB and every launch is latency. The
 // chain of tiled products this replaces took 13 launches on 1 to 8 CTAs that walked K = d or K = T
-// alone (the weight gradients up to 120 us each): 378 us. Six launches on 32 to 64 CTAs, chained by
-// programmatic dependent launch, take 23 us (narrow_ok() has more sizes). Sums run in a fixed order (a warp's
+// alone (the weight gradients up to 120 us each): 378 us. Four launches (narrow_step) on 32 to 96 CTAs,
+// chained by programmatic dependent launch, take 16 us (narrow_ok() has more sizes). Sums run in a fixed order (a warp's
 // part of K, the warps in order; a rank's tokens, the ranks in order): bitwise reproducible.
 #pragma once
 
@@ -29,9 +29,9 @@ constexpr int kNChunk = 512;   // columns of Z staged at a time (k_narrow_in)
 constexpr int kNCl = 8;        // CTAs per cluster (k_narrow_wgrad)
 
 // The wide kernels (generic.cu) take any m and r; these hold a row of each in one warp's width. A step's
-// time, wide -> narrow, fp32: T = 512, d = 256, r = m = 2: 371 -> 23 us; T = 2048, d = 1024, r = m = 8:
-// 892 -> 81 us, r = m = 32: 990 -> 193 us; T = 16384, d = 2048, r = m = 16: 2.15 -> 0.67 ms; T = 65536,
-// d = 64, r = m = 32: 1.77 -> 1.30 ms; T = 32768, d = 4096, r = m = 32: 5.8 -> 4.3 ms. bf16 alike.
+// time, wide -> narrow, fp32: T = 512, d = 256, r = m = 2: 371 -> 16 us; T = 2048, d = 1024, r = m = 8:
+// 892 -> 52 us, r = m = 32: 990 -> 131 us; T = 16384, d = 2048, r = m = 16: 2.15 -> 0.64 ms; T = 65536,
+// d = 64, r = m = 32: 1.77 -> 0.95 ms; T = 32768, d = 4096, r = m = 32: 5.8 -> 4.0 ms. bf16 alike.
 inline bool narrow_ok(const resbm_desc &d) { return d.m <= kNW && d.r <= kNW; }
 
 // element (t, j) of a rows x cols tile at src (row pitch ld) -> dst[t * 33 + j], zeros past `rows`

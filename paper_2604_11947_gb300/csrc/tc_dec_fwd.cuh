@@ -14,8 +14,8 @@
 //                    G while this tile's last chunk is being computed (no bubble between tiles)
 //   epilogue warps : G = phi(Q) -> bf16 -> shared memory (the A operand, K-major), then per
 //                    chunk TMEM -> registers, + B on the first r columns (chunk 0 only), -> bf16
-//                    -> swizzled staging -> TMA store of Y (boxes of 128 rows, or 16 rows for a
-//                    partial tile). Eight warps, two per TMEM lane quarter, each pair splitting
+//                    -> swizzled staging -> TMA store of Y (boxes of 32 rows x 64 columns, a
+//                    warp's own). Eight warps, two per TMEM lane quarter, each pair splitting
 //                    a chunk's columns: one warp's TMEM and shared-memory latencies overlap the
 //                    other's work (with one warp per quarter the epilogue set the pace).
 // HBM traffic per token: read B (2r bytes, once per segment), write Y (2d bytes); Wd2 is

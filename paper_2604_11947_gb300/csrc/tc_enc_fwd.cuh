@@ -1,7 +1,7 @@
 // tc_enc_fwd.cuh -- send side of the boundary on tensor cores (Sec. 3.2 encoder, Eq. Pid
 // truncating identity path):  P = F . We1 (saved, fp32),  B = X[:, :r] + phi(P) . We2.
 //
-// Persistent CTAs in pairs (clusters of 2; single CTAs for m = 128): each pair owns a
+// Persistent CTAs in pairs (clusters of 2): each pair owns a
 // contiguous run of whole 128-token tiles (balanced over the pairs) and splits it evenly in
 // 64-column chunks, so at most one tile is shared: rank 1 takes the shared tile's last chunks
 // first and pushes its partial P (128 x m fp32) into rank 0's shared memory (st.async, counted

@@ -1,5 +1,6 @@
 // tc_gemm.cuh -- a persistent tcgen05 GEMM with the boundary's epilogues fused in, for the
-// widths the fused boundary kernels do not take (m = r = 512, the r = 128 backward, m != r):
+// shapes the fused boundary kernels do not take or are slower at (m = r = 128 and wider, m != r,
+// the m = 64 encoder backward, few wide tokens: tc_preferred() in tc.cu):
 // there the two linear layers of Sec. 3.2's encoder and decoder, and their gradients, become a
 // chain of products C = A . B (bf16 operands, fp32 accumulation in TMEM), each with the
 // element-wise step that follows it in the chain (phi, phi', the identity-path merge of Eq. Pid,
@@ -9,13 +10,16 @@
 //   A: K-major (stored M x K row-major) or MN-major (stored K x M row-major, i.e. A^T in memory)
 //   B: K-major (stored N x K row-major) or MN-major (stored K x N row-major)
 //
-// Work units are (128-row block, BN-column block, K split); unit u runs on CTA u mod grid
+// Work units are (row block, BN-column block, K split); unit u runs on CTA (pair) u mod grid
 // (n fastest, then m, then the split: CTAs running at the same time share their A block and,
-// across a wave, their B rows in L2). Per CTA:
-//   producer warp  : TMA loads of 64-deep K slices of A (128 x 64) and B (BN x 64), 128-byte
-//                    swizzle, into a ring of NST stages
-//   MMA warp       : four 128 x BN x 16 tcgen05.mma per stage into one of two TMEM accumulators
-//                    (double-buffered: the next unit's products overlap this unit's epilogue)
+// across a wave, their B rows in L2). The row block is 256 rows on a pair of CTAs with two-CTA
+// MMAs (PAIR: every product of more than 128 columns and 128 rows), else 128 rows on one CTA. Per
+// CTA:
+//   producer warp  : TMA loads of 64-deep K slices of A (128 x 64) and B (BN x 64; PAIR: half of
+//                    it), 128-byte swizzle, into a ring of NST stages
+//   MMA warp       : four 128 x BN x 16 (PAIR: 256 x BN x 16, issued by the even CTA) tcgen05.mma
+//                    per stage into one of two TMEM accumulators (double-buffered: the next
+//                    unit's products overlap this unit's epilogue)
 //   With ALO the A operand is a bf16 pair hi + lo (hi = a value rounded to bf16, lo = the
 //   rounded remainder, two matrices of the same shape): each stage holds both A tiles and the
 //   MMA warp issues hi . B and lo . B into the same accumulator, so the product sees A to about
@@ -23,7 +27,13 @@
 //   decoder's dWd2 = G^T . dY, a long sum over tokens whose terms cancel for real gradients).
 //   epilogue warps : eight warps, two per TMEM lane quarter splitting the columns: TMEM ->
 //                    registers (one output row per thread, 32 columns at a time) -> the
-//                    epilogue's element-wise step -> global memory
+//                    epilogue's element-wise step -> shared-memory boxes -> TMA stores (TS), or
+//                    straight to global memory
+// What bounds it: long products (K = d or K = tokens) the tensor cores (d = 8192, m = 512: 533 to
+// 582 cycles a 64-deep slice on pairs, 512 at their rate; the last round of units is uneven);
+// products with K = m <= 512 that write T x d the epilogue and the stores (m = 512: dF 274 us with
+// one thread's dX read-modify-write and 128-thread boxes, 190 us now, 537 MB and 275 GFLOP); N <= 128
+// with K = d the reading of A.
 // Out-of-range rows, columns and K are read as zeros by TMA and never written, so any M, N, K
 // with 16-byte row pitches work. Each output element is summed by one CTA in K order (a split-K
 // launch writes per-split fp32 slots that a second kernel adds in slot order), so results are
@@ -113,7 +123,7 @@ struct GemmEp {
     float alpha, beta;   // AXPBY
     // ENCP launches (the encoder fused into the FFN down-projection): F = acc rounded to bf16
     // (stored at out if set), and the partial P_slice = F_tile . We1[cols of the tile] summed over
-    // a thread's BN / 2 columns, written to slot (nb * 2 + half) of pslots (slots T x pm fp32,
+    // half of the unit's columns, written to slot (nb * 2 + half) of pslots (slots T x pm fp32,
     // slot_stride apart)
     const __nv_bfloat16 *we1;   // d x pm
     float *pslots;
