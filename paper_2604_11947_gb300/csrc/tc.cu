@@ -846,25 +846,37 @@ bool tc_supported(const resbm_desc &d, int op)
 // write one d x m partial gradient per CTA or cluster, which weighs against their one pass over the data
 // when a CTA gets few tokens; the chain spreads both over the chip but reads the T x d input of a backward
 // op twice and takes three to six launches (20 to 30 us at least). Measured, us, fused / chain (T x d):
-//   encode fwd  m = 16: 1000 x 4096 24 / 19, 4096 x 4096 17 / 20;  m = 32: 1000 x 512 13 / 9 (but in a
-//               step 39 / 40 in all), 1000 x 4096 29 / 18, 4096 x 1024 10.7 / 11.2, 16384 x 2048 19 / 22;  m = 64: 256 x 512 16 / 11, 32768 x 8192 106 / 105,
-//               65536 x 4096 98 / 112;  m = 128: 256 x 512 39 / 12 ... 65536 x 4096 155 / 124 (no fused kernel)
-//   decode fwd  m = 64: 1000 x 4096 10 / 10, 65536 x 4096 82 / 103;  m = 128: 1000 x 512 17 / 12, 32768 x 8192
+//   encode fwd  m = 16: 1000 x 4096 24 / 19, 4096 x 4096 17 / 20;  m = 32: 1000 x 512 12 / 9 (but in a
+//               step 39 / 40 in all), 1000 x 4096 29 / 18, 4096 x 1024 10.3 / 10.8, 4096 x 4096 19.4 / 18.4 (but
+//               the same in a step), 16384 x 2048 18 / 22;  m = 128: 256 x 512 39 / 12 ... 65536 x 4096
+//               155 / 121 (no fused kernel).  m = 64 in a step, whose other kernels leave their writes in L2 (the
+//               four ops in turn): 33000 x 512 157 / 132, 49152 x 4096 544 / 530, 65536 x 1024 305 / 288, 65536 x
+//               4096 679 / 678, 98304 x 2048 632 / 598, 131072 x 4096 1224 / 1214;  65536 x 5120 798 / 800,
+//               65536 x 8192 1157 / 1166
+//   decode fwd  m = 64: 1000 x 4096 9 / 9, 65536 x 4096 83 / 102;  m = 128: 1000 x 512 17 / 11, 32768 x 8192
 //               104 / 103, 65536 x 4096 121 / 115
-//   decode bwd  m = 32: 1000 x 4096 38 / 34, 16384 x 2048 30 / 44;  m = 64: 1000 x 512 21 / 31, 1000 x 4096
-//               71 / 39, 65536 x 1024 97 / 110, 16384 x 2048 54 / 51, 32768 x 8192 234 / 223
-//   encode bwd  m = 16: 1000 x 4096 59 / 22, 4096 x 4096 50 / 32, 16384 x 8192 119 / 127;  m = 32: 1000 x 512
-//               16 / 21, 4096 x 4096 70 / 31, 16384 x 2048 42 / 55, 32768 x 8192 259 / 219, 65536 x 4096
-//               200 / 235;  m = 64: 256 x 512 26 / 21 ... 65536 x 4096 485 / 235 (no fused kernel)
+//   decode bwd  m = 32: 1000 x 4096 39 / 34, 1000 x 8192 65 / 44, 4096 x 8192 77 / 54 (in a step 181 / 171), 6144 x
+//               8192 79 / 70 (in a step 200 / 202), 2048 x 4096 42 / 36 (in a step 91 / 95), 16384 x 2048 30 / 46;
+//               m = 64: 1000 x 512 21 / 30, 1000 x 4096 71 / 40, 36864 x 1024 42 / 67, 65536 x 1024 96 / 108,
+//               81920 x 1024 149 / 129, 98304 x 1536 215 / 179, 262144 x 1024 410 / 340, 262144 x 512 258 / 305,
+//               16384 x 2048 54 / 51, 32768 x 8192 234 / 217
+//   encode bwd  m = 16: 1000 x 4096 59 / 24, 4096 x 4096 50 / 34, 16384 x 8192 117 / 130;  m = 32: 1000 x 512
+//               15 / 20, 4096 x 4096 70 / 31, 16384 x 2048 40 / 56, 32768 x 8192 259 / 221, 65536 x 4096
+//               198 / 235;  m = 64: 256 x 512 26 / 20 ... 65536 x 4096 485 / 235 (no fused kernel)
 // RESBM_CLUSTER set (the fused kernels' cluster size is being forced) keeps the fused kernels.
 bool tc_preferred(const resbm_desc &d, int op)
 {
     if (forced_cluster() || !gemm_supported(d, op)) return true;
     switch (op) {
     case RESBM_OP_ENCODE_FWD:
-        return d.m == 16 ? !(d.T <= 2048 && d.d >= 2048) : d.m == 32 ? !(d.T <= 2048 && d.d >= 1024) : d.T > 32768;
+        return d.m == 16   ? !(d.T <= 2048 && d.d >= 2048)
+               : d.m == 32 ? !(d.T <= 2048 && d.d >= 1024)
+                           : d.T > 49152 && d.d >= 5120;
     case RESBM_OP_DECODE_FWD: return d.m <= 64;
-    case RESBM_OP_DECODE_BWD: return d.m <= 32 || d.d < 2048;
+    case RESBM_OP_DECODE_BWD:
+        return d.m == 16   ? true
+               : d.m == 32 ? !(d.d >= 4096 && d.T <= d.d * 3 / 4 - 2048)
+                           : d.d < 1024 || (d.d < 2048 && d.T * d.d <= (int64_t)72 << 20);
     case RESBM_OP_ENCODE_BWD:
         return d.m == 16 ? d.d < 1024 + d.T / 2 : d.T > 38912 || d.d < 512 + d.T / 5;
     }

@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 
 # T, d, r = m
 SHAPES = [(2048, 2048, 16), (2049, 2048, 16), (700, 1408, 16), (2048, 1024, 32), (2049, 1024, 32), (1000, 768, 32),
-          (520, 2048, 64), (520, 1920, 64), (300, 256, 64), (260, 512, 128)]
+          (520, 2048, 64), (520, 1920, 64), (300, 256, 64), (260, 512, 128), (1024, 4096, 32), (1025, 4096, 32),
+          (73729, 1024, 64)]
 
 
 @pytest.mark.parametrize("T,d,r", SHAPES)
@@ -43,4 +44,16 @@ def test_gradients_not_16_byte_aligned(T, d, r):
     resbm.resbm_encode_bwd(desc, want["dB"], dev["F"], want["P"], dev["We1"], dev["We2"], dF, None, dWe1, dWe2,
                            resbm.workspace(desc, resbm.RESBM_OP_ENCODE_BWD))
     assert torch.equal(dF, want["dF"]) and torch.equal(dWe1, want["dWe1"]) and torch.equal(dWe2, want["dWe2"])
+    assert resbm.resbm_device_error() == 0
+
+
+@pytest.mark.parametrize("cluster", ["1", "2"])
+@pytest.mark.parametrize("T,d", [(1000, 512), (300, 192), (20000, 64)])
+def test_fused_m64_matches_oracle(T, d, cluster, monkeypatch):
+    """The fused m = 64 kernels at sizes that the chain takes by itself (a forced cluster size keeps them)."""
+    monkeypatch.setenv("RESBM_CLUSTER", cluster)
+    cfg = synth.BoundaryConfig("route_fused_%d_%d" % (T, d), T=T, d=d, r=64, m=64)
+    h = host_inputs(cfg)
+    dev = {k: to_dev(v, cfg) for k, v in h.items()}
+    _compare_all(cfg, gpu_step(cfg, dev), oracle_step(cfg, h), dev)
     assert resbm.resbm_device_error() == 0
