@@ -250,9 +250,8 @@ cudaError_t launch_enc_fwd(const resbm_desc &d, const void *X, const void *F, co
     const CUtensorMapSwizzle wswz = Cfg::WSW == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
                                     : Cfg::WSW == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                                                      : CU_TENSOR_MAP_SWIZZLE_32B;
-    CUtensorMap m_f128, m_f16, m_we1;
+    CUtensorMap m_f128, m_we1;
     if (!make_map(&m_f128, F, d.d, d.T, d.d * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m_f16, F, d.d, d.T, d.d * 2, 64, 16, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_we1, We1, d.m, d.d, d.m * 2, Cfg::WSW / 2, 64, wswz))
         return cudaErrorInvalidValue;
     static std::atomic<uint8_t> smem_set[kMaxDev];
@@ -278,8 +277,7 @@ cudaError_t launch_enc_fwd(const resbm_desc &d, const void *X, const void *F, co
             grid = 2 * pairs;
         }
     }
-    e = launch_clustered(tc::k_enc_fwd<M>, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, cl, c.stream, m_f128, m_f16,
-                         m_we1, a);
+    e = launch_clustered(tc::k_enc_fwd<M>, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, cl, c.stream, m_f128, m_we1, a);
     count_launches(1);
     return e;
 }
@@ -364,9 +362,8 @@ cudaError_t launch_dec_bwd(const resbm_desc &d, const void *dY, const void *B, c
     const BwdShape sh = bwd_shape(tc::k_dec_bwd<M>, d.T, c.sm_count, Cfg::THREADS, Cfg::SMEM_BYTES, Cfg::CLMAX,
                                   Cfg::CL_MIN_TOKENS, c.device, fit, true);
     const BwdPlan p = bwd_plan(d, c.sm_count, sh.grid, Cfg::NT, d.r * d.m, ws);
-    CUtensorMap m_dy128, m_dy16, m_wd2, m_b, m_yr;
+    CUtensorMap m_dy128, m_wd2, m_b, m_yr;
     if (!make_map(&m_dy128, dY, d.d, d.T, d.d * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m_dy16, dY, d.d, d.T, d.d * 2, 64, 16, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_wd2, Wd2, d.d, d.m, d.d * 2, 64, M, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_b, B, d.r, d.T, d.r * 2, M, 128, swizzle_for(Cfg::RB)) ||
         !make_map(&m_yr, dY, d.d, d.T, d.d * 2, M, 128, swizzle_for(Cfg::RB)))
@@ -375,7 +372,7 @@ cudaError_t launch_dec_bwd(const resbm_desc &d, const void *dY, const void *B, c
                      static_cast<__nv_bfloat16 *>(dB),
                      tc::WgradArgs{p.part_big, p.nch},
                      p.part_small, d.T, d.d, d.act, d.merge_identity, p.max_groups, after_independent ? 1 : 0};
-    e = launch_clustered(tc::k_dec_bwd<M>, p.grid, Cfg::THREADS, Cfg::SMEM_BYTES, sh.cl, c.stream, m_dy128, m_dy16,
+    e = launch_clustered(tc::k_dec_bwd<M>, p.grid, Cfg::THREADS, Cfg::SMEM_BYTES, sh.cl, c.stream, m_dy128,
                          m_wd2, m_b, m_yr, a);
     count_launches(1);
     if (e != cudaSuccess) return e;
@@ -427,9 +424,8 @@ cudaError_t launch_enc_bwd(const resbm_desc &d, const void *dB, const void *F, c
                                   Cfg::CL_MIN_TOKENS, c.device, fit, false);
     const EncBwdWs w = enc_bwd_ws(d, c.sm_count, sh.grid, ws);
     const BwdPlan &p = w.plan;
-    CUtensorMap m_f128, m_f16, m_we1, m_df32, m_db;
+    CUtensorMap m_f128, m_we1, m_df32, m_db;
     if (!make_map(&m_f128, F, d.d, d.T, d.d * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m_f16, F, d.d, d.T, d.d * 2, 64, 16, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_we1, We1, d.m, d.d, d.m * 2, M, 128, swizzle_for(Cfg::RB)) ||
         !make_map(&m_df32, dF, d.d, d.T, d.d * 2, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_db, dB, d.r, d.T, d.r * 2, M, 128, swizzle_for(Cfg::RB)))
@@ -441,8 +437,7 @@ cudaError_t launch_enc_bwd(const resbm_desc &d, const void *dB, const void *F, c
     }
     tc::EncBwdArgs a{P, static_cast<const __nv_bfloat16 *>(We2), static_cast<__nv_bfloat16 *>(dX),
                      tc::WgradArgs{p.part_big, p.nch}, p.part_small, d.T, d.d, d.act, p.max_groups};
-    e = launch_clustered(tc::k_enc_bwd<M>, p.grid, Cfg::THREADS, Cfg::SMEM_BYTES, sh.cl, c.stream, m_f128, m_f16,
-                         m_we1, m_df32, m_db, a);
+    e = launch_clustered(tc::k_enc_bwd<M>, p.grid, Cfg::THREADS, Cfg::SMEM_BYTES, sh.cl, c.stream, m_f128, m_we1, m_df32, m_db, a);
     count_launches(1);
     if (e != cudaSuccess) return e;
     const int64_t cap = (int64_t)c.sm_count * 8;
@@ -790,7 +785,7 @@ size_t slot_floats(int64_t M, int64_t N, int64_t K, int sms)
 
 // dWd1 = B^T . dQ takes dQ as a hi + lo pair (as dQ^T . B, transposed by its reduction) up to m = r = 64,
 // where the chain runs in place of a fused kernel that does.
-bool dwd1_pair(const resbm_desc &d) { return d.m == d.r && d.m <= 64; }
+bool dwd1_pair(const resbm_desc &d) { return d.m == d.r && tc_width_ok(d.m) && d.m <= 64; }
 
 GemmWs gemm_ws(const resbm_desc &d, int op, int sms, void *ws, bool have_P)
 {

@@ -102,9 +102,8 @@ struct DecBwdArgs {
 
 template <int M_>
 __global__ void __launch_bounds__(192, 1)
-    k_dec_bwd(const __grid_constant__ CUtensorMap tm_dy128, const __grid_constant__ CUtensorMap tm_dy16,
-              const __grid_constant__ CUtensorMap tm_wd2, const __grid_constant__ CUtensorMap tm_b,
-              const __grid_constant__ CUtensorMap tm_yr, const DecBwdArgs a)
+    k_dec_bwd(const __grid_constant__ CUtensorMap tm_dy128, const __grid_constant__ CUtensorMap tm_wd2,
+              const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ CUtensorMap tm_yr, const DecBwdArgs a)
 {
     using C = DecBwdCfg<M_>;
     extern __shared__ uint8_t smem_raw[];
@@ -191,7 +190,6 @@ __global__ void __launch_bounds__(192, 1)
         if (elect_one()) {
             const uint64_t stream_pol = l2_evict_first();   // read once
             tma_prefetch_desc(&tm_dy128);
-            tma_prefetch_desc(&tm_dy16);
             tma_prefetch_desc(&tm_wd2);
             tma_prefetch_desc(&tm_b);
             tma_prefetch_desc(&tm_yr);
@@ -228,22 +226,13 @@ __global__ void __launch_bounds__(192, 1)
                             ++wit;
                         }
                         const int64_t t0 = start + 128 * (int64_t)i;
-                        const int valid = (int)((end - t0) < 128 ? (end - t0) : 128);
-                        const int nb = (valid + 15) / 16;
                         const uint32_t s = yit % C::NSY, ph = (yit / C::NSY) & 1;
                         if (!mbar_wait(smem_u32(&y_empty[s]), ph ^ 1)) { ok = false; break; }
                         const uint32_t dst = smem_u32(smem + C::OFF_Y + s * C::Y_STAGE);
                         const uint32_t bar = smem_u32(&y_full[s]);
-                        mbar_expect_tx(bar, valid == 128 ? C::Y_STAGE : (uint32_t)nb * 2u * 2048u);
-                        for (int h = 0; h < 2; ++h) {
-                            if (valid == 128) {
-                                tma_load_2d_hint(dst + h * 16384, &tm_dy128, cc * 128 + 64 * h, (int32_t)t0, bar, stream_pol);
-                            } else {
-                                for (int rg = 0; rg < nb; ++rg)
-                                    tma_load_2d_hint(dst + h * 16384 + rg * 2048, &tm_dy16, cc * 128 + 64 * h,
-                                                (int32_t)(t0 + 16 * rg), bar, stream_pol);
-                            }
-                        }
+                        mbar_expect_tx(bar, C::Y_STAGE);
+                        for (int h = 0; h < 2; ++h)   // (rows past T arrive as zeros)
+                            tma_load_2d_hint(dst + h * 16384, &tm_dy128, cc * 128 + 64 * h, (int32_t)t0, bar, stream_pol);
                         ++yit;
                     }
                     if (!ok) break;

@@ -85,9 +85,8 @@ struct EncBwdArgs {
 
 template <int M_>
 __global__ void __launch_bounds__(192, 1)
-    k_enc_bwd(const __grid_constant__ CUtensorMap tm_f128, const __grid_constant__ CUtensorMap tm_f16,
-              const __grid_constant__ CUtensorMap tm_we1, const __grid_constant__ CUtensorMap tm_df32,
-              const __grid_constant__ CUtensorMap tm_db,
+    k_enc_bwd(const __grid_constant__ CUtensorMap tm_f128, const __grid_constant__ CUtensorMap tm_we1,
+              const __grid_constant__ CUtensorMap tm_df32, const __grid_constant__ CUtensorMap tm_db,
               const EncBwdArgs a)
 {
     using C = EncBwdCfg<M_>;
@@ -170,7 +169,6 @@ __global__ void __launch_bounds__(192, 1)
         if (elect_one()) {
             const uint64_t stream_pol = l2_evict_first();   // read once
             tma_prefetch_desc(&tm_f128);
-            tma_prefetch_desc(&tm_f16);
             tma_prefetch_desc(&tm_we1);
             tma_prefetch_desc(&tm_db);
             // F stages use slots 0, 1, ... from the start of every group (so that slots 1 and 2
@@ -207,8 +205,6 @@ __global__ void __launch_bounds__(192, 1)
                             ++wit;
                         }
                         const int64_t t0 = start + 128 * (int64_t)i;
-                        const int valid = (int)((end - t0) < 128 ? (end - t0) : 128);
-                        const int nb = (valid + 15) / 16;
                         const uint32_t s = j % C::NSF;
                         if (s >= (uint32_t)(C::NSF - 2) && !p0_seen) {   // phase-0 scratch released
                             if (!mbar_wait(smem_u32(&p0_done), g & 1)) { ok = false; break; }
@@ -219,16 +215,9 @@ __global__ void __launch_bounds__(192, 1)
                         filled |= 1u << s;
                         const uint32_t dst = smem_u32(smem + C::OFF_F + s * C::F_STAGE);
                         const uint32_t bar = smem_u32(&f_full[s]);
-                        mbar_expect_tx(bar, valid == 128 ? C::F_STAGE : (uint32_t)nb * 2u * 2048u);
-                        for (int h = 0; h < 2; ++h) {
-                            if (valid == 128) {
-                                tma_load_2d_hint(dst + h * 16384, &tm_f128, cc * 128 + 64 * h, (int32_t)t0, bar, stream_pol);
-                            } else {
-                                for (int rg = 0; rg < nb; ++rg)
-                                    tma_load_2d_hint(dst + h * 16384 + rg * 2048, &tm_f16, cc * 128 + 64 * h,
-                                                (int32_t)(t0 + 16 * rg), bar, stream_pol);
-                            }
-                        }
+                        mbar_expect_tx(bar, C::F_STAGE);
+                        for (int h = 0; h < 2; ++h)   // (rows past T arrive as zeros)
+                            tma_load_2d_hint(dst + h * 16384, &tm_f128, cc * 128 + 64 * h, (int32_t)t0, bar, stream_pol);
                         ++j;
                     }
                     if (!ok) break;
