@@ -841,39 +841,49 @@ bool tc_supported(const resbm_desc &d, int op)
 // write one d x m partial gradient per CTA or cluster, which weighs against their one pass over the data
 // when a CTA gets few tokens; the chain spreads both over the chip but reads the T x d input of a backward
 // op twice and takes three to six launches (20 to 30 us at least). Measured, us, fused / chain (T x d):
-//   encode fwd  m = 16: 1000 x 4096 24 / 19, 4096 x 4096 17 / 20;  m = 32: 1000 x 512 12 / 9 (but in a
-//               step 39 / 40 in all), 1000 x 4096 29 / 18, 4096 x 1024 10.3 / 10.8, 4096 x 4096 19.4 / 18.4 (but
-//               the same in a step), 16384 x 2048 18 / 22;  m = 128: 256 x 512 39 / 12 ... 65536 x 4096
-//               155 / 121 (no fused kernel).  m = 64 in a step, whose other kernels leave their writes in L2 (the
-//               four ops in turn): 33000 x 512 157 / 132, 49152 x 4096 544 / 530, 65536 x 1024 305 / 288, 65536 x
-//               4096 679 / 678, 98304 x 2048 632 / 598, 131072 x 4096 1224 / 1214;  65536 x 5120 798 / 800,
-//               65536 x 8192 1157 / 1166
+// ("step": the boundary step with that op by the one or the other, whose other kernels leave their writes in L2)
+//   encode fwd  m = 16: 256 x 2048 11 / 14, 1000 x 4096 18 / 19, 500 x 8192 30 / 30 (step 158 / 153), 4096 x 4096
+//               17 / 20;  m = 32: 1000 x 512 12 / 9 (but step 39 / 40), 1000 x 1024 14 / 10, 1000 x 6144 29 / 24,
+//               2000 x 1536 15 / 12, 2048 x 8192 32 / 29 (but step 227 / 240), 4096 x 1024 10.3 / 10.8, 16384 x
+//               2048 18 / 22;  m = 64, steps: 33000 x 512 157 / 132, 49152 x 4096 544 / 530, 65536 x 1024 305 / 288,
+//               65536 x 4096 679 / 678, 98304 x 2048 632 / 598, 131072 x 4096 1224 / 1214;  65536 x 5120 798 /
+//               800, 65536 x 8192 1157 / 1166;  m = 128: 256 x 512 39 / 12 ... 65536 x 4096 155 / 121 (no fused
+//               kernel)
 //   decode fwd  m = 64: 1000 x 4096 9 / 9, 65536 x 4096 83 / 102;  m = 128: 1000 x 512 17 / 11, 32768 x 8192
 //               104 / 103, 65536 x 4096 121 / 115
-//   decode bwd  m = 32: 1000 x 4096 39 / 34, 1000 x 8192 65 / 44, 4096 x 8192 77 / 54 (in a step 181 / 171), 6144 x
-//               8192 79 / 70 (in a step 200 / 202), 2048 x 4096 42 / 36 (in a step 91 / 95), 16384 x 2048 30 / 46;
-//               m = 64: 1000 x 512 21 / 30, 1000 x 4096 71 / 40, 36864 x 1024 42 / 67, 65536 x 1024 96 / 108,
-//               81920 x 1024 149 / 129, 98304 x 1536 215 / 179, 262144 x 1024 410 / 340, 262144 x 512 258 / 305,
-//               16384 x 2048 54 / 51, 32768 x 8192 234 / 217
-//   encode bwd  m = 16: 1000 x 4096 59 / 24, 4096 x 4096 50 / 34, 16384 x 8192 117 / 130;  m = 32: 1000 x 512
-//               15 / 20, 4096 x 4096 70 / 31, 16384 x 2048 40 / 56, 32768 x 8192 259 / 221, 65536 x 4096
-//               198 / 235;  m = 64: 256 x 512 26 / 20 ... 65536 x 4096 485 / 235 (no fused kernel)
+//   decode bwd  m = 32: 1000 x 4096 39 / 34, 1000 x 8192 65 / 44, 4096 x 8192 77 / 54, 2048 x 4096 42 / 36 (but step
+//               91 / 95), 6144 x 8192 79 / 70 (step 200 / 202), 16384 x 2048 30 / 46;  m = 64: 1000 x 512 21 / 30,
+//               1000 x 4096 71 / 40, 16384 x 1920 50 / 55, 36864 x 1024 42 / 67, 39000 x 1536 122 / 92, 50000 x 1280
+//               109 / 98, 76000 x 1024 99 / 123, 81920 x 1024 149 / 129, 262144 x 512 258 / 305;  steps: 19456 x 2048
+//               184 / 178, 20000 x 4096 272 / 284, 30000 x 2048 220 / 243, 24576 x 8192 510 / 516, 38912 x 4096
+//               426 / 435, 38912 x 6144 588 / 583, 45000 x 2048 366 / 324, 65536 x 4096 770 / 680
+//   encode bwd  m = 16, steps: 1000 x 1408 50 / 54, 1000 x 2048 55 / 52, 4096 x 3072 79 / 77, 6000 x 4096 103 / 108,
+//               8192 x 6144 149 / 153, 8192 x 8192 193 / 188;  m = 32, steps: 1 x 512 39 / 43, 1000 x 768 47 / 48,
+//               1000 x 1024 52 / 51, 4096 x 2048 82 / 70, 12000 x 3072 132 / 137, 16384 x 4608 207 / 202, 20000 x
+//               2048 140 / 142, 20000 x 3072 189 / 178, 32768 x 3072 238 / 235 (but alone 98 / 109), 32768 x 4096
+//               301 / 290, 45000 x 4096 353 / 365;  m = 64: 256 x 512 26 / 20 ... 65536 x 4096 485 / 235 (no
+//               fused kernel)
 // RESBM_CLUSTER set (the fused kernels' cluster size is being forced) keeps the fused kernels.
 bool tc_preferred(const resbm_desc &d, int op)
 {
     if (forced_cluster() || !gemm_supported(d, op)) return true;
     switch (op) {
     case RESBM_OP_ENCODE_FWD:
-        return d.m == 16   ? !(d.T <= 2048 && d.d >= 2048)
-               : d.m == 32 ? !(d.T <= 2048 && d.d >= 1024)
+        return d.m == 16   ? d.T > 1024 || d.d < 8192
+               : d.m == 32 ? !(d.T <= 2048 && d.d >= 1024 && (d.T <= 1024 || d.d <= 2048))
                            : d.T > 49152 && d.d >= 5120;
     case RESBM_OP_DECODE_FWD: return d.m <= 64;
     case RESBM_OP_DECODE_BWD:
-        return d.m == 16   ? true
-               : d.m == 32 ? !(d.d >= 4096 && d.T <= d.d * 3 / 4 - 2048)
-                           : d.d < 1024 || (d.d < 2048 && d.T * d.d <= (int64_t)72 << 20);
+        if (d.m == 16) return true;
+        if (d.m == 32) return !(d.d >= 4096 && d.T <= d.d * 3 / 4 - 2048);
+        if (d.d < 1024) return true;
+        // (one, two and four tiles a CTA on 152 SMs: 19456, 38912 and 77824 tokens)
+        if (d.d < 2048) return d.T <= 38912 || (d.T > 58368 && d.T * d.d <= (int64_t)76 << 20);
+        return d.T > 19456 && d.T <= 38912 && d.T * d.d <= (int64_t)200 << 20;
     case RESBM_OP_ENCODE_BWD:
-        return d.m == 16 ? d.d < 1024 + d.T / 2 : d.T > 38912 || d.d < 512 + d.T / 5;
+        if (d.m == 16) return d.d < 1024 + d.T / 2 || (d.T >= 6000 && d.d <= d.T * 3 / 4);
+        if (d.T > 38912 || d.d <= 768) return true;
+        return d.T > 19456 ? d.d <= 1024 + d.T / 16 : d.d < 512 + (d.T >= 8192 ? d.T / 4 : d.T / 5);
     }
     return true;
 }
