@@ -458,6 +458,17 @@ __device__ __forceinline__ void tridiag_top(const float *a, const float *b, int 
     __syncwarp();
 }
 
+// The power of two that brings a Gram matrix's trace to about 1. Both kernels multiply their products with
+// G by it: the sums of squares and the tridiagonal matrix, whose elements scale with sigma^4 where they are
+// squared, then keep to fp32's range for every G that does itself (the effective rank does not depend on
+// W's scale). Exact, and undone in fp64 in the results; 1 for a zero matrix, infinities and NaN.
+__device__ __forceinline__ float gram_scale(double trace)
+{
+    if (!(trace > 0.0) || isinf(trace)) return 1.0f;
+    const int e = ilogb(trace);
+    return ldexpf(1.0f, e < -126 ? 126 : e > 126 ? -126 : -e);
+}
+
 // The form for n <= kLzSmallN: every CTA keeps the whole of the cycle's vectors and repeats their
 // orthogonalisation, so that a step's only exchange is the product itself (each CTA's rows of G v into
 // every CTA's copy). With the vectors spread over the cluster (k_lanczos_top) a step takes three
@@ -525,6 +536,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_small(const float *__
     t2[1] = (double)q * q;
     sums(t2);
     const double trace = t2[0];
+    const float gs = gram_scale(trace);
     if (on) Q[tid] = q * (float)(1.0 / sqrt(t2[1]));
     cluster_sync();   // every CTA runs before anything is written into it (and Q, G are complete)
 
@@ -533,7 +545,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_small(const float *__
     uint32_t buf = 0;
     double lam = 0.0;
     for (;;) {
-        // y = G q_j, one warp per four rows, every row's sum into all CTAs' copies
+        // y = gs G q_j, one warp per four rows, every row's sum into all CTAs' copies
         {
             const float4 *v4 = reinterpret_cast<const float4 *>(Q + j * n);
             const uint32_t ydst = smem_u32(sm + L.y + buf * n);
@@ -555,7 +567,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_small(const float *__
                 const int r = lane & 3;   // eight CTAs x four rows
                 if (r <= last)
                     st_cluster_f32(map_shared(ydst + 4u * (uint32_t)(row0 + i0 + r), (uint32_t)(lane >> 2)),
-                                   r == 0 ? acc[0] : r == 1 ? acc[1] : r == 2 ? acc[2] : acc[3]);
+                                   gs * (r == 0 ? acc[0] : r == 1 ? acc[1] : r == 2 ? acc[2] : acc[3]));
             }
         }
         cluster_sync();
@@ -656,6 +668,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_small(const float *__
         __syncthreads();
     }
     if (rank == 0 && tid == 0) {
+        lam /= (double)gs;
         out[0] = lam;
         out[1] = trace;
         out[2] = lam > 0.0 ? trace / lam : 0.0;
@@ -731,6 +744,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__re
         for (int p = 0; p < kLzCl; ++p) send(tid, bs, p);
     cluster_sync();
     const double trace = total(buf, 0);
+    const float gs = gram_scale(trace);
     float scale = (float)(1.0 / sqrt(total(buf, 1)));   // 1 / ||v||: v is kept unnormalised
     buf ^= 1;
     for (int i = tid; i < nr; i += kLzThreads) Q[i] = sm[row0 + i] * scale;
@@ -740,7 +754,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__re
     double lam = 0.0;
     for (;;) {
         __syncthreads();   // y of the previous step has been read
-        // y = scale * G v, one warp per four rows
+        // y = scale * gs G v, one warp per four rows
         {
             const float4 *v4 = reinterpret_cast<const float4 *>(sm + cur * n);
             for (int i0 = 4 * warp; i0 < nr; i0 += 4 * NW) {
@@ -759,7 +773,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__re
                 for (int r = 0; r < 4; ++r)
                     for (int o = 16; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
                 if (lane < 4 && lane <= last)
-                    y[i0 + lane] = scale * (lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3]);
+                    y[i0 + lane] = scale * (gs * (lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3]));
             }
         }
         __syncthreads();
@@ -868,6 +882,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__re
         for (int i = tid; i < nr; i += kLzThreads) Q[i] = y[i] * scale;
     }
     if (rank == 0 && tid == 0) {
+        lam /= (double)gs;
         out[0] = lam;
         out[1] = trace;
         out[2] = lam > 0.0 ? trace / lam : 0.0;

@@ -137,3 +137,16 @@ def test_effective_rank_lanczos_edges(shape):
 def test_effective_rank_of_a_zero_matrix():
     out = _reff(torch.zeros(512, 64, dtype=torch.bfloat16, device="cuda"))
     assert out[0] == 0.0 and out[1] == 0.0 and out[2] == 0.0 and out[3] == 0.0
+
+
+@pytest.mark.parametrize("k", [20, 33, 55, -20, -36, -45, -55])
+@pytest.mark.parametrize("cols", [128, 520])
+def test_effective_rank_at_extreme_scales(cols, k):
+    """W scaled by 2^k, both kernels: the same arithmetic up to the power of two (at the ends the Gram matrix
+    is 2^-110 to 2^110, still in fp32's range with all its bits), so the same r_eff and sigma_max^2 but for
+    the last products' rounding near fp32's smallest numbers: 1e-6, and the same iterations within a cycle."""
+    W = torch.from_numpy(synth.matrix(1024, cols, seed=cols) / 32.0).to("cuda").to(torch.bfloat16)
+    want, got = _reff(W), _reff(W * 2.0 ** k)
+    assert abs(got[2] - want[2]) <= 1e-6 * want[2], (got, want)
+    assert abs(got[0] * 4.0 ** -k - want[0]) <= 1e-6 * want[0] and abs(got[1] * 4.0 ** -k - want[1]) <= 1e-6 * want[1]
+    assert got[3] <= want[3] + 32
