@@ -509,7 +509,7 @@ template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = f
 cudaError_t launch_gemm_t(const CUtensorMap &ma, const CUtensorMap &malo, const CUtensorMap &mb,
                           const tc::GemmShape &g, const tc::GemmEp &ep, const Ctx &c, const GemmOutMaps *out = nullptr)
 {
-    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB>;
+    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB, tc::gemm_halves(BN, AMN, ALO, ENCP, PAIR, BM2, TS, RB)>;
     const GemmOutMaps none{ma, ma, ma};   // not read
     const GemmOutMaps &mo = out ? *out : none;
     auto kernel = tc::k_gemm<BN, AMN, BMN, ALO, ENCP, PAIR, BM2, TS, RB>;
@@ -586,6 +586,18 @@ int gemm_ts(const tc::GemmEp &ep, int64_t M, int64_t N, int splits, bool lo, Gem
     return 0;
 }
 
+// The 64-deep K slices per piece of a sum (GemmShape::pc; launches without HALVES or PIECES do not read it), by the
+// product alone, so that every form of it adds in the same order. Up to m = 64, where the chain can stand in for a
+// fused kernel: a weight gradient's sum in pieces of 128 tokens, the least that a CTA of the fused decoder backward
+// sums in one accumulator; P's and dQ's (K = d) in two halves. nk: slices per split. (Cost: the encoder forward by
+// the chain 0.2 to 0.5 us of 10 to 20, the decoder backward 1 us of 50.)
+int gemm_piece(int mode, bool wg, int64_t M, int64_t N, int64_t nk)
+{
+    if (wg) return (int)(M <= 64 && nk > 2 ? 2 : nk);
+    const bool pre = mode == tc::GEP_F32 || mode == tc::GEP_P_A || mode == tc::GEP_ACT || mode == tc::GEP_DACT;
+    return (int)(pre && N <= 64 && nk >= 4 ? (nk + 1) / 2 : nk);
+}
+
 // splits: 1 for every product whose epilogue is not a plain fp32 store; with splits > 1 the
 // epilogue must be GEP_F32 into `splits` slots of M x N (ep.split_stride apart). A_lo: the lo
 // half of A as a bf16 hi + lo pair (same shape and layout as A), or null. form: the unit as the
@@ -634,6 +646,7 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
     g.nn = (int)((N + g.bnv - 1) / g.bnv);
     g.units = (int64_t)g.nm * g.nn * g.splits;
     g.rpc = 0;
+    g.pc = gemm_piece(ep.mode, a_mn, M, N, (g.kc + 63) / 64);
     if (bm2) {
         if (!a_mn && b_mn) return launch_gemm_t<256, false, true, false, false, false, true>(ma, malo, mbm, g, ep, c);
         if (!a_mn && !b_mn) return launch_gemm_t<256, false, false, false, false, false, true>(ma, malo, mbm, g, ep, c);

@@ -143,7 +143,22 @@ struct GemmShape {
     // so these launches keep one store box a warp and 64-column tiles where N allows: 6 stages of 16 KB of A, or 8.
     int rpc;
     int bnv;             // columns per unit (BN; on pairs with an MN-major A a multiple of 32 up to BN)
+    int pc;              // 64-deep K slices per piece of a sum (GemmCfg's HALVES and PIECES)
 };
+
+// Sums in pieces. The tensor core truncates as it adds to its accumulator, an error that grows with the number of
+// MMAs in one accumulator. Where a chain replaces a fused kernel whose accumulators hold shorter sums, the unit's
+// sum runs in pieces of GemmShape::pc slices, added in fp32 (to nearest) in K order.
+// HALVES: the products of up to 64 columns over d (P, dQ): two accumulators a unit, added as the epilogue reads
+// them. P over K = 8192, error against 64 bits: one accumulator 9.1e-6, the fused kernel 8.4e-6.
+// PIECES: the weight gradients of hi + lo operands, whose sums over the tokens are long: pieces alternate between
+// the two accumulators, and the epilogue warps add them in registers while the next piece runs. dWd2 at m = 64 over
+// 8192 tokens a split: one accumulator 1.9e-5, the fused kernel 2.5e-6 (~300 tokens in one).
+constexpr bool gemm_halves(int bn, bool amn, bool alo, bool encp, bool pair, bool bm2, int ts, bool rb)
+{
+    return bn <= (rb ? 64 : 128) && !amn && !alo && !encp && !pair && !bm2 && ts != 1;   // (RB with 128: N > 64)
+}
+constexpr bool gemm_pieces(bool amn, bool alo, bool pair, bool bm2) { return amn && alo && !pair && !bm2; }
 
 // BM2: 256-row units, two 128-row A sub-tiles per stage against one B tile, the two halves'
 // accumulators side by side in TMEM (one unit at a time: no accumulator double buffering).
@@ -156,7 +171,8 @@ struct GemmShape {
 // in a warp instruction: they, not the products, set the pace where K is short.
 // ENCP: one box of 32 rows x 64 columns per warp (F as the partial P's operand, and for F's store) and
 // We1's rows of the unit's columns.
-template <int BN_, bool ALO_ = false, bool BM2_ = false, int TS_ = 0, bool PAIR_ = false, bool ENCP_ = false, bool RB_ = false>
+template <int BN_, bool ALO_ = false, bool BM2_ = false, int TS_ = 0, bool PAIR_ = false, bool ENCP_ = false, bool RB_ = false,
+          bool HALVES_ = false>
 struct GemmCfg {
     static constexpr int BN = BN_;
     static constexpr uint32_t A_TILE = 128 * 64 * 2;        // 128 rows x 64 K, bf16
@@ -175,7 +191,7 @@ struct GemmCfg {
     static constexpr uint32_t OFF_WE1 = OFF_STG + 8 * STG_WARP;
     static constexpr uint32_t SMEM_BYTES = NST * STAGE + STG_BYTES + 1024;
     static_assert(SMEM_BYTES <= 232448 - 512, "shared memory budget");
-    static constexpr uint32_t TMEM_COLS = 2 * BN_;          // two accumulators
+    static constexpr uint32_t TMEM_COLS = (HALVES_ ? 4 : 2) * BN_;   // two accumulators (HALVES: two of two)
     static_assert(TMEM_COLS <= 512, "TMEM budget");
     static constexpr int EPI = 256;                         // epilogue threads (8 warps)
     static constexpr int THREADS = 64 + EPI;
@@ -233,6 +249,19 @@ __device__ __forceinline__ void st_f32x32(float *dst, const float (&v)[32], int 
     } else {
 #pragma unroll
         for (int j = 0; j < 32; ++j)
+            if (j < nv) dst[j] = v[j];
+    }
+}
+
+__device__ __forceinline__ void st_f32x16(float *dst, const float (&v)[16], int nv)
+{
+    if (nv == 16) {
+        float4 *o = reinterpret_cast<float4 *>(dst);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
             if (j < nv) dst[j] = v[j];
     }
 }
@@ -387,13 +416,16 @@ __global__ void __launch_bounds__(320, 1)
            const __grid_constant__ CUtensorMap tmo2, const __grid_constant__ CUtensorMap tmol, const GemmShape g,
            const GemmEp ep)
 {
-    using C = GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB>;
+    constexpr bool HALVES = gemm_halves(BN, AMN, ALO, ENCP, PAIR, BM2, TS, RB), PIECES = gemm_pieces(AMN, ALO, PAIR, BM2);
+    using C = GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB, HALVES>;
     // (a compile-time property so that the other launches keep their index arithmetic)
     constexpr bool ROWS = RB;
     const int bnv = PAIR && AMN ? g.bnv : BN;
     static_assert(!RB || (BN <= 128 && !AMN && !ALO && !ENCP && !PAIR && !BM2 && TS), "row-balanced: K-major A, one column block");
     static_assert(!(BM2 && (ALO || PAIR)), "256-row units without hi + lo A or pairs");
     static_assert(!(TS && (ENCP || BM2)), "TMA-store epilogue: plain 128-row units or pairs");
+    static_assert(!PIECES || (BMN && TS == 0 && !ENCP), "sums in pieces: the weight gradients on single CTAs");
+    const bool two = HALVES && (g.kc + 63) / 64 > g.pc;   // (HALVES: one split, so g.kc is K)
     constexpr int MH = BM2 ? 2 : 1;   // 128-row halves per unit (g.nm counts units of 128 * MH rows)
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -553,45 +585,53 @@ __global__ void __launch_bounds__(320, 1)
             constexpr uint64_t BK = BMN ? (2048 >> 4) : (32 >> 4);
             uint32_t it = 0, ti = 0;
             bool ok = true;
-            for (int64_t u = u_first; u < gp.units && ok; u += u_step, ++ti) {
+            for (int64_t u = u_first; u < gp.units && ok; u += u_step) {
                 int mb, nb, ks;
                 unit_of(u, mb, nb, ks);
                 int64_t k0;
                 const int nk = k_steps(ks, k0);
-                // double-buffered accumulators; BM2: one pair of half accumulators, every unit
-                const uint32_t ab = BM2 ? 0u : (ti & 1);
-                const uint32_t eph = BM2 ? ((ti & 1) ^ 1) : (((ti >> 1) & 1) ^ 1);
-                ok = mbar_wait(smem_u32(&acc_empty[ab]), eph);
-                tc_fence_after();
-                if (!ok) break;
-                const uint32_t d_tmem = tmem + ab * BN;
-                for (int kb = 0; kb < nk; ++kb, ++it) {
-                    const uint32_t s = it % C::NST, ph = (it / C::NST) & 1;
-                    ok = mbar_wait(smem_u32(&full[s]), ph);
-                    tc_fence_after();
-                    if (!ok) break;
-                    const uint64_t so = (uint64_t)((s * C::STAGE) >> 4);
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        if (PAIR) {
-                            mma_bf16_pair(d_tmem, ad0 + so + kk * AK, bd0 + so + kk * BK, idesc, kb > 0 || kk > 0);
-                            if (ALO)
-                                mma_bf16_pair(d_tmem, ad0 + so + (C::A_TILE >> 4) + kk * AK, bd0 + so + kk * BK, idesc, true);
-                            continue;
-                        }
-                        mma_bf16(d_tmem, ad0 + so + kk * AK, bd0 + so + kk * BK, idesc, kb > 0 || kk > 0);
-                        if (ALO) mma_bf16(d_tmem, ad0 + so + (C::A_TILE >> 4) + kk * AK, bd0 + so + kk * BK, idesc, true);
-                        if (BM2)   // the second 128-row half into the next BN columns
-                            mma_bf16(d_tmem + BN, ad0 + so + (C::A_TILE >> 4) + kk * AK, bd0 + so + kk * BK, idesc,
-                                     kb > 0 || kk > 0);
+                const int pc = HALVES || PIECES ? g.pc : nk;
+                for (int kp = 0; kp < nk && ok; kp += pc) {   // (one piece but for HALVES and PIECES)
+                    // double-buffered accumulators; BM2: one pair of half accumulators, every unit
+                    const uint32_t ab = BM2 ? 0u : (ti & 1);
+                    if (!HALVES || kp == 0) {
+                        const uint32_t eph = BM2 ? ((ti & 1) ^ 1) : (((ti >> 1) & 1) ^ 1);
+                        ok = mbar_wait(smem_u32(&acc_empty[ab]), eph);
+                        tc_fence_after();
+                        if (!ok) break;
                     }
-                    // the stage is free once these MMAs are done (a pair's: in both CTAs)
-                    if (PAIR) mma_commit_pair(smem_u32(&empty[s]));
-                    else mma_commit(smem_u32(&empty[s]));
+                    const uint32_t d_tmem = tmem + (HALVES ? (2 * ab + (kp ? 1 : 0)) * BN : ab * BN);
+                    const int ke = nk - kp < pc ? nk : kp + pc;
+                    for (int kb = kp; kb < ke; ++kb, ++it) {
+                        const uint32_t s = it % C::NST, ph = (it / C::NST) & 1;
+                        ok = mbar_wait(smem_u32(&full[s]), ph);
+                        tc_fence_after();
+                        if (!ok) break;
+                        const uint64_t so = (uint64_t)((s * C::STAGE) >> 4);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            if (PAIR) {
+                                mma_bf16_pair(d_tmem, ad0 + so + kk * AK, bd0 + so + kk * BK, idesc, kb > kp || kk > 0);
+                                if (ALO)
+                                    mma_bf16_pair(d_tmem, ad0 + so + (C::A_TILE >> 4) + kk * AK, bd0 + so + kk * BK, idesc, true);
+                                continue;
+                            }
+                            mma_bf16(d_tmem, ad0 + so + kk * AK, bd0 + so + kk * BK, idesc, kb > kp || kk > 0);
+                            if (ALO) mma_bf16(d_tmem, ad0 + so + (C::A_TILE >> 4) + kk * AK, bd0 + so + kk * BK, idesc, true);
+                            if (BM2)   // the second 128-row half into the next BN columns
+                                mma_bf16(d_tmem + BN, ad0 + so + (C::A_TILE >> 4) + kk * AK, bd0 + so + kk * BK, idesc,
+                                         kb > kp || kk > 0);
+                        }
+                        // the stage is free once these MMAs are done (a pair's: in both CTAs)
+                        if (PAIR) mma_commit_pair(smem_u32(&empty[s]));
+                        else mma_commit(smem_u32(&empty[s]));
+                    }
+                    if (!ok) break;
+                    if (HALVES && ke < nk) continue;   // the second half follows
+                    if (PAIR) mma_commit_pair(smem_u32(&acc_full[ab]));
+                    else mma_commit(smem_u32(&acc_full[ab]));
+                    ++ti;
                 }
-                if (!ok) break;
-                if (PAIR) mma_commit_pair(smem_u32(&acc_full[ab]));
-                else mma_commit(smem_u32(&acc_full[ab]));
             }
             if (PAIR) mma_commit_pair(smem_u32(&done_bar), 1);
             else mma_commit(smem_u32(&done_bar));
@@ -642,8 +682,24 @@ __global__ void __launch_bounds__(320, 1)
                 mbar_arrive(smem_u32(&acc_empty[ab]));
             }
         };
+        // 32 columns of the accumulator `ab` from column c (warp-collective): the loads, and their end (HALVES: w, the
+        // second half's)
+        auto acc_ld32 = [&](uint32_t ab, int c, float (&v)[32], float (&w)[32]) {
+            const uint32_t t = tmem + lane_base + ab * (HALVES ? 2 * BN : BN) + c;
+            tmem_ld32(t, v);
+            if (HALVES && two) tmem_ld32(t + BN, w);
+        };
+        auto acc_ready = [&](float (&v)[32], float (&w)[32]) {
+            tmem_ld_wait();
+            tmem_regs_ready(v);
+            if (HALVES && two) {
+                tmem_regs_ready(w);
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] += w[j];
+            }
+        };
         bool ok = true;
-        for (int64_t u = u_first; u < gp.units && ok; u += u_step, ++ti) {
+        for (int64_t u = u_first; u < gp.units && ok; u += u_step, ti += PIECES ? 0 : 1) {
             int mb, nb, ks;
             unit_of(u, mb, nb, ks);
             const uint32_t ab = BM2 ? 0u : (ti & 1);
@@ -665,6 +721,42 @@ __global__ void __launch_bounds__(320, 1)
             if (TS == 1 && ep.mode == GEP_DF && ep.rmw) {
                 const int64_t end = ts_col0 + BN / 2 < ep.aux_cols ? ts_col0 + BN / 2 : ep.aux_cols;
                 if (ts_col0 < end) rmw_rows(ep, ts_row0, m_end, ts_col0, end);   // dX[:, :r] += dB, while the products run
+            }
+            if (PIECES) {
+                float sum[BN / 32][16];   // this thread's columns
+#pragma unroll
+                for (int i = 0; i < BN / 32; ++i)
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sum[i][j] = 0.0f;
+                int64_t k0;
+                const int nk = k_steps(ks, k0);
+#pragma unroll 1
+                for (int kp = 0; kp < nk; kp += g.pc, ++ti) {
+                    const uint32_t pb = ti & 1;
+                    ok = mbar_wait(smem_u32(&acc_full[pb]), (ti >> 1) & 1);
+                    tc_fence_after();
+                    if (!ok) break;
+#pragma unroll
+                    for (int i = 0; i < BN / 32; ++i) {   // (16 at a time: 32 made the loop spill)
+                        float v[16];
+                        tmem_ld16(tmem + lane_base + pb * BN + half * (BN / 2) + 16 * i, v);   // warp-collective
+                        tmem_ld_wait();
+                        tmem_regs_ready(v);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) sum[i][j] += v[j];
+                    }
+                    release_acc(pb);
+                }
+                if (!ok) break;
+                const int64_t row = (int64_t)mb * 128 + rin;   // (the epilogue step is GEP_F32)
+                float *dst = static_cast<float *>(ep.out) + ks * ep.split_stride + row * ep.ldo;
+#pragma unroll
+                for (int i = 0; i < BN / 32; ++i) {
+                    const int64_t col = (int64_t)nb * BN + half * (BN / 2) + 16 * i;
+                    if (row >= g.M || col >= g.N) continue;
+                    st_f32x16(dst + col, sum[i], g.N - col < 16 ? (int)(g.N - col) : 16);
+                }
+                continue;
             }
             ok = mbar_wait(smem_u32(&acc_full[ab]), BM2 ? (ti & 1) : ((ti >> 1) & 1));
             tc_fence_after();
@@ -740,8 +832,9 @@ __global__ void __launch_bounds__(320, 1)
                     const int64_t col0 = (int64_t)nb * bnv + c0;
                     const bool last = c0 + CW >= (half + 1) * (BN / 2);
                     float v[CW / 32][32];
+                    float w[32];   // (HALVES: the second half)
 #pragma unroll
-                    for (int h = 0; h < CW / 32; ++h) tmem_ld32(tmem + lane_base + ab * BN + c0 + 32 * h, v[h]);   // warp-collective
+                    for (int h = 0; h < CW / 32; ++h) acc_ld32(ab, c0 + 32 * h, v[h], w);
                     if (row0 >= m_end || col0 >= g.N || c0 >= bnv) {   // nothing of it exists (the same for the whole warp)
                         tmem_ld_wait();
                         if (last) release_acc(ab);
@@ -778,8 +871,7 @@ __global__ void __launch_bounds__(320, 1)
                         uint8_t *box = next_box();
                         if (ep.mode == GEP_DACT && row < m_end)
                             ld_f32x32(static_cast<const float *>(ep.aux) + row * ep.lda + col0, x, g.N - col0 < 32 ? (int)(g.N - col0) : 32);
-                        tmem_ld_wait();
-                        tmem_regs_ready(v[0]);
+                        acc_ready(v[0], w);
                         if (last) release_acc(ab);
                         float *f32 = static_cast<float *>(ep.mode == GEP_ACT ? ep.out2 : ep.mode == GEP_DACT ? nullptr : ep.out);
                         if (f32) {   // P, Q, or a plain fp32 output
@@ -825,13 +917,12 @@ __global__ void __launch_bounds__(320, 1)
 #pragma unroll 1
             for (int h = 0; h < MH; ++h) {   // the unit's 128-row halves (one unless BM2)
                 const int64_t row = (int64_t)mb * (128 * MH) + 128 * h + rin;
-                const uint32_t acc_col = (ab + (uint32_t)h) * BN;
+                const uint32_t acc = ab + (uint32_t)h;
 #pragma unroll 1
                 for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
-                    float v[32];
-                    tmem_ld32(tmem + lane_base + acc_col + c, v);   // warp-collective: every lane
-                    tmem_ld_wait();
-                    tmem_regs_ready<32>(v);
+                    float v[32], w[32];
+                    acc_ld32(acc, c, v, w);
+                    acc_ready(v, w);
                     const int64_t col = (int64_t)nb * bnv + c;
                     if (col < g.N && row < g.M && c < bnv)
                         gemm_epilogue(ep, row, col, v, g.N - col < 32 ? (int)(g.N - col) : 32, ks);

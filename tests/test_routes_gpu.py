@@ -58,3 +58,40 @@ def test_fused_m64_matches_oracle(T, d, cluster, monkeypatch):
     dev = {k: to_dev(v, cfg) for k, v in h.items()}
     _compare_all(cfg, gpu_step(cfg, dev), oracle_step(cfg, h), dev)
     assert resbm.resbm_device_error() == 0
+
+
+@pytest.mark.parametrize("T,d,r,encoder", [(33000, 512, 64, True), (16384, 4096, 64, True), (45000, 2048, 64, True),
+                                           (1000, 4096, 64, True), (4096, 8192, 32, False)])   # (False: fused anyway)
+def test_chain_sums_are_as_exact_as_the_fused_kernels(T, d, r, encoder, monkeypatch):
+    """Where the chain replaces a fused kernel, the error of its long sums (P over d, the weight gradients of hi + lo
+    operands over the tokens) against 64 bits is no larger than the fused kernel's (which a forced cluster size
+    keeps): at most 1.05 of it, for the error's own spread from one order of summation to another (a few per cent of
+    a 2-norm over at least 10^3 elements)."""
+    cfg = synth.BoundaryConfig("route_err_%d_%d" % (T, d), T=T, d=d, r=r, m=r)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    X, F, dY, B = rand(T, d), rand(T, d), rand(T, d), rand(T, r)
+    We1, We2, Wd1, Wd2 = rand(d, r) * d ** -0.5, rand(r, r) * r ** -0.5, rand(r, r) * r ** -0.5, rand(r, d) * r ** -0.5
+    desc = resbm.desc_from_config(cfg)
+    ws = resbm.workspace(desc, resbm.RESBM_OP_BOUNDARY_STEP)
+    D = torch.Tensor.double
+    Q = D(B) @ D(Wd1)
+    s = torch.sigmoid(Q)
+    dQ = (D(dY) @ D(Wd2).T) * (s * (1 + Q * (1 - s)))
+    want = {"dWd2": (Q * s).T @ D(dY), "dWd1": D(B).T @ dQ}
+    if encoder:
+        want["P"] = D(F) @ D(We1)
+
+    def errors():
+        o = resbm.step_outputs(desc)
+        resbm.resbm_encode_fwd(desc, X, F, We1, We2, o["B"], o["P"], ws)
+        resbm.resbm_decode_bwd(desc, dY, B, Wd1, Wd2, o["dB"], o["dWd1"], o["dWd2"], ws)
+        return {k: float((D(o[k]) - w).norm() / w.norm()) for k, w in want.items()}
+
+    chain = errors()
+    monkeypatch.setenv("RESBM_CLUSTER", "4")
+    fused = errors()
+    for k in want:
+        assert chain[k] <= 1.05 * fused[k], (k, chain, fused)
+    assert resbm.resbm_device_error() == 0
