@@ -509,7 +509,7 @@ template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = f
 cudaError_t launch_gemm_t(const CUtensorMap &ma, const CUtensorMap &malo, const CUtensorMap &mb,
                           const tc::GemmShape &g, const tc::GemmEp &ep, const Ctx &c, const GemmOutMaps *out = nullptr)
 {
-    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB, tc::gemm_halves(BN, AMN, ALO, ENCP, PAIR, BM2, TS, RB)>;
+    using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB, tc::gemm_halves(BN, AMN, ALO, ENCP, PAIR, BM2, TS)>;
     const GemmOutMaps none{ma, ma, ma};   // not read
     const GemmOutMaps &mo = out ? *out : none;
     auto kernel = tc::k_gemm<BN, AMN, BMN, ALO, ENCP, PAIR, BM2, TS, RB>;
@@ -659,25 +659,29 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
     // dWe1 of d = 8192, m = 128 went 84 -> 91 us)
     const bool ts_ok = ep.mode == tc::GEP_F32 ? pair && !lo : (pair || bn == 128) && !a_mn && g.splits == 1;
     const int ts = ts_ok ? gemm_ts(ep, M, N, g.splits, lo, &mo) : 0;
-    if (ts == 2 && bn == 128 && g.nm > c.sm_count && K >= 1024) {   // P, dQ of m <= 128: row-balanced units
+    if (ts == 2 && bn == 128) {   // P, dQ of m <= 128
+        // 64-column tiles where N allows: A is what such a product reads, and beside the store boxes six stages of
+        // it fit against five (N = 8, T = 12000, d = 3072 P 27.8 us by per-thread stores with six, 30.7 with five)
+        const bool narrow = N <= 64;
         const int64_t rpc = (M + 32 * (int64_t)c.sm_count - 1) / (32 * (int64_t)c.sm_count) * 32;
-        if (rpc < INT32_MAX) {
-            const bool narrow = N <= 64;
-            CUtensorMap mrest, mbr;
-            if (!make_map(&mrest, A, K, M, K * 2, 64, rpc % 128 ? (uint32_t)(rpc % 128) : 128u, CU_TENSOR_MAP_SWIZZLE_128B) ||
-                !(b_mn ? make_map(&mbr, B, N, K, N * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
-                       : make_map(&mbr, B, K, N, K * 2, 64, narrow ? 64 : 128, CU_TENSOR_MAP_SWIZZLE_128B)))
+        const bool rb = g.nm > c.sm_count && K >= 1024 && rpc < INT32_MAX;   // row-balanced units
+        if (narrow && !b_mn && !make_map(&mbm, B, K, N, K * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)) return cudaErrorInvalidValue;
+        if (rb) {
+            CUtensorMap mrest;
+            if (!make_map(&mrest, A, K, M, K * 2, 64, rpc % 128 ? (uint32_t)(rpc % 128) : 128u, CU_TENSOR_MAP_SWIZZLE_128B))
                 return cudaErrorInvalidValue;
             g.rpc = (int)rpc;
-            if (narrow) return b_mn ? launch_gemm_t<64, false, true, false, false, false, false, 2, true>(ma, mrest, mbr, g, ep, c, &mo)
-                                    : launch_gemm_t<64, false, false, false, false, false, false, 2, true>(ma, mrest, mbr, g, ep, c, &mo);
-            return b_mn ? launch_gemm_t<128, false, true, false, false, false, false, 2, true>(ma, mrest, mbr, g, ep, c, &mo)
-                        : launch_gemm_t<128, false, false, false, false, false, false, 2, true>(ma, mrest, mbr, g, ep, c, &mo);
+            if (narrow) return b_mn ? launch_gemm_t<64, false, true, false, false, false, false, 2, true>(ma, mrest, mbm, g, ep, c, &mo)
+                                    : launch_gemm_t<64, false, false, false, false, false, false, 2, true>(ma, mrest, mbm, g, ep, c, &mo);
+            return b_mn ? launch_gemm_t<128, false, true, false, false, false, false, 2, true>(ma, mrest, mbm, g, ep, c, &mo)
+                        : launch_gemm_t<128, false, false, false, false, false, false, 2, true>(ma, mrest, mbm, g, ep, c, &mo);
         }
+        if (narrow) return b_mn ? launch_gemm_t<64, false, true, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo)
+                                : launch_gemm_t<64, false, false, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo);
+        return b_mn ? launch_gemm_t<128, false, true, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo)
+                    : launch_gemm_t<128, false, false, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo);
     }
     if (ts && bn == 128) {
-        if (ts == 2) return b_mn ? launch_gemm_t<128, false, true, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo)
-                                 : launch_gemm_t<128, false, false, false, false, false, false, 2>(ma, malo, mbm, g, ep, c, &mo);
         if (b_mn) return lo ? launch_gemm_t<128, false, true, true, false, false, false, 1>(ma, malo, mbm, g, ep, c, &mo)
                             : launch_gemm_t<128, false, true, false, false, false, false, 1>(ma, malo, mbm, g, ep, c, &mo);
         return lo ? launch_gemm_t<128, false, false, true, false, false, false, 1>(ma, malo, mbm, g, ep, c, &mo)

@@ -154,9 +154,9 @@ struct GemmShape {
 // PIECES: the weight gradients of hi + lo operands, whose sums over the tokens are long: pieces alternate between
 // the two accumulators, and the epilogue warps add them in registers while the next piece runs. dWd2 at m = 64 over
 // 8192 tokens a split: one accumulator 1.9e-5, the fused kernel 2.5e-6 (~300 tokens in one).
-constexpr bool gemm_halves(int bn, bool amn, bool alo, bool encp, bool pair, bool bm2, int ts, bool rb)
+constexpr bool gemm_halves(int bn, bool amn, bool alo, bool encp, bool pair, bool bm2, int ts)
 {
-    return bn <= (rb ? 64 : 128) && !amn && !alo && !encp && !pair && !bm2 && ts != 1;   // (RB with 128: N > 64)
+    return (bn == 64 || (bn == 128 && ts == 0)) && !amn && !alo && !encp && !pair && !bm2;   // (TS: N <= 64 by BN = 64)
 }
 constexpr bool gemm_pieces(bool amn, bool alo, bool pair, bool bm2) { return amn && alo && !pair && !bm2; }
 
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(320, 1)
            const __grid_constant__ CUtensorMap tmo2, const __grid_constant__ CUtensorMap tmol, const GemmShape g,
            const GemmEp ep)
 {
-    constexpr bool HALVES = gemm_halves(BN, AMN, ALO, ENCP, PAIR, BM2, TS, RB), PIECES = gemm_pieces(AMN, ALO, PAIR, BM2);
+    constexpr bool HALVES = gemm_halves(BN, AMN, ALO, ENCP, PAIR, BM2, TS), PIECES = gemm_pieces(AMN, ALO, PAIR, BM2);
     using C = GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB, HALVES>;
     // (a compile-time property so that the other launches keep their index arithmetic)
     constexpr bool ROWS = RB;
