@@ -11,6 +11,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <numeric>
 #include <utility>
 
 #include "tc.h"
@@ -507,7 +508,7 @@ struct GemmOutMaps {
 };
 template <int BN, bool AMN, bool BMN, bool ALO, bool ENCP = false, bool PAIR = false, bool BM2 = false, int TS = 0, bool RB = false>
 cudaError_t launch_gemm_t(const CUtensorMap &ma, const CUtensorMap &malo, const CUtensorMap &mb,
-                          const tc::GemmShape &g, const tc::GemmEp &ep, const Ctx &c, const GemmOutMaps *out = nullptr)
+                          tc::GemmShape g, const tc::GemmEp &ep, const Ctx &c, const GemmOutMaps *out = nullptr)
 {
     using Cfg = tc::GemmCfg<BN, ALO, BM2, TS, PAIR, ENCP, RB, tc::gemm_halves(BN, AMN, ALO, ENCP, PAIR, BM2, TS)>;
     const GemmOutMaps none{ma, ma, ma};   // not read
@@ -522,10 +523,12 @@ cudaError_t launch_gemm_t(const CUtensorMap &ma, const CUtensorMap &malo, const 
         const int64_t pair_units = (int64_t)((g.nm + 1) / 2) * g.nn * g.splits;
         const int64_t pairs = pair_units < pairs_fit ? pair_units : pairs_fit;
         if (pairs < 1) return cudaErrorNotSupported;
+        g.turn = (int)(pairs / std::gcd<int64_t>(pairs, g.nn));
         e = launch_clustered(kernel, (unsigned)(2 * pairs), Cfg::THREADS, Cfg::SMEM_BYTES, 2, c.stream, ma, malo, mb, mo.o,
                              mo.o2, mo.lo, g, ep);
     } else {
         const int64_t grid = RB ? (g.M + g.rpc - 1) / g.rpc : g.units < c.sm_count ? g.units : c.sm_count;
+        g.turn = (int)(grid / std::gcd<int64_t>(grid, g.nn));
         e = launch(kernel, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, c.stream, ma, malo, mb, mo.o, mo.o2, mo.lo, g, ep);
     }
     count_launches(1);
@@ -645,6 +648,7 @@ cudaError_t gemm(const Ctx &c, int64_t M, int64_t N, int64_t K, const void *A, b
     }
     g.nn = (int)((N + g.bnv - 1) / g.bnv);
     g.units = (int64_t)g.nm * g.nn * g.splits;
+    if (g.units > INT32_MAX) return cudaErrorNotSupported;   // (2^38 rows, beyond any memory)
     g.rpc = 0;
     g.pc = gemm_piece(ep.mode, a_mn, M, N, (g.kc + 63) / 64);
     if (bm2) {

@@ -143,6 +143,7 @@ struct GemmShape {
     // so these launches keep one store box a warp and 64-column tiles where N allows: 6 stages of 16 KB of A, or 8.
     int rpc;
     int bnv;             // columns per unit (BN; on pairs with an MN-major A a multiple of 32 up to BN)
+    int turn;            // row blocks between shifts of the column blocks' order (gemm_unit)
     int pc;              // 64-deep K slices per piece of a sum (GemmCfg's HALVES and PIECES)
 };
 
@@ -197,14 +198,20 @@ struct GemmCfg {
     static constexpr int THREADS = 64 + EPI;
 };
 
-__device__ __forceinline__ void gemm_unit(const GemmShape &g, int64_t u, int &mb, int &nb, int &ks)
+// (in 32 bits, which hold every unit, as the host checks: a 64-bit division costs 0.2 us, and the first ones delay
+// the first load)
+__device__ __forceinline__ void gemm_unit(const GemmShape &g, uint32_t u, int &mb, int &nb, int &ks)
 {
-    const int64_t rest = u / g.nn;
-    // the column blocks rotate with the row block: with a fixed start the grid's stride gave some CTAs
-    // every column block that carries the identity path's extra work and others none
-    nb = (int)((u + rest) % g.nn);
-    mb = (int)(rest % g.nm);
-    ks = (int)(rest / g.nm);
+    const uint32_t nn = (uint32_t)g.nn, rest = u / nn;
+    // The column blocks that carry the identity path's extra work must not keep falling to the same CTAs. With one
+    // order of the columns, block 0 of row block t is unit t * nn, on worker t * nn mod W: only every gcd(nn, W)-th
+    // worker, in turns of W / gcd row blocks. So each turn starts one column later: every worker in W row blocks
+    // gets one. (A start that moves with every row block met the grid's stride instead: 16 x 20 blocks on 76 pairs
+    // put four of the 16 identity blocks on one pair, T = 4096, d = 5120, r = 96 20.4 us; so 17.0.)
+    const uint32_t at = u - rest * nn, shift = rest < (uint32_t)g.turn ? 0 : rest / (uint32_t)g.turn % nn;
+    nb = (int)(at >= shift ? at - shift : at + nn - shift);
+    ks = g.splits > 1 ? (int)(rest / (uint32_t)g.nm) : 0;
+    mb = (int)rest - ks * g.nm;
 }
 
 // ---- the epilogue's element-wise steps on 32 consecutive columns of one row ----------------
@@ -442,15 +449,16 @@ __global__ void __launch_bounds__(320, 1)
     // this CTA's units: every gridDim.x-th from blockIdx.x, or for a pair every (gridDim.x / 2)-th
     // pair unit from the cluster index, the row block 2 * (pair row block) + rank
     const uint32_t crank = PAIR ? cluster_rank() : 0u;
-    const int64_t u_first = PAIR ? (int64_t)cluster_index() : ROWS ? 0 : (int64_t)blockIdx.x;
-    const int64_t u_step = PAIR ? (int64_t)(gridDim.x / 2) : ROWS ? 1 : (int64_t)gridDim.x;
+    const uint32_t u_first = PAIR ? cluster_index() : ROWS ? 0u : blockIdx.x;
+    const uint32_t u_step = PAIR ? gridDim.x / 2 : ROWS ? 1u : gridDim.x;
     GemmShape gp = g;
     if (ROWS) gp.units = (g.rpc + 127) / 128;
     if (PAIR) {
         gp.nm = (g.nm + 1) / 2;
         gp.units = (int64_t)gp.nm * gp.nn * gp.splits;
     }
-    auto unit_of = [&](int64_t u, int &mb, int &nb, int &ks) {
+    const uint32_t units = (uint32_t)gp.units;
+    auto unit_of = [&](uint32_t u, int &mb, int &nb, int &ks) {
         if (ROWS) {
             mb = (int)u;
             nb = ks = 0;
@@ -497,7 +505,7 @@ __global__ void __launch_bounds__(320, 1)
             tma_prefetch_desc(&tmb);
             uint32_t it = 0;
             bool ok = true;
-            for (int64_t u = u_first; u < gp.units && ok; u += u_step) {
+            for (uint32_t u = u_first; u < units && ok; u += u_step) {
                 int mb, nb, ks;
                 unit_of(u, mb, nb, ks);
                 int64_t k0;
@@ -585,7 +593,7 @@ __global__ void __launch_bounds__(320, 1)
             constexpr uint64_t BK = BMN ? (2048 >> 4) : (32 >> 4);
             uint32_t it = 0, ti = 0;
             bool ok = true;
-            for (int64_t u = u_first; u < gp.units && ok; u += u_step) {
+            for (uint32_t u = u_first; u < units && ok; u += u_step) {
                 int mb, nb, ks;
                 unit_of(u, mb, nb, ks);
                 int64_t k0;
@@ -699,7 +707,7 @@ __global__ void __launch_bounds__(320, 1)
             }
         };
         bool ok = true;
-        for (int64_t u = u_first; u < gp.units && ok; u += u_step, ti += PIECES ? 0 : 1) {
+        for (uint32_t u = u_first; u < units && ok; u += u_step, ti += PIECES ? 0 : 1) {
             int mb, nb, ks;
             unit_of(u, mb, nb, ks);
             const uint32_t ab = BM2 ? 0u : (ti & 1);
