@@ -572,7 +572,7 @@ int gemm_ts(const tc::GemmEp &ep, int64_t M, int64_t N, int splits, bool lo, Gem
     case tc::GEP_P_A:
     case tc::GEP_ACT:
     case tc::GEP_DACT: {
-        if (lo || (ep.mode == tc::GEP_DACT && ep.lo && ep.out2)) return 0;   // (a box holds two bf16 outputs)
+        if (lo || (ep.mode == tc::GEP_DACT && ep.lo && ep.out2 && N > 64)) return 0;   // (three: 64-column tiles only)
         const bool p_a = ep.mode == tc::GEP_P_A;
         const void *act = p_a ? ep.out2 : ep.out;   // the bf16 activation (or dQ, dP): always there
         map(p_a ? &m->o2 : &m->o, act, p_a ? ep.ldo2 : ep.ldo, false, 32);

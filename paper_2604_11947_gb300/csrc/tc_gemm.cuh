@@ -168,7 +168,8 @@ constexpr bool gemm_pieces(bool amn, bool alo, bool pair, bool bm2) { return amn
 // TS: the outputs leave by TMA stores from shared-memory boxes, two 4 KB boxes per epilogue warp (one
 // fills while the other's store reads it; RB: one box), each warp on its own: no barrier between warps. 1: one bf16
 // output in boxes of 32 rows x 64 columns (128-byte swizzle); 2: an fp32 output in boxes of 32 rows x 32
-// columns and / or up to two bf16 outputs of 32 x 32 in one box (64-byte rows). Per-thread 16-byte stores put 32 different rows
+// columns and / or up to two bf16 outputs of 32 x 32 in one box (64-byte rows; BN = 64 a third in the next box: dP's hi and lo
+// and phi(P); the encoder backward at m = 64, T = 32768, d = 1024 65.5 us with dP by per-thread stores, 60.6 so). Per-thread 16-byte stores put 32 different rows
 // in a warp instruction: they, not the products, set the pace where K is short.
 // ENCP: one box of 32 rows x 64 columns per warp (F as the partial P's operand, and for F's store) and
 // We1's rows of the unit's columns.
@@ -899,6 +900,11 @@ __global__ void __launch_bounds__(320, 1)
                             for (int j = 0; j < 32; ++j) v[0][j] *= dx[j];
                         } else {
                             act_fast_row<32>(ep.act, v[0]);
+                        }
+                        if (BN == 64 && ep.mode == GEP_DACT && ep.lo && ep.out2) {   // three results: A = phi(P) in a box of its own
+                            put_bf16(box, x, 0, 64);
+                            store_box(tmo2, box, col0, row0);
+                            box = next_box();
                         }
                         // the bf16 result in the box's first half, its remainder or A = phi(P) in the second
                         put_bf16(box, v[0], 0, 64);
