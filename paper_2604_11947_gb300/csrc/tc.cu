@@ -251,8 +251,9 @@ cudaError_t launch_enc_fwd(const resbm_desc &d, const void *X, const void *F, co
     const CUtensorMapSwizzle wswz = Cfg::WSW == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
                                     : Cfg::WSW == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                                                      : CU_TENSOR_MAP_SWIZZLE_32B;
-    CUtensorMap m_f128, m_we1;
+    CUtensorMap m_f128, m_frest, m_we1;
     if (!make_map(&m_f128, F, d.d, d.T, d.d * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map(&m_frest, F, d.d, d.T, d.d * 2, 64, d.T % 128 ? (uint32_t)(d.T % 128) : 128u, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m_we1, We1, d.m, d.d, d.m * 2, Cfg::WSW / 2, 64, wswz))
         return cudaErrorInvalidValue;
     static std::atomic<uint8_t> smem_set[kMaxDev];
@@ -278,7 +279,8 @@ cudaError_t launch_enc_fwd(const resbm_desc &d, const void *X, const void *F, co
             grid = 2 * pairs;
         }
     }
-    e = launch_clustered(tc::k_enc_fwd<M>, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, cl, c.stream, m_f128, m_we1, a);
+    e = launch_clustered(tc::k_enc_fwd<M>, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, cl, c.stream, m_f128, m_frest,
+                         m_we1, a);
     count_launches(1);
     return e;
 }

@@ -10,7 +10,7 @@
 // paced by its stages, not by bytes, so at T = 65536 the pairs make at most 3.5 tile passes
 // instead of 4 (the tensor's last tile may be partial).
 //   producer warp : for each tile, d in chunks of 64 columns: F tile chunk (128 x 64, K-major,
-//                   128B swizzle; rows past T as zeros) + We1 rows (64 x m, MN-major),
+//                   128B swizzle; of the last tile its rows) + We1 rows (64 x m, MN-major),
 //                   two consecutive chunks per ring stage for m <= 32
 //   MMA warp      : P (128 x m fp32 in TMEM, double-buffered per tile) += F_chunk . We1_chunk
 //   epilogue warps: TMEM -> registers (one token per thread), store P, A = phi(P) as a bf16
@@ -102,7 +102,8 @@ __device__ __forceinline__ EncFwdWork enc_fwd_work(int64_t T, int nk, uint32_t c
 
 template <int M_>
 __global__ void __launch_bounds__(192, 1)
-    k_enc_fwd(const __grid_constant__ CUtensorMap tm_f128, const __grid_constant__ CUtensorMap tm_we1, const EncFwdArgs a)
+    k_enc_fwd(const __grid_constant__ CUtensorMap tm_f128, const __grid_constant__ CUtensorMap tm_frest,
+              const __grid_constant__ CUtensorMap tm_we1, const EncFwdArgs a)
 {
     using C = EncFwdCfg<M_>;
     extern __shared__ uint8_t smem_raw[];
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(192, 1)
         // the peer's partial P of the shared tile: 128 rows of m fp32
         if (wk.recv_last) mbar_expect_tx(smem_u32(&rx_full), 128 * C::M * 4);
         tma_prefetch_desc(&tm_f128);
+        tma_prefetch_desc(&tm_frest);
         tma_prefetch_desc(&tm_we1);
     }
     // Barriers, TMEM and (in clusters) the peers are set up before the wait for the previous kernel, whose last
@@ -176,6 +178,8 @@ __global__ void __launch_bounds__(192, 1)
             bool ok = true;
             for (int ti = 0; ti < ntiles && ok; ++ti) {
                 const int64_t t0 = (wk.t_begin + ti) * 128;
+                const bool rest = valid_of(ti) < 128;   // the tensor's last tile: a box of its rows
+                const uint32_t fbytes = (uint32_t)valid_of(ti) * 128u;
                 int kc0, kc1;
                 chunks_of(ti, kc0, kc1);
                 for (int kc = kc0; kc < kc1; kc += C::SUB) {
@@ -186,14 +190,15 @@ __global__ void __launch_bounds__(192, 1)
                         break;
                     }
                     const uint32_t bar = smem_u32(&full[s]);
-                    mbar_expect_tx(bar, (uint32_t)nsub * (C::F_BYTES + C::W_BYTES));
+                    mbar_expect_tx(bar, (uint32_t)nsub * (fbytes + C::W_BYTES));
                     for (int j = 0; j < nsub; ++j) {
                         const uint32_t fdst = smem_u32(smem + C::OFF_STAGE + (s * C::SUB + j) * C::STAGE_BYTES);
                         const uint32_t wdst = fdst + C::F_BYTES;
-                        // (rows past T arrive as zeros and are not read from memory: a last tile of 104 rows in
-                        // seven 16-row boxes a chunk was bound by their issue. T = 1000, d = 2048, m = 16: 14.8 ->
-                        // 12.3 us)
-                        tma_load_2d_hint(fdst, &tm_f128, (kc + j) * 64, (int32_t)t0, bar, stream_pol);
+                        // (a partial tile's rows past T keep what the stage held: a row of P, A and B depends on its
+                        // own row of F only. In the 128-row box they would arrive as zeros, but slowly: T = 50000,
+                        // d = 2048, m = 32 43 us, with whole tiles at T = 50048 40; and seven 16-row boxes a chunk were
+                        // bound by their issue: T = 1000, d = 2048, m = 16 14.8 against 12.3 us)
+                        tma_load_2d_hint(fdst, rest ? &tm_frest : &tm_f128, (kc + j) * 64, (int32_t)t0, bar, stream_pol);
                         for (int wb = 0; wb < C::WBOXES; ++wb)
                             tma_load_2d(wdst + wb * 64 * C::WSW, &tm_we1, wb * 64, (kc + j) * 64, bar);
                     }
