@@ -458,6 +458,19 @@ __device__ __forceinline__ void tridiag_top(const float *a, const float *b, int 
     __syncwarp();
 }
 
+// One warp: the cycle's top Ritz vector s after k vectors (tridiag_top), and in *stop whether its residual's estimate,
+// the new direction's norm beta times its last component, is below half the stop.
+__device__ __forceinline__ void ritz_converged(const float *a, const float *b, int k, float *d, float *u, float *s, float beta,
+                                               float tol, float lam, int *stop)
+{
+    tridiag_top(a, b, k, d, u, s);
+    if ((threadIdx.x & 31) == 0) {
+        float s2 = 0.0f;
+        for (int v = 0; v < k; ++v) s2 = fmaf(s[v], s[v], s2);
+        *stop = beta * fabsf(s[k - 1]) <= 0.5f * tol * fabsf(lam) * sqrtf(s2);
+    }
+}
+
 // The power of two that brings a Gram matrix's trace to about 1. Both kernels multiply their products with
 // G by it: the sums of squares and the tridiagonal matrix, whose elements scale with sigma^4 where they are
 // squared, then keep to fp32's range for every G that does itself (the effective rank does not depend on
@@ -632,14 +645,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_small(const float *__
         bool more = j + 1 < kmax && it < max_iter && beta > 1e-6f * fabsf((float)lam);
         bool have_s = false;
         if (more && (j + 1 == 8 || j + 1 == 16)) {
-            if (warp == 0) {
-                tridiag_top(al, be, j + 1, pd, pu, sv);
-                if (lane == 0) {
-                    float s2 = 0.0f;
-                    for (int v = 0; v <= j; ++v) s2 = fmaf(sv[v], sv[v], s2);
-                    stop_early = beta * fabsf(sv[j]) <= 0.5f * tol * fabsf((float)lam) * sqrtf(s2);
-                }
-            }
+            if (warp == 0) ritz_converged(al, be, j + 1, pd, pu, sv, beta, tol, (float)lam, &stop_early);
             __syncthreads();
             if (stop_early) {
                 more = false;
@@ -686,6 +692,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__re
     __shared__ float hslots[2][kLzK][kLzCl];   // the same for the projections
     __shared__ double red[3][kLzThreads / 32];
     __shared__ float hs[kLzK], al[kLzK], be[kLzK + 1], sv[kLzK], pd[kLzK], pu[kLzK];
+    __shared__ int stop_early;
     const LanczosLayout L = lanczos_layout(n);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NW = kLzThreads / 32;
@@ -851,7 +858,16 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__re
         cluster_sync();
         const float beta = (float)sqrt(total(buf, 0));
         buf ^= 1;
-        if (j + 1 < kmax && it < max_iter && beta > 1e-6f * fabsf((float)lam)) {
+        bool more = j + 1 < kmax && it < max_iter && beta > 1e-6f * fabsf((float)lam), have_s = false;
+        // an early end of the cycle as in k_lanczos_small, from 2 vectors on (a product costs more here): one
+        // dominant singular value needs three (2048 x 520, all but rank one: 358 us by whole cycles)
+        if (more && (j + 1 == 2 || j + 1 == 4 || j + 1 == 16)) {
+            if (warp == 0) ritz_converged(al, be, j + 1, pd, pu, sv, beta, tol, (float)lam, &stop_early);
+            __syncthreads();
+            have_s = stop_early != 0;
+            more = !have_s;
+        }
+        if (more) {
             if (tid == 0) be[j + 1] = beta;
             scale = 1.0f / beta;
             cur ^= 1;
@@ -860,7 +876,7 @@ __global__ void __launch_bounds__(kLzThreads, 1) k_lanczos_top(const float *__re
             continue;   // (Q and be are read after later barriers)
         }
         // the cycle's top Ritz vector starts the next cycle
-        if (warp == 0) tridiag_top(al, be, j + 1, pd, pu, sv);
+        if (!have_s && warp == 0) tridiag_top(al, be, j + 1, pd, pu, sv);
         __syncthreads();
         t1[0] = 0.0;
         for (int i = tid; i < nr; i += kLzThreads) {
