@@ -193,9 +193,9 @@ template <size_t N> bool any_overlap(const Range (&outs)[N], const Range *ins, s
 
 // Which kernels run an op: the fused tensor-core kernels where they take the shape and are the faster
 // ones (unless a flag says otherwise), else the tensor-core GEMM chain, else the portable CUDA-core kernels.
-bool use_tc(const resbm_desc &d, int op)
+bool use_tc(const resbm_desc &d, int op, const Ctx &c)
 {
-    return !(d.flags & (RESBM_FLAG_GENERIC | RESBM_FLAG_GEMM)) && tc_supported(d, op) && tc_preferred(d, op);
+    return !(d.flags & (RESBM_FLAG_GENERIC | RESBM_FLAG_GEMM)) && tc_supported(d, op) && tc_preferred(d, op, c.sm_count);
 }
 // ... and where the chain does not take the call's pointers after all
 bool can_tc(const resbm_desc &d, int op)
@@ -383,7 +383,7 @@ resbm_status run_encode_fwd(const resbm_desc &d, const void *X, const void *F, c
                             const void *We2, void *B, float *P, void *ws, const Ctx &c)
 {
     if (d.T == 0) return RESBM_OK;
-    if (use_tc(d, RESBM_OP_ENCODE_FWD)) {
+    if (use_tc(d, RESBM_OP_ENCODE_FWD, c)) {
         cudaError_t e = tc_encode_fwd(d, X, F, We1, We2, B, P, ws, c);
         if (e != cudaErrorNotSupported) return finish(e);
     }
@@ -402,7 +402,7 @@ resbm_status run_decode_fwd(const resbm_desc &d, const void *B, const void *Wd1,
     if (on_tc) *on_tc = false;
     if (kept_q) *kept_q = false;
     if (d.T == 0) return RESBM_OK;
-    if (use_tc(d, RESBM_OP_DECODE_FWD)) {
+    if (use_tc(d, RESBM_OP_DECODE_FWD, c)) {
         cudaError_t e = tc_decode_fwd(d, B, Wd1, Wd2, Y, ws, c);
         if (e != cudaErrorNotSupported) {
             if (on_tc) *on_tc = e == cudaSuccess;
@@ -410,7 +410,7 @@ resbm_status run_decode_fwd(const resbm_desc &d, const void *B, const void *Wd1,
         }
     }
     if (use_gemm(d, RESBM_OP_DECODE_FWD)) {
-        const bool keep = kept_q && !use_tc(d, RESBM_OP_DECODE_BWD);
+        const bool keep = kept_q && !use_tc(d, RESBM_OP_DECODE_BWD, c);
         cudaError_t e = gemm_decode_fwd(d, B, Wd1, Wd2, Y, ws, c, keep);
         if (e != cudaErrorNotSupported) {
             if (keep) *kept_q = e == cudaSuccess;
@@ -429,7 +429,7 @@ resbm_status run_decode_bwd(const resbm_desc &d, const void *dY, const void *B, 
         resbm_status s = zero_f32(dWd1, d.r * d.m, c.stream);
         return s != RESBM_OK ? s : zero_f32(dWd2, d.m * d.d, c.stream);
     }
-    if (use_tc(d, RESBM_OP_DECODE_BWD)) {
+    if (use_tc(d, RESBM_OP_DECODE_BWD, c)) {
         cudaError_t e = tc_decode_bwd(d, dY, B, Wd1, Wd2, dB, dWd1, dWd2, ws, c, after_independent);
         if (e != cudaErrorNotSupported) return finish(e);
     }
@@ -452,7 +452,7 @@ resbm_status run_encode_bwd(const resbm_desc &d, const void *dB, const void *F, 
         resbm_status s = zero_f32(dWe1, d.d * d.m, c.stream);
         return s != RESBM_OK ? s : zero_f32(dWe2, d.m * d.r, c.stream);
     }
-    if (use_tc(d, RESBM_OP_ENCODE_BWD)) {
+    if (use_tc(d, RESBM_OP_ENCODE_BWD, c)) {
         cudaError_t e = tc_encode_bwd(d, dB, F, P, We1, We2, dF, dX, dWe1, dWe2, ws, c);
         if (e != cudaErrorNotSupported) return finish(e);
     }
@@ -573,7 +573,7 @@ resbm_status enqueue_step(const resbm_desc &d, const resbm_step_args &a, void *w
     }
     // no tensor-core path for any op, and nothing to wait for in between: the portable kernels' own step
     bool portable = narrow_step_ok(e) && !fwd_done && !bwd_ready;
-    for (int op = RESBM_OP_ENCODE_FWD; op <= RESBM_OP_ENCODE_BWD; ++op) portable = portable && !use_tc(e, op) && !use_gemm(e, op);
+    for (int op = RESBM_OP_ENCODE_FWD; op <= RESBM_OP_ENCODE_BWD; ++op) portable = portable && !use_tc(e, op, c) && !use_gemm(e, op);
     if (s == RESBM_OK && portable) return finish(generic_narrow_step(e, a, We2, Wd1, P, dWe2, dWd1, inner, c));
     if (s == RESBM_OK) s = run_encode_fwd(e, a.X, a.F, a.We1, We2, a.B, P, inner, c);
     bool dec_fwd_tc = false, kept_q = false;

@@ -886,27 +886,30 @@ bool tc_supported(const resbm_desc &d, int op)
 //               2048 140 / 142, 20000 x 3072 189 / 178, 32768 x 3072 238 / 235 (but alone 98 / 109), 32768 x 4096
 //               301 / 290, 45000 x 4096 353 / 365;  m = 64: 256 x 512 26 / 20 ... 65536 x 4096 485 / 235 (no
 //               fused kernel)
+// One rule for an op alone and in a step, whose outputs are the ops' bit for bit. (Every entry on a device of 152 SMs:
+// 19456 tokens give every CTA one whole tile there.)
 // RESBM_CLUSTER set (the fused kernels' cluster size is being forced) keeps the fused kernels.
-bool tc_preferred(const resbm_desc &d, int op)
+bool tc_preferred(const resbm_desc &d, int op, int sms)
 {
     if (forced_cluster() || !gemm_supported(d, op)) return true;
+    const int64_t round = 128 * (int64_t)sms;   // tokens: one whole tile per CTA
     switch (op) {
     case RESBM_OP_ENCODE_FWD:
         return d.m == 16   ? d.T > 1024 || d.d < 8192
                : d.m == 32 ? !(d.T <= 2048 && d.d >= 1024 && (d.T <= 1024 || d.d <= 2048))
-                           : d.T > 49152 && d.d >= 5120;
+                           : 2 * d.T > 5 * round && d.d >= 5120;
     case RESBM_OP_DECODE_FWD: return d.m <= 64;
     case RESBM_OP_DECODE_BWD:
         if (d.m == 16) return true;
         if (d.m == 32) return !(d.d >= 4096 && d.T <= d.d * 3 / 4 - 2048);
         if (d.d < 1024) return true;
-        // (one, two and four tiles a CTA on 152 SMs: 19456, 38912 and 77824 tokens)
-        if (d.d < 2048) return d.T <= 38912 || (d.T > 58368 && d.T * d.d <= (int64_t)76 << 20);
-        return d.T > 19456 && d.T <= 38912 && d.T * d.d <= (int64_t)200 << 20;
+        // (whole tiles a CTA: up to two; four, while the tensor is not much larger than L2; two of wide rows)
+        if (d.d < 2048) return d.T <= 2 * round || (d.T > 3 * round && d.T * d.d <= (int64_t)76 << 20);
+        return d.T > round && d.T <= 2 * round && d.T * d.d <= (int64_t)200 << 20;
     case RESBM_OP_ENCODE_BWD:
-        if (d.m == 16) return d.d < 1024 + d.T / 2 || (d.T >= 6000 && d.d <= d.T * 3 / 4);
-        if (d.T > 38912 || d.d <= 768) return true;
-        return d.T > 19456 ? d.d <= 1024 + d.T / 16 : d.d < 512 + (d.T >= 8192 ? d.T / 4 : d.T / 5);
+        if (d.m == 16) return d.d < 1024 + d.T / 2 || d.d < d.T * 3 / 4;
+        if (d.T > 2 * round || d.d <= 768) return true;
+        return d.T > round ? d.d <= 1024 + d.T / 16 : d.d < 512 + (d.T >= 8192 ? d.T / 4 : d.T / 5);
     }
     return true;
 }
@@ -1099,7 +1102,7 @@ cudaError_t gemm_decode_bwd(const resbm_desc &d, const void *dY, const void *B, 
 namespace {
 cudaError_t recompute_P(const resbm_desc &d, const void *F, const void *We1, const void *We2, float *P, const Ctx &c)
 {
-    if (!(d.flags & RESBM_FLAG_GEMM) && tc_supported(d, RESBM_OP_ENCODE_FWD) && tc_preferred(d, RESBM_OP_ENCODE_FWD) &&
+    if (!(d.flags & RESBM_FLAG_GEMM) && tc_supported(d, RESBM_OP_ENCODE_FWD) && tc_preferred(d, RESBM_OP_ENCODE_FWD, c.sm_count) &&
         al16(We2))
         return d.m == 16   ? launch_enc_fwd<16>(d, nullptr, F, We1, We2, nullptr, P, c)
                : d.m == 32 ? launch_enc_fwd<32>(d, nullptr, F, We1, We2, nullptr, P, c)

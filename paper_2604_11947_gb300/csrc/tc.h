@@ -9,7 +9,7 @@ namespace resbm {
 // their tiles); otherwise the portable kernels run.
 bool tc_supported(const resbm_desc &d, int op);
 // Whether they are the better choice there against the GEMM chain below.
-bool tc_preferred(const resbm_desc &d, int op);
+bool tc_preferred(const resbm_desc &d, int op, int sms);
 
 // Reads (and optionally clears) the error word of the tensor-core kernels; synchronizing.
 cudaError_t tc_device_error(unsigned int *code, bool clear);
@@ -45,7 +45,8 @@ cudaError_t tc_encode_bwd(const resbm_desc &d, const void *dB, const void *F, co
                           float *dWe2, void *ws, const Ctx &c);
 
 // The GEMM chain (tc_gemm.cuh): every op as a sequence of tcgen05 products with fused
-// epilogues, for bf16 shapes the fused kernels do not take or are slower at (tc_preferred). Needs d, r, m multiples of 8 and 16-byte aligned pointers (else cudaErrorNotSupported
+// epilogues, for bf16 shapes the fused kernels do not take or are slower at (tc_preferred). Needs
+// d, r, m multiples of 8 and 16-byte aligned pointers (else cudaErrorNotSupported
 // before anything is enqueued).
 bool gemm_supported(const resbm_desc &d, int op);
 size_t gemm_ws_bytes(const resbm_desc &d, int op, int sms);
