@@ -868,10 +868,11 @@ bool tc_supported(const resbm_desc &d, int op)
 //   encode fwd  m = 16: 256 x 2048 11 / 14, 1000 x 4096 18 / 19, 500 x 8192 30 / 30 (step 158 / 153), 4096 x 4096
 //               17 / 20;  m = 32: 1000 x 512 12 / 9 (but step 39 / 40), 1000 x 1024 14 / 10, 1000 x 6144 29 / 24,
 //               2000 x 1536 15 / 12, 2048 x 8192 32 / 29 (but step 227 / 240), 4096 x 1024 10.3 / 10.8, 16384 x
-//               2048 18 / 22;  m = 64, steps: 33000 x 512 157 / 132, 49152 x 4096 544 / 530, 65536 x 1024 305 / 288,
-//               65536 x 4096 679 / 678, 98304 x 2048 632 / 598, 131072 x 4096 1224 / 1214;  65536 x 5120 798 /
-//               800, 65536 x 8192 1157 / 1166;  m = 128: 256 x 512 39 / 12 ... 65536 x 4096 155 / 121 (no fused
-//               kernel)
+//               2048 18 / 22;  m = 64: 50000 x 2048 50 / 50 (but step 339 / 333), 65536 x 512 44 / 31, 65536 x
+//               1024 48 / 42, 98304 x 768 61 / 53, 131072 x 1024 73 / 75 (but step 504 / 488), 65536 x 2048 60 / 64
+//               (but step 419 / 414), 98304 x 2048 82 / 91 (step 576 / 577), 65536 x 4096 96 / 107 (step 653 / 658),
+//               131072 x 2048 101 / 115 (step 719 / 726), 49152 x 4096 step 544 / 530, 65536 x 5120 step 798 / 800;
+//               m = 128: 256 x 512 39 / 12 ... 65536 x 4096 155 / 121 (no fused kernel)
 //   decode fwd  m = 64: 1000 x 4096 9 / 9, 65536 x 4096 83 / 102;  m = 128: 1000 x 512 17 / 11, 32768 x 8192
 //               104 / 103, 65536 x 4096 121 / 115
 //   decode bwd  m = 32: 1000 x 4096 39 / 34, 1000 x 8192 65 / 44, 4096 x 8192 77 / 54, 2048 x 4096 42 / 36 (but step
@@ -897,7 +898,7 @@ bool tc_preferred(const resbm_desc &d, int op, int sms)
     case RESBM_OP_ENCODE_FWD:
         return d.m == 16   ? d.T > 1024 || d.d < 8192
                : d.m == 32 ? !(d.T <= 2048 && d.d >= 1024 && (d.T <= 1024 || d.d <= 2048))
-                           : 2 * d.T > 5 * round && d.d >= 5120;
+                           : d.d >= 5120 ? 2 * d.T > 5 * round : d.d >= 2048 && d.T > 3 * round;
     case RESBM_OP_DECODE_FWD: return d.m <= 64;
     case RESBM_OP_DECODE_BWD:
         if (d.m == 16) return true;

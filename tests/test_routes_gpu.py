@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(2048, 2048, 16), (2049, 2048, 16), (700, 1408, 16), (2048, 1024, 32), (2049, 1024, 32), (1000, 768, 32),
           (520, 2048, 64), (520, 1920, 64), (300, 256, 64), (260, 512, 128), (1024, 4096, 32), (1025, 4096, 32),
           (73729, 1024, 64), (77824, 1024, 64), (39000, 1024, 64), (19457, 2048, 64), (1000, 8192, 16),
-          (6000, 4096, 16), (1, 512, 32), (8192, 2432, 32), (19500, 2432, 32)]
+          (6000, 4096, 16), (1, 512, 32), (8192, 2432, 32), (19500, 2432, 32), (58400, 2048, 64)]
 
 
 @pytest.mark.parametrize("T,d,r", SHAPES)
