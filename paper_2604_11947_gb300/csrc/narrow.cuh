@@ -181,8 +181,9 @@ template <bool ENC> struct NarrowOutSmem {
     float ws[ENC ? kNThr * 33 : 1];                  // ENC: this block's columns of W
 };
 
-// One tile and block of 256 columns
-template <typename E, bool ENC>
+// One tile and block of 256 columns, a thread per column. DC: 256, or 64 where d is no larger: the tile's tokens then
+// go round the block's four groups of threads (the same sums).
+template <typename E, bool ENC, int DC>
 __device__ __forceinline__ void narrow_out_tile(const NarrowOut &a, int64_t tile, int64_t cblk, NarrowOutSmem<ENC> &sh)
 {
     float *ws = sh.ws, *in = sh.in, *vs = sh.vs;
@@ -225,38 +226,40 @@ __device__ __forceinline__ void narrow_out_tile(const NarrowOut &a, int64_t tile
             *x = from_f32<E>(to_f32(*x) + in[t * 33 + n]);
         }
     __syncthreads();
-    const int64_t c = c0 + tid;
-    if (tid >= nc) return;
-    float acc[kNT];
+    constexpr int NTG = kNT / (kNThr / DC);   // this thread's tokens, from tb on
+    const int cl = DC == kNThr ? tid : tid % DC, tb = DC == kNThr ? 0 : tid / DC * NTG;
+    const int64_t c = c0 + cl;
+    if (cl >= nc) return;
+    float acc[NTG];
 #pragma unroll
-    for (int t = 0; t < kNT; ++t) acc[t] = 0.0f;
+    for (int t = 0; t < NTG; ++t) acc[t] = 0.0f;
 #pragma unroll 4
     for (int k = 0; k < a.m; ++k) {
-        const float w = ENC ? ws[tid * 33 + k] : to_f32(W[k * a.sj + c]);
+        const float w = ENC ? ws[cl * 33 + k] : to_f32(W[k * a.sj + c]);
 #pragma unroll
-        for (int q = 0; q < kNT / 4; ++q) {
-            const float4 g = *reinterpret_cast<const float4 *>(&gs[k][4 * q]);
+        for (int q = 0; q < NTG / 4; ++q) {
+            const float4 g = *reinterpret_cast<const float4 *>(&gs[k][tb + 4 * q]);
             acc[4 * q] = fmaf(g.x, w, acc[4 * q]);
             acc[4 * q + 1] = fmaf(g.y, w, acc[4 * q + 1]);
             acc[4 * q + 2] = fmaf(g.z, w, acc[4 * q + 2]);
             acc[4 * q + 3] = fmaf(g.w, w, acc[4 * q + 3]);
         }
     }
-    E *o = static_cast<E *>(a.out) + t0 * a.d + c;
+    E *o = static_cast<E *>(a.out) + (t0 + tb) * a.d + c;
 #pragma unroll
-    for (int t = 0; t < kNT; ++t)
-        if (t < nt) {
-            const float skip = (!ENC && a.merge && c < a.r) ? in[t * 33 + c] : 0.0f;
+    for (int t = 0; t < NTG; ++t)
+        if (tb + t < nt) {
+            const float skip = (!ENC && a.merge && c < a.r) ? in[(tb + t) * 33 + c] : 0.0f;
             o[t * a.d] = from_f32<E>(skip + acc[t]);
         }
 }
 
-template <typename E, bool ENC> __global__ void __launch_bounds__(kNThr) k_narrow_out(const NarrowOut a)
+template <typename E, bool ENC, int DC> __global__ void __launch_bounds__(kNThr) k_narrow_out(const NarrowOut a)
 {
     __shared__ NarrowOutSmem<ENC> sh;
     griddep_wait();
     griddep_launch_dependents();
-    narrow_out_tile<E, ENC>(a, blockIdx.x, blockIdx.y, sh);
+    narrow_out_tile<E, ENC, DC>(a, blockIdx.x, blockIdx.y, sh);
 }
 
 // The step's two decoder ops in one launch (both read B only): blocks [0, tiles) run the backward's tiles, the
@@ -273,7 +276,7 @@ template <typename E, int MP> __global__ void __launch_bounds__(kNThr) k_narrow_
         narrow_in_tile<E, MP, true>(i, blockIdx.x, sh.in);
     } else {
         const int64_t k = (int64_t)blockIdx.x - tiles;
-        narrow_out_tile<E, false>(o, k % tiles, k / tiles, sh.out);
+        narrow_out_tile<E, false, kNThr>(o, k % tiles, k / tiles, sh.out);
     }
 }
 
@@ -442,8 +445,9 @@ template <typename E, bool DEC> cudaError_t narrow_in(const NarrowIn &a, const C
 }
 template <typename E, bool ENC> cudaError_t narrow_out(const NarrowOut &a, const Ctx &c)
 {
-    return launch_narrow(k_narrow_out<E, ENC>, dim3((unsigned)((a.T + kNT - 1) / kNT), (unsigned)((a.d + kNThr - 1) / kNThr)),
-                         1, a, c);
+    const dim3 grid((unsigned)((a.T + kNT - 1) / kNT), (unsigned)((a.d + kNThr - 1) / kNThr));
+    return a.d <= 64 ? launch_narrow(k_narrow_out<E, ENC, 64>, grid, 1, a, c)
+                     : launch_narrow(k_narrow_out<E, ENC, kNThr>, grid, 1, a, c);
 }
 template <typename E> cudaError_t narrow_wgrad(const NarrowWgrads &w, const Ctx &c)
 {
