@@ -98,11 +98,11 @@ def measured_peaks():
             "source": "fallback"}
 
 
-# The files that define the fused boundary kernels the bench workload runs (their device code):
-# the committed DRAM traffic is valid while these hash the same. Their launch rules are in tc.cu: a
-# change of a grid or a cluster size there needs a fresh capture too.
+# The files that define what the bench workload runs: the fused boundary kernels' device code, and
+# the routing and launch rules (which kernel takes a shape, its grid, its clusters). The committed
+# DRAM traffic is valid while these hash the same.
 BENCH_KERNEL_FILES = ("common.cuh", "tc_common.cuh", "tc_wgrad.cuh", "tc_enc_fwd.cuh", "tc_dec_fwd.cuh",
-                      "tc_dec_bwd.cuh", "tc_enc_bwd.cuh")
+                      "tc_dec_bwd.cuh", "tc_enc_bwd.cuh", "tc.cu", "tc.h", "internal.h", "resbm_abi.cu")
 
 
 def kernel_sources_sha():

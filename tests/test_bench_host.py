@@ -23,6 +23,22 @@ def test_traffic_is_read_for_the_sources_it_was_captured_on():
         assert bench.traffic_for(op, cfg) == j["ops"][cfg.name][op]["dram_bytes_per_launch"]
 
 
+def test_the_hash_covers_kernels_and_routes(tmp_path, monkeypatch):
+    """A changed byte in a kernel, a launch rule or a route makes the committed traffic stale."""
+    import shutil
+    csrc = os.path.join(ROOT, "paper_2604_11947_gb300", "csrc")
+    copy = tmp_path / "paper_2604_11947_gb300" / "csrc"
+    shutil.copytree(csrc, copy)
+    want = bench.kernel_sources_sha()
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    assert bench.kernel_sources_sha() == want
+    for name in ("tc_enc_bwd.cuh", "tc.cu", "resbm_abi.cu"):
+        text = (copy / name).read_text()
+        (copy / name).write_text(text + "\n")
+        assert bench.kernel_sources_sha() != want, name
+        (copy / name).write_text(text)
+
+
 def test_traffic_is_dropped_when_the_sources_change(monkeypatch):
     monkeypatch.setattr(bench, "kernel_sources_sha", lambda: "0" * 16)
     assert bench.traffic_for("enc_bwd", synth.CONFIGS["large_bf16"]) is None
