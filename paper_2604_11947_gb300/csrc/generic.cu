@@ -233,6 +233,8 @@ GenericWs carve(const resbm_desc &d, int op, void *base, size_t *bytes)
     case RESBM_OP_DECODE_BWD:
         g.Q = w.take<float>(T * d.m);
         g.dG = w.take<float>(T * d.m);
+        // (the narrow kernels leave the partials untouched; the sizes that callers are told, and what the call with
+        // fixed scratch refuses, stay)
         g.part1 = w.take<float>(S * d.m * d.d);
         g.part2 = w.take<float>(S * d.r * d.m);
         break;

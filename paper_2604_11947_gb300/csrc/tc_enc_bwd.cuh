@@ -44,9 +44,8 @@ template <int M_> struct EncBwdCfg {
     static constexpr int NW = M_ <= 16 ? 4 : 2;                  // We1 slice ring depth
     static constexpr int CLMAX = 4;                              // CTAs per cluster (weight-gradient exchange)
     static constexpr int CL_MIN_TOKENS = 256;                 // clusters only from this many tokens per CTA
-    static constexpr int NWB = CLMAX > 1 ? 3 : 2;                // dWe1 accumulators in TMEM
+    static constexpr int NWB = 3;                                // dWe1 accumulators in TMEM
     static constexpr int NDA = NT;                               // dA TMEM regions (a ring)
-    static constexpr bool DPLO = true;                           // dP kept as bf16 hi + lo for dF
     static constexpr uint32_t RB = M_ * 2;                       // row bytes (= swizzle) of r / m wide tiles
     static constexpr uint32_t F_STAGE = 128 * 128 * 2;
     static constexpr uint32_t STG_BOX = 32 * 64 * 2;             // dF staging: 32 rows x 64 columns, two per warp
@@ -57,8 +56,8 @@ template <int M_> struct EncBwdCfg {
     static constexpr uint32_t OFF_STG = OFF_F + NSF * F_STAGE;
     static constexpr uint32_t OFF_W = OFF_STG + 8 * STG_BOX;
     static constexpr uint32_t OFF_DP = OFF_W + NW * W_STAGE;     // dP (hi) tiles [token][m]
-    static constexpr uint32_t OFF_DPLO = OFF_DP + NT * TILE;     // dP lo tiles (if DPLO)
-    static constexpr uint32_t OFF_WE2 = OFF_DPLO + (DPLO ? NT * TILE : 0);  // We2 [m][r], K-major
+    static constexpr uint32_t OFF_DPLO = OFF_DP + NT * TILE;     // dP lo tiles (dF takes dP as bf16 hi + lo)
+    static constexpr uint32_t OFF_WE2 = OFF_DPLO + NT * TILE;    // We2 [m][r], K-major
     static constexpr uint32_t OFF_RX = OFF_WE2 + WE2_BYTES;      // weight-gradient receive buffer
     static constexpr uint32_t SMEM_BYTES = OFF_RX + wgrad_rx_bytes<M_>(CLMAX) + 1024;
     // phase-0 scratch in F-ring slots 1 and 2
@@ -113,7 +112,7 @@ __global__ void __launch_bounds__(192, 1)
         if (threadIdx.x == 0) flag_error(kErrPlan);
         ngroups = 0;
     }
-    WgradXchg<C::M, C::CLMAX> xg{C::CLMAX > 1 ? cluster_size() : 1u, cluster_rank(), cluster_index(),
+    WgradXchg<C::M, C::CLMAX> xg{cluster_size(), cluster_rank(), cluster_index(),
                                  smem_u32(smem + C::OFF_RX), smem_u32(&rx_full), smem_u32(&rx_free[0]), 0};
 
     if (threadIdx.x == 0) {
@@ -151,7 +150,7 @@ __global__ void __launch_bounds__(192, 1)
     // CTAs may still run: only what follows touches global memory.
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_sh), C::TMEM_COLS);
     __syncthreads();
-    if (C::CLMAX > 1 && xg.cl > 1) cluster_sync();   // every CTA's barriers are initialized before any exchange
+    if (xg.cl > 1) cluster_sync();   // every CTA's barriers are initialized before any exchange
     griddep_wait();               // the previous kernel of the stream has completed
     griddep_launch_dependents();  // the next one may be scheduled on SMs as they free up
     if (warp >= 2) {  // We2 (m x r) as a swizzled K-major operand
@@ -324,10 +323,8 @@ __global__ void __launch_bounds__(192, 1)
                         // dF = dP . We1_chunk^T (K = m in steps of 16 = 32 bytes of a swizzled row)
 #pragma unroll
                         for (int k = 0; k < C::M / 16; ++k) mma_bf16(d_df, pk + 2 * k, wd + 2 * k, id_df, k > 0);
-                        if (C::DPLO) {
 #pragma unroll
-                            for (int k = 0; k < C::M / 16; ++k) mma_bf16(d_df, pk + LO16 + 2 * k, wd + 2 * k, id_df, true);
-                        }
+                        for (int k = 0; k < C::M / 16; ++k) mma_bf16(d_df, pk + LO16 + 2 * k, wd + 2 * k, id_df, true);
                         mma_commit(smem_u32(&df_full[ad_buf]));
                         // dWe1^T_chunk += F^T . dP  (K = the tile's tokens in steps of 16)
                         if (valid == 128) {
@@ -369,7 +366,6 @@ __global__ void __launch_bounds__(192, 1)
                 const int64_t tok = start + 128 * (int64_t)i + row;
                 if (tok < end) {
                     prefetch_l2(a.P + tok * C::M);
-                    if (C::M * 4 > 128) prefetch_l2(a.P + tok * C::M + 32);
                     if (a.dX) prefetch_l2(a.dX + tok * a.d);
                 }
             }
@@ -411,7 +407,7 @@ __global__ void __launch_bounds__(192, 1)
                     av[jj] = active ? av[jj] : 0.0f;
                 }
                 store_bf16_swz_row<C::M>(smem + C::OFF_DP + (i - tb) * C::TILE, row, da);
-                if (C::DPLO) store_bf16_swz_row<C::M>(smem + C::OFF_DPLO + (i - tb) * C::TILE, row, pv);
+                store_bf16_swz_row<C::M>(smem + C::OFF_DPLO + (i - tb) * C::TILE, row, pv);
                 store_bf16_swz_row<C::M>(smem + C::OFF_A + (i - tb) * C::TILE, row, av);
                 // identity path: dX[:, :r] += dB
                 if (active && a.dX) {
@@ -550,7 +546,7 @@ __global__ void __launch_bounds__(192, 1)
         tc_fence_after();
         tmem_dealloc(tmem, C::TMEM_COLS);
     }
-    if (C::CLMAX > 1 && xg.cl > 1) cluster_sync();   // no peer addresses this CTA's shared memory any more
+    if (xg.cl > 1) cluster_sync();   // no peer addresses this CTA's shared memory any more
 }
 
 }  // namespace tc

@@ -338,7 +338,7 @@ def resbm_newton_schulz(G, steps, X, ws, stream=None):
 
 
 def resbm_effective_rank(W, out, ws, stream=None):
-    """out (device float64, 4): sigma_max^2, ||W||_F^2, r_eff, power iterations taken."""
+    """out (device float64, 4): sigma_max^2, ||W||_F^2, r_eff, the iterations taken (products with the Gram matrix)."""
     rows, cols = W.shape
     _check("resbm_effective_rank", load().resbm_effective_rank(rows, cols, _p(W), _p(out), _p(ws), _nbytes(ws),
                                                                _stream(stream)))
