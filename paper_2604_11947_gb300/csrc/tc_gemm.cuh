@@ -433,7 +433,6 @@ __global__ void __launch_bounds__(320, 1)
     static_assert(!(BM2 && (ALO || PAIR)), "256-row units without hi + lo A or pairs");
     static_assert(!(TS && (ENCP || BM2)), "TMA-store epilogue: plain 128-row units or pairs");
     static_assert(!PIECES || (BMN && TS == 0 && !ENCP), "sums in pieces: the weight gradients on single CTAs");
-    const bool two = HALVES && (g.kc + 63) / 64 > g.pc;   // (HALVES: one split, so g.kc is K)
     constexpr int MH = BM2 ? 2 : 1;   // 128-row halves per unit (g.nm counts units of 128 * MH rows)
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -691,6 +690,7 @@ __global__ void __launch_bounds__(320, 1)
                 mbar_arrive(smem_u32(&acc_empty[ab]));
             }
         };
+        bool two = false;   // HALVES: the unit has a second half (a split product's last split can be too short for one)
         // 32 columns of the accumulator `ab` from column c (warp-collective): the loads, and their end (HALVES: w, the
         // second half's)
         auto acc_ld32 = [&](uint32_t ab, int c, float (&v)[32], float (&w)[32]) {
@@ -712,6 +712,10 @@ __global__ void __launch_bounds__(320, 1)
             int mb, nb, ks;
             unit_of(u, mb, nb, ks);
             const uint32_t ab = BM2 ? 0u : (ti & 1);
+            if (HALVES) {
+                int64_t k0;
+                two = k_steps(ks, k0) > g.pc;
+            }
             if (ENCP) {   // this half's rows of We1 (zeros past the last column), while the products run
                 constexpr int HC = BN / 2;
                 uint8_t *w = smem + C::OFF_WE1 + half * C::WE1_HALF;

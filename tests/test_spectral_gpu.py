@@ -120,11 +120,12 @@ def test_newton_schulz_extreme_scales(scale):
     assert np.isfinite(got).all() and np.linalg.norm(got - want) <= NS_FRO_TOL * np.linalg.norm(want) + 1e-30
 
 
-@pytest.mark.parametrize("shape", [(8, 8), (8, 4096), (40, 4096), (264, 1000), (512, 520), (600, 520), (1032, 1024),
-                                   (2048, 1536)])
+@pytest.mark.parametrize("shape", [(8, 8), (8, 4096), (40, 4096), (40, 4200), (64, 2312), (264, 1000), (512, 520),
+                                   (600, 520), (1032, 1024), (2048, 1536)])
 def test_effective_rank_lanczos_edges(shape):
-    """Fewer columns than a cycle's vectors, CTAs without rows, both sides of the line between the two
-    kernels (512), the Gram matrix too large for shared memory; bounds as in test_effective_rank_matches_oracle."""
+    """Fewer columns than a cycle's vectors, a Gram product whose last split is shorter than half of the others,
+    CTAs without rows, both sides of the line between the two kernels (512), the Gram matrix too large for shared
+    memory; bounds as in test_effective_rank_matches_oracle."""
     W = torch.from_numpy(synth.matrix(*shape, seed=sum(shape)) / np.sqrt(shape[0])).to("cuda").to(torch.bfloat16)
     Wh = W.double().cpu().numpy()
     lam, fro2, reff, iters = _reff(W)
