@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(320, 1)
         const int row = q * 32 + lane;
         const int et = threadIdx.x - 64;    // 0..255
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        const bool short_rows = a.d <= 1024;
+        const bool short_rows = NORM == 0 && a.d <= 1024;
         uint32_t acc_it = 0, store_it = 0;
         uint8_t *const boxes = smem + C::OFF_STG + (warp - 2) * C::WBOX * C::BOX;   // this warp's
         bool ok = true;
@@ -349,7 +349,8 @@ __global__ void __launch_bounds__(320, 1)
             // In short rows the warps that write no G go straight on to the tile's last chunk (T = 65536, d = 1024,
             // m = 32 26.5 -> 25.2 us; d = 512 16.7 -> 15.6). In long ones, where that chunk is few of many, keeping the
             // eight together is the faster way (d = 4096 84.9 against 86.6, m = 16, d = 2048 41.8 against 43.8).
-            if (half == 0 || !short_rows) named_barrier(1, short_rows ? C::EPI / 2 : C::EPI);
+            if (!short_rows) named_barrier(1, C::EPI);
+            else if (half == 0) named_barrier(1, C::EPI / 2);
             if (et == 0) mbar_arrive(smem_u32(&g_full[k % C::NGB]));
         };
         auto valid_of = [&](int64_t tile) -> int {
