@@ -31,7 +31,9 @@ constexpr int kNCl = 8;        // CTAs per cluster (k_narrow_wgrad)
 // The wide kernels (generic.cu) take any m and r; these hold a row of each in one warp's width. A step's
 // time, wide -> narrow, fp32: T = 512, d = 256, r = m = 2: 371 -> 16 us; T = 2048, d = 1024, r = m = 8:
 // 892 -> 52 us, r = m = 32: 990 -> 131 us; T = 16384, d = 2048, r = m = 16: 2.15 -> 0.64 ms; T = 65536,
-// d = 64, r = m = 32: 1.77 -> 0.95 ms; T = 32768, d = 4096, r = m = 32: 5.8 -> 4.0 ms. bf16 alike.
+// d = 64, r = m = 32: 1.77 -> 0.95 ms; T = 32768, d = 4096, r = m = 32: 5.8 -> 4.0 ms. bf16 alike. Of the ops alone
+// only the forward ones at r = m = 32 and d <= 64 over many tokens are the wide kernels' (T = 65536, d = 64 encoder
+// forward 45 -> 50 us, decoder forward 33.5 -> 36.3); the step's outputs are the ops', so they stay on one path.
 inline bool narrow_ok(const resbm_desc &d) { return d.m <= kNW && d.r <= kNW; }
 
 // element (t, j) of a rows x cols tile at src (row pitch ld) -> dst[t * 33 + j], zeros past `rows`
@@ -443,6 +445,8 @@ template <typename E, bool DEC> cudaError_t narrow_in(const NarrowIn &a, const C
            : a.m <= 16 ? launch_narrow(k_narrow_in<E, 16, DEC>, grid, 1, a, c)
                        : launch_narrow(k_narrow_in<E, 32, DEC>, grid, 1, a, c);
 }
+// (rows of up to 64: fp32 m = 32 decoder forward T = 16384, d = 64 18.1 us with 256 columns a block, 12.4 with 64;
+// 33 columns 17.8 and 12.3; T = 100 3.8 and 3.2. Of 65 to 255 columns a block of 256 leaves fewer threads idle)
 template <typename E, bool ENC> cudaError_t narrow_out(const NarrowOut &a, const Ctx &c)
 {
     const dim3 grid((unsigned)((a.T + kNT - 1) / kNT), (unsigned)((a.d + kNThr - 1) / kNThr));
