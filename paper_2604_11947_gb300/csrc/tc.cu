@@ -243,21 +243,23 @@ cudaError_t launch_dec_fwd(const resbm_desc &d, const void *B, const void *Wd1, 
     return e;
 }
 
-template <int M>
-cudaError_t launch_enc_fwd(const resbm_desc &d, const void *X, const void *F, const void *We1, const void *We2,
-                           void *B, float *P, const Ctx &c)
+template <int M, bool REST>
+cudaError_t launch_enc_fwd_t(const resbm_desc &d, const void *X, const void *F, const void *We1, const void *We2,
+                             void *B, float *P, const Ctx &c)
 {
     using Cfg = tc::EncFwdCfg<M>;
     const CUtensorMapSwizzle wswz = Cfg::WSW == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
                                     : Cfg::WSW == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                                                      : CU_TENSOR_MAP_SWIZZLE_32B;
-    CUtensorMap m_f128, m_frest, m_we1;
-    if (!make_map(&m_f128, F, d.d, d.T, d.d * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m_frest, F, d.d, d.T, d.d * 2, 64, d.T % 128 ? (uint32_t)(d.T % 128) : 128u, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m_we1, We1, d.m, d.d, d.m * 2, Cfg::WSW / 2, 64, wswz))
-        return cudaErrorInvalidValue;
+    tc::EncFwdMaps<REST> m;
+    bool ok = make_map(&m.f128, F, d.d, d.T, d.d * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
+              make_map(&m.we1, We1, d.m, d.d, d.m * 2, Cfg::WSW / 2, 64, wswz);
+    if constexpr (REST)
+        ok = ok && make_map(&m.frest, F, d.d, d.T, d.d * 2, 64, (uint32_t)(d.T % 128), CU_TENSOR_MAP_SWIZZLE_128B);
+    if (!ok) return cudaErrorInvalidValue;
+    auto kernel = tc::k_enc_fwd<M, REST>;
     static std::atomic<uint8_t> smem_set[kMaxDev];
-    cudaError_t e = ensure_smem(tc::k_enc_fwd<M>, Cfg::SMEM_BYTES, c.device, smem_set);
+    cudaError_t e = ensure_smem(kernel, Cfg::SMEM_BYTES, c.device, smem_set);
     if (e != cudaSuccess) return e;
     tc::EncFwdArgs a{static_cast<const __nv_bfloat16 *>(X), static_cast<const __nv_bfloat16 *>(We2),
                      static_cast<__nv_bfloat16 *>(B), P, d.T, d.d, d.act};
@@ -274,15 +276,20 @@ cudaError_t launch_enc_fwd(const resbm_desc &d, const void *X, const void *F, co
     if (forced != 1 && (forced != 0 || tiles > c.sm_count)) {
         static std::atomic<int> fit[kMaxDev][2];
         int64_t pairs = tiles < c.sm_count / 2 ? (tiles < 1 ? 1 : tiles) : c.sm_count / 2;
-        if (pairs >= 1 && coresident_clusters(tc::k_enc_fwd<M>, 2, Cfg::THREADS, Cfg::SMEM_BYTES, c.device, fit) >= pairs) {
+        if (pairs >= 1 && coresident_clusters(kernel, 2, Cfg::THREADS, Cfg::SMEM_BYTES, c.device, fit) >= pairs) {
             cl = 2;
             grid = 2 * pairs;
         }
     }
-    e = launch_clustered(tc::k_enc_fwd<M>, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, cl, c.stream, m_f128, m_frest,
-                         m_we1, a);
+    e = launch_clustered(kernel, (unsigned)grid, Cfg::THREADS, Cfg::SMEM_BYTES, cl, c.stream, m, a);
     count_launches(1);
     return e;
+}
+template <int M>
+cudaError_t launch_enc_fwd(const resbm_desc &d, const void *X, const void *F, const void *We1, const void *We2,
+                           void *B, float *P, const Ctx &c)
+{
+    return d.T % 128 ? launch_enc_fwd_t<M, true>(d, X, F, We1, We2, B, P, c) : launch_enc_fwd_t<M, false>(d, X, F, We1, We2, B, P, c);
 }
 
 // Scratch layout of the backward kernels: the d x m weight gradient has one fp32 slot per
